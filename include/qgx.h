@@ -260,11 +260,10 @@ enum { QGX_SPLIT_AUTO = 0, QGX_SPLIT_NEVER = 1, QGX_SPLIT_ALWAYS = 2, QGX_SPLIT_
 qgx_status qgx_set_decode_split(qgx_ctx *ctx, int mode);
 /* Which kernel the encode pass of the fused calls uses (no counterpart in the paper; the streams are the same bit
  * for bit).  QGX_ENCODE_REGISTERS: one CTA per bucket, the bucket held in registers between the norm and the
- * rounding.  QGX_ENCODE_STAGED: whole buckets of 1024, 2048, 4096, 8192 or 16384 coordinates of 16-byte aligned
- * vectors whose rows lie a multiple of 32 floats apart are staged in shared memory by bulk tensor copies, three
- * buffers deep, and packed 32 coordinates per lane; what does not qualify (other bucket sizes, a short last
- * bucket) still goes through the first kernel.  QGX_ENCODE_AUTO (the default) takes the kernel that measured
- * faster on B200: the first. */
+ * rounding.  QGX_ENCODE_STAGED: buckets of 1024, 2048, 4096, 8192 or 16384 coordinates (whatever the alignment and the
+ * length of the vectors) are staged in shared memory by asynchronous copies and packed 32 coordinates per lane by warps
+ * that do not wait for one another's buckets; other bucket sizes still go through the first kernel.  QGX_ENCODE_AUTO
+ * (the default) takes the kernel that measured faster on B200. */
 enum { QGX_ENCODE_AUTO = 0, QGX_ENCODE_REGISTERS = 1, QGX_ENCODE_STAGED = 2 };
 qgx_status qgx_set_encode_path(qgx_ctx *ctx, int mode);
 /* The receiving side alone (Algorithm 1: decode, aggregate): decodes the streams that the last qgx_exchange with

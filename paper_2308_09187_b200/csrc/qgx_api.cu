@@ -96,6 +96,24 @@ void make_round_table(const float* lev, int nlev, RoundTable* out) {
   }
   margin16 = (margin16 + 2.0) * 1.01;
   bool usable = std::isfinite(margin) && margin < S / 4.0 && std::isfinite(margin16) && margin16 < S / 4.0;
+  // the fixed-point variant: units of 2^-16 of an interval, results in [2^23, 2^24).  What it can be off by, e, either way: u2
+  // against the correctly rounded quotient, b, the knot, db and the difference u2 - knot (at most 12 roundings of relative
+  // size 2^-24 of (1.25 l_{tau+1} + 2^-16) / width -- a bin that a knot divides reaches at most an eighth past it), the
+  // rounding of afix, two roundings to whole numbers, the exact routine's own.  The dropped variate bits add up to one unit
+  // on one side, so with a bias of e the safe outcomes are those at least 2 e + 1 above a multiple of 2^16.
+  double e_fix = 0.0;
+  for (int t = 0; t <= nlev - 2; ++t) {
+    const double wmin = std::min(width[t], t + 1 <= nlev - 2 ? width[t + 1] : width[t]);
+    const double exact = 8388608.0 + 65536.0 * (t + 1) - 65536.0 / width[t] * ((double)lev[t] + c0);
+    const double ulp = (double)std::nextafter(std::fabs((float)exact) + 64.0f, INFINITY) - ((double)std::fabs((float)exact) + 64.0);
+    e_fix = std::max(e_fix, 12.0 * 65536.0 * 0x1p-24 * (1.25 * (double)lev[t + 1] + c0) / wmin + std::max(ulp, 1.0) + 1.5);
+  }
+  const bool fix_ok = std::isfinite(e_fix) && e_fix < 4096.0;
+  const double bias = fix_ok ? std::ceil(e_fix) : 0.0;
+  for (int t = 0; t <= nlev - 2; ++t)
+    out->afix[t] = (float)(8388608.0 + 65536.0 * (t + 1) + bias - 65536.0 / width[t] * ((double)lev[t] + c0));
+  out->fix_scale = (float)(65536.0 / S);
+  out->thrfix = fix_ok ? (uint32_t)(2.0 * bias) + 2u : 65536u;
   // the coarsest bins that still hold at most one level each (coarser bins are stored in more copies: see kKeyShiftMin)
   int shift = -1;
   for (int sh = kKeyShiftMax; sh >= kKeyShiftMin && usable && shift < 0; --sh) {
@@ -107,7 +125,13 @@ void make_round_table(const float* lev, int nlev, RoundTable* out) {
       std::memcpy(&lo, &lo_bits, 4);
       std::memcpy(&hi, &hi_bits, 4);
       int inside = 0;
-      for (int j = 1; j <= nlev - 2; ++j) inside += (out->knot[j] > lo && out->knot[j] <= hi) ? 1 : 0;
+      for (int j = 1; j <= nlev - 2; ++j) {
+        if (!(out->knot[j] > lo && out->knot[j] <= hi)) continue;
+        ++inside;
+        // the lower piece is evaluated up to the bin's end before the slope change past the level is added: keep that
+        // value small enough for the fixed-point map
+        if (j + ((double)hi - (double)out->knot[j]) / width[j - 1] > 96.0) ok = false;
+      }
       if (inside > 1) ok = false;
     }
     if (ok) shift = sh;
@@ -115,6 +139,7 @@ void make_round_table(const float* lev, int nlev, RoundTable* out) {
   if (shift < 0) usable = false;
   out->key_shift = shift < 0 ? kKeyShiftMin : shift;
   out->usable = usable ? 1 : 0;
+  if (!usable) out->thrfix = 65536u;
   out->thr = usable ? (float)(S / 2.0 - margin) : -1.0f;
   out->neg_qscale = (float)(-S / 8388608.0);
   out->thr16 = usable ? (float)(S / 2.0 - margin16) : -1.0f;

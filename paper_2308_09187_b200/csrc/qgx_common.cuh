@@ -224,10 +224,18 @@ struct RoundTable {
   float a16[QGX_MAX_LEVELS];             // S tau - b (l_tau + 2^-16) + S / 2 - S 2^-17 + 2^23 S 2^-16
   float thr16;                           // S / 2 - (margin + what the dropped variate bits can move)
   float neg_qscale16;                    // -S / 2^16
+  // and in fixed point, 2^-16 of an interval per unit, for the pipelined encoder: 2^23 + 2^16 (F(u) + 1) + bias comes out of
+  // the multiply-adds as a whole number in the float's mantissa; less the variate's leading 16 bits, bits 16..20 are the
+  // level and bits 0..15 the distance to the point below which it would be one lower
+  float afix[QGX_MAX_LEVELS];
+  float fix_scale;                       // 2^16 / S: turns b and db into the fixed-point map's slopes (a power of two)
+  uint32_t thrfix;                       // distances below this go to the exact routine (2^16: all of them)
 };
 
-// one entry per bin and copy: {a (or a16), b, knot, db} of the interval of the bin's lowest value
-__device__ __forceinline__ void fill_bin_table(float4* bin, const RoundTable& rt, bool octet_encoder = false) {
+// one entry per bin and copy: {a (or a16, afix), b, knot, db} of the interval of the bin's lowest value
+enum class BinKind { kQuad, kOctet, kFixed };
+__device__ __forceinline__ void fill_bin_table(float4* bin, const RoundTable& rt, BinKind kind = BinKind::kQuad) {
+  const float scale = kind == BinKind::kFixed ? rt.fix_scale : 1.0f;
   const int rep_log = rt.key_shift - kKeyShiftMin;
   const int nbins = (int)((kKeyTop - kKeyBase) >> rt.key_shift) + 1;
   for (int i = threadIdx.x; i < (nbins << rep_log); i += blockDim.x) {
@@ -237,7 +245,8 @@ __device__ __forceinline__ void fill_bin_table(float4* bin, const RoundTable& rt
     int t0 = 0;
     for (int j = 1; j <= rt.nlev - 2; ++j) t0 = (rt.knot[j] <= lo) ? j : t0;
     const bool straddle = (t0 + 1 <= rt.nlev - 2) && (rt.knot[t0 + 1] <= hi);
-    bin[i] = make_float4(octet_encoder ? rt.a16[t0] : rt.a[t0], rt.b[t0], straddle ? rt.knot[t0 + 1] : 4.0f, straddle ? rt.db[t0 + 1] : 0.0f);
+    const float icpt = kind == BinKind::kFixed ? rt.afix[t0] : (kind == BinKind::kOctet ? rt.a16[t0] : rt.a[t0]);
+    bin[i] = make_float4(icpt, rt.b[t0] * scale, straddle ? rt.knot[t0 + 1] : 4.0f, straddle ? rt.db[t0 + 1] * scale : 0.0f);
   }
 }
 

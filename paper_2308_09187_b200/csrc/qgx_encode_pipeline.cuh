@@ -1,0 +1,772 @@
+// The fused quantize + encode pass for buckets of 1024, 2048, 4096, 8192 or 16384 coordinates: one CTA per SM whose
+// warps only meet at mbarriers, so no warp ever waits for the whole CTA.
+//   16 quantizers  take chunks of 1024 coordinates round-robin, 32 consecutive coordinates per lane: asynchronous copies
+//                  into two private stages (one comes in while the other is worked on), the operator's value added,
+//                  norms (fp64), variates, rounding, codewords, every lane's bits as a stream of its own in shared
+//                  memory.  No atomics per coordinate, one wait per bucket for the other quantizers' partial norms;
+//   1 dispatcher   draws the work units;
+//   2 scanners     turn the chunks' bit counts into places: offsets inside the buckets, the buckets' places in the
+//                  worker's stream (a look-back over the work units before this one);
+//   5 copiers      shift the lanes' bits to where they belong, and write the headers.
+// What bounds it: instruction issue and latency.  A quantizer's core alone (data already in shared memory, 16 warps) takes
+// 0.40 cycles per coordinate and SM: 33 instructions at 65 % issue, with the ALU, the integer multiplier (the generator's
+// wide products run at a quarter of the rate) and the shared-memory pipe each 55-60 % busy.  With copies, norms and
+// placing it is 65 instructions at about 57 %.  Shared memory (two stages and two to four images per quantizer) sets the
+// number of warps.  Measured per 2^27 coordinates against the bucket-in-registers kernel, whose CTAs load, norm, round
+// and write one after the other with three CTA barriers per bucket: buckets of 16384 395 us (433), 8192 392 us (508),
+// 4096 390 us (480), 1024 379 us (883); rows that are not 16-byte aligned, 16 x 10^6 coordinates, 69 us (234), since
+// there the rounding map serves, too, and a row costs four-byte instead of 16-byte copies.
+// Tried: loaders as warps of their own (they share the issue slots of one warp each and fall behind), and quantizers that
+// copy their own bits out (fewer warps to hide latency behind): 5-30 % slower.
+//
+// Included by qgx_exchange.cu (uses its status words, look-back and EncodeArgs).
+#pragma once
+
+namespace qgx {
+
+constexpr int kChunk = 1024;                             // coordinates per chunk: 32 lanes x 32
+constexpr int kLaneCoords = 32;                          // coordinates per lane: one 128-byte line of the stage
+constexpr int kQuantizers = 16, kDispatchers = 1, kScanners = 2, kCopiers = 5;
+constexpr int kPipeThreads = 32 * (kQuantizers + kDispatchers + kScanners + kCopiers);
+constexpr unsigned kUnitRing = 64;                       // unit descriptors: more than are ever under way
+constexpr int kMaxImageTurns = 4, kMaxImageUnits = kMaxImageTurns * kQuantizers / 4;
+constexpr unsigned kTurnRing = 4;
+
+// a unit of work ...
+struct __align__(16) PipeUnit {
+  unsigned long long lo;                                 // its first coordinate in the worker's vector
+  const float* src;                                      // where that is in memory (the first source)
+  uint32_t k;
+  int len;                                               // coordinates, 0: there are no more units
+};
+// ... the norm of a bucket
+struct __align__(16) PipeNorm {
+  float norm;
+  float rn;                                              // RN(1 / norm), 0 where every coordinate goes to the exact routine
+  uint32_t thr;                                          // fractions below this go to the exact routine
+  int live;                                              // 0: every coordinate is level 0
+};
+// what the scanners hand on per chunk
+struct __align__(16) PipePlace {
+  unsigned long long word;                               // of its bucket's first word in the worker's stream
+  uint32_t bit;                                          // of the chunk's first bit in the bucket
+  uint32_t nbits;                                        // the bucket's bits; 0: do not write
+};
+
+__host__ __device__ constexpr int pipe_lane_stride(int maxlen) { return (maxlen + 1) | 1; }   // words per lane, odd: no bank conflicts
+struct PipeSmem {                                        // byte offsets into the dynamic shared memory
+  uint32_t stage, image, bin, pair, lut, lev, cnt, tot, inorm, last, unit, norm, place, bars, part, posted, bytes;
+};
+// turns: how many of a quantizer's chunks may hold bits at a time (2, 3 or 4)
+__host__ __device__ constexpr PipeSmem pipe_smem(int nlev, int maxlen, int turns) {
+  const uint32_t images = (uint32_t)turns * kQuantizers;
+  PipeSmem s{};
+  s.stage = 0;
+  s.image = 2u * kQuantizers * kChunk * 4u;
+  s.bin = s.image + images * 32u * (uint32_t)pipe_lane_stride(maxlen) * 4u;
+  s.pair = s.bin + (uint32_t)kBinEntries * 16u;
+  s.lut = s.pair + (uint32_t)(4 * nlev * nlev) * 4u;
+  s.lev = s.lut + 2u * QGX_MAX_LEVELS * 4u;
+  s.cnt = s.lev + QGX_MAX_LEVELS * 4u;
+  s.tot = s.cnt + 2u * images * 32u * 2u;
+  s.inorm = s.tot + images * 4u;
+  s.last = s.inorm + images * 4u;
+  s.unit = s.last + 2u * images * 4u;
+  s.norm = s.unit + kUnitRing * (uint32_t)sizeof(PipeUnit);
+  s.place = s.norm + 2u * kQuantizers * (uint32_t)sizeof(PipeNorm);
+  s.bars = s.place + images * (uint32_t)sizeof(PipePlace);
+  s.part = s.bars + (kUnitRing + 2u * kQuantizers + 3u * kMaxImageUnits + kTurnRing) * 8u;
+  s.posted = s.part + 2u * kQuantizers * 8u;
+  s.bytes = s.posted + 2u * kQuantizers * 4u;
+  return s;
+}
+constexpr size_t kPipeSmemMax = 226u * 1024u;
+static_assert(pipe_smem(QGX_MAX_LEVELS, QGX_MAX_CODE_LEN, 2).bytes <= kPipeSmemMax, "shared memory of one CTA");
+
+// What the host works out for a launch.  Everything here is read from the constant bank where it is used: kept in registers,
+// or derived in the kernel, it would push the quantizers' loop over its 80 registers.
+struct PipeShape {
+  PipeSmem smem;
+  int b_log, m_log, m;                                   // bucket = 1024 * m = 2^b_log
+  int unit, u_log;                                       // chunks per unit of work
+  unsigned per_turn;                                     // units that the quantizers work on side by side: 16 / unit
+  int image_turns;
+  uint32_t lane_words;                                   // words per lane of an image
+  int nlev;
+  uint32_t weights, neg4;                                // of the pair table: byte offsets of the two symbols; nlev in every byte
+  uint32_t bin_mask, bin_copy;                           // of the rounding table: see RoundFix; bytes of a bin's copies less 16
+  size_t units;                                          // per worker
+  size_t status_ld, status_first;                        // status words per worker, the first one used (the diagnostic leaves some unpublished)
+};
+// ---- mbarriers by 32-bit shared address ----
+__device__ __forceinline__ void bar_init(uint32_t bar, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint32_t bar) {
+  asm volatile("{ .reg .b64 st; mbarrier.arrive.shared::cta.b64 st, [%0]; }" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void bar_arrive_n(uint32_t bar, unsigned n) {
+  asm volatile("{ .reg .b64 st; mbarrier.arrive.shared::cta.b64 st, [%0], %1; }" ::"r"(bar), "r"(n) : "memory");
+}
+// Waits for the phase of the given parity; called by whole warps.  False if the bounded wait ran out or another warp of
+// the CTA gave up (*quit, shared memory).  The warp is suspended between its looks (at most 20 us each): polls would take
+// issue slots from the warps that compute.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* quit) {
+  unsigned done = 0;
+  for (int i = 0; i < kSpinLimit; ++i) {
+    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(done) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
+    if (done) break;
+    if ((i & 15) == 15 && *quit) break;
+  }
+  return __all_sync(0xffffffffu, done != 0);
+}
+
+// 16 (4) bytes from global to shared memory without passing through registers; `bytes` of them are read, the rest is zero
+__device__ __forceinline__ void copy_async16(uint32_t dst, const float* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void copy_async4(uint32_t dst, const float* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// byte offset, inside a chunk, of 16-byte piece u (0..255): the pieces of a 128-byte line are permuted by the line number,
+// so that both a loader's lanes (consecutive pieces) and a quantizer's (the same piece of 8 consecutive lines) spread
+// over the banks
+__device__ __forceinline__ uint32_t piece_at(uint32_t u) { return ((u & ~7u) | ((u ^ (u >> 3)) & 7u)) << 4; }
+
+// ---- the generator, with what the blocks of a lane share worked out once ----
+// Counter words 2 and 3 (worker, exchange) and, but for carries, word 1 are the same for all blocks of a bucket: the second
+// product of round 1 and the first of round 2 do not depend on word 0.
+struct PhiloxShared {
+  uint32_t x0, a, b, c;
+};
+__device__ __forceinline__ PhiloxShared philox_shared(uint32_t c1, uint32_t k, uint32_t xid, const PhiloxKey& key) {
+  const uint64_t p1 = (uint64_t)0xCD9E8D57u * (uint64_t)k;
+  const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ key.k0[0];
+  const uint64_t p0 = (uint64_t)0xD2511F53u * (uint64_t)n0;
+  PhiloxShared s;
+  s.x0 = xid ^ key.k1[0];
+  s.a = (uint32_t)p1 ^ key.k0[1];
+  s.b = (uint32_t)(p0 >> 32) ^ key.k1[1];
+  s.c = (uint32_t)p0;
+  return s;
+}
+// both halves of a * b in one instruction (left to itself the compiler sometimes computes them apart)
+__device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t* hi, uint32_t* lo) {
+  asm("{ .reg .b64 p; mul.wide.u32 p, %2, %3; mov.b64 {%0, %1}, p; }" : "=r"(*lo), "=r"(*hi) : "r"(a), "r"(b));
+}
+// blocks c0 and c0 + 1
+__device__ __forceinline__ void philox_pair(uint32_t c0, const PhiloxShared& s, const PhiloxKey& key, uint32_t* w) {
+  uint32_t s0[2], s1[2], s2[2], s3[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    uint32_t hi, lo, hi1;
+    mul_wide(c0 + (uint32_t)j, 0xD2511F53u, &hi, &lo);
+    mul_wide(hi ^ s.x0, 0xCD9E8D57u, &hi1, &s1[j]);                    // after round 1: word 2
+    s0[j] = hi1 ^ s.a;                                                 // after round 2
+    s2[j] = s.b ^ lo;
+    s3[j] = s.c;
+  }
+#pragma unroll
+  for (int r = 2; r < 10; ++r) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      uint32_t hi0, lo0, hi1, lo1;
+      mul_wide(s0[j], 0xD2511F53u, &hi0, &lo0);
+      mul_wide(s2[j], 0xCD9E8D57u, &hi1, &lo1);
+      s0[j] = hi1 ^ s1[j] ^ key.k0[r];
+      s2[j] = hi0 ^ s3[j] ^ key.k1[r];
+      s1[j] = lo1;
+      s3[j] = lo0;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) { w[4 * j] = s0[j]; w[4 * j + 1] = s1[j]; w[4 * j + 2] = s2[j]; w[4 * j + 3] = s3[j]; }
+}
+
+// ---- rounding: the level map in fixed point (see RoundTable::afix) ----
+struct RoundFix {
+  float rn;
+  uint32_t thr;
+  uint32_t mask;                                         // clears the bits of pattern >> kBinAddrShift below a bin's copies
+  uint32_t base;                                         // shared address of this lane's copies, minus kBinAddrBase
+};
+// Fixed-point decision variable of one coordinate: bits 16..20 the level, bits 0..15 how far it is above the point where
+// the level would be one lower (in 2^-16 of an interval).
+__device__ __forceinline__ uint32_t round_fixed(float x, uint32_t w, const RoundFix& c) {
+  const float u2 = fmaf(fabsf(x), c.rn, kRoundShift);
+  const float4 e = lds_table128(((__float_as_uint(u2) >> kBinAddrShift) & c.mask) + c.base);
+  float z = fmaf(u2, e.y, e.x);
+  z = fmaf(__saturatef(__fsub_rn(u2, e.z)), e.w, z);                   // in [2^23, 2^24): the mantissa is a whole number
+  return __float_as_uint(z) - (w >> 16);
+}
+__device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+// Definition 1 for one coordinate in IEEE operations, given a level near the outcome (the interval is looked for from there);
+// r24 = the 24-bit variate.
+__device__ __forceinline__ uint32_t level_exact_near(float absv, float norm, uint32_t r24, int near_level, uint32_t lev_sa, int nlev) {
+  auto lev = [&](int j) { return __uint_as_float(lds_table32(lev_sa + 4u * (uint32_t)j)); };
+  float u = (norm > 0.0f) ? __fdiv_rn(absv, norm) : 0.0f;
+  u = fminf(u, 1.0f);
+  int tau = min(max(near_level - 1, 0), nlev - 2);
+  while (tau < nlev - 2 && lev(tau + 1) <= u) ++tau;
+  while (tau > 0 && lev(tau) > u) --tau;
+  const float lo = lev(tau), hi = lev(tau + 1);
+  const float xi = __fdiv_rn(__fsub_rn(u, lo), __fsub_rn(hi, lo));
+  const float r = __fmul_rn(__uint2float_rn(r24), 5.9604644775390625e-8f);        // exact
+  return (uint32_t)(tau + ((r < xi) ? 1 : 0));
+}
+
+// Stream bits of a lane as they are produced: a 64-bit window that new bits enter at the top (two funnel shifts, no masks);
+// the oldest 32 go to the lane's words in shared memory once they are there.
+struct LaneBits {
+  uint32_t lo, hi;
+  int pos;                                               // 64 - bits waiting in the window
+  uint32_t wa;                                           // shared address of the next word
+  __device__ __forceinline__ void open(uint32_t addr) { lo = hi = 0u; pos = 64; wa = addr; }
+  // the low n bits of e (n <= 26, the entry's upper 6 bits; fewer than 32 bits are waiting)
+  __device__ __forceinline__ void put(uint32_t e) {
+    const uint32_t n = e >> 26;
+    lo = __funnelshift_r(lo, hi, n);
+    hi = __funnelshift_r(hi, e, n);
+    pos -= (int)n;
+    if (pos <= 32) {
+      sts32(wa, __funnelshift_rc(lo, hi, (uint32_t)pos));
+      wa += 4u;
+      pos += 32;
+    }
+  }
+  // stores what is waiting; the bits put since open(addr)
+  __device__ __forceinline__ uint32_t close(uint32_t addr) {
+    if (pos < 64) sts32(wa, hi >> ((uint32_t)pos - 32u));
+    return 8u * (wa - addr) + (uint32_t)(64 - pos);
+  }
+};
+
+// Two octets (first, first + 1) of one lane's 32 coordinates (of the first `count` of them when MASKED): lx = the shared
+// address of its line, plus 16 times the line's permutation (piece p is at lx ^ 16 p), q0 the generator's counter of its
+// first quad.  The loop runs at the register limit: what only its rare branches need is fetched there.
+template <bool MASKED>
+__device__ __forceinline__ void quantize_line(int first, uint32_t lx, uint64_t q0, int count, const PipeNorm* norm, uint32_t k, uint32_t xid,
+                                              const PhiloxKey& key, const RoundFix& rc, const PipeShape& h, uint32_t sa, LaneBits& out) {
+  const PhiloxShared ps = philox_shared((uint32_t)(q0 >> 32), k, xid, key);
+#pragma unroll 1
+  for (int o = first; o < first + 2; ++o) {
+    if (MASKED && 8 * o >= count) break;
+    uint32_t w[8];
+    if (!MASKED) {
+      philox_pair((uint32_t)q0 + 2u * (uint32_t)o, ps, key, w);
+    } else {                                                           // also where the counter's low word wraps around
+      uint4 wa, wb;
+      philox4x32_10_x2(q0 + 2ull * (uint64_t)o, q0 + 2ull * (uint64_t)o + 1ull, k, xid, key, &wa, &wb);
+      w[0] = wa.x; w[1] = wa.y; w[2] = wa.z; w[3] = wa.w; w[4] = wb.x; w[5] = wb.y; w[6] = wb.z; w[7] = wb.w;
+    }
+    const float4 xa = lds128(lx ^ (32u * (uint32_t)o)), xb = lds128(lx ^ (32u * (uint32_t)o + 16u));
+    const float x[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+    uint32_t d[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) d[i] = round_fixed(x[i], w[i], rc);
+    uint32_t m = min_u16x2(prmt(d[0], d[1], 0x5410u), prmt(d[2], d[3], 0x5410u));
+    m = min_u16x2(min_u16x2(prmt(d[4], d[5], 0x5410u), prmt(d[6], d[7], 0x5410u)), m);
+    uint32_t lv[2];                                                    // the levels, one per byte
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      lv[q] = prmt(prmt(d[4 * q], d[4 * q + 1], 0x0062u), prmt(d[4 * q + 2], d[4 * q + 3], 0x0062u), 0x5410u) & 0x1f1f1f1fu;
+    if (min(m & 0xffffu, m >> 16) < rc.thr) {
+      // Some coordinate needs the exact routine (3 % of a warp's octets; every octet of a bucket without a usable norm).  In
+      // line, its inputs taken from their sources again, one coordinate at a time: a call, or anything kept for it, would
+      // cost the loop its registers.
+      const PipeNorm pn = *norm;
+      uint32_t todo = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) todo |= (d[i] & 0xffffu) < rc.thr ? 1u << i : 0u;
+      if (!pn.live) { lv[0] = lv[1] = 0u; todo = 0u; }
+#pragma unroll 1
+      while (todo) {
+        const uint32_t i = (uint32_t)__ffs((int)todo) - 1u;
+        todo &= todo - 1u;
+        const uint64_t ctr = q0 + 2ull * (uint64_t)o + (uint64_t)(i >> 2);
+        const uint4 wb = philox4x32_10((uint32_t)ctr, (uint32_t)(ctr >> 32), k, xid, key);
+        const uint32_t word = (i & 2u) ? ((i & 1u) ? wb.w : wb.z) : ((i & 1u) ? wb.y : wb.x);
+        const float xv = __uint_as_float(lds32((lx ^ (32u * (uint32_t)o + 16u * (i >> 2))) + 4u * (i & 3u)));
+        const uint32_t sh = 8u * (i & 3u), was = i < 4u ? lv[0] : lv[1];
+        const uint32_t fixed = level_exact_near(fabsf(xv), pn.norm, word >> 8, (int)((was >> sh) & 0x1fu), sa + h.smem.lev, h.nlev);
+        const uint32_t put = (was & ~(0xffu << sh)) | (fixed << sh);
+        if (i < 4u) lv[0] = put; else lv[1] = put;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const uint32_t s4 = prmt(prmt(__float_as_uint(x[4 * q]), __float_as_uint(x[4 * q + 1]), 0x00fbu),
+                               prmt(__float_as_uint(x[4 * q + 2]), __float_as_uint(x[4 * q + 3]), 0x00fbu), 0x5410u);
+      const uint32_t c4 = lv[q] + (s4 & h.neg4);                       // level, plus nlev for a negative coordinate
+      if (!MASKED) {
+        out.put(lds_table32(__dp2a_lo(h.weights, c4, sa + h.smem.pair)));
+        out.put(lds_table32(__dp2a_hi(h.weights, c4, sa + h.smem.pair)));
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t cc = (c4 >> (8 * i)) & 0xffu;
+          const uint32_t one = lds_table32(sa + h.smem.lut + 4u * (cc < (uint32_t)h.nlev ? cc : cc - (uint32_t)h.nlev + 32u));
+          if (8 * o + 4 * q + i < count) out.put((one & 0xffffu) | ((one >> 16) << 26));
+        }
+      }
+    }
+  }
+}
+
+// ---- the kernel ----------------------------------------------------------------------------------
+// The launch's work is cut into units of `h.unit` chunks of one worker: one bucket of 16384 coordinates, or several smaller
+// ones in a row (one look-back for all of them).  Tickets are drawn in the order unit-major, worker-minor by the
+// dispatcher, so within a CTA units n = 0, 1, 2, ... carry increasing tickets.  The smallest ticket of the device that has
+// no place yet belongs to a CTA that has placed -- and therefore copies, without waiting for anybody else -- everything
+// before it: the image it needs becomes free, its look-back finds only placed units, and every wait ends.
+// A barrier's parity tells a phase from the one before it, not from the one before that: whoever waits at a place of a
+// ring has seen the place's last phase complete, because it waits there every turn or because what it took last from the
+// ring implies it.
+template <int G>
+__global__ void __launch_bounds__(kPipeThreads, 1)
+k_encode_pipeline(const __grid_constant__ EncodeArgs a, const __grid_constant__ PipeShape h, const __grid_constant__ LevelTable lt, const __grid_constant__ CodeTable ct,
+                  const __grid_constant__ PhiloxKey key, const __grid_constant__ RoundTable rt) {
+  extern __shared__ __align__(1024) unsigned char s_pipe[];
+  __shared__ int s_quit;
+  const PipeSmem& L = h.smem;
+  const uint32_t sa = smem_addr(s_pipe);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b_log = h.b_log, m_log = h.m_log, m = h.m;                 // log2 of the bucket; chunks per bucket: 1, 2, 4, 8 or 16
+  const int U = h.unit, u_log = h.u_log;                               // chunks per unit: 4, 8 or 16, at least m
+  const unsigned per_turn = h.per_turn;                                // units that the quantizers work on side by side
+  const int NT = h.image_turns;
+  const uint32_t dealt = sa + L.bars, ready = dealt + 8u * kUnitRing, coded = ready + 8u * 2u * kQuantizers;
+  const uint32_t placed = coded + 8u * kMaxImageUnits, written = placed + 8u * kMaxImageUnits;
+  const uint32_t turned = written + 8u * kMaxImageUnits;
+  PipeUnit* s_unit = reinterpret_cast<PipeUnit*>(s_pipe + L.unit);
+  PipeNorm* s_norm = reinterpret_cast<PipeNorm*>(s_pipe + L.norm);
+  uint16_t* s_cnt = reinterpret_cast<uint16_t*>(s_pipe + L.cnt);
+  uint32_t* s_tot = reinterpret_cast<uint32_t*>(s_pipe + L.tot);
+  float* s_inorm = reinterpret_cast<float*>(s_pipe + L.inorm);
+  uint32_t* s_last = reinterpret_cast<uint32_t*>(s_pipe + L.last);
+  PipePlace* s_place = reinterpret_cast<PipePlace*>(s_pipe + L.place);
+  volatile double* s_part = reinterpret_cast<volatile double*>(s_pipe + L.part);
+  unsigned* s_posted = reinterpret_cast<unsigned*>(s_pipe + L.posted);
+  float* s_lev = reinterpret_cast<float*>(s_pipe + L.lev);
+  const uint32_t lane_words = h.lane_words;
+
+  {                                                                    // the tables of the configuration
+    const uint4* gb = reinterpret_cast<const uint4*>(a.tables->bin_fix);
+    uint4* sb = reinterpret_cast<uint4*>(s_pipe + L.bin);
+    for (int i = threadIdx.x; i < kBinEntries; i += kPipeThreads) sb[i] = __ldg(gb + i);
+    uint32_t* sp = reinterpret_cast<uint32_t*>(s_pipe + L.pair);
+    for (int i = threadIdx.x; i < 4 * lt.nlev * lt.nlev; i += kPipeThreads) sp[i] = __ldg(a.tables->pair_fix + i);
+    if (threadIdx.x < 2 * QGX_MAX_LEVELS) reinterpret_cast<uint32_t*>(s_pipe + L.lut)[threadIdx.x] = __ldg(a.tables->lut.e + threadIdx.x);
+    if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
+  }
+  if (threadIdx.x < kUnitRing) bar_init(dealt + 8u * threadIdx.x, 1);
+  if (threadIdx.x < 2 * kQuantizers) { bar_init(ready + 8u * threadIdx.x, 1); s_posted[threadIdx.x] = 0u; }
+  if (threadIdx.x < kMaxImageUnits) {
+    bar_init(coded + 8u * threadIdx.x, (unsigned)U);
+    bar_init(placed + 8u * threadIdx.x, 1);
+    bar_init(written + 8u * threadIdx.x, kCopiers);
+  }
+  if (threadIdx.x == 0) s_quit = 0;
+  if (threadIdx.x < kTurnRing) bar_init(turned + 8u * threadIdx.x, kQuantizers);
+  __syncthreads();
+  volatile int* quit = &s_quit;
+  // a wait that ran out: everybody gives up, the launch ends and reports it
+  auto give_up = [&]() {
+    if (lane == 0) {
+      if (!*quit) latch_error(a.st, QGX_ERR_TIMEOUT);
+      *quit = 1;
+    }
+  };
+
+  if (warp < kQuantizers) {
+    // ================================ quantizers ================================
+    const bool two = a.src.v && a.src.a;
+    // copies and norms: a lane's pieces of a chunk are 32 j + lane, byte offsets 512 j + off[j & 1]
+    const uint32_t off0 = piece_at((uint32_t)lane), off1 = off0 ^ 64u;
+    RoundFix rc;
+    rc.mask = h.bin_mask;
+    rc.base = sa + L.bin - kBinAddrBase + (((uint32_t)lane << 4) & h.bin_copy);
+    // the copies of chunk c = 16 turn + warp; its length in *len (0: there are no more units)
+    auto issue = [&](unsigned c, int* len) -> bool {
+      const unsigned n = c >> u_log;
+      if (!bar_wait(dealt + 8u * (n & (kUnitRing - 1u)), (n / kUnitRing) & 1u, quit)) return false;
+      const PipeUnit pu = s_unit[n & (kUnitRing - 1u)];
+      *len = pu.len;
+      const int i = (int)(c & (unsigned)(U - 1));
+      const int left = pu.len - i * kChunk;                            // coordinates of the chunk, if fewer than 1024
+      if (left > 0) {
+        const uint32_t dst = sa + L.stage + (c & (2u * kQuantizers - 1u)) * (kChunk * 4u);
+        const float* from = pu.src + i * kChunk;
+        if (a.v_vec && left >= kChunk) {
+          const float* p = from + 4 * lane;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) copy_async16(dst + 512u * (uint32_t)q + ((q & 1) ? off1 : off0), p + 128 * q, 16);
+        } else if (a.v_vec) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            const int e = 4 * (32 * q + lane);
+            const int bytes = max(0, min(16, 4 * (left - e)));
+            copy_async16(dst + 512u * (uint32_t)q + ((q & 1) ? off1 : off0), bytes > 0 ? from + e : from, bytes);
+          }
+        } else {
+#pragma unroll 8
+          for (int q = 0; q < 32; ++q) {
+            const int e = 32 * q + lane;
+            copy_async4(dst + piece_at((uint32_t)(e >> 2)) + 4u * (uint32_t)(e & 3), e < left ? from + e : from, e < left ? 4 : 0);
+          }
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      return true;
+    };
+    // The copies of chunk c have landed: the operator's value added, the partial norm posted; whoever posts a bucket's last
+    // one forms the norm.
+    auto norm_of = [&](unsigned c) {
+      const unsigned n = c >> u_log, cs = c & (2u * kQuantizers - 1u);
+      const PipeUnit pu = s_unit[n & (kUnitRing - 1u)];
+      const int i = (int)(c & (unsigned)(U - 1)), left = pu.len - i * kChunk;
+      double part = 0.0;
+      const bool l2 = a.norm_type == QGX_NORM_L2;
+      if (left > 0) {
+        const uint32_t st = sa + L.stage + cs * (kChunk * 4u);
+        const float* pa = two ? a.src.a + (size_t)pu.lo + i * kChunk : nullptr;
+        const bool whole = a.a_vec && left >= kChunk;
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        float mx = 0.0f;
+        bool bad = false;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float4 av[4];
+          if (two) {
+            if (whole) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) av[q] = __ldg(reinterpret_cast<const float4*>(pa + 4 * lane) + 32 * (4 * h + q));
+            } else {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int e = 4 * (32 * (4 * h + q) + lane);
+                av[q] = make_float4(e + 0 < left ? pa[e + 0] : 0.f, e + 1 < left ? pa[e + 1] : 0.f, e + 2 < left ? pa[e + 2] : 0.f, e + 3 < left ? pa[e + 3] : 0.f);
+              }
+            }
+          }
+          if (h == 0) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            if (!a.v_vec) __syncwarp();                                // 4-byte copies: a piece comes from four lanes
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint32_t at = st + 512u * (uint32_t)(4 * h + q) + ((q & 1) ? off1 : off0);
+            float4 x = lds128(at);
+            if (two) {
+              x = dual_combine(av[q], x, a.src.mul);
+              asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w) : "memory");
+            }
+            if (l2) {
+              const double x0 = x.x, x1 = x.y, x2 = x.z, x3 = x.w;
+              acc[0] = fma(x0, x0, acc[0]); acc[1] = fma(x1, x1, acc[1]); acc[2] = fma(x2, x2, acc[2]); acc[3] = fma(x3, x3, acc[3]);
+            } else {
+              bad = bad || (x.x != x.x) || (x.y != x.y) || (x.z != x.z) || (x.w != x.w);
+              mx = fmaxf(mx, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
+            }
+          }
+        }
+        if (l2) {
+          part = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+        } else {
+          mx = warp_max(mx);
+          part = __any_sync(0xffffffffu, bad) ? (double)__int_as_float(0x7fc00000) : (double)mx;
+        }
+      }
+      const unsigned c0 = cs & ~(unsigned)(m - 1);                     // the bucket's first place in the stage
+      bool last = true;
+      if (m > 1) {
+        unsigned before = 0;
+        if (lane == 0) {
+          s_part[cs] = part;
+          __threadfence_block();
+          before = atomicAdd(s_posted + c0, 1u);
+          __threadfence_block();
+        }
+        last = __shfl_sync(0xffffffffu, before, 0) == (unsigned)(m - 1);
+      }
+      if (last) {
+        double x = part;
+        if (m > 1) {
+          x = lane < m ? s_part[c0 + (unsigned)lane] : 0.0;
+          for (int o = 1; o < m; o <<= 1) {
+            const double y = __shfl_xor_sync(0xffffffffu, x, o);
+            x = l2 ? x + y : ((x != x || y != y) ? (double)__int_as_float(0x7fc00000) : fmax(x, y));
+          }
+        }
+        if (lane == 0) {
+          const float norm = l2 ? (float)sqrt(x) : (float)x;
+          const bool finite = (norm - norm) == 0.0f, fast = rt.usable && norm > 7.9e-31f && norm < 1.2e30f;
+          PipeNorm pn;
+          pn.norm = norm;
+          pn.rn = fast ? __frcp_rn(norm) : 0.0f;
+          pn.thr = fast ? rt.thrfix : 0x10000u;
+          pn.live = finite && norm != 0.0f ? 1 : 0;
+          s_norm[c0] = pn;
+          s_posted[c0] = 0u;
+          const int blo = (i & ~(m - 1)) * kChunk;                     // the bucket's first coordinate in the unit
+          if (blo < pu.len) {
+            a.norms[(size_t)pu.k * a.nb + (((size_t)pu.lo + (size_t)blo) >> b_log)] = norm;
+            if (!finite) latch_error(a.st, QGX_ERR_NONFINITE);
+          }
+          bar_arrive(ready + 8u * c0);
+        }
+        __syncwarp();
+      }
+    };
+
+    // Chunk by chunk.  While chunk c is quantized, c + 16 comes in; half way through its norm is formed, so that the other
+    // quantizers of its bucket have theirs posted, too, by the time it is its turn; its successor is asked for when c is done.
+    // (The first two turns of the loop only bring in and norm.)
+    // Bits wait in one of NT images for the copiers.
+    int len_next = 0;                                                  // of the unit of chunk c + 16
+    int it = NT - 2;                                                   // turn_no mod NT: the image,
+    uint32_t par = 1u;                                                 // and turn_no / NT mod 2
+    bool ok = true;
+    for (int turn_no = -2; ok; ++turn_no) {
+      const bool now = turn_no >= 0;
+      const unsigned c = (unsigned)warp + (unsigned)(turn_no * kQuantizers);          // wraps around before the first
+      const unsigned n = c >> u_log, i = c & (unsigned)(U - 1), cs = c & (2u * kQuantizers - 1u);
+      const unsigned ci = (unsigned)(it * kQuantizers + warp), ci2 = ci + par * (unsigned)(NT * kQuantizers);
+      if (now) {
+        ok = bar_wait(ready + 8u * (cs & ~(unsigned)(m - 1)), (c / (2u * kQuantizers)) & 1u, quit);
+        if (ok && turn_no >= NT) ok = bar_wait(written + 8u * ((unsigned)it * per_turn + (n & (per_turn - 1u))), par ^ 1u, quit);
+        if (!ok) break;
+      }
+      const PipeUnit pu = s_unit[n & (kUnitRing - 1u)];
+      const PipeNorm* norm = s_norm + (cs & ~(unsigned)(m - 1));
+      const uint32_t lx = sa + L.stage + cs * (kChunk * 4u) + (uint32_t)lane * 128u + (((uint32_t)lane & 7u) << 4);
+      const int count = max(0, min(kLaneCoords, pu.len - (int)i * kChunk - lane * kLaneCoords));
+      const uint64_t q0 = a.quad_base + (uint64_t)(pu.lo >> 2) + (uint64_t)(i * (kChunk / 4) + (unsigned)lane * (kLaneCoords / 4));
+      rc.rn = norm->rn;
+      rc.thr = norm->thr;
+      if (now && !norm->live) {                                        // NaN or infinite coordinates would leave the tables
+#pragma unroll 1
+        for (uint32_t p = 0; p < 8u; ++p)
+          asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(lx ^ (16u * p)), "f"(0.0f) : "memory");
+      }
+      const uint32_t img = sa + L.image + (ci * 32u + (unsigned)lane) * lane_words * 4u;
+      LaneBits out;
+      out.open(img);
+      const bool plain = __all_sync(0xffffffffu, count == kLaneCoords && (uint32_t)q0 < 0xfffffff0u);
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        if (now && plain)
+          quantize_line<false>(2 * half, lx, q0, count, norm, pu.k, a.xid, key, rc, h, sa, out);
+        else if (now)
+          quantize_line<true>(2 * half, lx, q0, count, norm, pu.k, a.xid, key, rc, h, sa, out);
+        if (half == 0 && len_next > 0) norm_of(c + kQuantizers);
+      }
+      if (now) {
+        if (lane == 31) s_last[ci2] = out.hi;                          // the chunk's last 32 bits, for the chunk after it
+        const uint32_t bits = out.close(img);
+        s_cnt[ci2 * 32u + (unsigned)lane] = (uint16_t)bits;
+        const uint32_t chunk_bits = __reduce_add_sync(0xffffffffu, bits);
+        if (lane == 0) {
+          s_tot[ci] = chunk_bits;
+          s_inorm[ci] = norm->norm;
+        }
+        __syncwarp();
+        if (lane == 0) {
+          bar_arrive(coded + 8u * ((unsigned)it * per_turn + (n & (per_turn - 1u))));
+          bar_arrive(turned + 8u * ((unsigned)turn_no & (kTurnRing - 1u)));
+        }
+      }
+      if (len_next <= 0 && turn_no > -2) break;
+      ok = issue(c + 2u * kQuantizers, &len_next);
+      if (++it == NT) { it = 0; par ^= 1u; }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!ok) give_up();
+    return;
+  }
+
+  if (warp < kQuantizers + kDispatchers) {
+    // ================================ dispatcher ================================
+    const unsigned total = (unsigned)h.units * (unsigned)a.K;          // below 2^31: the host checks
+    const size_t unit_coords = (size_t)U * kChunk;
+    const float* v = a.src.v ? a.src.v : a.src.a;
+    const size_t row = a.src.v ? (a.src.ld ? a.src.ld : a.d) : 0;
+    unsigned ticket = lane == 0 ? atomicAdd(a.ticket, 1u) : 0u;        // drawn a unit early: nobody waits for the counter
+    bool ok = true;
+    for (unsigned n = 0; ok; ++n) {
+      const unsigned turn = n / per_turn;                              // three turns are under way at most
+      if (turn >= 3u && n % per_turn == 0u) ok = bar_wait(turned + 8u * ((turn - 3u) & (kTurnRing - 1u)), ((turn - 3u) / kTurnRing) & 1u, quit);
+      if (!ok) break;
+      PipeUnit pu;
+      pu.lo = 0ull; pu.src = nullptr; pu.k = 0u; pu.len = 0;
+      if (lane == 0) {
+        if (ticket < total) {
+          const unsigned u = ticket / (unsigned)a.K;
+          pu.k = ticket - u * (unsigned)a.K;
+          const size_t lo = a.b_first * (size_t)a.bucket + (size_t)u * unit_coords;
+          pu.lo = (unsigned long long)lo;
+          pu.src = v + (size_t)pu.k * row + lo;
+          pu.len = (int)min(unit_coords, a.d - lo);
+          ticket = atomicAdd(a.ticket, 1u);
+        }
+        s_unit[n & (kUnitRing - 1u)] = pu;
+        bar_arrive(dealt + 8u * (n & (kUnitRing - 1u)));
+      }
+      if (__shfl_sync(0xffffffffu, pu.len, 0) > 0) continue;
+      // No more units: end markers for everybody who asks for one.
+      if (lane == 0)
+        for (unsigned e = n + 1u; e < n + max(per_turn, (unsigned)kScanners); ++e) {
+          s_unit[e & (kUnitRing - 1u)] = pu;
+          bar_arrive(dealt + 8u * (e & (kUnitRing - 1u)));
+        }
+      break;
+    }
+    if (!ok) give_up();
+    return;
+  }
+
+  if (warp < kQuantizers + kDispatchers + kScanners) {
+    // ================================ scanners: where a unit's bits go ================================
+    for (unsigned n = (unsigned)(warp - kQuantizers - kDispatchers);; n += kScanners) {
+      if (!bar_wait(dealt + 8u * (n & (kUnitRing - 1u)), (n / kUnitRing) & 1u, quit)) { give_up(); return; }
+      const PipeUnit pu = s_unit[n & (kUnitRing - 1u)];
+      if (pu.len == 0) return;
+      const unsigned turn = n / per_turn, it = turn % (unsigned)NT, ui = it * per_turn + (n & (per_turn - 1u));
+      const unsigned ci0 = it * kQuantizers + ((n * (unsigned)U) & (kQuantizers - 1u));    // the unit's first image
+      if (!bar_wait(coded + 8u * ui, (turn / (unsigned)NT) & 1u, quit)) { give_up(); return; }
+      const size_t k = (size_t)pu.k, b0 = (size_t)pu.lo >> b_log;
+      // lane i: chunk i.  Its first bit in the bucket's payload, then the bucket's words, then the words before the bucket
+      const uint32_t bits = lane < U ? s_tot[ci0 + (unsigned)lane] : 0u;
+      uint32_t upto = bits;
+      for (int o = 1; o < m; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, upto, o);
+        if ((lane & (m - 1)) >= o) upto += y;
+      }
+      const uint32_t payload = __shfl_sync(0xffffffffu, upto, lane | (m - 1));
+      const int blen = min(a.bucket, pu.len - (lane & ~(m - 1)) * kChunk);
+      const bool first = lane < U && (lane & (m - 1)) == 0 && blen > 0;          // the bucket's first chunk
+      const uint32_t nsub = blen > 0 ? (uint32_t)((blen + G - 1) / G) : 0u, hdr_bits = kNormBits + 16u * nsub;
+      const uint32_t nbits = hdr_bits + payload, nwords = (nbits + 31u) >> 5;
+      const uint32_t words_upto = warp_incl_scan(first ? nwords : 0u, lane);
+      const uint32_t words = __shfl_sync(0xffffffffu, words_upto, 31);
+      unsigned long long* srow = a.status + k * h.status_ld;
+      const size_t su = ((b0 - a.b_first) >> (u_log - m_log)) + h.status_first;
+      if (lane == 0) st_status(srow + su, kStAggregate | (unsigned long long)words);
+      unsigned long long all_bits = first ? (unsigned long long)nbits : 0ull;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) all_bits += __shfl_xor_sync(0xffffffffu, all_bits, o);
+      if (lane == 0) atomicAdd(a.total_bits + k, all_bits);
+      bool timed_out = false;
+      const unsigned long long base = lookback_prefix(srow, (long long)su, lane, a.spin_limit, &timed_out);
+      const bool skip = timed_out || base + words > (unsigned long long)a.cap_words;
+      if (lane == 0) {
+        st_status(srow + su, kStPrefix | (base + (unsigned long long)words));
+        if (timed_out) latch_error(a.st, QGX_ERR_TIMEOUT);
+        else if (skip) latch_error(a.st, QGX_ERR_CAPACITY);
+      }
+      const uint32_t before = __shfl_sync(0xffffffffu, words_upto - (first ? nwords : 0u), lane & ~(m - 1));   // words before the bucket
+      if (first) {
+        const size_t kb = k * a.nb + b0 + (size_t)(lane >> m_log);
+        a.bucket_bits[kb] = nbits;
+        a.offsets[kb] = (uint32_t)min(base + before, 0xffffffffull);
+      }
+      if (lane < U) {
+        PipePlace pp;
+        pp.word = base + before;
+        pp.bit = hdr_bits + upto - bits;
+        pp.nbits = skip ? 0u : nbits;
+        s_place[ci0 + (unsigned)lane] = pp;
+      }
+      __syncwarp();
+      if (lane == 0) bar_arrive(placed + 8u * ui);
+    }
+  }
+
+  {
+    // ================================ copiers: the lanes' bits into the stream ================================
+    const int w = warp - kQuantizers - kDispatchers - kScanners;
+    for (unsigned n = 0;; ++n) {
+      if (!bar_wait(dealt + 8u * (n & (kUnitRing - 1u)), (n / kUnitRing) & 1u, quit)) { give_up(); return; }
+      const PipeUnit pu = s_unit[n & (kUnitRing - 1u)];
+      if (pu.len == 0) return;
+      const unsigned turn = n / per_turn, it = turn % (unsigned)NT, ui = it * per_turn + (n & (per_turn - 1u)), par = (turn / (unsigned)NT) & 1u;
+      const unsigned ci0 = it * kQuantizers + ((n * (unsigned)U) & (kQuantizers - 1u));    // the unit's first image
+      if (!bar_wait(placed + 8u * ui, par, quit)) { give_up(); return; }
+      for (int i = w; i < U; i += kCopiers) {
+        if (pu.len - i * kChunk <= 0) break;
+        const unsigned cs = ci0 + (unsigned)i, cs2 = cs + par * (unsigned)(NT * kQuantizers);   // the image; of twice the ring
+        const PipePlace pp = s_place[cs];
+        if (pp.nbits == 0u) continue;                               // no place was found for the unit
+        uint32_t* dst = a.stream + (size_t)pu.k * a.cap_words + pp.word;
+        const int ib = i & (m - 1);                                    // the chunk's place in its bucket
+        const uint32_t cnt_sa = sa + L.cnt + cs2 * 64u;                // its 32 lane counts, two bytes each
+        const uint32_t nsub = (uint32_t)((min(a.bucket, pu.len - (i - ib) * kChunk) + G - 1) / G);
+        // The header's words of this chunk: two sub-blocks each, G / 32 lane counts per sub-block.
+        constexpr uint32_t kWords = kChunk / G / 2;                    // 16, 8 or 4
+        if ((uint32_t)lane < kWords && (uint32_t)ib * kWords + (uint32_t)lane < nsub / 2u) {
+          uint32_t h;
+          if (G == 32) {
+            h = lds32(cnt_sa + 4u * (uint32_t)lane);
+          } else {
+            uint32_t f0 = 0, f1 = 0;
+#pragma unroll
+            for (int j = 0; j < G / 64; ++j) {
+              const uint32_t c0 = lds32(cnt_sa + (uint32_t)lane * (G / 8) + 4u * j), c1 = lds32(cnt_sa + (uint32_t)lane * (G / 8) + (G / 16) + 4u * j);
+              f0 += (c0 & 0xffffu) + (c0 >> 16);
+              f1 += (c1 & 0xffffu) + (c1 >> 16);
+            }
+            h = f0 | (f1 << 16);
+          }
+          dst[1u + (uint32_t)ib * kWords + (uint32_t)lane] = h;
+        }
+        if (ib == 0 && lane == 0) dst[0] = __float_as_uint(s_inorm[cs]);
+        const uint32_t n_l = s_cnt[cs2 * 32u + (unsigned)lane];
+        const uint32_t p = pp.bit + warp_incl_scan(n_l, lane) - n_l, sh = p & 31u, nw = ((p + n_l) >> 5) - (p >> 5);
+        uint32_t* out = dst + (p >> 5);
+        const uint32_t img = sa + L.image + (cs * 32u + (unsigned)lane) * lane_words * 4u;
+        // Word j of the lane's part of the stream takes the end of its bits' word j - 1 and the beginning of word j; words
+        // 0 .. nw - 1 end inside its bits, word nw is for the lane after it (past the lane's words the reads run into its
+        // neighbour's: those bits are masked off).
+        const uint32_t most = __reduce_max_sync(0xffffffffu, nw);
+        uint32_t prev = lds32(img), tail = 0;
+        const uint32_t first = prev << sh;
+#pragma unroll
+        for (uint32_t j = 1; j <= (uint32_t)QGX_MAX_CODE_LEN + 2u; ++j) {
+          if (j > most) break;
+          const uint32_t cur = lds32(img + 4u * j), x = __funnelshift_l(prev, cur, sh);
+          if (j < nw) out[j] = x;
+          if (j == nw) tail = x;
+          prev = cur;
+        }
+        const uint32_t over = (p + n_l) & 31u, mask = (1u << over) - 1u;
+        tail &= mask;
+        uint32_t before = __shfl_up_sync(0xffffffffu, tail, 1);
+        if (lane == 0) {
+          before = 0;
+          if (sh != 0u) {
+            if (ib != 0) {
+              before = s_last[cs2 - 1u] >> (32u - sh);                 // the last bits of the chunk before
+            } else {                                                   // an odd number of sub-blocks: the last length shares a word
+              const uint16_t* cnt = s_cnt + cs2 * 32u;
+#pragma unroll
+              for (int j = 0; j < G / kLaneCoords; ++j) before += cnt[(nsub - 1u) * (G / kLaneCoords) + j];
+            }
+          }
+        }
+        if (nw > 0u) out[0] = first | before;
+        // the bucket's last word, when it is not whole
+        if (n_l > 0u && p + n_l == pp.nbits && over != 0u) out[nw] = nw > 0u ? tail : ((first & mask) | before);
+      }
+      __syncwarp();
+      if (lane == 0) bar_arrive(written + 8u * ui);
+    }
+  }
+}
+
+}  // namespace qgx

@@ -4,8 +4,6 @@
 #include "qgx_bucket.cuh"
 #include "qgx_codec.cuh"
 
-#include <cuda.h>
-
 #include <algorithm>
 #include <cstring>
 #include <limits>
@@ -74,6 +72,7 @@ struct EncodeArgs {
   uint32_t xid;
   uint64_t quad_base;           // (index of the vector's first coordinate in the generator's counter space) / 4
   bool vec_ok;
+  bool v_vec, a_vec;            // the workers' rows / the shared vector are 16-byte aligned (whatever d is)
   uint32_t* stream;
   size_t cap_words;
   uint32_t* bucket_bits;        // [K][nb]
@@ -84,8 +83,7 @@ struct EncodeArgs {
   unsigned int* ticket;         // zeroed before the launch
   const struct EncodeTables* tables;   // the shared-memory tables of the configuration, built once (null: every CTA builds them)
   DevStatus* st;
-  size_t nb_whole;              // buckets [0, nb_whole) of every worker belong to k_encode_staged ...
-  size_t b_first;               // ... and buckets [b_first, nb) to k_exchange_encode
+  size_t b_first;               // first bucket of every worker to encode (0 but for the diagnostic)
   int spin_limit;               // polls of a wait for another bucket's count before it gives up
 };
 
@@ -236,6 +234,9 @@ struct EncodeTables {
   float4 bin[kBinEntries];
   uint32_t pair[kPairLutSize];
   EncLut lut;
+  float4 bin_fix[kBinEntries];             // the fixed-point rounding map of k_encode_pipeline
+  uint32_t pair_fix[kPairLutSize];         // its pair table, (2 nlev)^2 entries: first + 2 nlev * second, a symbol being its level,
+                                           // plus nlev for a negative coordinate
 };
 static_assert(sizeof(EncodeTables) % 16 == 0, "copied in 16-byte pieces");
 
@@ -245,13 +246,24 @@ __global__ void __launch_bounds__(512) k_build_encode_tables(const __grid_consta
   __shared__ __align__(16) uint32_t s_pair[kPairLutSize];
   __shared__ EncLut s_lut;
   fill_enc_lut(&s_lut, ct);
-  fill_bin_table(s_bin, rt, true);
+  fill_bin_table(s_bin, rt, BinKind::kOctet);
   __syncthreads();
   fill_pair_lut_signed(s_pair, &s_lut);
   __syncthreads();
   for (int i = threadIdx.x; i < kBinEntries; i += blockDim.x) out->bin[i] = s_bin[i];
   for (int i = threadIdx.x; i < kPairLutSize; i += blockDim.x) out->pair[i] = s_pair[i];
   for (int i = threadIdx.x; i < 2 * QGX_MAX_LEVELS; i += blockDim.x) out->lut.e[i] = s_lut.e[i];
+  __syncthreads();
+  fill_bin_table(s_bin, rt, BinKind::kFixed);
+  const int n2 = 2 * ct.nlev;
+  for (int i = threadIdx.x; i < n2 * n2; i += blockDim.x) {
+    const int f = i % n2, g = i / n2;
+    const uint32_t x = s_lut.e[f < ct.nlev ? f : f - ct.nlev + 32], y = s_lut.e[g < ct.nlev ? g : g - ct.nlev + 32];
+    const uint32_t nx = x >> 16, ny = y >> 16;
+    out->pair_fix[i] = ((x & 0xffffu) | ((y & 0xffffu) << nx)) | ((nx + ny) << 26);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < kBinEntries; i += blockDim.x) out->bin_fix[i] = s_bin[i];
 }
 
 // One persistent CTA per SM slot; each ticket is one bucket (k = ticket % K, b = ticket / K).
@@ -293,7 +305,7 @@ k_exchange_encode(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
     for (int i = threadIdx.x; i < 2 * QGX_MAX_LEVELS; i += blockDim.x) s_lut.e[i] = __ldg(a.tables->lut.e + i);
   } else {
     fill_enc_lut(&s_lut, ct);
-    fill_bin_table(s_bin, rt, true);
+    fill_bin_table(s_bin, rt, BinKind::kOctet);
   }
   if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
   if (threadIdx.x == 0) s_ticket[0] = atomicAdd(a.ticket, 1u);
@@ -446,7 +458,7 @@ k_exchange_encode(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
 
 }  // namespace qgx
 
-#include "qgx_encode_staged.cuh"
+#include "qgx_encode_pipeline.cuh"
 
 namespace qgx {
 
@@ -1086,7 +1098,6 @@ struct LaunchShape { size_t smem; int per_sm; };      // smem == 0: not asked ye
 struct TableCache {
   CachedTables e[kTableCacheSlots];
   LaunchShape enc[3][3];                // [octets per thread 1, 2, 4][sub-block 32, 64, 128]
-  LaunchShape enc_staged[3];            // [sub-block]
   LaunchShape dec[3][6];                // [sub-block][symbol mode]
   LaunchShape dec_walk[3][6];           // the walk alone
 };
@@ -1194,33 +1205,6 @@ static qgx_status cached_tables(qgx_ctx* c, const qgx_quant_cfg* cfg, const Cach
   return QGX_OK;
 }
 
-// Tensor map of `rows` rows of 32 floats (128 bytes) starting at base, copied `box_rows` rows at a time with the
-// 128-byte swizzle: what k_encode_staged's bulk copies read.  The encoder of the map is a driver entry point,
-// looked up once (the library does not link the driver).
-static bool make_rows_map(const float* base, unsigned long long rows, unsigned box_rows, CUtensorMap* out) {
-  typedef CUresult (*encode_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static encode_fn encode = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess && qres == cudaDriverEntryPointSuccess)
-      encode = reinterpret_cast<encode_fn>(fn);
-    else
-      cudaGetLastError();
-  });
-  if (!encode || rows == 0) return false;
-  const cuuint64_t gdim[2] = {(cuuint64_t)kLaneCoords, (cuuint64_t)rows};
-  const cuuint64_t gstride[1] = {(cuuint64_t)(kLaneCoords * sizeof(float))};
-  const cuuint32_t box[2] = {(cuuint32_t)kLaneCoords, (cuuint32_t)box_rows};
-  const cuuint32_t estride[2] = {1u, 1u};
-  return encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), gdim, gstride, box, estride,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // The whole exchange.  sym_mode 1 keeps the decoded symbols (and the norms) in the workspace; sym_mode 2
 // adds sum_k ||vhat_k kept by the other slot - vhat_k decoded in this exchange||^2 to *sum_sq.
 qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_quant_cfg* cfg, uint32_t xid, int slot,
@@ -1249,7 +1233,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   uint32_t* bbits = (uint32_t*)ws_get(c, base + 1, sizeof(uint32_t) * (size_t)K * nb);
   uint32_t* offs = (uint32_t*)ws_get(c, base + 2, sizeof(uint32_t) * (size_t)K * nb);
   // one block per slot, zeroed by one memset: the per-worker bit totals, the ticket counter, the status words of the scan
-  unsigned long long* tot = (unsigned long long*)ws_get(c, base + 3, sizeof(uint64_t) * ((size_t)K + 2 + (size_t)K * nb));
+  unsigned long long* tot = (unsigned long long*)ws_get(c, base + 3, sizeof(uint64_t) * ((size_t)K + 2 + (size_t)K * (nb + 1)));
   unsigned long long* status = tot ? tot + K + 2 : nullptr;
   float* norms = (float*)ws_get(c, slot == 0 ? WS_NORMS : WS_NORMS2, sizeof(float) * (size_t)K * nb);
   const DecEntry* lut = tables->lut_dev;
@@ -1259,12 +1243,13 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   c->slot_nb[slot] = nb;
 
   const bool do_encode = !c->decode_only;               // the decode-only entry point works on the streams that are there
-  if (do_encode && cudaMemsetAsync(tot, 0, sizeof(uint64_t) * ((size_t)K + 2 + (size_t)K * nb), c->stream) != cudaSuccess) return QGX_ERR_CUDA;
 
   EncodeArgs ea;
   ea.src = src; ea.d = d; ea.bucket = bucket; ea.K = K; ea.nb = nb; ea.norm_type = cfg->norm_type; ea.xid = xid; ea.quad_base = coord_base / kQuad;
   ea.vec_ok = (d % kQuad == 0) && (src.ld % kQuad == 0) && ((reinterpret_cast<uintptr_t>(src.v) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(src.a) & 15u) == 0);
-  ea.stream = stream; ea.cap_words = cap; ea.bucket_bits = bbits; ea.offsets = offs; ea.total_bits = tot; ea.norms = norms;
+  ea.v_vec = (reinterpret_cast<uintptr_t>(src.v ? src.v : src.a) & 15u) == 0 && (!src.v || K == 1 || (src.ld ? src.ld : d) % kQuad == 0);
+  ea.a_vec = (reinterpret_cast<uintptr_t>(src.a) & 15u) == 0;
+    ea.stream = stream; ea.cap_words = cap; ea.bucket_bits = bbits; ea.offsets = offs; ea.total_bits = tot; ea.norms = norms;
   ea.status = status; ea.ticket = reinterpret_cast<unsigned int*>(tot + K); ea.st = c->dstatus; ea.tables = tables->enc_dev;
   uint8_t* sym_out = nullptr;
   const uint8_t* sym_prev = nullptr;
@@ -1316,60 +1301,64 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     else if (ct.G == 64) QGX_LAUNCH_E(V, 64);              \
     else QGX_LAUNCH_E(V, 128);                             \
   } while (0)
-  // Whole buckets of a multiple of 1024 coordinates that divides 16384 go through the staged kernel; what is left
-  // (a short last bucket, other bucket sizes, unaligned vectors) through the bucket-in-registers kernel.
-  bool staged_ok = ea.vec_ok && bucket % kWarpCoords == 0 && kStageCoords % bucket == 0 && coord_base % 8 == 0 &&
-                   c->encode_path == QGX_ENCODE_STAGED && d / (size_t)bucket > 0 && c->skip_buckets == 0;
-  CUtensorMap tmap;
-  std::memset(&tmap, 0, sizeof(tmap));
-  if (staged_ok) {
-    // the staged source: the workers' rows (worker k at k * ld) or, without them, the shared vector a
-    const size_t ldv = src.ld ? src.ld : d;
-    const size_t whole = (d / (size_t)bucket) * (size_t)bucket;
-    const float* base = src.v ? src.v : src.a;
-    const unsigned long long floats = src.v ? (unsigned long long)(K - 1) * ldv + whole : whole;
-    staged_ok = (!src.v || ldv % kLaneCoords == 0) &&
-                make_rows_map(base, floats / kLaneCoords, (unsigned)std::min(256, bucket / kLaneCoords), &tmap);
+  // Buckets of 1024 * 2^j coordinates go through the pipelined kernel, other sizes through the bucket-in-registers kernel.
+  // (So do a few hundred buckets of 4096, which that kernel holds all at once: 36864 coordinates of 16 workers 15 us
+  // against 17 us; from some 600 buckets on the pipeline is ahead.)
+  const bool pipelined = bucket % kChunk == 0 && (bucket & (bucket - 1)) == 0 && c->encode_path != QGX_ENCODE_REGISTERS &&
+                         (unsigned long long)nb * (unsigned long long)K < (1ull << 31) &&
+                         (bucket != 4 * kChunk || c->encode_path == QGX_ENCODE_STAGED || nb * (size_t)K >= 4 * (size_t)c->num_sms);
+  ea.b_first = std::min(c->skip_buckets, nb);
+  size_t status_ld = nb;
+  PipeShape ps;
+  std::memset(&ps, 0, sizeof(ps));
+  if (pipelined) {
+    ps.b_log = 31 - __builtin_clz((unsigned)bucket);
+    ps.m = bucket / kChunk;
+    ps.m_log = ps.b_log - 10;
+    // units of 16 chunks; fewer where that would leave SMs without any
+    const size_t chunks = (nb - ea.b_first) * (size_t)ps.m;
+    ps.unit = 16;
+    while (ps.unit > std::max(ps.m, 4) && (chunks + (size_t)ps.unit - 1) / (size_t)ps.unit * (size_t)K < 4 * (size_t)c->num_sms) ps.unit /= 2;
+    ps.u_log = 31 - __builtin_clz((unsigned)ps.unit);
+    ps.per_turn = (unsigned)(kQuantizers / ps.unit);
+    ps.units = (chunks + (size_t)ps.unit - 1) / (size_t)ps.unit;
+    ps.status_first = (ea.b_first * (size_t)ps.m + (size_t)ps.unit - 1) / (size_t)ps.unit;
+    ps.status_ld = status_ld = ps.status_first + ps.units;          // at most nb + 1
+    ps.image_turns = kMaxImageTurns;
+    while (ps.image_turns > 2 && pipe_smem(ct.nlev, ct.maxlen, ps.image_turns).bytes > kPipeSmemMax) --ps.image_turns;
+    ps.smem = pipe_smem(ct.nlev, ct.maxlen, ps.image_turns);
+    ps.lane_words = (uint32_t)pipe_lane_stride(ct.maxlen);
+    ps.nlev = ct.nlev;
+    ps.weights = 4u | ((uint32_t)(8 * ct.nlev) << 16);
+    ps.neg4 = (uint32_t)ct.nlev * 0x01010101u;
+    ps.bin_copy = (16u << (tables->rt.key_shift - kKeyShiftMin)) - 16u;
+    ps.bin_mask = ~(ps.bin_copy + 15u);
   }
-  ea.nb_whole = staged_ok ? d / (size_t)bucket : 0;
-  ea.b_first = staged_ok ? ea.nb_whole : std::min(c->skip_buckets, nb);
+  if (do_encode && cudaMemsetAsync(tot, 0, sizeof(uint64_t) * ((size_t)K + 2 + (size_t)K * status_ld), c->stream) != cudaSuccess) return QGX_ERR_CUDA;
   c->skip_buckets = 0;
   ea.spin_limit = c->wait_limit;
-  if (do_encode) {
+  if (do_encode && ea.b_first < nb) {
     ScopedKernelTimer timer(c, QGX_KERNEL_ENCODE);
-    if (ea.nb_whole > 0) {
-      const size_t smem_st = sizeof(float) * kStageCoords * kStageBuffers;
-      const unsigned long long per_group = (unsigned long long)(kStageCoords / bucket);
-      const unsigned long long groups = ((unsigned long long)ea.nb_whole * (unsigned long long)K + per_group - 1ull) / per_group;
-#define QGX_LAUNCH_SG(GG)                                                                                            \
-  do {                                                                                                               \
-    allow_max_dynamic_smem(k_encode_staged<GG>, c->device);                                                          \
-    LaunchShape& shape = table_cache(c)->enc_staged[GG == 32 ? 0 : (GG == 64 ? 1 : 2)];                              \
-    if (shape.smem == 0) {                                                                                           \
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_encode_staged<GG>, kStagedThreads, smem_st);          \
-      shape.smem = 1;                                                                                                \
-      shape.per_sm = per_sm < 1 ? 1 : per_sm;                                                                        \
-    }                                                                                                                \
-    const unsigned grid = (unsigned)std::min<unsigned long long>((groups + 1ull) / 2ull, (unsigned long long)c->num_sms * (unsigned long long)shape.per_sm); \
-    /* a cooperative launch: the static assignment of groups needs every CTA of the grid resident at once, */       \
-    /* also when other kernels (another exchange on a helper stream) share the device                      */       \
-    void* kargs[] = {(void*)&ea, (void*)&lt, (void*)&ct, (void*)&key, (void*)&qt, (void*)&tmap};                     \
-    cudaLaunchCooperativeKernel((const void*)k_encode_staged<GG>, dim3(grid), dim3(kStagedThreads), kargs, smem_st, c->stream); \
+    if (pipelined) {
+      const unsigned long long units = (unsigned long long)ps.units * (unsigned long long)K;
+      const unsigned grid = (unsigned)std::min<unsigned long long>(units, (unsigned long long)c->num_sms);
+#define QGX_LAUNCH_P(GG)                                                                        \
+  do {                                                                                          \
+    allow_max_dynamic_smem(k_encode_pipeline<GG>, c->device);                                   \
+    k_encode_pipeline<GG><<<grid, kPipeThreads, ps.smem.bytes, c->stream>>>(ea, ps, lt, ct, key, qt);   \
   } while (0)
-      if (ct.G == 32) QGX_LAUNCH_SG(32);
-      else if (ct.G == 64) QGX_LAUNCH_SG(64);
-      else QGX_LAUNCH_SG(128);
-#undef QGX_LAUNCH_SG
-      count_launch(c);
-    }
-    if (ea.b_first < nb) {
+      if (ct.G == 32) QGX_LAUNCH_P(32);
+      else if (ct.G == 64) QGX_LAUNCH_P(64);
+      else QGX_LAUNCH_P(128);
+#undef QGX_LAUNCH_P
+    } else {
       switch (pp) {
         case 1: QGX_LAUNCH_EG(1); break;
         case 2: QGX_LAUNCH_EG(2); break;
         default: QGX_LAUNCH_EG(4); break;
       }
-      count_launch(c);
     }
+    count_launch(c);
   }
 #undef QGX_LAUNCH_EG
 #undef QGX_LAUNCH_E
