@@ -212,6 +212,7 @@ void qgx_destroy(qgx_ctx* c) {
   if (c->timing_ev) timing_free(c);
   free_seg_children(c);
   free_table_cache(c);
+  free_step_cache(c);
   for (int i = 0; i < 24; ++i)
     if (c->ws[i]) cudaFree(c->ws[i]);
   cudaFree(c->dstatus);

@@ -126,4 +126,90 @@ __device__ __forceinline__ float bucket_norm(const BucketRegs<V4>& r, int norm_t
   return (float)red[32];
 }
 
+// Norm of the bucket held by the CTA, one barrier: per-warp partials go to shared memory and every
+// warp then reduces them in the same order (so all warps hold the same value).
+template <int V4>
+__device__ __forceinline__ float bucket_norm_all(const BucketRegs<V4>& r, int norm_type, double* red) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  double acc = 0.0;
+  if (norm_type == QGX_NORM_L2) {
+#pragma unroll
+    for (int j = 0; j < V4; ++j) {
+      const double a = r.x[j].x, b = r.x[j].y, c = r.x[j].z, e = r.x[j].w;
+      acc = fma(a, a, acc); acc = fma(b, b, acc); acc = fma(c, c, acc); acc = fma(e, e, acc);
+    }
+    acc = warp_sum(acc);
+  } else {
+    float m = 0.0f;
+    bool bad = false;
+#pragma unroll
+    for (int j = 0; j < V4; ++j) {
+      const float4 x = r.x[j];
+      bad = bad || (x.x != x.x) || (x.y != x.y) || (x.z != x.z) || (x.w != x.w);
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
+    }
+    m = warp_max(m);
+    acc = __any_sync(0xffffffffu, bad) ? (double)__int_as_float(0x7fc00000) : (double)m;
+  }
+  if (lane == 0) red[warp] = acc;
+  __syncthreads();
+  double t = lane < nwarps ? red[lane] : 0.0;
+  if (norm_type == QGX_NORM_L2) return (float)sqrt(warp_sum(t));
+  const bool bad = __any_sync(0xffffffffu, t != t);
+  const float m = warp_max((float)t);
+  return bad ? __int_as_float(0x7fc00000) : m;
+}
+
+// Loads bucket [lo, lo + len) of worker k: warp w holds coordinates [w * 256 * P, (w + 1) * 256 * P), row j of
+// them 32 octets (8 consecutive coordinates: two quads), lane l the l-th octet of the row.
+template <int P>
+__device__ __forceinline__ void load_bucket_octets(BucketRegs<2 * P>& r, const DualSource& s, size_t k, size_t d,
+                                                   size_t lo, int len, bool vec_ok) {
+  const size_t ld = s.ld ? s.ld : d;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (vec_ok && len == 256 * P * (int)(blockDim.x >> 5)) {
+    // every lane holds full octets: the kind of source is decided once, not per quad
+    const float4* pv = s.v ? reinterpret_cast<const float4*>(s.v + k * ld + lo) + ((warp * P * 32 + lane) << 1) : nullptr;
+    const float4* pa = s.a ? reinterpret_cast<const float4*>(s.a + lo) + ((warp * P * 32 + lane) << 1) : nullptr;
+    if (pa == nullptr) {
+#pragma unroll
+      for (int j = 0; j < 2 * P; ++j) r.x[j] = __ldcs(pv + (j >> 1) * 64 + (j & 1));
+    } else if (pv == nullptr) {
+#pragma unroll
+      for (int j = 0; j < 2 * P; ++j) r.x[j] = __ldg(pa + (j >> 1) * 64 + (j & 1));
+    } else if (s.mul) {
+#pragma unroll
+      for (int j = 0; j < 2 * P; ++j) r.x[j] = dual_combine(__ldg(pa + (j >> 1) * 64 + (j & 1)), __ldcs(pv + (j >> 1) * 64 + (j & 1)), 1);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 2 * P; ++j) r.x[j] = dual_combine(__ldg(pa + (j >> 1) * 64 + (j & 1)), __ldcs(pv + (j >> 1) * 64 + (j & 1)), 0);
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 2 * P; ++j) {
+    const int e = ((((warp * P + (j >> 1)) * 32 + lane) << 1) + (j & 1)) * kQuad;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (e + kQuad <= len && vec_ok) {
+      if (s.a == nullptr) {
+        x = __ldcs(reinterpret_cast<const float4*>(s.v + k * ld + lo + e));
+      } else {
+        const float4 av = __ldg(reinterpret_cast<const float4*>(s.a + lo + e));
+        if (s.v) {
+          const float4 u = __ldcs(reinterpret_cast<const float4*>(s.v + k * ld + lo + e));
+          x = dual_combine(av, u, s.mul);
+        } else {
+          x = av;
+        }
+      }
+    } else {
+      if (e + 0 < len) x.x = dual_value(s, k, d, lo + e + 0);
+      if (e + 1 < len) x.y = dual_value(s, k, d, lo + e + 1);
+      if (e + 2 < len) x.z = dual_value(s, k, d, lo + e + 2);
+      if (e + 3 < len) x.w = dual_value(s, k, d, lo + e + 3);
+    }
+    r.x[j] = x;
+  }
+}
+
 }  // namespace qgx

@@ -163,6 +163,54 @@ __device__ __forceinline__ bool decode_symbol(BitReader& br, const uint16_t* lut
   return true;
 }
 
+// ---- chained scan of bucket lengths ("decoupled look-back") ----------------------------------
+// status word of bucket (k, b): bits 62..63 state, bits 0..61 a word count.
+constexpr unsigned long long kStEmpty = 0ull, kStAggregate = 1ull << 62, kStPrefix = 2ull << 62;
+constexpr unsigned long long kStMask = 3ull << 62;
+
+__device__ __forceinline__ unsigned long long ld_status(const unsigned long long* p) {
+  return *reinterpret_cast<const volatile unsigned long long*>(p);
+}
+__device__ __forceinline__ void st_status(unsigned long long* p, unsigned long long v) {
+  *reinterpret_cast<volatile unsigned long long*>(p) = v;
+}
+
+// Exclusive prefix (in words) of bucket b of one worker, by warp 0 of the CTA.  Buckets are handed
+// out by a ticket counter in the order b-major, k-minor, so every predecessor (k, b') with b' < b
+// belongs to a CTA that is already running or done: the wait below always ends; it is bounded all
+// the same, and *timed_out reports a wait that ran out.
+__device__ __forceinline__ unsigned long long lookback_prefix(unsigned long long* row /* status of worker k */, long long b,
+                                                              int lane, int spin_limit, bool* timed_out) {
+  unsigned long long prefix = 0;
+  long long hi = b - 1;                                 // nearest predecessor not yet accounted for
+  int spins = 0;
+  bool fail = false;
+  while (hi >= 0 && !fail) {
+    const long long mine = hi - lane;
+    unsigned long long s = kStPrefix;                   // positions before bucket 0 act as a zero prefix
+    if (mine >= 0) s = ld_status(row + mine);
+    const unsigned empty = __ballot_sync(0xffffffffu, (s & kStMask) == kStEmpty);
+    const unsigned pref = __ballot_sync(0xffffffffu, (s & kStMask) == kStPrefix);
+    // lanes are ordered from the nearest predecessor outwards
+    const int first_pref = pref ? __ffs(pref) - 1 : 32;
+    const int first_empty = empty ? __ffs(empty) - 1 : 32;
+    if (first_empty < first_pref) {                     // a predecessor has not published yet
+      if (++spins > spin_limit) fail = true;
+      __nanosleep(64);
+      continue;
+    }
+    const int take = first_pref < 32 ? first_pref + 1 : 32;
+    unsigned long long part = lane < take ? (s & ~kStMask) : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    prefix += part;
+    if (first_pref < 32) break;
+    hi -= 32;
+  }
+  *timed_out = fail;
+  return prefix;
+}
+
 void build_dec_lut_host(const CodeTable& ct, uint16_t* lut /*[1 << maxlen]*/);
 
 }  // namespace qgx

@@ -53,6 +53,7 @@ struct qgx_ctx {
   // host-side cache of the fused calls: tables derived from a quantizer configuration (with their device copies)
   // and launch shapes; owned by qgx_exchange.cu
   void* table_cache;
+  void* step_cache;                      // the same for the separate calls; owned by qgx_quantize.cu
   // helper contexts (own streams and workspaces) that run the tensors of a layer-wise exchange side by side;
   // owned by qgx_exchange.cu
   void* seg_children;
@@ -412,6 +413,94 @@ static __device__ __noinline__ int quantize_level_exact(float absv, float norm, 
   return tau + ((r < xi) ? 1 : 0);
 }
 
+// ---- the generator, with what the blocks of a lane share worked out once ----
+// Counter words 2 and 3 (worker, exchange) and, but for carries, word 1 are the same for all blocks of a bucket: the second
+// product of round 1 and the first of round 2 do not depend on word 0.
+struct PhiloxShared {
+  uint32_t x0, a, b, c;
+};
+__device__ __forceinline__ PhiloxShared philox_shared(uint32_t c1, uint32_t k, uint32_t xid, const PhiloxKey& key) {
+  const uint64_t p1 = (uint64_t)0xCD9E8D57u * (uint64_t)k;
+  const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ key.k0[0];
+  const uint64_t p0 = (uint64_t)0xD2511F53u * (uint64_t)n0;
+  PhiloxShared s;
+  s.x0 = xid ^ key.k1[0];
+  s.a = (uint32_t)p1 ^ key.k0[1];
+  s.b = (uint32_t)(p0 >> 32) ^ key.k1[1];
+  s.c = (uint32_t)p0;
+  return s;
+}
+// both halves of a * b in one instruction (left to itself the compiler sometimes computes them apart)
+__device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t* hi, uint32_t* lo) {
+  asm("{ .reg .b64 p; mul.wide.u32 p, %2, %3; mov.b64 {%0, %1}, p; }" : "=r"(*lo), "=r"(*hi) : "r"(a), "r"(b));
+}
+// blocks c0 and c0 + 1
+__device__ __forceinline__ void philox_pair(uint32_t c0, const PhiloxShared& s, const PhiloxKey& key, uint32_t* w) {
+  uint32_t s0[2], s1[2], s2[2], s3[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    uint32_t hi, lo, hi1;
+    mul_wide(c0 + (uint32_t)j, 0xD2511F53u, &hi, &lo);
+    mul_wide(hi ^ s.x0, 0xCD9E8D57u, &hi1, &s1[j]);                    // after round 1: word 2
+    s0[j] = hi1 ^ s.a;                                                 // after round 2
+    s2[j] = s.b ^ lo;
+    s3[j] = s.c;
+  }
+#pragma unroll
+  for (int r = 2; r < 10; ++r) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      uint32_t hi0, lo0, hi1, lo1;
+      mul_wide(s0[j], 0xD2511F53u, &hi0, &lo0);
+      mul_wide(s2[j], 0xCD9E8D57u, &hi1, &lo1);
+      s0[j] = hi1 ^ s1[j] ^ key.k0[r];
+      s2[j] = hi0 ^ s3[j] ^ key.k1[r];
+      s1[j] = lo1;
+      s3[j] = lo0;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) { w[4 * j] = s0[j]; w[4 * j + 1] = s1[j]; w[4 * j + 2] = s2[j]; w[4 * j + 3] = s3[j]; }
+}
+
+// ---- rounding: the level map in fixed point (see RoundTable::afix) ----
+struct RoundFix {
+  float rn;
+  uint32_t thr;
+  uint32_t mask;                                         // clears the bits of pattern >> kBinAddrShift below a bin's copies
+  uint32_t base;                                         // shared address of this lane's copies, minus kBinAddrBase
+};
+// Fixed-point decision variable of one coordinate: bits 16..20 the level, bits 0..15 how far it is above the point where
+// the level would be one lower (in 2^-16 of an interval).
+template <bool kClamp = false>
+__device__ __forceinline__ uint32_t round_fixed(float x, uint32_t w, const RoundFix& c) {
+  float u2 = fmaf(fabsf(x), c.rn, kRoundShift);
+  if (kClamp) u2 = fminf(u2, 1.0f + kRoundShift);
+  const float4 e = lds_table128(((__float_as_uint(u2) >> kBinAddrShift) & c.mask) + c.base);
+  float z = fmaf(u2, e.y, e.x);
+  z = fmaf(__saturatef(__fsub_rn(u2, e.z)), e.w, z);                   // in [2^23, 2^24): the mantissa is a whole number
+  return __float_as_uint(z) - (w >> 16);
+}
+__device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+// Definition 1 for one coordinate in IEEE operations, given a level near the outcome (the interval is looked for from there);
+// r24 = the 24-bit variate.
+__device__ __forceinline__ uint32_t level_exact_near(float absv, float norm, uint32_t r24, int near_level, uint32_t lev_sa, int nlev) {
+  auto lev = [&](int j) { return __uint_as_float(lds_table32(lev_sa + 4u * (uint32_t)j)); };
+  float u = (norm > 0.0f) ? __fdiv_rn(absv, norm) : 0.0f;
+  u = fminf(u, 1.0f);
+  int tau = min(max(near_level - 1, 0), nlev - 2);
+  while (tau < nlev - 2 && lev(tau + 1) <= u) ++tau;
+  while (tau > 0 && lev(tau) > u) --tau;
+  const float lo = lev(tau), hi = lev(tau + 1);
+  const float xi = __fdiv_rn(__fsub_rn(u, lo), __fsub_rn(hi, lo));
+  const float r = __fmul_rn(__uint2float_rn(r24), 5.9604644775390625e-8f);        // exact
+  return (uint32_t)(tau + ((r < xi) ? 1 : 0));
+}
+
 __device__ __forceinline__ uint32_t symbol_of(float v, int idx) {
   const uint32_t neg = (__float_as_uint(v) >> 31) & (idx != 0 ? 1u : 0u);
   return (uint32_t)idx | (neg << 7);
@@ -456,9 +545,12 @@ qgx_status make_code_table(const qgx_codebook* cb, int bucket, CodeTable* out);
 void make_round_table(const float* lev, int nlev, RoundTable* out);
 void* ws_get(qgx_ctx* c, int which, size_t bytes);          // nullptr on failure
 void free_table_cache(qgx_ctx* c);
+void free_step_cache(qgx_ctx* c);
+qgx_status step_code(qgx_ctx* c, const qgx_codebook* cb, int bucket, const CodeTable** ct, const uint16_t** lut /*[dev]*/);
 void free_seg_children(qgx_ctx* c);
 uint64_t seg_children_launches(const qgx_ctx* c);
 qgx_status cuda_status(cudaError_t e);
+void allow_max_dynamic_smem(const void* kernel, int device);
 inline void count_launch(qgx_ctx* c, int n = 1) { c->launches += (uint64_t)n; }
 
 // Brackets an instrumented kernel launch with two events when timing is on (qgx_timing_enable).

@@ -19,12 +19,14 @@
 // Tried: loaders as warps of their own (they share the issue slots of one warp each and fall behind), and quantizers that
 // copy their own bits out (fewer warps to hide latency behind): 5-30 % slower.
 //
-// Included by qgx_exchange.cu (uses its status words, look-back and EncodeArgs).
-#pragma once
+// In a translation unit of its own: the quantizers' loop runs at the register limit.
+#include "qgx_encode.cuh"
+
+#include <algorithm>
+#include <cstring>
 
 namespace qgx {
 
-constexpr int kChunk = 1024;                             // coordinates per chunk: 32 lanes x 32
 constexpr int kLaneCoords = 32;                          // coordinates per lane: one 128-byte line of the stage
 constexpr int kQuantizers = 16, kDispatchers = 1, kScanners = 2, kCopiers = 5;
 constexpr int kPipeThreads = 32 * (kQuantizers + kDispatchers + kScanners + kCopiers);
@@ -134,92 +136,6 @@ __device__ __forceinline__ void copy_async4(uint32_t dst, const float* src, int 
 // so that both a loader's lanes (consecutive pieces) and a quantizer's (the same piece of 8 consecutive lines) spread
 // over the banks
 __device__ __forceinline__ uint32_t piece_at(uint32_t u) { return ((u & ~7u) | ((u ^ (u >> 3)) & 7u)) << 4; }
-
-// ---- the generator, with what the blocks of a lane share worked out once ----
-// Counter words 2 and 3 (worker, exchange) and, but for carries, word 1 are the same for all blocks of a bucket: the second
-// product of round 1 and the first of round 2 do not depend on word 0.
-struct PhiloxShared {
-  uint32_t x0, a, b, c;
-};
-__device__ __forceinline__ PhiloxShared philox_shared(uint32_t c1, uint32_t k, uint32_t xid, const PhiloxKey& key) {
-  const uint64_t p1 = (uint64_t)0xCD9E8D57u * (uint64_t)k;
-  const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ key.k0[0];
-  const uint64_t p0 = (uint64_t)0xD2511F53u * (uint64_t)n0;
-  PhiloxShared s;
-  s.x0 = xid ^ key.k1[0];
-  s.a = (uint32_t)p1 ^ key.k0[1];
-  s.b = (uint32_t)(p0 >> 32) ^ key.k1[1];
-  s.c = (uint32_t)p0;
-  return s;
-}
-// both halves of a * b in one instruction (left to itself the compiler sometimes computes them apart)
-__device__ __forceinline__ void mul_wide(uint32_t a, uint32_t b, uint32_t* hi, uint32_t* lo) {
-  asm("{ .reg .b64 p; mul.wide.u32 p, %2, %3; mov.b64 {%0, %1}, p; }" : "=r"(*lo), "=r"(*hi) : "r"(a), "r"(b));
-}
-// blocks c0 and c0 + 1
-__device__ __forceinline__ void philox_pair(uint32_t c0, const PhiloxShared& s, const PhiloxKey& key, uint32_t* w) {
-  uint32_t s0[2], s1[2], s2[2], s3[2];
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    uint32_t hi, lo, hi1;
-    mul_wide(c0 + (uint32_t)j, 0xD2511F53u, &hi, &lo);
-    mul_wide(hi ^ s.x0, 0xCD9E8D57u, &hi1, &s1[j]);                    // after round 1: word 2
-    s0[j] = hi1 ^ s.a;                                                 // after round 2
-    s2[j] = s.b ^ lo;
-    s3[j] = s.c;
-  }
-#pragma unroll
-  for (int r = 2; r < 10; ++r) {
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      uint32_t hi0, lo0, hi1, lo1;
-      mul_wide(s0[j], 0xD2511F53u, &hi0, &lo0);
-      mul_wide(s2[j], 0xCD9E8D57u, &hi1, &lo1);
-      s0[j] = hi1 ^ s1[j] ^ key.k0[r];
-      s2[j] = hi0 ^ s3[j] ^ key.k1[r];
-      s1[j] = lo1;
-      s3[j] = lo0;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 2; ++j) { w[4 * j] = s0[j]; w[4 * j + 1] = s1[j]; w[4 * j + 2] = s2[j]; w[4 * j + 3] = s3[j]; }
-}
-
-// ---- rounding: the level map in fixed point (see RoundTable::afix) ----
-struct RoundFix {
-  float rn;
-  uint32_t thr;
-  uint32_t mask;                                         // clears the bits of pattern >> kBinAddrShift below a bin's copies
-  uint32_t base;                                         // shared address of this lane's copies, minus kBinAddrBase
-};
-// Fixed-point decision variable of one coordinate: bits 16..20 the level, bits 0..15 how far it is above the point where
-// the level would be one lower (in 2^-16 of an interval).
-__device__ __forceinline__ uint32_t round_fixed(float x, uint32_t w, const RoundFix& c) {
-  const float u2 = fmaf(fabsf(x), c.rn, kRoundShift);
-  const float4 e = lds_table128(((__float_as_uint(u2) >> kBinAddrShift) & c.mask) + c.base);
-  float z = fmaf(u2, e.y, e.x);
-  z = fmaf(__saturatef(__fsub_rn(u2, e.z)), e.w, z);                   // in [2^23, 2^24): the mantissa is a whole number
-  return __float_as_uint(z) - (w >> 16);
-}
-__device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b) {
-  uint32_t d;
-  asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-// Definition 1 for one coordinate in IEEE operations, given a level near the outcome (the interval is looked for from there);
-// r24 = the 24-bit variate.
-__device__ __forceinline__ uint32_t level_exact_near(float absv, float norm, uint32_t r24, int near_level, uint32_t lev_sa, int nlev) {
-  auto lev = [&](int j) { return __uint_as_float(lds_table32(lev_sa + 4u * (uint32_t)j)); };
-  float u = (norm > 0.0f) ? __fdiv_rn(absv, norm) : 0.0f;
-  u = fminf(u, 1.0f);
-  int tau = min(max(near_level - 1, 0), nlev - 2);
-  while (tau < nlev - 2 && lev(tau + 1) <= u) ++tau;
-  while (tau > 0 && lev(tau) > u) --tau;
-  const float lo = lev(tau), hi = lev(tau + 1);
-  const float xi = __fdiv_rn(__fsub_rn(u, lo), __fsub_rn(hi, lo));
-  const float r = __fmul_rn(__uint2float_rn(r24), 5.9604644775390625e-8f);        // exact
-  return (uint32_t)(tau + ((r < xi) ? 1 : 0));
-}
 
 // Stream bits of a lane as they are produced: a 64-bit window that new bits enter at the top (two funnel shifts, no masks);
 // the oldest 32 go to the lane's words in shared memory once they are there.
@@ -767,6 +683,55 @@ k_encode_pipeline(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
       if (lane == 0) bar_arrive(written + 8u * ui);
     }
   }
+}
+
+PipePlan plan_encode_pipeline(const qgx_ctx* c, int bucket, size_t nb, size_t b_first, int K) {
+  PipePlan p;
+  const int m = bucket / kChunk;
+  // units of 16 chunks; fewer where that would leave SMs without any
+  const size_t chunks = (nb - b_first) * (size_t)m;
+  p.unit = 16;
+  while (p.unit > std::max(m, 4) && (chunks + (size_t)p.unit - 1) / (size_t)p.unit * (size_t)K < 4 * (size_t)c->num_sms) p.unit /= 2;
+  p.units = (chunks + (size_t)p.unit - 1) / (size_t)p.unit;
+  p.status_first = (b_first * (size_t)m + (size_t)p.unit - 1) / (size_t)p.unit;
+  p.status_ld = p.status_first + p.units;                // at most nb + 1
+  return p;
+}
+
+qgx_status launch_encode_pipeline(qgx_ctx* c, const EncodeArgs& ea, const LevelTable& lt, const CodeTable& ct, const PhiloxKey& key,
+                                  const RoundTable& rt, const PipePlan& plan) {
+  PipeShape ps;
+  std::memset(&ps, 0, sizeof(ps));
+  ps.b_log = 31 - __builtin_clz((unsigned)ea.bucket);
+  ps.m = ea.bucket / kChunk;
+  ps.m_log = ps.b_log - 10;
+  ps.unit = plan.unit;
+  ps.u_log = 31 - __builtin_clz((unsigned)ps.unit);
+  ps.per_turn = (unsigned)(kQuantizers / ps.unit);
+  ps.units = plan.units;
+  ps.status_first = plan.status_first;
+  ps.status_ld = plan.status_ld;
+  ps.image_turns = kMaxImageTurns;
+  while (ps.image_turns > 2 && pipe_smem(ct.nlev, ct.maxlen, ps.image_turns).bytes > kPipeSmemMax) --ps.image_turns;
+  ps.smem = pipe_smem(ct.nlev, ct.maxlen, ps.image_turns);
+  ps.lane_words = (uint32_t)pipe_lane_stride(ct.maxlen);
+  ps.nlev = ct.nlev;
+  ps.weights = 4u | ((uint32_t)(8 * ct.nlev) << 16);
+  ps.neg4 = (uint32_t)ct.nlev * 0x01010101u;
+  ps.bin_copy = (16u << (rt.key_shift - kKeyShiftMin)) - 16u;
+  ps.bin_mask = ~(ps.bin_copy + 15u);
+  const unsigned long long units = (unsigned long long)ps.units * (unsigned long long)ea.K;
+  const unsigned grid = (unsigned)std::min<unsigned long long>(units, (unsigned long long)c->num_sms);
+#define QGX_LAUNCH_P(GG)                                                                              \
+  do {                                                                                                \
+    allow_max_dynamic_smem((const void*)k_encode_pipeline<GG>, c->device);                            \
+    k_encode_pipeline<GG><<<grid, kPipeThreads, ps.smem.bytes, c->stream>>>(ea, ps, lt, ct, key, rt); \
+  } while (0)
+  if (ct.G == 32) QGX_LAUNCH_P(32);
+  else if (ct.G == 64) QGX_LAUNCH_P(64);
+  else QGX_LAUNCH_P(128);
+#undef QGX_LAUNCH_P
+  return cuda_status(cudaGetLastError());
 }
 
 }  // namespace qgx

@@ -1,8 +1,7 @@
 // Fused exchange: one pass over the dual vectors writes the compact streams (quantize + encode),
 // one pass over the streams writes the mean (decode + average).  Same streams, bit for bit, and
 // the same mean as qgx_quantize -> qgx_encode -> qgx_decode -> qgx_average.
-#include "qgx_bucket.cuh"
-#include "qgx_codec.cuh"
+#include "qgx_encode.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -13,165 +12,6 @@
 #include <vector>
 
 namespace qgx {
-
-// ---- chained scan of bucket lengths ("decoupled look-back") ----------------------------------
-// status word of bucket (k, b): bits 62..63 state, bits 0..61 a word count.
-constexpr unsigned long long kStEmpty = 0ull, kStAggregate = 1ull << 62, kStPrefix = 2ull << 62;
-constexpr unsigned long long kStMask = 3ull << 62;
-
-__device__ __forceinline__ unsigned long long ld_status(const unsigned long long* p) {
-  return *reinterpret_cast<const volatile unsigned long long*>(p);
-}
-__device__ __forceinline__ void st_status(unsigned long long* p, unsigned long long v) {
-  *reinterpret_cast<volatile unsigned long long*>(p) = v;
-}
-
-// Exclusive prefix (in words) of bucket b of one worker, by warp 0 of the CTA.  Buckets are handed
-// out by a ticket counter in the order b-major, k-minor, so every predecessor (k, b') with b' < b
-// belongs to a CTA that is already running or done: the wait below always ends; it is bounded all
-// the same, and *timed_out reports a wait that ran out.
-__device__ __forceinline__ unsigned long long lookback_prefix(unsigned long long* row /* status of worker k */, long long b,
-                                                              int lane, int spin_limit, bool* timed_out) {
-  unsigned long long prefix = 0;
-  long long hi = b - 1;                                 // nearest predecessor not yet accounted for
-  int spins = 0;
-  bool fail = false;
-  while (hi >= 0 && !fail) {
-    const long long mine = hi - lane;
-    unsigned long long s = kStPrefix;                   // positions before bucket 0 act as a zero prefix
-    if (mine >= 0) s = ld_status(row + mine);
-    const unsigned empty = __ballot_sync(0xffffffffu, (s & kStMask) == kStEmpty);
-    const unsigned pref = __ballot_sync(0xffffffffu, (s & kStMask) == kStPrefix);
-    // lanes are ordered from the nearest predecessor outwards
-    const int first_pref = pref ? __ffs(pref) - 1 : 32;
-    const int first_empty = empty ? __ffs(empty) - 1 : 32;
-    if (first_empty < first_pref) {                     // a predecessor has not published yet
-      if (++spins > spin_limit) fail = true;
-      __nanosleep(64);
-      continue;
-    }
-    const int take = first_pref < 32 ? first_pref + 1 : 32;
-    unsigned long long part = lane < take ? (s & ~kStMask) : 0ull;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    prefix += part;
-    if (first_pref < 32) break;
-    hi -= 32;
-  }
-  *timed_out = fail;
-  return prefix;
-}
-
-struct EncodeArgs {
-  DualSource src;
-  size_t d;
-  int bucket;
-  int K;
-  size_t nb;
-  int norm_type;
-  uint32_t xid;
-  uint64_t quad_base;           // (index of the vector's first coordinate in the generator's counter space) / 4
-  bool vec_ok;
-  bool v_vec, a_vec;            // the workers' rows / the shared vector are 16-byte aligned (whatever d is)
-  uint32_t* stream;
-  size_t cap_words;
-  uint32_t* bucket_bits;        // [K][nb]
-  uint32_t* offsets;            // [K][nb] word offset of each bucket
-  unsigned long long* total_bits;   // [K], zeroed before the launch
-  float* norms;                 // [K][nb] (kept for the caller; the streams carry them too)
-  unsigned long long* status;   // [K][nb], zeroed before the launch
-  unsigned int* ticket;         // zeroed before the launch
-  const struct EncodeTables* tables;   // the shared-memory tables of the configuration, built once (null: every CTA builds them)
-  DevStatus* st;
-  size_t b_first;               // first bucket of every worker to encode (0 but for the diagnostic)
-  int spin_limit;               // polls of a wait for another bucket's count before it gives up
-};
-
-// Norm of the bucket held by the CTA, one barrier: per-warp partials go to shared memory and every
-// warp then reduces them in the same order (so all warps hold the same value).
-template <int V4>
-__device__ __forceinline__ float bucket_norm_all(const BucketRegs<V4>& r, int norm_type, double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  double acc = 0.0;
-  if (norm_type == QGX_NORM_L2) {
-#pragma unroll
-    for (int j = 0; j < V4; ++j) {
-      const double a = r.x[j].x, b = r.x[j].y, c = r.x[j].z, e = r.x[j].w;
-      acc = fma(a, a, acc); acc = fma(b, b, acc); acc = fma(c, c, acc); acc = fma(e, e, acc);
-    }
-    acc = warp_sum(acc);
-  } else {
-    float m = 0.0f;
-    bool bad = false;
-#pragma unroll
-    for (int j = 0; j < V4; ++j) {
-      const float4 x = r.x[j];
-      bad = bad || (x.x != x.x) || (x.y != x.y) || (x.z != x.z) || (x.w != x.w);
-      m = fmaxf(m, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
-    }
-    m = warp_max(m);
-    acc = __any_sync(0xffffffffu, bad) ? (double)__int_as_float(0x7fc00000) : (double)m;
-  }
-  if (lane == 0) red[warp] = acc;
-  __syncthreads();
-  double t = lane < nwarps ? red[lane] : 0.0;
-  if (norm_type == QGX_NORM_L2) return (float)sqrt(warp_sum(t));
-  const bool bad = __any_sync(0xffffffffu, t != t);
-  const float m = warp_max((float)t);
-  return bad ? __int_as_float(0x7fc00000) : m;
-}
-
-// Loads bucket [lo, lo + len) of worker k: warp w holds coordinates [w * 256 * P, (w + 1) * 256 * P), row j of
-// them 32 octets (8 consecutive coordinates: two quads), lane l the l-th octet of the row.
-template <int P>
-__device__ __forceinline__ void load_bucket_octets(BucketRegs<2 * P>& r, const DualSource& s, size_t k, size_t d,
-                                                   size_t lo, int len, bool vec_ok) {
-  const size_t ld = s.ld ? s.ld : d;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (vec_ok && len == 256 * P * (int)(blockDim.x >> 5)) {
-    // every lane holds full octets: the kind of source is decided once, not per quad
-    const float4* pv = s.v ? reinterpret_cast<const float4*>(s.v + k * ld + lo) + ((warp * P * 32 + lane) << 1) : nullptr;
-    const float4* pa = s.a ? reinterpret_cast<const float4*>(s.a + lo) + ((warp * P * 32 + lane) << 1) : nullptr;
-    if (pa == nullptr) {
-#pragma unroll
-      for (int j = 0; j < 2 * P; ++j) r.x[j] = __ldcs(pv + (j >> 1) * 64 + (j & 1));
-    } else if (pv == nullptr) {
-#pragma unroll
-      for (int j = 0; j < 2 * P; ++j) r.x[j] = __ldg(pa + (j >> 1) * 64 + (j & 1));
-    } else if (s.mul) {
-#pragma unroll
-      for (int j = 0; j < 2 * P; ++j) r.x[j] = dual_combine(__ldg(pa + (j >> 1) * 64 + (j & 1)), __ldcs(pv + (j >> 1) * 64 + (j & 1)), 1);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 2 * P; ++j) r.x[j] = dual_combine(__ldg(pa + (j >> 1) * 64 + (j & 1)), __ldcs(pv + (j >> 1) * 64 + (j & 1)), 0);
-    }
-    return;
-  }
-#pragma unroll
-  for (int j = 0; j < 2 * P; ++j) {
-    const int e = ((((warp * P + (j >> 1)) * 32 + lane) << 1) + (j & 1)) * kQuad;
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (e + kQuad <= len && vec_ok) {
-      if (s.a == nullptr) {
-        x = __ldcs(reinterpret_cast<const float4*>(s.v + k * ld + lo + e));
-      } else {
-        const float4 av = __ldg(reinterpret_cast<const float4*>(s.a + lo + e));
-        if (s.v) {
-          const float4 u = __ldcs(reinterpret_cast<const float4*>(s.v + k * ld + lo + e));
-          x = dual_combine(av, u, s.mul);
-        } else {
-          x = av;
-        }
-      }
-    } else {
-      if (e + 0 < len) x.x = dual_value(s, k, d, lo + e + 0);
-      if (e + 1 < len) x.y = dual_value(s, k, d, lo + e + 1);
-      if (e + 2 < len) x.z = dual_value(s, k, d, lo + e + 2);
-      if (e + 3 < len) x.w = dual_value(s, k, d, lo + e + 3);
-    }
-    r.x[j] = x;
-  }
-}
 
 // ---- rounding of one octet (eight consecutive coordinates of one lane) ---------------------------
 // The rare way through an octet, out of line: every coordinate is tested again and the ones whose outcome the
@@ -227,18 +67,6 @@ __device__ __forceinline__ uint32_t pair_entry(uint32_t pair, float z_first, flo
   const float t = fmaf(z_second, 64.0f * four_over_S, fmaf(z_first, four_over_S, 12582912.0f));   // 1.5 * 2^23 + 4 first + 256 second
   return lds_table32(pair + (__float_as_uint(t) & 0x3ffcu));
 }
-
-// The encoder's shared-memory tables as one block of global memory: built by one CTA when a configuration is first
-// used and copied by every encode CTA after that (building them costs a CTA of a small bucket more than the bucket).
-struct EncodeTables {
-  float4 bin[kBinEntries];
-  uint32_t pair[kPairLutSize];
-  EncLut lut;
-  float4 bin_fix[kBinEntries];             // the fixed-point rounding map of k_encode_pipeline
-  uint32_t pair_fix[kPairLutSize];         // its pair table, (2 nlev)^2 entries: first + 2 nlev * second, a symbol being its level,
-                                           // plus nlev for a negative coordinate
-};
-static_assert(sizeof(EncodeTables) % 16 == 0, "copied in 16-byte pieces");
 
 __global__ void __launch_bounds__(512) k_build_encode_tables(const __grid_constant__ RoundTable rt, const __grid_constant__ CodeTable ct,
                                                              EncodeTables* out) {
@@ -458,7 +286,6 @@ k_exchange_encode(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
 
 }  // namespace qgx
 
-#include "qgx_encode_pipeline.cuh"
 
 namespace qgx {
 
@@ -1105,21 +932,19 @@ struct TableCache {
 // Lets a kernel use all the dynamic shared memory that the device allows, once per kernel and device.  (The
 // attribute belongs to the function, not to a context: a per-context "largest size asked so far" would be undone
 // by another context asking for less.)
-template <typename Kernel>
-static void allow_max_dynamic_smem(Kernel kernel, int device) {
+void allow_max_dynamic_smem(const void* fn, int device) {
   struct Seen { const void* fn; int device; };
-  static Seen seen[256];                                // all template instances of a kernel share this function
+  static Seen seen[256];
   static int nseen = 0;
   static std::mutex guard;                              // contexts may be driven from different host threads
   std::lock_guard<std::mutex> lock(guard);
-  const void* fn = reinterpret_cast<const void*>(kernel);
   for (int i = 0; i < nseen; ++i)
     if (seen[i].fn == fn && seen[i].device == device) return;
   int optin = 0;
   cudaFuncAttributes fa;
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) == cudaSuccess &&
-      cudaFuncGetAttributes(&fa, kernel) == cudaSuccess && optin > (int)fa.sharedSizeBytes)
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+      cudaFuncGetAttributes(&fa, fn) == cudaSuccess && optin > (int)fa.sharedSizeBytes)
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
   else
     cudaGetLastError();
   if (nseen < 256) { seen[nseen].fn = fn; seen[nseen].device = device; ++nseen; }
@@ -1283,7 +1108,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   int per_sm = 1;
 #define QGX_LAUNCH_E(V, GG)                                                                                    \
   do {                                                                                                         \
-    allow_max_dynamic_smem(k_exchange_encode<V, GG>, c->device);                                               \
+    allow_max_dynamic_smem((const void*)k_exchange_encode<V, GG>, c->device);                                               \
     LaunchShape& shape = table_cache(c)->enc[V == 1 ? 0 : (V == 2 ? 1 : 2)][GG == 32 ? 0 : (GG == 64 ? 1 : 2)];  \
     if (shape.smem != smem + 1 + (size_t)threads * 0x100000) {   /* occupancy asked once per shape */          \
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_exchange_encode<V, GG>, threads, smem);         \
@@ -1309,30 +1134,11 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
                          (bucket != 4 * kChunk || c->encode_path == QGX_ENCODE_STAGED || nb * (size_t)K >= 4 * (size_t)c->num_sms);
   ea.b_first = std::min(c->skip_buckets, nb);
   size_t status_ld = nb;
-  PipeShape ps;
-  std::memset(&ps, 0, sizeof(ps));
+  PipePlan plan;
+  std::memset(&plan, 0, sizeof(plan));
   if (pipelined) {
-    ps.b_log = 31 - __builtin_clz((unsigned)bucket);
-    ps.m = bucket / kChunk;
-    ps.m_log = ps.b_log - 10;
-    // units of 16 chunks; fewer where that would leave SMs without any
-    const size_t chunks = (nb - ea.b_first) * (size_t)ps.m;
-    ps.unit = 16;
-    while (ps.unit > std::max(ps.m, 4) && (chunks + (size_t)ps.unit - 1) / (size_t)ps.unit * (size_t)K < 4 * (size_t)c->num_sms) ps.unit /= 2;
-    ps.u_log = 31 - __builtin_clz((unsigned)ps.unit);
-    ps.per_turn = (unsigned)(kQuantizers / ps.unit);
-    ps.units = (chunks + (size_t)ps.unit - 1) / (size_t)ps.unit;
-    ps.status_first = (ea.b_first * (size_t)ps.m + (size_t)ps.unit - 1) / (size_t)ps.unit;
-    ps.status_ld = status_ld = ps.status_first + ps.units;          // at most nb + 1
-    ps.image_turns = kMaxImageTurns;
-    while (ps.image_turns > 2 && pipe_smem(ct.nlev, ct.maxlen, ps.image_turns).bytes > kPipeSmemMax) --ps.image_turns;
-    ps.smem = pipe_smem(ct.nlev, ct.maxlen, ps.image_turns);
-    ps.lane_words = (uint32_t)pipe_lane_stride(ct.maxlen);
-    ps.nlev = ct.nlev;
-    ps.weights = 4u | ((uint32_t)(8 * ct.nlev) << 16);
-    ps.neg4 = (uint32_t)ct.nlev * 0x01010101u;
-    ps.bin_copy = (16u << (tables->rt.key_shift - kKeyShiftMin)) - 16u;
-    ps.bin_mask = ~(ps.bin_copy + 15u);
+    plan = plan_encode_pipeline(c, bucket, nb, ea.b_first, K);
+    status_ld = plan.status_ld;
   }
   if (do_encode && cudaMemsetAsync(tot, 0, sizeof(uint64_t) * ((size_t)K + 2 + (size_t)K * status_ld), c->stream) != cudaSuccess) return QGX_ERR_CUDA;
   c->skip_buckets = 0;
@@ -1340,17 +1146,8 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   if (do_encode && ea.b_first < nb) {
     ScopedKernelTimer timer(c, QGX_KERNEL_ENCODE);
     if (pipelined) {
-      const unsigned long long units = (unsigned long long)ps.units * (unsigned long long)K;
-      const unsigned grid = (unsigned)std::min<unsigned long long>(units, (unsigned long long)c->num_sms);
-#define QGX_LAUNCH_P(GG)                                                                        \
-  do {                                                                                          \
-    allow_max_dynamic_smem(k_encode_pipeline<GG>, c->device);                                   \
-    k_encode_pipeline<GG><<<grid, kPipeThreads, ps.smem.bytes, c->stream>>>(ea, ps, lt, ct, key, qt);   \
-  } while (0)
-      if (ct.G == 32) QGX_LAUNCH_P(32);
-      else if (ct.G == 64) QGX_LAUNCH_P(64);
-      else QGX_LAUNCH_P(128);
-#undef QGX_LAUNCH_P
+      rc = launch_encode_pipeline(c, ea, lt, ct, key, qt, plan);
+      if (rc != QGX_OK) return rc;
     } else {
       switch (pp) {
         case 1: QGX_LAUNCH_EG(1); break;
@@ -1443,7 +1240,7 @@ static qgx_status launch_decode_gs(qgx_ctx* c, const DecodeArgs& da, const CodeT
   int per_sm = 1;
   {
     ScopedKernelTimer timer(c, QGX_KERNEL_DECODE);
-    allow_max_dynamic_smem(k_exchange_decode<G, SYM, VAL>, c->device);
+    allow_max_dynamic_smem((const void*)k_exchange_decode<G, SYM, VAL>, c->device);
     TableCache* tc = table_cache(c);
     LaunchShape& shape = (VAL ? tc->dec : tc->dec_walk)[G == 32 ? 0 : (G == 64 ? 1 : 2)][SYM];
     if (shape.smem != lut_bytes + 1) {                       // occupancy asked once per shape, not per call

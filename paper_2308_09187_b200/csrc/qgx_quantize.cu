@@ -1,95 +1,302 @@
 // qgx_quantize (Definition 1 per bucket) and qgx_average (the aggregation of Algorithm 1).
 #include "qgx_bucket.cuh"
+#include "qgx_codec.cuh"
+
+#include <algorithm>
+#include <cstring>
+#include <new>
+#include <vector>
 
 namespace qgx {
 
-// One CTA per (bucket, worker).  The bucket stays in registers between the norm reduction and
-// the rounding pass, so v is read from HBM exactly once.
-template <int V4>
-__global__ void __launch_bounds__(512) k_quantize(DualSource src, size_t d, int bucket, const __grid_constant__ LevelTable lt,
-                                                   const __grid_constant__ PhiloxKey key, const __grid_constant__ RoundTable rt,
-                                                   uint32_t xid, int norm_type, int norms_supplied, bool vec_ok,
-                                                   float* __restrict__ norms, uint8_t* __restrict__ sym, DevStatus* st) {
-  __shared__ float s_lev[QGX_MAX_LEVELS];
-  __shared__ float4 s_bin[kBinEntries];
-  fill_bin_table(s_bin, rt);
-  __shared__ double s_red[34];
-  const size_t b = blockIdx.x, k = blockIdx.y;
-  const size_t nb = gridDim.x;
-  const size_t lo = b * (size_t)bucket;
-  const int len = (int)min((size_t)bucket, d - lo);
-  if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
+// ---- what the separate calls derive from their levels and codes, kept between calls ---------------
+// Building the rounding table costs the host some 50 us, the decoder table a copy to the device: a program calls with a
+// handful of tables, so a context keeps the last few (compared in full on a hit).
+struct StepLevels {
+  bool valid;
+  int nlev;
+  float lev[QGX_MAX_LEVELS];
+  RoundTable rt;
+  float4* bins;                          // [dev] the fixed-point map's bin table, owned
+};
+struct StepCode {
+  bool valid;
+  int bucket;
+  qgx_codebook cb;
+  CodeTable ct;
+  uint16_t* lut;                         // [dev] decoder table, owned
+};
+constexpr int kStepSlots = 8;
+struct StepCache {
+  StepLevels lev[kStepSlots];
+  StepCode code[kStepSlots];
+};
 
-  BucketRegs<V4> r;
-  load_bucket<V4>(r, src, k, d, lo, len, vec_ok);
-  float norm;
-  if (norms_supplied) {
-    norm = norms[k * nb + b];
-    __syncthreads();
-  } else {
-    norm = bucket_norm<V4>(r, norm_type, s_red);
-    if (threadIdx.x == 0) norms[k * nb + b] = norm;
+__global__ void __launch_bounds__(512) k_build_bins(const __grid_constant__ RoundTable rt, float4* out) {
+  fill_bin_table(out, rt, BinKind::kFixed);
+}
+
+static StepCache* step_cache(qgx_ctx* c) {
+  if (!c->step_cache) c->step_cache = new (std::nothrow) StepCache();          // value-initialized: all zero
+  return (StepCache*)c->step_cache;
+}
+void free_step_cache(qgx_ctx* c) {
+  StepCache* sc = (StepCache*)c->step_cache;
+  if (!sc) return;
+  for (int i = 0; i < kStepSlots; ++i) {
+    if (sc->lev[i].bins) cudaFree(sc->lev[i].bins);
+    if (sc->code[i].lut) cudaFree(sc->code[i].lut);
   }
-  const bool finite = (norm - norm) == 0.0f;
-  if (!finite && threadIdx.x == 0) latch_error(st, QGX_ERR_NONFINITE);
-  const RoundConsts rc = round_consts(rt, norm);
+  delete sc;
+  c->step_cache = nullptr;
+}
+static uint32_t mix_bytes(uint32_t h, const void* p, size_t n) {
+  const unsigned char* b = (const unsigned char*)p;
+  for (size_t i = 0; i < n; ++i) { h ^= b[i]; h *= 16777619u; }
+  return h;
+}
 
-  uint8_t* out = sym + k * d + lo;
-  const bool sym_vec = vec_ok;            // d % 4 == 0 and bucket % 4 == 0: every quad is 4-byte aligned
-#pragma unroll
-  for (int j = 0; j < V4; ++j) {
-    const int q = j * (int)blockDim.x + (int)threadIdx.x;
-    const int e = q * kQuad;
-    if (e >= len) continue;
-    uint32_t packed = 0;
-    if (finite && norm != 0.0f) {
-      const uint64_t ctr = (uint64_t)(lo >> 2) + (uint64_t)q;      // (coordinate index) / 4
-      const uint4 w = philox4x32_10((uint32_t)ctr, (uint32_t)(ctr >> 32), (uint32_t)k, xid, key);
-      const float4 x = r.x[j];
-      const uint32_t code4 = quantize_quad_codes(x, w, rc, norm, s_bin, s_lev, lt.nlev);
-      packed = (code4 & 0x1f1f1f1fu) | ((code4 & 0x20202020u) << 2);      // symbol bytes: level | sign << 7
+static qgx_status step_levels(qgx_ctx* c, const float* lev, int nlev, const StepLevels** out) {
+  StepCache* sc = step_cache(c);
+  if (!sc) return QGX_ERR_CUDA;
+  StepLevels* e = &sc->lev[mix_bytes(2166136261u, lev, sizeof(float) * (size_t)nlev) % kStepSlots];
+  if (!(e->valid && e->nlev == nlev && std::memcmp(e->lev, lev, sizeof(float) * (size_t)nlev) == 0)) {
+    e->valid = false;
+    make_round_table(lev, nlev, &e->rt);
+    if (!e->bins && cudaMalloc((void**)&e->bins, sizeof(float4) * kBinEntries) != cudaSuccess) {
+      cudaGetLastError();
+      e->bins = nullptr;
+      return QGX_ERR_CUDA;
     }
-    if (e + kQuad <= len && sym_vec) {
-      *reinterpret_cast<uint32_t*>(out + e) = packed;
+    k_build_bins<<<1, 512, 0, c->stream>>>(e->rt, e->bins);           // ordered after the kernels that still read the old one
+    count_launch(c);
+    if (cudaGetLastError() != cudaSuccess) return QGX_ERR_CUDA;
+    e->nlev = nlev;
+    std::memcpy(e->lev, lev, sizeof(float) * (size_t)nlev);
+    e->valid = true;
+  }
+  *out = e;
+  return QGX_OK;
+}
+
+qgx_status step_code(qgx_ctx* c, const qgx_codebook* cb, int bucket, const CodeTable** ct, const uint16_t** lut) {
+  StepCache* sc = step_cache(c);
+  if (!sc) return QGX_ERR_CUDA;
+  if (cb == nullptr || cb->nlev < 2 || cb->nlev > QGX_MAX_LEVELS) return QGX_ERR_INVALID_ARG;
+  uint32_t h = mix_bytes(2166136261u, cb->len, (size_t)cb->nlev);
+  h = mix_bytes(mix_bytes(h, &cb->subblock, sizeof(int)), &bucket, sizeof(int));
+  StepCode* e = &sc->code[h % kStepSlots];
+  if (!(e->valid && e->bucket == bucket && e->cb.nlev == cb->nlev && e->cb.subblock == cb->subblock &&
+        std::memcmp(e->cb.len, cb->len, (size_t)cb->nlev) == 0 && std::memcmp(e->cb.code, cb->code, sizeof(uint32_t) * (size_t)cb->nlev) == 0)) {
+    e->valid = false;
+    const qgx_status rc = make_code_table(cb, bucket, &e->ct);
+    if (rc != QGX_OK) return rc;
+    if (!e->lut && cudaMalloc((void**)&e->lut, sizeof(uint16_t) << QGX_MAX_CODE_LEN) != cudaSuccess) {
+      cudaGetLastError();
+      e->lut = nullptr;
+      return QGX_ERR_CUDA;
+    }
+    std::vector<uint16_t> table((size_t)1 << e->ct.maxlen);
+    build_dec_lut_host(e->ct, table.data());
+    // pageable source: the runtime stages it before returning, so the vector may go out of scope
+    if (cudaMemcpyAsync(e->lut, table.data(), table.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
+      return QGX_ERR_CUDA;
+    e->bucket = bucket;
+    e->cb = *cb;
+    e->valid = true;
+  }
+  *ct = &e->ct;
+  *lut = e->lut;
+  return QGX_OK;
+}
+
+struct QuantizeArgs {
+  DualSource src;
+  size_t d;
+  int bucket;
+  size_t nb, total;                      // buckets per worker, of all workers
+  int norm_type, norms_supplied;
+  uint32_t xid;
+  bool vec_ok;                           // 16-byte loads
+  int store;                             // bytes per symbol store: 8, 4 or 1
+  const float4* bins;
+  float* norms;
+  uint8_t* sym;
+  DevStatus* st;
+};
+
+// Persistent CTAs, one bucket at a time held in registers between the norm and the rounding (v is read from HBM once); a
+// thread works on P octets of consecutive coordinates.  What bounds it: instruction issue -- about 26 instructions per
+// coordinate are the generator and the rounding map.  The map's table comes ready made from global memory, once per CTA:
+// built by every CTA for its one bucket, as before, it cost more than a small bucket.
+template <int P>
+__global__ void __launch_bounds__(P == 1 ? 256 : 512, P == 1 ? 4 : 2)
+k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ LevelTable lt, const __grid_constant__ PhiloxKey key,
+           const __grid_constant__ RoundTable rt) {
+  __shared__ __align__(128) float4 s_bin[kBinEntries];
+  __shared__ float s_lev[QGX_MAX_LEVELS];
+  __shared__ double s_red[2][32];
+  for (int i = threadIdx.x; i < kBinEntries; i += blockDim.x) s_bin[i] = __ldg(a.bins + i);
+  if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t lev_sa = smem_addr(s_lev);
+  RoundFix rc;
+  const uint32_t copies = 16u << (rt.key_shift - kKeyShiftMin);
+  rc.mask = ~(copies - 1u);
+  rc.base = smem_addr(s_bin) - kBinAddrBase + (((uint32_t)lane << 4) & (copies - 1u));
+  int par = 0;
+  for (size_t t = blockIdx.x; t < a.total; t += gridDim.x, par ^= 1) {
+    const size_t k = a.total <= 0xffffffffull ? (size_t)((uint32_t)t / (uint32_t)a.nb) : t / a.nb;
+    const uint32_t ku = (uint32_t)k;
+    const size_t lo = (t - k * a.nb) * (size_t)a.bucket;
+    const int len = (int)min((size_t)a.bucket, a.d - lo);
+    BucketRegs<2 * P> r;
+    load_bucket_octets<P>(r, a.src, k, a.d, lo, len, a.vec_ok);
+    float norm;
+    if (a.norms_supplied) {
+      norm = a.norms[t];
     } else {
-      for (int c = 0; c < kQuad && e + c < len; ++c) out[e + c] = (uint8_t)(packed >> (8 * c));
+      norm = bucket_norm_all<2 * P>(r, a.norm_type, s_red[par]);
+      if (threadIdx.x == 0) a.norms[t] = norm;
+    }
+    const bool finite = (norm - norm) == 0.0f;
+    if (!finite && threadIdx.x == 0) latch_error(a.st, QGX_ERR_NONFINITE);
+    const bool live = finite && norm != 0.0f;
+    const bool fast = rt.usable && norm > 7.9e-31f && norm < 1.2e30f;
+    rc.rn = fast ? __frcp_rn(norm) : 0.0f;
+    rc.thr = fast ? rt.thrfix : 0x10000u;
+    uint8_t* out = a.sym + k * a.d + lo;
+    const uint64_t q0 = (uint64_t)(lo >> 2);
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+      const int o = (warp * P + j) * 32 + lane, e = 8 * o;
+      if (e >= len) continue;
+      uint32_t sy[2] = {0u, 0u};
+      if (live) {
+        const uint64_t ctr = q0 + 2ull * (uint64_t)o;
+        uint32_t w[8];
+        if ((uint32_t)ctr != 0xffffffffu) {
+          philox_pair((uint32_t)ctr, philox_shared((uint32_t)(ctr >> 32), ku, a.xid, key), key, w);
+        } else {
+          uint4 wa, wb;
+          philox4x32_10_x2(ctr, ctr + 1ull, ku, a.xid, key, &wa, &wb);
+          w[0] = wa.x; w[1] = wa.y; w[2] = wa.z; w[3] = wa.w; w[4] = wb.x; w[5] = wb.y; w[6] = wb.z; w[7] = wb.w;
+        }
+        const float x[8] = {r.x[2 * j].x, r.x[2 * j].y, r.x[2 * j].z, r.x[2 * j].w, r.x[2 * j + 1].x, r.x[2 * j + 1].y, r.x[2 * j + 1].z, r.x[2 * j + 1].w};
+        uint32_t d[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) d[i] = round_fixed<true>(x[i], w[i], rc);        // a supplied norm may be smaller than |v|
+        uint32_t m = min_u16x2(prmt(d[0], d[1], 0x5410u), prmt(d[2], d[3], 0x5410u));
+        m = min_u16x2(min_u16x2(prmt(d[4], d[5], 0x5410u), prmt(d[6], d[7], 0x5410u)), m);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          sy[q] = prmt(prmt(d[4 * q], d[4 * q + 1], 0x0062u), prmt(d[4 * q + 2], d[4 * q + 3], 0x0062u), 0x5410u) & 0x1f1f1f1fu;
+        if (min(m & 0xffffu, m >> 16) < rc.thr) {
+          // some coordinate needs the exact routine: its inputs are fetched again, one coordinate at a time
+          uint32_t todo = 0;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) todo |= (d[i] & 0xffffu) < rc.thr ? 1u << i : 0u;
+#pragma unroll 1
+          while (todo) {
+            const uint32_t i = (uint32_t)__ffs((int)todo) - 1u;
+            todo &= todo - 1u;
+            if (e + (int)i >= len) continue;
+            const float xv = dual_value(a.src, k, a.d, lo + (size_t)e + i);
+            const uint32_t r24 = variate_bits(4ull * ctr + i, ku, a.xid, key);
+            const uint32_t sh = 8u * (i & 3u), was = i < 4u ? sy[0] : sy[1];
+            const uint32_t fixed = level_exact_near(fabsf(xv), norm, r24, (int)((was >> sh) & 0x1fu), lev_sa, lt.nlev);
+            const uint32_t put = (was & ~(0xffu << sh)) | (fixed << sh);
+            if (i < 4u) sy[0] = put; else sy[1] = put;
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {                                  // the sign of a nonzero level at bit 7
+          const uint32_t s4 = prmt(prmt(__float_as_uint(x[4 * q]), __float_as_uint(x[4 * q + 1]), 0x00fbu),
+                                   prmt(__float_as_uint(x[4 * q + 2]), __float_as_uint(x[4 * q + 3]), 0x00fbu), 0x5410u);
+          sy[q] |= s4 & (sy[q] + 0x7f7f7f7fu) & 0x80808080u;
+        }
+      }
+      if (e + 8 <= len && a.store == 8) {
+        *reinterpret_cast<uint2*>(out + e) = make_uint2(sy[0], sy[1]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          if (e + 4 * q + 4 <= len && a.store >= 4) *reinterpret_cast<uint32_t*>(out + e + 4 * q) = sy[q];
+          else
+            for (int i = 0; i < 4; ++i)
+              if (e + 4 * q + i < len) out[e + 4 * q + i] = (uint8_t)(sy[q] >> (8 * i));
+        }
+      }
     }
   }
 }
 
-// out[i] = (sum_k vhat[k][i]) / K, the sum taken in the order k = 0..K-1; one thread per quad.
-__global__ void __launch_bounds__(256) k_average(const float* __restrict__ norms, const uint8_t* __restrict__ sym, int K,
-                                                 size_t d, int bucket, size_t nb, LevelTable lt, bool vec_ok,
-                                                 float* __restrict__ out, DevStatus* st) {
-  __shared__ float s_lev[QGX_MAX_LEVELS];
-  if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 0.0f;
+// out[i] = (sum_k vhat[k][i]) / K, the sum taken in the order k = 0..K-1.  A thread takes V consecutive coordinates of one
+// bucket (V = 16: one 16-byte load of symbols per worker), two workers' loads ahead of the additions; the level values are
+// read from a table with one copy per lane (bank = lane).  Memory-bound in principle (K symbol bytes and 4 output bytes per
+// coordinate); the version before divided by the bucket size for every coordinate and worker.
+template <int V>
+__global__ void __launch_bounds__(256) k_average(const float* __restrict__ norms, const uint8_t* __restrict__ sym, int K, size_t d,
+                                                 int bucket, size_t nb, const __grid_constant__ LevelTable lt, float* __restrict__ out, DevStatus* st) {
+  __shared__ float s_lev[QGX_MAX_LEVELS * 32];
+  for (int i = threadIdx.x; i < QGX_MAX_LEVELS * 32; i += blockDim.x) s_lev[i] = (i >> 5) < lt.nlev ? lt.lev[i >> 5] : 0.0f;
   __syncthreads();
-  const size_t nquads = (d + kQuad - 1) / kQuad;
+  const size_t groups = (d + V - 1) / V;
   const float Kf = (float)K;
-  bool bad = false;
-  for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < nquads; q += (size_t)gridDim.x * blockDim.x) {
-    const size_t e = q * kQuad;
-    const int nval = (int)min((size_t)kQuad, d - e);
-    float acc[kQuad] = {0.f, 0.f, 0.f, 0.f};
-    for (int k = 0; k < K; ++k) {
-      uint32_t packed = 0;
-      if (nval == kQuad && vec_ok) {
-        packed = __ldcs(reinterpret_cast<const uint32_t*>(sym + (size_t)k * d + e));
-      } else {
-        for (int c = 0; c < nval; ++c) packed |= (uint32_t)sym[(size_t)k * d + e + c] << (8 * c);
-      }
+  const uint32_t lev_sa = smem_addr(s_lev) + 4u * (threadIdx.x & 31u);
+  const uint32_t limit4 = (uint32_t)(128 - lt.nlev) * 0x01010101u;    // carries into bit 7 of a byte >= nlev
+  uint32_t bad = 0;
+  for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < groups; g += (size_t)gridDim.x * blockDim.x) {
+    const size_t e = g * V;
+    float acc[V];
 #pragma unroll
-      for (int c = 0; c < kQuad; ++c) {
-        if (c < nval) {
-          const uint32_t s = (packed >> (8 * c)) & 0xffu;
-          bad = bad || ((s & 31u) >= (uint32_t)lt.nlev);
-          // a bucket never splits a quad when bucket % 4 == 0, but the tail of d may
-          const float norm = norms[(size_t)k * nb + (e + c) / (size_t)bucket];
-          acc[c] = __fadd_rn(acc[c], dequantize_symbol(s, norm, s_lev));
+    for (int i = 0; i < V; ++i) acc[i] = 0.0f;
+    // the bucket of the group (V = 16: the host sees to it that no bucket ends inside a group)
+    const size_t b = d <= 0xffffffffull ? (size_t)((uint32_t)e / (uint32_t)bucket) : e / (size_t)bucket;
+    if constexpr (V == 16) {
+      const uint4* p = reinterpret_cast<const uint4*>(sym + e);
+      const size_t ld = d / 16;
+      auto add = [&](const uint4 q, float norm) {
+        const uint32_t wd[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          bad |= ((wd[j] & 0x1f1f1f1fu) + limit4) & 0x80808080u;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint32_t s = (wd[j] >> (8 * i)) & 0xffu;
+            const float val = __fmul_rn(norm, __uint_as_float(lds_table32(lev_sa + ((s & 31u) << 7))));
+            acc[4 * j + i] = __fadd_rn(acc[4 * j + i], __uint_as_float(__float_as_uint(val) ^ ((s & 0x80u) << 24)));
+          }
+        }
+      };
+      int k = 0;
+      for (; k + 1 < K; k += 2) {
+        const uint4 q0 = __ldcs(p + (size_t)k * ld), q1 = __ldcs(p + (size_t)(k + 1) * ld);
+        const float n0 = norms[(size_t)k * nb + b], n1 = norms[(size_t)(k + 1) * nb + b];
+        add(q0, n0);
+        add(q1, n1);
+      }
+      if (k < K) add(__ldcs(p + (size_t)k * ld), norms[(size_t)k * nb + b]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        *reinterpret_cast<float4*>(out + e + 4 * j) = make_float4(__fdiv_rn(acc[4 * j], Kf), __fdiv_rn(acc[4 * j + 1], Kf), __fdiv_rn(acc[4 * j + 2], Kf), __fdiv_rn(acc[4 * j + 3], Kf));
+    } else {
+#pragma unroll 4
+      for (int k = 0; k < K; ++k) {
+        const uint32_t wd = V == 4 ? __ldcs(reinterpret_cast<const uint32_t*>(sym + (size_t)k * d + e)) : (uint32_t)sym[(size_t)k * d + e];
+        const float norm = norms[(size_t)k * nb + b];
+        bad |= ((wd & 0x1f1f1f1fu) + limit4) & 0x80808080u;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+          const uint32_t s = (wd >> (8 * i)) & 0xffu;
+          const float val = __fmul_rn(norm, __uint_as_float(lds_table32(lev_sa + ((s & 31u) << 7))));
+          acc[i] = __fadd_rn(acc[i], __uint_as_float(__float_as_uint(val) ^ ((s & 0x80u) << 24)));
         }
       }
+#pragma unroll
+      for (int i = 0; i < V; ++i) out[e + i] = __fdiv_rn(acc[i], Kf);
     }
-    for (int c = 0; c < nval; ++c) out[e + c] = __fdiv_rn(acc[c], Kf);
   }
   if (bad) latch_error(st, QGX_ERR_CORRUPT);
 }
@@ -103,24 +310,28 @@ static bool all_aligned16(std::initializer_list<const void*> ps) {
 qgx_status launch_quantize(qgx_ctx* c, DualSource src, int K, size_t d, int bucket, const LevelTable& lt, int norm_type,
                            uint64_t seed, uint32_t xid, int norms_supplied, float* norms, uint8_t* sym) {
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
-  const bool vec_ok = (d % kQuad == 0) && all_aligned16({src.v, src.a}) &&
-                      ((reinterpret_cast<uintptr_t>(sym) & 3u) == 0);
+  const StepLevels* tables = nullptr;
+  const qgx_status rc = step_levels(c, lt.lev, lt.nlev, &tables);
+  if (rc != QGX_OK) return rc;
   const PhiloxKey key = make_philox_key(seed);
-  RoundTable qt;
-  make_round_table(lt.lev, lt.nlev, &qt);
-  const int v4 = bucket_v4(bucket);
-  const dim3 grid((unsigned)nb, (unsigned)K);
-  const int threads = bucket_threads(bucket, v4);
-#define QGX_LAUNCH_Q(V)                                                                                      \
-  k_quantize<V><<<grid, threads, 0, c->stream>>>(src, d, bucket, lt, key, qt, xid, norm_type, norms_supplied, \
-                                                 vec_ok, norms, sym, c->dstatus)
-  switch (v4) {
-    case 1: QGX_LAUNCH_Q(1); break;
-    case 2: QGX_LAUNCH_Q(2); break;
-    case 4: QGX_LAUNCH_Q(4); break;
-    default: QGX_LAUNCH_Q(8); break;
+  QuantizeArgs a;
+  a.src = src; a.d = d; a.bucket = bucket; a.nb = nb; a.total = nb * (size_t)K;
+  a.norm_type = norm_type; a.norms_supplied = norms_supplied; a.xid = xid;
+  a.vec_ok = (d % kQuad == 0) && all_aligned16({src.v, src.a});
+  const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
+  a.store = (d % 8 == 0 && bucket % 8 == 0 && (at & 7u) == 0) ? 8 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
+  a.bins = tables->bins; a.norms = norms; a.sym = sym; a.st = c->dstatus;
+  // octets per thread so that CTAs have at most 256 / 512 / 512 threads; as many CTAs as an SM holds (registers: 1024
+  // threads; shared memory: 12 tables of 17 KB)
+  const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
+  const int threads = bucket_threads(bucket, 2 * pp);
+  const unsigned per_sm = (unsigned)std::min(12, std::max(2, 1024 / threads));
+  const unsigned grid = (unsigned)std::min<size_t>(a.total, (size_t)c->num_sms * per_sm);
+  switch (pp) {
+    case 1: k_quantize<1><<<grid, threads, 0, c->stream>>>(a, lt, key, tables->rt); break;
+    case 2: k_quantize<2><<<grid, threads, 0, c->stream>>>(a, lt, key, tables->rt); break;
+    default: k_quantize<4><<<grid, threads, 0, c->stream>>>(a, lt, key, tables->rt); break;
   }
-#undef QGX_LAUNCH_Q
   count_launch(c);
   return cuda_status(cudaGetLastError());
 }
@@ -155,11 +366,14 @@ qgx_status qgx_average(qgx_ctx* c, const float* norms, const uint8_t* sym, int K
   lt.nlev = nlev;
   for (int j = 0; j < QGX_MAX_LEVELS; ++j) lt.lev[j] = j < nlev ? levels[j] : 0.0f;
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
-  const size_t nquads = (d + kQuad - 1) / kQuad;
-  const bool vec_ok = (d % kQuad == 0) && ((reinterpret_cast<uintptr_t>(sym) & 3u) == 0);
-  const int threads = 256;
-  const unsigned blocks = (unsigned)std::min<size_t>((nquads + threads - 1) / threads, (size_t)c->num_sms * 16u);
-  k_average<<<blocks, threads, 0, c->stream>>>(norms, sym, K, d, bucket, nb, lt, vec_ok, out, c->dstatus);
+  // sixteen coordinates per thread where symbols come in whole 16-byte pieces and no bucket ends inside one
+  const bool wide = d % 16 == 0 && bucket % 16 == 0 && all_aligned16({sym, out});
+  const bool quads = d % 4 == 0 && bucket % 4 == 0 && (reinterpret_cast<uintptr_t>(sym) & 3u) == 0;
+  const size_t groups = wide ? d / 16 : (quads ? d / 4 : d);
+  const unsigned blocks = (unsigned)std::min<size_t>((groups + 255) / 256, (size_t)c->num_sms * 16u);
+  if (wide) k_average<16><<<blocks, 256, 0, c->stream>>>(norms, sym, K, d, bucket, nb, lt, out, c->dstatus);
+  else if (quads) k_average<4><<<blocks, 256, 0, c->stream>>>(norms, sym, K, d, bucket, nb, lt, out, c->dstatus);
+  else k_average<1><<<blocks, 256, 0, c->stream>>>(norms, sym, K, d, bucket, nb, lt, out, c->dstatus);
   count_launch(c);
   return cuda_status(cudaGetLastError());
 }
