@@ -3,6 +3,7 @@
 #include "qgx_bucket.cuh"
 #include "qgx_codec.cuh"
 
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
@@ -68,43 +69,54 @@ __global__ void __launch_bounds__(512) k_bucket_bits(const uint8_t* __restrict__
 }
 
 // One CTA per worker: off[k][b] = sum_{b' < b} ceil(bits[k][b'] / 32); total_bits[k]; a worker whose
-// words exceed cap_words is flagged (flags[k] = 1) and err_code is latched.
-__global__ void __launch_bounds__(256) k_scan_offsets(const uint32_t* __restrict__ bucket_bits, size_t nb, size_t cap_words,
-                                                      uint64_t* __restrict__ off, uint64_t* __restrict__ total_bits,
-                                                      uint32_t* __restrict__ flags, unsigned int err_code, DevStatus* st) {
-  __shared__ uint64_t s_words[8], s_bits[8];
-  __shared__ uint64_t s_carry_w, s_carry_b;
+// words exceed cap_words is flagged (flags[k] = 1) and err_code is latched.  4096 buckets per turn of the loop: a worker's
+// lengths are a serial chain of turns, each a few barriers long.
+constexpr int kScanThreads = 1024, kScanEach = 4;
+__global__ void __launch_bounds__(kScanThreads) k_scan_offsets(const uint32_t* __restrict__ bucket_bits, size_t nb, size_t cap_words,
+                                                               uint64_t* __restrict__ off, uint64_t* __restrict__ total_bits,
+                                                               uint32_t* __restrict__ flags, unsigned int err_code, DevStatus* st) {
+  __shared__ uint64_t s_words[2][32], s_bits[2][32];
   const size_t k = blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  if (threadIdx.x == 0) { s_carry_w = 0; s_carry_b = 0; }
-  __syncthreads();
-  for (size_t base = 0; base < nb; base += blockDim.x) {
-    const size_t b = base + threadIdx.x;
-    const uint64_t bits = b < nb ? (uint64_t)bucket_bits[k * nb + b] : 0ull;
-    const uint64_t words = (bits + 31) >> 5;
-    uint64_t iw = words, ib = bits;                     // warp-inclusive scans of words and bits
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint64_t carry_w = 0, carry_b = 0;
+  int par = 0;
+  for (size_t base = 0; base < nb; base += kScanThreads * kScanEach, par ^= 1) {
+    const size_t b0 = base + (size_t)threadIdx.x * kScanEach;
+    uint32_t bits[kScanEach];
+    uint64_t words = 0, sum = 0;
+#pragma unroll
+    for (int j = 0; j < kScanEach; ++j) {
+      bits[j] = b0 + j < nb ? bucket_bits[k * nb + b0 + j] : 0u;
+      words += ((uint64_t)bits[j] + 31) >> 5;
+      sum += bits[j];
+    }
+    uint64_t iw = words, ib = sum;                      // warp-inclusive scans of words and bits
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint64_t yw = __shfl_up_sync(0xffffffffu, iw, o), yb = __shfl_up_sync(0xffffffffu, ib, o);
       if (lane >= o) { iw += yw; ib += yb; }
     }
-    if (lane == 31) { s_words[warp] = iw; s_bits[warp] = ib; }
-    __syncthreads();
-    uint64_t before = s_carry_w;
-    for (int w = 0; w < warp; ++w) before += s_words[w];
-    if (b < nb) off[k * nb + b] = before + iw - words;
-    __syncthreads();                                    // every thread has read the carry
-    if (threadIdx.x == 0) {
-      uint64_t tw = 0, tb = 0;
-      for (int w = 0; w < nwarps; ++w) { tw += s_words[w]; tb += s_bits[w]; }
-      s_carry_w += tw;
-      s_carry_b += tb;
+    if (lane == 31) { s_words[par][warp] = iw; s_bits[par][warp] = ib; }
+    __syncthreads();                                    // (double-buffered: the next turn writes the other half)
+    uint64_t tw = s_words[par][lane], tb = s_bits[par][lane];
+    const uint64_t mine_w = tw;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t yw = __shfl_up_sync(0xffffffffu, tw, o), yb = __shfl_up_sync(0xffffffffu, tb, o);
+      if (lane >= o) { tw += yw; tb += yb; }
     }
-    __syncthreads();
+    uint64_t at = carry_w + __shfl_sync(0xffffffffu, tw - mine_w, warp) + iw - words;
+#pragma unroll
+    for (int j = 0; j < kScanEach; ++j) {
+      if (b0 + j < nb) off[k * nb + b0 + j] = at;
+      at += ((uint64_t)bits[j] + 31) >> 5;
+    }
+    carry_w += __shfl_sync(0xffffffffu, tw, 31);
+    carry_b += __shfl_sync(0xffffffffu, tb, 31);
   }
   if (threadIdx.x == 0) {
-    if (total_bits) total_bits[k] = s_carry_b;
-    const bool over = s_carry_w > (uint64_t)cap_words;
+    if (total_bits) total_bits[k] = carry_b;
+    const bool over = carry_w > (uint64_t)cap_words;
     flags[k] = over ? 1u : 0u;
     if (over) latch_error(st, err_code);
   }
@@ -185,89 +197,315 @@ __global__ void __launch_bounds__(512) k_bit_scatter(const float* __restrict__ n
   for (uint32_t i = threadIdx.x; i < nwords; i += blockDim.x) dst[i] = s_img[i];
 }
 
-// One CTA per (bucket, worker); one thread per sub-block walks its part of the stream.
-__global__ void __launch_bounds__(256) k_decode(const uint32_t* __restrict__ stream, size_t cap_words,
-                                                const uint32_t* __restrict__ bucket_bits, const uint64_t* __restrict__ off,
-                                                const uint32_t* __restrict__ flags, size_t d, int bucket, CodeTable ct,
-                                                const uint16_t* __restrict__ g_lut, bool vec_ok, float* __restrict__ norms,
-                                                uint8_t* __restrict__ sym, DevStatus* st) {
-  extern __shared__ uint32_t s_dyn[];
-  const size_t b = blockIdx.x, k = blockIdx.y, nb = gridDim.x;
-  const size_t lo = b * (size_t)bucket;
-  const int len = (int)min((size_t)bucket, d - lo);
-  const int lane = threadIdx.x & 31;
-  const uint32_t nsub = ct.has_header ? (uint32_t)((len + ct.G - 1) / ct.G) : 1u;
-  const uint32_t hdr_bits = kNormBits + (ct.has_header ? 16u * nsub : 0u);
-  uint32_t* s_start = s_dyn;                            // nsub + 1 payload-relative start bits
-  uint16_t* s_lut = reinterpret_cast<uint16_t*>(s_dyn + (bucket / ct.G + 2));
-  const int lut_n = 1 << ct.maxlen;
-  for (int i = threadIdx.x; i < lut_n; i += blockDim.x) s_lut[i] = g_lut[i];
+// ---- encode in one pass ----------------------------------------------------------------------------
+// The status word of a bucket in the look-back carries two sums at once: words in bits 0..32, unused bits at the ends of
+// the buckets' last words in bits 33..61 -- so the last bucket of a worker knows the stream's bits, too.
+constexpr int kPadShift = 33;
 
-  uint8_t* out = sym + k * d + lo;
-  const bool dead = flags[k] != 0;
-  const uint32_t nbits = dead ? 0u : bucket_bits[k * nb + b];
-  const uint32_t nwords = (nbits + 31) >> 5;
-  const uint32_t* w = stream + k * cap_words + (dead ? 0 : off[k * nb + b]);
-  bool bad = !dead && nbits < hdr_bits;
-  if (dead || bad) {                                    // nothing trustworthy to read: zero output
-    for (int i = threadIdx.x; i < len; i += blockDim.x) out[i] = 0;
-    if (threadIdx.x == 0) { norms[k * nb + b] = 0.0f; if (bad) latch_error(st, QGX_ERR_CORRUPT); }
-    return;
-  }
-  if (threadIdx.x == 0) norms[k * nb + b] = __uint_as_float(w[0]);
-  // start bit of every sub-block: exclusive scan of the 16-bit header fields
-  if (threadIdx.x < 32) {
-    uint32_t carry = 0;
-    if (ct.has_header) {
-      for (uint32_t base = 0; base < nsub; base += 32) {
-        const uint32_t s = base + lane;
-        uint32_t L = 0;
-        if (s < nsub) {
-          const uint32_t bit = kNormBits + 16u * s;
-          L = (w[bit >> 5] >> (bit & 31u)) & 0xffffu;   // inside the header, which nbits covers
-        }
-        const uint32_t incl = warp_incl_scan(L, lane);
-        if (s < nsub) s_start[s] = carry + incl - L;
-        carry += __shfl_sync(0xffffffffu, incl, 31);
-      }
-    } else {
-      if (lane == 0) s_start[0] = 0;
-      carry = nbits - hdr_bits;
-    }
-    if (lane == 0) s_start[nsub] = carry;
+struct PackArgs {
+  const float* norms;
+  const uint8_t* sym;
+  size_t d;
+  int bucket, K;
+  size_t nb;
+  int load;                              // bytes per symbol load: 8, 4 or 1
+  uint32_t* stream;
+  size_t cap_words;
+  uint32_t* bucket_bits;
+  uint64_t* total_bits;
+  unsigned long long* status;            // [K][nb], zeroed before the launch
+  unsigned int* ticket;                  // zeroed before the launch
+  int spin_limit;
+  DevStatus* st;
+};
+
+// Persistent CTAs, a bucket at a time (in the order b-major, k-minor, by a ticket counter: see lookback_prefix), P octets of
+// eight symbols per thread.  One pass over the symbols instead of three kernels and two passes; the symbols' codewords come
+// from a table of pairs.  For streams whose capacity is the worst case, so that no worker can turn out not to fit after
+// its first buckets are written; codes with sub-blocks of 32, 64 or 128 or with none.  Instruction-bound, about 20 per symbol.
+template <int P>
+__global__ void __launch_bounds__(P == 1 ? 256 : 512, P == 1 ? 4 : 2)
+k_pack(const __grid_constant__ PackArgs a, const __grid_constant__ CodeTable ct) {
+  extern __shared__ __align__(16) uint32_t s_dyn[];                    // two images, then the pair table
+  __shared__ EncLut s_lut;
+  __shared__ uint32_t s_wtot[2][32];
+  __shared__ unsigned int s_ticket[2];
+  __shared__ unsigned long long s_prefix[2];
+  __shared__ int s_skip[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int nlev = ct.nlev, n2 = 2 * nlev;
+  const int img_words = (int)((((((uint32_t)a.bucket * (uint32_t)(ct.maxlen + 1) + 16u * (uint32_t)(a.bucket / ct.G + 1) + kNormBits + 31u) >> 5) + 4) + 3u) & ~3u);
+  uint32_t* s_pair = s_dyn + 2 * img_words;
+  fill_enc_lut(&s_lut, ct);
+  if (threadIdx.x == 0) s_ticket[0] = atomicAdd(a.ticket, 1u);
+  for (int i = threadIdx.x; i < 2 * img_words; i += blockDim.x) s_dyn[i] = 0;
+  __syncthreads();
+  for (int i = threadIdx.x; i < n2 * n2; i += blockDim.x) {            // (first, second): a level, plus nlev for a negative one
+    const int f = i % n2, g = i / n2;
+    const uint32_t x = s_lut.e[f < nlev ? f : f - nlev + 32], y = s_lut.e[g < nlev ? g : g - nlev + 32];
+    s_pair[i] = ((x & 0xffffu) | ((y & 0xffffu) << (x >> 16))) | (((x >> 16) + (y >> 16)) << 26);
   }
   __syncthreads();
-  if (s_start[nsub] != nbits - hdr_bits) bad = true;    // the lengths must add up to the bucket's payload
-  const uint32_t mask = (uint32_t)lut_n - 1u;
-  for (uint32_t s = threadIdx.x; s < nsub; s += blockDim.x) {
-    const int first = (int)s * ct.G;
-    const int count = min(ct.G, len - first);
-    const uint32_t want = s_start[s + 1] - s_start[s];
-    BitReader br;
-    br.w = w;
-    br.nwords = nwords;
-    br.seek(hdr_bits + s_start[s]);
-    uint32_t used = 0;
-    bool ok = !bad;
-    for (int i = 0; i < count; i += kQuad) {
-      uint32_t packed = 0;
-      const int nvalid = min(kQuad, count - i);
-      for (int c = 0; c < nvalid; ++c) {
-        uint32_t one = 0;
-        if (ok) ok = decode_symbol(br, s_lut, mask, &one, &used) && used <= want;
-        if (!ok) one = 0;
-        packed |= one << (8 * c);
-      }
-      uint8_t* o = out + first + i;
-      if (nvalid == kQuad && vec_ok) {
-        *reinterpret_cast<uint32_t*>(o) = packed;
-      } else {
-        for (int c = 0; c < nvalid; ++c) o[c] = (uint8_t)(packed >> (8 * c));
+  const uint32_t pair_sa = smem_addr(s_pair), weights = 4u | ((uint32_t)(8 * nlev) << 16);
+  const uint32_t limit4 = (uint32_t)(128 - nlev) * 0x01010101u;        // carries into bit 7 of a byte >= nlev
+  const unsigned long long total = (unsigned long long)a.nb * (unsigned long long)a.K;
+  const int seg = ct.has_header ? ct.G / 8 : 32;                       // lanes per sub-block
+  uint32_t used_words[2] = {0u, 0u};
+  bool bad = false;
+  for (int par = 0;; par ^= 1) {
+    const unsigned long long t = s_ticket[par];
+    if (t >= total) break;
+    const size_t b = total <= 0xffffffffull ? (size_t)((uint32_t)t / (uint32_t)a.K) : (size_t)(t / (unsigned long long)a.K);
+    const size_t k = (size_t)(t - (unsigned long long)b * (unsigned long long)a.K);
+    const size_t lo = b * (size_t)a.bucket;
+    const int len = (int)min((size_t)a.bucket, a.d - lo);
+    uint32_t* s_img = s_dyn + par * img_words;
+    const uint8_t* src = a.sym + k * a.d + lo;
+    uint32_t sy[P][2];
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+      const int e = ((warp * P + j) * 32 + lane) * 8;
+      sy[j][0] = sy[j][1] = 0u;
+      if (e + 8 <= len && a.load == 8) {
+        const uint2 x = __ldcs(reinterpret_cast<const uint2*>(src + e));
+        sy[j][0] = x.x; sy[j][1] = x.y;
+      } else if (e < len) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) sy[j][q] = load_quad_syms(src + e + 4 * q, max(0, min(kQuad, len - e - 4 * q)), a.load >= 4);
       }
     }
-    if (!ok || used != want) bad = true;
+    {
+      // this image was last read by the copy-out two buckets ago; two barriers have passed since
+      uint4* z = reinterpret_cast<uint4*>(s_img);
+      const int n4 = (int)((used_words[par] + 6u) >> 2);
+      for (int i = threadIdx.x; i < n4; i += blockDim.x) z[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    uint64_t qbits[2 * P];
+    uint32_t qn[P], qoff[P];
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+      const int e = ((warp * P + j) * 32 + lane) * 8;
+      uint32_t n01[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        uint32_t lv = sy[j][q] & 0x1f1f1f1fu;
+        if ((lv + limit4) & 0x80808080u) {                             // not a level of this code: sent as level 0
+          bad = true;
+          lv = 0u; sy[j][q] = 0u;
+        }
+        if (e + 4 * q + kQuad <= len) {
+          const uint32_t c4 = lv + ((sy[j][q] >> 7) & 0x01010101u) * (uint32_t)nlev;
+          pack_pair_entries(lds_table32(__dp2a_lo(weights, c4, pair_sa)), lds_table32(__dp2a_hi(weights, c4, pair_sa)), &qbits[2 * j + q], &n01[q]);
+        } else {
+          pack_quad(sy[j][q], max(0, min(kQuad, len - e - 4 * q)), &s_lut, &qbits[2 * j + q], &n01[q]);
+        }
+      }
+      qn[j] = n01[0] | (n01[1] << 8);
+    }
+    __syncthreads();                                                   // the image is zero
+    const uint32_t nsub = ct.has_header ? (uint32_t)((len + ct.G - 1) / ct.G) : 0u;
+    const uint32_t hdr_bits = kNormBits + 16u * nsub;
+    uint32_t warp_bits = 0;
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+      const uint32_t n = (qn[j] & 0xffu) + (qn[j] >> 8);
+      const uint32_t incl = warp_incl_scan(n, lane);
+      const uint32_t before = __shfl_up_sync(0xffffffffu, incl, seg & 31);
+      qoff[j] = warp_bits + incl - n;
+      warp_bits += __shfl_sync(0xffffffffu, incl, 31);
+      if (ct.has_header && (lane + 1) % seg == 0) {
+        const uint32_t sb = (uint32_t)((warp * P + j) * (32 / seg) + lane / seg);
+        if (sb < nsub) reinterpret_cast<uint16_t*>(s_img)[2 + sb] = (uint16_t)(incl - (lane >= seg ? before : 0u));
+      }
+    }
+    if (threadIdx.x == 0) s_img[0] = __float_as_uint(a.norms[k * a.nb + b]);
+    if (lane == 0) s_wtot[par][warp] = warp_bits;
+    __syncthreads();
+    const uint32_t wt = lane < nwarps ? s_wtot[par][lane] : 0u;
+    const uint32_t wincl = warp_incl_scan(wt, lane);
+    const uint32_t base = hdr_bits + __shfl_sync(0xffffffffu, wincl - wt, warp);
+    const uint32_t nbits = hdr_bits + __shfl_sync(0xffffffffu, wincl, 31), nwords = (nbits + 31) >> 5;
+    used_words[par] = nwords;
+    const unsigned long long mine = (unsigned long long)nwords | ((unsigned long long)(32u * nwords - nbits) << kPadShift);
+    unsigned long long* row = a.status + k * a.nb;
+    if (threadIdx.x == 0) {
+      st_status(row + b, kStAggregate | mine);
+      a.bucket_bits[k * a.nb + b] = nbits;
+    }
+#pragma unroll
+    for (int j = 0; j < P; ++j) put_bits2(s_img, base + qoff[j], qbits[2 * j], qn[j] & 0xffu, qbits[2 * j + 1], qn[j] >> 8);
+    if (warp == 0) {
+      bool timed_out = false;
+      const unsigned long long excl = lookback_prefix(row, (long long)b, lane, a.spin_limit, &timed_out);
+      if (lane == 0) {
+        const unsigned long long incl = excl + mine, words = incl & ((1ull << kPadShift) - 1ull);
+        st_status(row + b, kStPrefix | incl);
+        if (timed_out) latch_error(a.st, QGX_ERR_TIMEOUT);
+        if (b + 1 == a.nb) a.total_bits[k] = 32ull * words - (incl >> kPadShift);
+        s_prefix[par] = excl & ((1ull << kPadShift) - 1ull);
+        s_skip[par] = timed_out || words > (unsigned long long)a.cap_words ? 1 : 0;
+        s_ticket[par ^ 1] = atomicAdd(a.ticket, 1u);
+      }
+    }
+    __syncthreads();
+    if (!s_skip[par]) {
+      uint32_t* dst = a.stream + k * a.cap_words + s_prefix[par];
+      for (uint32_t i = threadIdx.x; i < nwords; i += blockDim.x) dst[i] = s_img[i];
+    }
   }
-  if (bad) latch_error(st, QGX_ERR_CORRUPT);
+  if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
+}
+
+// ---- decode ------------------------------------------------------------------------------------------
+struct UnpackArgs {
+  const uint32_t* stream;
+  size_t cap_words;
+  const uint32_t* bucket_bits;
+  const uint64_t* off;
+  const uint32_t* flags;
+  size_t d;
+  int bucket, K;
+  size_t nb;
+  const uint16_t* lut;                   // [1 << maxlen]: level | codeword length << 8
+  int store;                             // bytes per symbol store: 16, 4 or 1
+  float* norms;
+  uint8_t* sym;
+  DevStatus* st;
+};
+
+// One thread per sub-block (per bucket without sub-blocks), a warp on consecutive ones of one bucket or of several small
+// buckets; persistent CTAs, so that the table is built once per CTA and not once per bucket.  Every read is bounded by the
+// bucket's words.  A serial walk per thread: latency-bound with few sub-blocks, instruction-bound (14 per symbol) with many.
+__global__ void __launch_bounds__(128) k_unpack(const __grid_constant__ UnpackArgs a, const __grid_constant__ CodeTable ct) {
+  extern __shared__ uint16_t s_tab[];    // [2 << maxlen]: the next maxlen + 1 bits -> symbol byte | bits consumed << 8, 0: none
+  const int tab_n = 2 << ct.maxlen;
+  for (int i = threadIdx.x; i < tab_n; i += blockDim.x) {
+    const uint32_t w = a.lut[i & ((tab_n >> 1) - 1)], L = w >> 8, idx = w & 0xffu;
+    s_tab[i] = (uint16_t)(L == 0 ? 0u : (idx == 0 ? L << 8 : ((L + 1u) << 8) | idx | ((((uint32_t)i >> L) & 1u) << 7)));
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const uint32_t mask = (uint32_t)tab_n - 1u;
+  const int G = ct.G, spb = ct.has_header ? (a.bucket + G - 1) / G : 1;         // sub-blocks of a whole bucket
+  int group = 1;                                                                // lanes per bucket
+  while (group < spb && group < 32) group <<= 1;
+  const int rows = (spb + 31) / 32, per_warp = 32 / group;                      // warps per bucket, or buckets per warp
+  const size_t buckets = a.nb * (size_t)a.K;
+  const size_t warps = rows > 1 ? buckets * (size_t)rows : (buckets + (size_t)per_warp - 1) / (size_t)per_warp;
+  const bool small = warps <= 0xffffffffull && buckets <= 0xffffffffull;
+  bool bad = false;
+  for (size_t w = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < warps; w += ((size_t)gridDim.x * blockDim.x) >> 5) {
+    size_t bi;
+    int row = 0;
+    if (rows > 1) {
+      bi = small ? (size_t)((uint32_t)w / (uint32_t)rows) : w / (size_t)rows;
+      row = (int)(w - bi * (size_t)rows);
+    } else {
+      bi = w * (size_t)per_warp + (size_t)(lane / group);
+    }
+    const bool there = bi < buckets;
+    if (!there) bi = buckets - 1;
+    const size_t k = small ? (size_t)((uint32_t)bi / (uint32_t)a.nb) : bi / a.nb, b = bi - k * a.nb;
+    const int s = rows > 1 ? row * 32 + lane : lane % group;
+    const size_t lo = b * (size_t)a.bucket;
+    const int len = (int)min((size_t)a.bucket, a.d - lo);
+    const uint32_t nsub = ct.has_header ? (uint32_t)((len + G - 1) / G) : 1u;
+    const uint32_t hdr_bits = kNormBits + (ct.has_header ? 16u * nsub : 0u);
+    const bool dead = a.flags[k] != 0u;
+    const uint32_t nbits = dead ? 0u : a.bucket_bits[bi];
+    const uint32_t nwords = (nbits + 31u) >> 5;
+    const bool sound = !dead && nbits >= hdr_bits;                              // otherwise nothing trustworthy to read: zeros
+    const uint32_t* words = a.stream + k * a.cap_words + (sound ? a.off[bi] : 0ull);
+    const bool mine = there && s < (int)nsub;
+    // where the sub-block starts: the header's lengths before it
+    uint32_t L = 0, start = 0;
+    if (ct.has_header) {
+      auto field = [&](uint32_t i) { return (words[(kNormBits + 16u * i) >> 5] >> ((kNormBits + 16u * i) & 31u)) & 0xffffu; };
+      if (mine && sound) L = field((uint32_t)s);
+      uint32_t incl = L;
+      for (int o = 1; o < group; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((lane & (group - 1)) >= o) incl += y;
+      }
+      start = incl - L;
+      if (row > 0) {
+        uint32_t before = 0;
+        if (sound)
+          for (uint32_t i = (uint32_t)lane; i < 32u * (uint32_t)row && i < nsub; i += 32u) before += field(i);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        start += before;
+      }
+    } else if (sound) {
+      L = nbits - hdr_bits;
+    }
+    if (!mine) continue;
+    const uint32_t payload = nbits - hdr_bits;
+    bool ok = sound && start + L <= payload && ((uint32_t)s + 1u < nsub || start + L == payload);
+    if (s == 0) a.norms[bi] = sound ? __uint_as_float(words[0]) : 0.0f;
+    if (!ok && !dead) bad = true;
+    const int first = s * G, count = min(G, len - first);
+    uint8_t* out = a.sym + k * a.d + lo + first;
+    // the window: bits not yet consumed, refilled a word at a time
+    uint64_t buf = 0;
+    int avail = 0;
+    uint32_t next = 0, left = L;                                                // left: bits the sub-block still has (mod 2^32)
+    auto fetch = [&](uint32_t i) { return i < nwords ? words[i] : 0u; };
+    uint32_t ahead = 0;
+    if (ok) {
+      const uint32_t bit = hdr_bits + start;
+      next = bit >> 5;
+      buf = (((uint64_t)fetch(next + 1) << 32) | fetch(next)) >> (bit & 31u);
+      avail = 64 - (int)(bit & 31u);
+      next += 2;
+      ahead = fetch(next);
+    }
+    auto symbol = [&]() -> uint32_t {
+      const uint32_t e = s_tab[(uint32_t)buf & mask], n = e >> 8;
+      if (n == 0u) ok = false;                                                  // (stays at this bit: zeros from here on)
+      buf >>= n;
+      avail -= (int)n;
+      left -= n;
+      return ok ? e & 0xffu : 0u;
+    };
+    auto refill = [&]() {
+      if (avail <= 32) {
+        buf |= (uint64_t)ahead << avail;
+        avail += 32;
+        ahead = fetch(++next);
+      }
+    };
+    int i = 0;
+    if (a.store == 16) {
+      for (; i + 16 <= count; i += 16) {
+        uint32_t wd[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          refill();
+          uint32_t x = symbol();
+          x |= symbol() << 8;
+          refill();
+          x |= symbol() << 16;
+          x |= symbol() << 24;
+          wd[q] = x;
+        }
+        *reinterpret_cast<uint4*>(out + i) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+      }
+    }
+    for (; i < count; i += kQuad) {
+      const int nv = min(kQuad, count - i);
+      uint32_t x = 0;
+      for (int q = 0; q < nv; ++q) {
+        refill();
+        x |= symbol() << (8 * q);
+      }
+      if (nv == kQuad && a.store >= 4) *reinterpret_cast<uint32_t*>(out + i) = x;
+      else
+        for (int q = 0; q < nv; ++q) out[i + q] = (uint8_t)(x >> (8 * q));
+    }
+    if (!dead && (!ok || left != 0u)) bad = true;
+  }
+  if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
 }
 
 }  // namespace qgx
@@ -289,6 +527,38 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
   if (rc != QGX_OK) return rc;
   if (cudaSetDevice(c->device) != cudaSuccess) return QGX_ERR_CUDA;
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
+  const size_t img_words = (((size_t)bucket * (ct.maxlen + 1) + 16u * (bucket / ct.G + 1) + kNormBits + 31u) >> 5) + 4;
+  // one pass where the capacity is the worst case (nothing may be written for a worker that does not fit) and the layout
+  // of the sub-blocks is a warp's; the totals of a worker have to fit the status words
+  const bool layout = !ct.has_header || ct.G == 32 || ct.G == 64 || ct.G == 128;
+  const size_t worst = qgx_stream_capacity_words(d, bucket, cb->subblock, ct.maxlen);
+  if (layout && cap_words >= worst && worst < ((size_t)1 << (kPadShift - 1)) && nb < ((size_t)1 << 23) && nb * (size_t)K < ((size_t)1 << 31)) {
+    unsigned long long* status = (unsigned long long*)ws_get(c, 0, sizeof(uint64_t) * ((size_t)K * nb + 2));
+    if (!status) return QGX_ERR_CUDA;
+    if (cudaMemsetAsync(status, 0, sizeof(uint64_t) * ((size_t)K * nb + 2), c->stream) != cudaSuccess) return QGX_ERR_CUDA;
+    PackArgs a;
+    a.norms = norms; a.sym = sym; a.d = d; a.bucket = bucket; a.K = K; a.nb = nb; a.stream = stream; a.cap_words = cap_words;
+    a.bucket_bits = bucket_bits; a.total_bits = total_bits; a.status = status + 2; a.ticket = reinterpret_cast<unsigned int*>(status);
+    a.spin_limit = kSpinLimit; a.st = c->dstatus;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
+    a.load = (d % 8 == 0 && bucket % 8 == 0 && (at & 7u) == 0) ? 8 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
+    const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
+    const int threads = bucket_threads(bucket, 2 * pp);
+    const size_t smem = sizeof(uint32_t) * (2 * ((img_words + 3) & ~(size_t)3) + (size_t)(4 * ct.nlev * ct.nlev));
+    const unsigned fit = (unsigned)std::max<size_t>(1, std::min<size_t>((size_t)(1024 / threads), (220u * 1024u) / (smem + 2048u)));
+    const unsigned grid = (unsigned)std::min<unsigned long long>((unsigned long long)nb * (unsigned long long)K, (unsigned long long)c->num_sms * fit);
+#define QGX_LAUNCH_K(V)                                              \
+  do {                                                               \
+    allow_max_dynamic_smem((const void*)k_pack<V>, c->device);       \
+    k_pack<V><<<grid, threads, smem, c->stream>>>(a, ct);            \
+  } while (0)
+    if (pp == 1) QGX_LAUNCH_K(1);
+    else if (pp == 2) QGX_LAUNCH_K(2);
+    else QGX_LAUNCH_K(4);
+#undef QGX_LAUNCH_K
+    count_launch(c);
+    return cuda_status(cudaGetLastError());
+  }
   uint64_t* off = (uint64_t*)ws_get(c, 0, sizeof(uint64_t) * (size_t)K * nb);
   uint32_t* flags = (uint32_t*)ws_get(c, 1, sizeof(uint32_t) * (size_t)K);
   if (!off || !flags) return QGX_ERR_CUDA;
@@ -297,8 +567,7 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
   const int threads = bucket_threads(bucket, v4);
   const dim3 grid((unsigned)nb, (unsigned)K);
   k_bucket_bits<<<grid, threads, 0, c->stream>>>(sym, d, bucket, ct, vec_ok, bucket_bits, c->dstatus);
-  k_scan_offsets<<<K, 256, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus);
-  const size_t img_words = (((size_t)bucket * (ct.maxlen + 1) + 16u * (bucket / ct.G + 1) + kNormBits + 31u) >> 5) + 4;
+  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus);
   const size_t smem = sizeof(uint32_t) * (img_words + (size_t)(bucket / ct.G) + 2);
 #define QGX_LAUNCH_S(V)                                                                                         \
   do {                                                                                                          \
@@ -320,32 +589,31 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
 qgx_status qgx_decode(qgx_ctx* c, const uint32_t* stream, size_t cap_words, const uint32_t* bucket_bits, int K, size_t d,
                       int bucket, const qgx_codebook* cb, float* norms, uint8_t* sym) {
   if (!codec_args_ok(c, K, d, bucket) || !norms || !sym || !stream || !bucket_bits) return QGX_ERR_INVALID_ARG;
-  CodeTable ct;
-  qgx_status rc = make_code_table(cb, bucket, &ct);
-  if (rc != QGX_OK) return rc;
   if (cudaSetDevice(c->device) != cudaSuccess) return QGX_ERR_CUDA;
+  const CodeTable* ct = nullptr;
+  const uint16_t* lut = nullptr;
+  const qgx_status rc = step_code(c, cb, bucket, &ct, &lut);
+  if (rc != QGX_OK) return rc;
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
   uint64_t* off = (uint64_t*)ws_get(c, 0, sizeof(uint64_t) * (size_t)K * nb);
   uint32_t* flags = (uint32_t*)ws_get(c, 1, sizeof(uint32_t) * (size_t)K);
-  uint16_t* lut = (uint16_t*)ws_get(c, 2, sizeof(uint16_t) * kDecLutMax);
-  if (!off || !flags || !lut) return QGX_ERR_CUDA;
-  std::vector<uint16_t> h_lut((size_t)1 << ct.maxlen);
-  build_dec_lut_host(ct, h_lut.data());
-  // pageable source: the runtime stages it before returning, so the vector may go out of scope
-  if (cudaMemcpyAsync(lut, h_lut.data(), h_lut.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
-    return QGX_ERR_CUDA;
-  const bool vec_ok = (d % kQuad == 0) && ((reinterpret_cast<uintptr_t>(sym) & 3u) == 0);
-  k_scan_offsets<<<K, 256, 0, c->stream>>>(bucket_bits, nb, cap_words, off, nullptr, flags, QGX_ERR_CORRUPT, c->dstatus);
-  const uint32_t nsub_max = (uint32_t)(bucket / ct.G);
-  const int threads = (int)std::min<uint32_t>(256u, ((std::max<uint32_t>(nsub_max, 1u) + 31u) / 32u) * 32u);
-  const size_t smem = sizeof(uint32_t) * (nsub_max + 2) + sizeof(uint16_t) * ((size_t)1 << ct.maxlen);
-  const dim3 grid((unsigned)nb, (unsigned)K);
-  k_decode<<<grid, threads, smem, c->stream>>>(stream, cap_words, bucket_bits, off, flags, d, bucket, ct, lut, vec_ok, norms,
-                                               sym, c->dstatus);
+  if (!off || !flags) return QGX_ERR_CUDA;
+  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, nullptr, flags, QGX_ERR_CORRUPT, c->dstatus);
+  UnpackArgs a;
+  a.stream = stream; a.cap_words = cap_words; a.bucket_bits = bucket_bits; a.off = off; a.flags = flags; a.d = d; a.bucket = bucket;
+  a.K = K; a.nb = nb; a.lut = lut; a.norms = norms; a.sym = sym; a.st = c->dstatus;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
+  a.store = (d % 16 == 0 && bucket % 16 == 0 && ct->G % 16 == 0 && (at & 15u) == 0) ? 16 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
+  const size_t spb = ct->has_header ? (size_t)((bucket + ct->G - 1) / ct->G) : 1;
+  size_t lanes = 1;
+  while (lanes < spb && lanes < 32) lanes *= 2;
+  const size_t warps = spb > 32 ? nb * (size_t)K * ((spb + 31) / 32) : (nb * (size_t)K * lanes + 31) / 32;
+  const size_t smem = sizeof(uint16_t) * ((size_t)2 << ct->maxlen);
+  const unsigned grid = (unsigned)std::max<size_t>(1, std::min<size_t>((warps + 3) / 4, (size_t)c->num_sms * 12u));
+  k_unpack<<<grid, 128, smem, c->stream>>>(a, *ct);
   count_launch(c, 2);
   return cuda_status(cudaGetLastError());
 }
-
 
 // Device address of g_noalloc_scratch on the current device.  In host code the array's name only stands
 // in for the symbol; the address a kernel can use has to be asked for, once per device.
@@ -390,7 +658,7 @@ qgx_status qgx_encode_noalloc(qgx_ctx* c, const float* norms, const uint8_t* sym
   const int threads = bucket_threads(bucket, v4);
   const dim3 grid((unsigned)nb, (unsigned)K);
   k_bucket_bits<<<grid, threads, 0, c->stream>>>(sym, d, bucket, ct, vec_ok, bucket_bits, c->dstatus);
-  k_scan_offsets<<<K, 256, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus);
+  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus);
   const size_t img_words = (((size_t)bucket * (ct.maxlen + 1) + 16u * (bucket / ct.G + 1) + kNormBits + 31u) >> 5) + 4;
   const size_t smem = sizeof(uint32_t) * (img_words + (size_t)(bucket / ct.G) + 2);
 #define QGX_LAUNCH_S(V)                                                                                         \

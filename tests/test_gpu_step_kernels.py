@@ -1,0 +1,76 @@
+"""The separate calls at the sizes where their kernels branch: symbols that can be loaded eight, four or one at a time,
+several buckets per warp and several warps per bucket, codes without sub-blocks, more buckets than one turn of the offset
+scan, capacities below the worst case -- against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import qgx_inputs as gen
+from oracle import qgx_oracle as o
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # K, d, bucket, nlev, subblock
+    (1, 5, 4, 2, 0),
+    (3, 1003, 256, 9, 32),                  # one symbol at a time, 8 sub-blocks: four buckets per warp
+    (2, 4100, 512, 17, 128),                # four at a time
+    (5, 4808, 1024, 9, 0),                  # eight at a time, no sub-blocks
+    (4, 16 * 500, 500, 5, 100),             # a layout that only the three-kernel encoder takes
+    (2, 3 * 8192 + 4112, 8192, 32, 64),     # four warps per bucket
+    (3, 16384 + 16368, 16384, 17, 32),
+    (2, 4 * 5000, 4, 3, 0),                 # 5000 buckets: the scan's second turn
+]
+
+
+@pytest.mark.parametrize("K,d,bucket,nlev,sub", CASES)
+@pytest.mark.parametrize("roomy", [True, False])
+def test_steps_match_oracle(K, d, bucket, nlev, sub, roomy):
+    import paper_2308_09187_b200 as qgx
+    ctx = qgx.qgx_create(0)
+    try:
+        rng = np.random.default_rng(d + nlev)
+        v = gen.gaussian_mixture((K, d), seed=d, device="cuda")
+        v[0, : min(d, bucket)] = 0.0
+        lev = np.r_[0.0, np.sort(rng.uniform(0.001, 0.5, size=nlev - 2)), 1.0].astype(np.float32)
+        cb = qgx.qgx_build_codebook_huffman(list(rng.dirichlet(np.ones(nlev))), sub)
+        cbo = o.codebook_from(cb.lengths(), cb.codes(), subblock=sub)
+        norms, sym = qgx.qgx_quantize(ctx, v, bucket, lev, qgx.QGX_NORM_L2, 5, 2)
+        qgx.qgx_sync_status(ctx)
+        n = norms.cpu().numpy()
+        assert np.all(np.abs(n - o.bucket_norms(v.cpu().numpy(), bucket)) <= np.spacing(n))
+        s_ref = o.quantize(v.cpu().numpy(), bucket, lev, n, 5, 2)
+        assert np.array_equal(sym.cpu().numpy(), s_ref)
+        half = torch.full_like(norms, float(n.max()) * 0.25)         # supplied norms below the coordinates
+        _, sym2 = qgx.qgx_quantize(ctx, v, bucket, lev, qgx.QGX_NORM_L2, 5, 2, flags=qgx.QGX_NORMS_SUPPLIED, norms=half)
+        qgx.qgx_sync_status(ctx)
+        assert np.array_equal(sym2.cpu().numpy(), o.quantize(v.cpu().numpy(), bucket, lev, half.cpu().numpy(), 5, 2))
+        st_ref, bb_ref, tot_ref = o.encode(n, s_ref, bucket, cbo)
+        used = ((bb_ref.astype(np.int64) + 31) // 32).sum(axis=1)
+        cap = None if roomy else int(used.max())                     # just enough
+        stream, bits, total = qgx.qgx_encode(ctx, norms, sym, bucket, cb, cap_words=cap)
+        qgx.qgx_sync_status(ctx)
+        assert np.array_equal(bits.cpu().numpy().view(np.uint32), bb_ref)
+        assert np.array_equal(total.cpu().numpy().astype(np.uint64), tot_ref)
+        got = stream.cpu().numpy().view(np.uint32)
+        for k in range(K):
+            assert np.array_equal(got[k, : used[k]], st_ref[k, : used[k]]) and not got[k, used[k]:].any()
+        norms2, sym3 = qgx.qgx_decode(ctx, stream, bits, d, bucket, cb)
+        qgx.qgx_sync_status(ctx)
+        assert torch.equal(norms2, norms) and torch.equal(sym3, sym)
+        mean = qgx.qgx_average(ctx, norms, sym, bucket, lev)
+        qgx.qgx_sync_status(ctx)
+        assert np.array_equal(mean.cpu().numpy(), o.average(n, s_ref, bucket, lev))
+        if used.max() > 1:                                           # one word too few: nothing is written for that worker
+            tight = torch.zeros((K, int(used.max()) - 1), dtype=torch.int32, device="cuda")
+            qgx.qgx_encode(ctx, norms, sym, bucket, cb, cap_words=tight.shape[1], stream=tight)
+            assert qgx.qgx_sync_status(ctx, check=False) == qgx.QGX_ERR_CAPACITY
+            assert not tight[int(np.argmax(used))].any()
+        if nlev < 32:
+            sym[K - 1, d - 1] = 31                                   # no level of this code
+            qgx.qgx_encode(ctx, norms, sym, bucket, cb)
+            assert qgx.qgx_sync_status(ctx, check=False) == qgx.QGX_ERR_CORRUPT
+            qgx.qgx_average(ctx, norms, sym, bucket, lev)
+            assert qgx.qgx_sync_status(ctx, check=False) == qgx.QGX_ERR_CORRUPT
+    finally:
+        qgx.qgx_destroy(ctx)
