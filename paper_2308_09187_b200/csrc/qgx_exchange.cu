@@ -2,6 +2,7 @@
 // one pass over the streams writes the mean (decode + average).  Same streams, bit for bit, and
 // the same mean as qgx_quantize -> qgx_encode -> qgx_decode -> qgx_average.
 #include "qgx_encode.cuh"
+#include "qgx_small.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -885,7 +886,7 @@ namespace qgx {
 
 // workspace slots of a context
 enum { WS_OFF64 = 0, WS_FLAGS = 1, WS_LUT = 2, WS_SLOT0 = 3 /* stream, bits, offsets, total: 3..6 and 7..10 */,
-       WS_NORMS = 12, WS_SYM = 13, WS_NORMS2 = 14, WS_OPVAL = 15, WS_MEAN = 16, WS_DLUT = 18, WS_SEGBITS = 19, WS_VALUES = 20, WS_SYMTMP = 21, WS_NORMSDEC = 22 };
+       WS_NORMS = 12, WS_SYM = 13, WS_NORMS2 = 14, WS_OPVAL = 15, WS_MEAN = 16, WS_DLUT = 18, WS_SEGBITS = 19, WS_VALUES = 20, WS_SYMTMP = 21, WS_NORMSDEC = 22, WS_SMALL = 23 };
 
 // Small vectors, second part: mean_i = (((0 + v_{0,i}) + v_{1,i}) + ...) / K in worker order (the same sequential
 // sum as in the fused decode pass), then the optional state update.
@@ -1074,7 +1075,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   ea.vec_ok = (d % kQuad == 0) && (src.ld % kQuad == 0) && ((reinterpret_cast<uintptr_t>(src.v) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(src.a) & 15u) == 0);
   ea.v_vec = (reinterpret_cast<uintptr_t>(src.v ? src.v : src.a) & 15u) == 0 && (!src.v || K == 1 || (src.ld ? src.ld : d) % kQuad == 0);
   ea.a_vec = (reinterpret_cast<uintptr_t>(src.a) & 15u) == 0;
-    ea.stream = stream; ea.cap_words = cap; ea.bucket_bits = bbits; ea.offsets = offs; ea.total_bits = tot; ea.norms = norms;
+  ea.stream = stream; ea.cap_words = cap; ea.bucket_bits = bbits; ea.offsets = offs; ea.total_bits = tot; ea.norms = norms;
   ea.status = status; ea.ticket = reinterpret_cast<unsigned int*>(tot + K); ea.st = c->dstatus; ea.tables = tables->enc_dev;
   uint8_t* sym_out = nullptr;
   const uint8_t* sym_prev = nullptr;
@@ -1100,6 +1101,29 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   const PhiloxKey key = make_philox_key(cfg->seed);
   const RoundTable& qt = tables->rt;
   if (!ct.has_header || bucket % ct.G != 0 || (ct.G != 32 && ct.G != 64 && ct.G != 128)) return QGX_ERR_INVALID_ARG;
+  // small vectors: everything in one launch (the other ways are there when a caller asks for one of them)
+  if (do_encode && c->skip_buckets == 0 && c->encode_path == QGX_ENCODE_AUTO && c->decode_split == QGX_SPLIT_AUTO &&
+      small_exchange_fits(c, K, nb, bucket)) {
+    const size_t had = c->ws_bytes[WS_SMALL];
+    unsigned long long* words = (unsigned long long*)ws_get(c, WS_SMALL, sizeof(uint64_t) * ((size_t)K * nb + 2));
+    if (!words) return QGX_ERR_CUDA;
+    if (c->ws_bytes[WS_SMALL] != had && cudaMemsetAsync(words, 0, c->ws_bytes[WS_SMALL], c->stream) != cudaSuccess) return QGX_ERR_CUDA;
+    EncodeArgs es = ea;
+    es.status = words + 2;                              // zero between launches: the kernel sees to it
+    es.ticket = reinterpret_cast<unsigned int*>(words);
+    es.b_first = 0;
+    es.spin_limit = c->wait_limit;
+    SmallArgs sm;
+    std::memset(&sm, 0, sizeof(sm));
+    sm.lut_len = reinterpret_cast<const uint32_t*>(lut) + 1;
+    sm.mean = mean_out;
+    sm.update = upd ? upd->mode : 0; sm.xin = upd ? upd->xin : nullptr; sm.xout = upd ? upd->xout : nullptr; sm.scalars = upd ? upd->scalars : nullptr;
+    sm.sym_out = sym_out; sm.sym_prev = sym_prev; sm.sym_ld = sym_ld; sm.norms_prev = norms_prev;
+    sm.sum_sq = sum_sq; sm.square = (sym_mode & 4) ? 1 : 0; sm.total_out = total_bits_out;
+    ScopedKernelTimer timer(c, QGX_KERNEL_ENCODE);
+    const qgx_status done = launch_exchange_small(c, es, sm, lt, lt_kept, ct, key, qt);
+    if (done != QGX_ERR_TOO_LARGE) return done;
+  }
   // octets per thread chosen so that CTAs have at most 256 / 512 / 512 threads
   const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
   const int threads = bucket_threads(bucket, 2 * pp);

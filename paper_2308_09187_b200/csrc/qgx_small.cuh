@@ -1,0 +1,33 @@
+// The one-launch exchange of small vectors (qgx_exchange_small.cu).
+#pragma once
+
+#include "qgx_encode.cuh"
+
+namespace qgx {
+
+constexpr int kSmallMaxWorkers = 16;     // the largest cluster (more than 8 where the device allows it)
+
+struct SmallArgs {
+  const uint32_t* lut_len;               // second words of the decoder table's entries, 8 bytes apart
+  float* mean;
+  int update;                            // as DecodeArgs
+  const float* xin;
+  float* xout;
+  const double* scalars;
+  uint8_t* sym_out;
+  const uint8_t* sym_prev;
+  size_t sym_ld;
+  const float* norms_prev;
+  double* sum_sq;
+  int square;                            // add the squared values themselves
+  uint64_t* total_out;                   // the caller's copy of the totals, or null
+  uint32_t img_words, off_img, off_sym, off_tab;
+};
+
+bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket);
+// ea.status [K][nb] and ea.ticket [2] are zero before the launch and again after it.  QGX_ERR_TOO_LARGE: nothing was
+// launched, the device has no clusters of that many CTAs.
+qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, const LevelTable& lt, const LevelTable& lt_kept,
+                                 const CodeTable& ct, const PhiloxKey& key, const RoundTable& rt);
+
+}  // namespace qgx
