@@ -192,6 +192,7 @@ qgx_status qgx_create(qgx_ctx** out, int device, void* cuda_stream) {
   c->wait_limit = kSpinLimit;
   c->num_sms = 1;
   if (cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || c->num_sms < 1) { cudaGetLastError(); c->num_sms = 1; }
+  c->all_sms = c->num_sms;
   c->stream = (cudaStream_t)cuda_stream;
   if (cudaMalloc((void**)&c->dstatus, sizeof(DevStatus)) != cudaSuccess ||
       cudaMemsetAsync(c->dstatus, 0, sizeof(DevStatus), c->stream) != cudaSuccess ||

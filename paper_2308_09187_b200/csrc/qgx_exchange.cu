@@ -1315,7 +1315,16 @@ qgx_status launch_decode_average(qgx_ctx* c, const DecodeArgs& da, const CodeTab
 // The tensors of a layer-wise vector are independent; most are small, so one after the other they leave the GPU
 // mostly idle.  They are spread over a few helper contexts, each with its own stream and workspace; the caller's
 // stream forks into them and joins them again (events), so the call stays asynchronous and ordered on that stream.
-constexpr int kSegStreams = 4;
+// Each tensor is still a chain of launches with gaps, ends that not all SMs reach together and a start that fills slowly,
+// and the persistent kernels of two streams do not share an SM.  So, once there is enough work to fill the GPU, every
+// stream runs on the SMs of its share of the work: the chains then run side by side and a gap in one idles only its SMs.
+// 16 tensors of 1728 to 2.4 * 10^6 coordinates, 16 workers, bucket 4096: 905 us on 4 streams over all SMs, 766 on 4 with
+// shares, 706 on 8; 24 tensors of 10^3 to 1.3 * 10^6, 8 workers: 485, 440, 370.  Below kSegSplitCoords there is
+// nothing to share out and each further stream costs two events (8 tensors, 60 * 10^3 coordinates: 59 us on 4, 62 on 8).
+constexpr int kSegStreams = 8;
+constexpr int kSegStreamsSmall = 4;
+constexpr double kSegSplitCoordsPerSm = 16384.0;        // workers * coordinates per SM
+constexpr double kSegFixed = 1e6;                       // the chain of a tensor's launches, in coordinates of the whole GPU
 struct SegChildren {
   qgx_ctx* ctx[kSegStreams];
   cudaEvent_t fork, join[kSegStreams];
@@ -1363,6 +1372,7 @@ static SegChildren* seg_children(qgx_ctx* c) {
     h->decode_split = c->decode_split;
     h->encode_path = c->encode_path;
     h->num_sms = c->num_sms;
+    h->all_sms = c->all_sms;
     h->dstatus = c->dstatus;                            // errors latch into the parent's status block
     if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&sc->join[i], cudaEventDisableTiming) != cudaSuccess) {
@@ -1447,31 +1457,50 @@ qgx_status qgx_exchange_segments(qgx_ctx* c, const float* v, int K, size_t d, co
   if (total_bits && cudaMemsetAsync(total_bits, 0, sizeof(uint64_t) * (size_t)K, c->stream) != cudaSuccess) return QGX_ERR_CUDA;
   SegChildren* sc = nseg > 1 ? seg_children(c) : nullptr;
   if (nseg > 1 && !sc) return QGX_ERR_CUDA;
-  const int lanes = sc ? std::min(nseg, kSegStreams) : 0;
-  if (sc) {                                             // fork: the helpers start after everything queued so far
-    if (cudaEventRecord(sc->fork, c->stream) != cudaSuccess) return QGX_ERR_CUDA;
+  const bool shares = (double)K * (double)d > (double)c->num_sms * kSegSplitCoordsPerSm;
+  const int lanes = sc ? std::min(nseg, shares ? kSegStreams : kSegStreamsSmall) : 0;
+  std::vector<int> order((size_t)nseg), lane_of((size_t)nseg, 0);
+  for (int s = 0; s < nseg; ++s) order[(size_t)s] = s;
+  if (sc) {
+    // largest first, each to the stream with the least work; a stream's kernels get the SMs of its share of the work
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return segs[x].length > segs[y].length; });
+    double load[kSegStreams] = {}, part[kSegStreams] = {}, all = 0.0;
+    for (int s : order) {
+      const int l = (int)(std::min_element(load, load + lanes) - load);
+      const double w = (double)K * (double)segs[s].length;
+      const size_t bucket = (size_t)std::max(segs[s].cfg->bucket, 1);
+      const bool one_launch = small_exchange_fits(c, K, (segs[s].length + bucket - 1) / bucket, (int)bucket);
+      lane_of[(size_t)s] = l;
+      load[l] += w + kSegFixed;
+      part[l] += one_launch ? w : w + kSegFixed;        // (a tensor done in one launch takes the SMs that it finds)
+      all += one_launch ? w : w + kSegFixed;
+    }
+    if (cudaEventRecord(sc->fork, c->stream) != cudaSuccess) return QGX_ERR_CUDA;   // the helpers start after everything queued so far
     for (int i = 0; i < lanes; ++i) {
       sc->ctx[i]->decode_split = c->decode_split;
       sc->ctx[i]->encode_path = c->encode_path;
+      sc->ctx[i]->num_sms = shares ? std::max(1, (int)(c->num_sms * part[i] / all)) : c->num_sms;
       if (cudaStreamWaitEvent(sc->ctx[i]->stream, sc->fork, 0) != cudaSuccess) return QGX_ERR_CUDA;
     }
   }
   qgx_status rc = QGX_OK;
-  for (int s = 0; s < nseg && rc == QGX_OK; ++s) {
-    qgx_ctx* h = sc ? sc->ctx[s % lanes] : c;
+  int rc_seg = nseg;                                    // the first segment that failed decides the status
+  for (int s : order) {
+    qgx_ctx* h = sc ? sc->ctx[lane_of[(size_t)s]] : c;
     uint64_t* seg_bits = nullptr;
     if (total_bits) {
       seg_bits = (uint64_t*)ws_get(h, WS_SEGBITS, sizeof(uint64_t) * (size_t)K);
       if (!seg_bits) { rc = QGX_ERR_CUDA; break; }
     }
     DualSource src{v + segs[s].offset, nullptr, d, 0};
-    rc = exchange_impl(h, src, K, segs[s].length, segs[s].cfg, exchange_id, 0, mean_out + segs[s].offset, seg_bits,
-                       nullptr, 0, nullptr, segs[s].offset);
-    if (rc == QGX_OK && total_bits) {
+    const qgx_status mine = exchange_impl(h, src, K, segs[s].length, segs[s].cfg, exchange_id, 0, mean_out + segs[s].offset, seg_bits,
+                                          nullptr, 0, nullptr, segs[s].offset);
+    if (mine == QGX_OK && total_bits) {
       k_add_u64_atomic<<<(K + 255) / 256, 256, 0, h->stream>>>(reinterpret_cast<unsigned long long*>(total_bits),
                                                                reinterpret_cast<const unsigned long long*>(seg_bits), K);
       count_launch(h);
     }
+    if (mine != QGX_OK && s < rc_seg) { rc = mine; rc_seg = s; }
   }
   if (sc) {                                             // join, also after an error: the caller's stream waits for the helpers
     for (int i = 0; i < lanes; ++i)

@@ -328,7 +328,7 @@ static bool cluster_fits(const void* fn, int device, int workers, int threads, s
 // of bucket 16384 1.6 x 10^6 24.6 : 34.9.
 bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket) {
   if (K > kSmallMaxWorkers || bucket < 128 || bucket % 128 != 0 || nb > 65536) return false;
-  return nb * (size_t)K * (size_t)bucket <= (size_t)c->num_sms * (bucket >= 4096 ? 12288 : 7168);
+  return nb * (size_t)K * (size_t)bucket <= (size_t)c->all_sms * (bucket >= 4096 ? 12288 : 7168);
 }
 
 qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, const LevelTable& lt, const LevelTable& lt_kept,

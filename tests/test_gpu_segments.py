@@ -1,0 +1,43 @@
+"""The layer-wise exchange at the edges of the rule that shares the SMs out among its streams: just below and above the
+amount of work where it begins, more tensors than streams, one tensor with nearly all of the work.  Every tensor against
+the oracle, and the whole against the way without shares of the encode pass."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import qgx_oracle as o
+
+pytestmark = pytest.mark.gpu
+
+EDGE = 148 * 16384                                           # workers * coordinates where the SMs are shared out
+
+
+@pytest.mark.parametrize("K,sizes,bucket", [
+    (4, [EDGE // 8, EDGE // 8 - 8 * 3, 8, 4, 4], 1024),       # below the edge
+    (4, [EDGE // 8, EDGE // 8, 8, 4, 7], 1024),               # above it, a ragged end
+    (2, [64, 2000000, 4, 1028], 4096),                        # one tensor has nearly everything
+    (16, [4000, 52000] * 5 + [12, 33], 2048),                 # more tensors than streams
+])
+def test_segments_shared_out(K, sizes, bucket):
+    import paper_2308_09187_b200 as qgx
+    d = sum(sizes)
+    v = torch.randn((K, d), device="cuda", generator=torch.Generator("cuda").manual_seed(d))
+    lev = np.array([0.0, 0.004, 0.01, 0.02, 0.03, 0.05, 0.1, 0.3, 1.0], dtype=np.float32)
+    cfgs = [qgx.make_quant_cfg(lev, bucket, qgx.qgx_build_codebook_fixed(9, 32), 7 + s) for s in range(len(sizes))]
+    ctx, plain = qgx.qgx_create(0), qgx.qgx_create(0)
+    qgx.qgx_set_encode_path(plain, qgx.QGX_ENCODE_REGISTERS)
+    qgx.qgx_set_decode_split(plain, qgx.QGX_SPLIT_NEVER)
+    got = [qgx.qgx_exchange_segments(c, v, sizes, cfgs, 5) for c in (ctx, plain)]
+    qgx.qgx_sync_status(ctx)
+    qgx.qgx_sync_status(plain)
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    mean, at = got[0][0].cpu().numpy(), 0
+    for n, cfg in zip(sizes, cfgs):
+        if n <= 4096:                                        # the small ones against the oracle
+            part = np.ascontiguousarray(v[:, at:at + n].cpu().numpy())
+            norms = o.bucket_norms(part, bucket)
+            ref = o.average(norms, o.quantize(part, bucket, lev, norms, cfg.seed, 5, coord_base=at), bucket, lev)
+            assert np.max(np.abs(mean[at:at + n] - ref)) <= 1e-5 * float(norms.max())
+        at += n
+    qgx.qgx_destroy(ctx)
+    qgx.qgx_destroy(plain)
