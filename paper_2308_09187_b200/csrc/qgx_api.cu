@@ -53,12 +53,12 @@ qgx_status make_code_table(const qgx_codebook* cb, int bucket, CodeTable* out) {
   return QGX_OK;
 }
 
-// Tables of round_fast.  The margin bounds, in units of 1 / S of an interval, everything by which the
+// Tables of the level map.  The margin bounds, in units of 1 / S of an interval, everything by which the
 // kernel's S (F - r) can differ from the exact routine's decision variable: u2 against the correctly
 // rounded quotient and the rounding of b and of the knot (together under 2 * 2^-22 (l_{tau+1} + 2^-16) / width,
-// with the narrower of the two intervals around a level), the rounding of a, three fused multiply-adds of
+// with the narrower of the two intervals around a level), the rounding of a16, three fused multiply-adds of
 // results below 2^24, the slope-change term, and the exact routine's own roundings of xi plus the variate's
-// dropped last bit (3.02 S / 2^24).
+// dropped bits (1.01 S / 2^17).
 void make_round_table(const float* lev, int nlev, RoundTable* out) {
   std::memset(out, 0, sizeof(*out));
   out->nlev = nlev;
@@ -69,22 +69,13 @@ void make_round_table(const float* lev, int nlev, RoundTable* out) {
     width[t] = (double)(float)(lev[t + 1] - lev[t]);             // the fp32 difference the exact routine divides by
     b[t] = S / width[t];
     out->b[t] = (float)b[t];
-    out->a[t] = (float)(S * t - b[t] * ((double)lev[t] + c0) + 1.5 * S);
   }
   for (int j = 0; j < QGX_MAX_LEVELS; ++j) {
     const bool interior = j >= 1 && j <= nlev - 2;
     out->knot[j] = interior ? (float)((double)lev[j] + c0) : 4.0f;
     out->db[j] = interior ? (float)(b[j] - b[j - 1]) : 0.0f;
   }
-  double margin = 0.0;
-  for (int t = 0; t <= nlev - 2; ++t) {
-    const double wmin = std::min(width[t], t + 1 <= nlev - 2 ? width[t + 1] : width[t]);
-    const double a_ulp = (double)std::nextafter(std::fabs(out->a[t]), INFINITY) - (double)std::fabs(out->a[t]);
-    const double e = 2.0 * S * 0x1p-22 * ((double)lev[t + 1] + c0) / wmin + a_ulp + 1.5 + 1.0 + 3.02 * S / 16777216.0;
-    margin = std::max(margin, e);
-  }
-  margin = (margin + 2.0) * 1.01;
-  // the octet encoder's variant: only the leading 16 bits h of the variate are subtracted, as the float 2^23 + h
+  // only the leading 16 bits h of the variate are subtracted, as the float 2^23 + h
   // times -S 2^-16 (the 2^23 part is folded into a16); r lies within 2^-17 of the centre (h + 1/2) 2^-16
   double margin16 = 0.0;
   for (int t = 0; t <= nlev - 2; ++t) {
@@ -95,7 +86,7 @@ void make_round_table(const float* lev, int nlev, RoundTable* out) {
     margin16 = std::max(margin16, e);
   }
   margin16 = (margin16 + 2.0) * 1.01;
-  bool usable = std::isfinite(margin) && margin < S / 4.0 && std::isfinite(margin16) && margin16 < S / 4.0;
+  bool usable = std::isfinite(margin16) && margin16 < S / 4.0;
   // the fixed-point variant: units of 2^-16 of an interval, results in [2^23, 2^24).  What it can be off by, e, either way: u2
   // against the correctly rounded quotient, b, the knot, db and the difference u2 - knot (at most 12 roundings of relative
   // size 2^-24 of (1.25 l_{tau+1} + 2^-16) / width -- a bin that a knot divides reaches at most an eighth past it), the
@@ -140,8 +131,6 @@ void make_round_table(const float* lev, int nlev, RoundTable* out) {
   out->key_shift = shift < 0 ? kKeyShiftMin : shift;
   out->usable = usable ? 1 : 0;
   if (!usable) out->thrfix = 65536u;
-  out->thr = usable ? (float)(S / 2.0 - margin) : -1.0f;
-  out->neg_qscale = (float)(-S / 8388608.0);
   out->thr16 = usable ? (float)(S / 2.0 - margin16) : -1.0f;
   out->neg_qscale16 = (float)(-S / 65536.0);
   out->magic = (float)(1.5 * 8388608.0 * S);

@@ -159,70 +159,24 @@ __device__ __forceinline__ void philox4x32_10_x2(uint64_t ctr_a, uint64_t ctr_b,
   *out_b = make_uint4(b0, b1, b2, b3);
 }
 
-// four blocks with consecutive counters ctr, ctr + 1, ctr + 2, ctr + 3 (same last two counter words), round by round
-__device__ __forceinline__ void philox4x32_10_x4(uint64_t ctr, uint32_t c2, uint32_t c3, const PhiloxKey& key, uint4* out) {
-  uint32_t s0[4], s1[4], s2[4], s3[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const uint64_t c = ctr + (uint64_t)j;
-    s0[j] = (uint32_t)c; s1[j] = (uint32_t)(c >> 32); s2[j] = c2; s3[j] = c3;
-  }
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    const uint32_t k0 = key.k0[r], k1 = key.k1[r];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint64_t p0 = (uint64_t)0xD2511F53u * (uint64_t)s0[j], p1 = (uint64_t)0xCD9E8D57u * (uint64_t)s2[j];
-      const uint32_t n0 = (uint32_t)(p1 >> 32) ^ s1[j] ^ k0, n2 = (uint32_t)(p0 >> 32) ^ s3[j] ^ k1;
-      s0[j] = n0; s1[j] = (uint32_t)p1; s2[j] = n2; s3[j] = (uint32_t)p0;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) out[j] = make_uint4(s0[j], s1[j], s2[j], s3[j]);
-}
-
-// ---- Definition 1 for one normalized coordinate, every operation one IEEE rounding ----------
-// returns the level index; lev points to the table in shared memory
-__device__ __forceinline__ int quantize_level(float absv, float norm, const float* lev, int nlev, uint32_t word) {
-  float u = (norm > 0.0f) ? __fdiv_rn(absv, norm) : 0.0f;
-  u = fminf(u, 1.0f);
-  int tau = 0;
-  for (int j = 1; j <= nlev - 2; ++j) tau = (lev[j] <= u) ? j : tau;
-  const float num = __fsub_rn(u, lev[tau]);
-  const float den = __fsub_rn(lev[tau + 1], lev[tau]);
-  const float xi = __fdiv_rn(num, den);
-  const float r = __fmul_rn(__uint2float_rn(word >> 8), 5.9604644775390625e-8f);   // exact
-  return tau + ((r < xi) ? 1 : 0);
-}
-
-// The exact routine as one out-of-line copy (it runs for about 1e-5 of the coordinates).
-static __device__ __noinline__ int quantize_level_slow(float absv, float norm, const float* lev, int nlev, uint32_t word) {
-  return quantize_level(absv, norm, lev, nlev, word);
-}
-
 // ---- rounding through the level map -----------------------------------------------------------
 // F(u) = tau + (u - l_tau) / (l_{tau+1} - l_tau) is continuous and piecewise linear, and Definition 1
 // rounds u to level floor(F(u) - r) + 1 (r the uniform variate) unless F(u) - r is an integer.  The
 // kernels evaluate S F(u) with S = 2^19 (2^18 above 17 levels) from a table over the float pattern
 // of u2 = |v| RN(1 / norm) + 2^-16 (64 bins per octave, every bin holding at most one level: the lower
-// piece plus a slope change past that level), subtract S r, and read the level index off the mantissa
-// after adding 1.5 * 2^23 * S.  Whenever S (F - r) comes closer than `margin` to a multiple of S the
-// exact routine decides instead; the margin (see make_round_table) covers the difference between u2 and
-// the exact quotient, the table's roundings and the three fused multiply-adds.
+// piece plus a slope change past that level), subtract S r, r by its leading 16 bits, and read the level
+// off the nearest multiple of S.  Whenever S (F - r) comes closer than a margin (see make_round_table) to
+// where the outcome would change the exact routine decides instead.
 constexpr float kRoundShift = 1.52587890625e-05f;       // 2^-16: keeps u2 inside the table
 struct RoundTable {
   int nlev;
   int usable;                            // 0: some bin holds two levels, or the margin is too wide
   int key_shift;                         // layout of the bin table: kKeyShiftMin..kKeyShiftMax
-  float thr;                             // S / 2 - margin
-  float neg_qscale;                      // -S / 2^23
   float magic;                           // 1.5 * 2^23 * S
-  float a[QGX_MAX_LEVELS];               // per interval: S tau - b (l_tau + 2^-16) + 1.5 S
-  float b[QGX_MAX_LEVELS];               //               S / (l_{tau+1} - l_tau)
+  float b[QGX_MAX_LEVELS];               // per interval: S / (l_{tau+1} - l_tau)
   float knot[QGX_MAX_LEVELS];            // l_j + 2^-16 for interior levels j, else a value never reached
   float db[QGX_MAX_LEVELS];              // b[j] - b[j - 1]
-  // the same map for the octet encoder, which subtracts only the leading 16 bits h of the variate (as the float
-  // 2^23 + h) and leaves the rest to the exact routine:
+  // the leading 16 bits h of the variate are subtracted as the float 2^23 + h:
   float a16[QGX_MAX_LEVELS];             // S tau - b (l_tau + 2^-16) + S / 2 - S 2^-17 + 2^23 S 2^-16
   float thr16;                           // S / 2 - (margin + what the dropped variate bits can move)
   float neg_qscale16;                    // -S / 2^16
@@ -234,9 +188,9 @@ struct RoundTable {
   uint32_t thrfix;                       // distances below this go to the exact routine (2^16: all of them)
 };
 
-// one entry per bin and copy: {a (or a16, afix), b, knot, db} of the interval of the bin's lowest value
-enum class BinKind { kQuad, kOctet, kFixed };
-__device__ __forceinline__ void fill_bin_table(float4* bin, const RoundTable& rt, BinKind kind = BinKind::kQuad) {
+// one entry per bin and copy: {a16 or afix, b, knot, db} of the interval of the bin's lowest value
+enum class BinKind { kOctet, kFixed };
+__device__ __forceinline__ void fill_bin_table(float4* bin, const RoundTable& rt, BinKind kind) {
   const float scale = kind == BinKind::kFixed ? rt.fix_scale : 1.0f;
   const int rep_log = rt.key_shift - kKeyShiftMin;
   const int nbins = (int)((kKeyTop - kKeyBase) >> rt.key_shift) + 1;
@@ -247,7 +201,7 @@ __device__ __forceinline__ void fill_bin_table(float4* bin, const RoundTable& rt
     int t0 = 0;
     for (int j = 1; j <= rt.nlev - 2; ++j) t0 = (rt.knot[j] <= lo) ? j : t0;
     const bool straddle = (t0 + 1 <= rt.nlev - 2) && (rt.knot[t0 + 1] <= hi);
-    const float icpt = kind == BinKind::kFixed ? rt.afix[t0] : (kind == BinKind::kOctet ? rt.a16[t0] : rt.a[t0]);
+    const float icpt = kind == BinKind::kFixed ? rt.afix[t0] : rt.a16[t0];
     bin[i] = make_float4(icpt, rt.b[t0] * scale, straddle ? rt.knot[t0 + 1] : 4.0f, straddle ? rt.db[t0 + 1] * scale : 0.0f);
   }
 }
@@ -256,67 +210,6 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   uint32_t d;
   asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
   return d;
-}
-
-struct RoundConsts {
-  float rn;                              // RN(1 / norm)
-  float thr;                             // negative: every coordinate goes to the exact routine
-  float neg_qscale, magic;
-  uint32_t bin_mask;                     // keeps the bin part of pattern >> kBinAddrShift
-  uint32_t bin_lane;                     // byte offset of this lane's copy inside a bin
-};
-
-__device__ __forceinline__ RoundConsts round_consts(const RoundTable& rt, float norm) {
-  const bool ok = rt.usable && norm > 7.9e-31f && norm < 1.2e30f;
-  RoundConsts c;
-  c.rn = ok ? __frcp_rn(norm) : 0.0f;
-  c.thr = ok ? rt.thr : -1.0f;
-  c.neg_qscale = rt.neg_qscale;
-  c.magic = rt.magic;
-  const uint32_t copy_bytes = 16u << (rt.key_shift - kKeyShiftMin);
-  c.bin_mask = ~(copy_bytes - 1u);
-  c.bin_lane = ((threadIdx.x & 31u) << 4) & (copy_bytes - 1u);
-  return c;
-}
-
-// pattern of the float whose low mantissa bits are the level index; *unsafe: ask the exact routine
-__device__ __forceinline__ uint32_t round_fast(float absv, const RoundConsts& c, const float4* bin, uint32_t word, bool* unsafe) {
-  const float u2 = fminf(fmaf(absv, c.rn, kRoundShift), 1.0f + kRoundShift);   // a supplied norm may be smaller than |v|
-  const uint32_t off = ((__float_as_uint(u2) >> kBinAddrShift) & c.bin_mask) | c.bin_lane;
-  const float4 e = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(bin) + off - kBinAddrBase);
-  float X = fmaf(u2, e.y, e.x);
-  X = fmaf(__saturatef(__fsub_rn(u2, e.z)), e.w, X);
-  const float mb = __uint_as_float(0x4B000000u | (word >> 9));                    // 2^23 + (m >> 1), exact
-  const float D = fmaf(mb, c.neg_qscale, X);                                       // S (F - r) + S / 2
-  const float Z = __fadd_rn(D, c.magic);
-  const float rho = __fsub_rn(D, __fsub_rn(Z, c.magic));                            // D minus the nearest multiple of S
-  *unsafe = fabsf(rho) > c.thr;
-  return __float_as_uint(Z);
-}
-
-// The four coordinates of a quad as 6-bit codes, one per byte: level index, bit 5 the sign of a
-// nonzero level.
-__device__ __forceinline__ uint32_t quantize_quad_codes(const float4 x, const uint4 w, const RoundConsts& c, float norm,
-                                                        const float4* bin, const float* lev, int nlev) {
-  bool u0, u1, u2, u3;
-  const uint32_t z0 = round_fast(fabsf(x.x), c, bin, w.x, &u0);
-  const uint32_t z1 = round_fast(fabsf(x.y), c, bin, w.y, &u1);
-  const uint32_t z2 = round_fast(fabsf(x.z), c, bin, w.z, &u2);
-  const uint32_t z3 = round_fast(fabsf(x.w), c, bin, w.w, &u3);
-  uint32_t idx4 = prmt(prmt(z0, z1, 0x0040u), prmt(z2, z3, 0x0040u), 0x5410u);    // the low bytes
-  if (u0 | u1 | u2 | u3) {
-    uint32_t i0 = idx4 & 0xffu, i1 = (idx4 >> 8) & 0xffu, i2 = (idx4 >> 16) & 0xffu, i3 = idx4 >> 24;
-    if (u0) i0 = (uint32_t)quantize_level_slow(fabsf(x.x), norm, lev, nlev, w.x);
-    if (u1) i1 = (uint32_t)quantize_level_slow(fabsf(x.y), norm, lev, nlev, w.y);
-    if (u2) i2 = (uint32_t)quantize_level_slow(fabsf(x.z), norm, lev, nlev, w.z);
-    if (u3) i3 = (uint32_t)quantize_level_slow(fabsf(x.w), norm, lev, nlev, w.w);
-    idx4 = i0 | (i1 << 8) | (i2 << 16) | (i3 << 24);
-  }
-  // sign bytes (0x00 / 0xff) of the four floats, kept at bit 5 where the level is not zero
-  const uint32_t s4 = prmt(prmt(__float_as_uint(x.x), __float_as_uint(x.y), 0x00fbu),
-                           prmt(__float_as_uint(x.z), __float_as_uint(x.w), 0x00fbu), 0x5410u);
-  const uint32_t nz = (idx4 + 0x1f1f1f1fu) & 0x20202020u;                          // level indices are < 0x20
-  return idx4 | (s4 & nz);
 }
 
 // ---- the octet encoder's rounding ---------------------------------------------------------------
