@@ -422,7 +422,7 @@ def qgx_update_levels(ctx, v, cfg, refit, hist=None):
     host = (C.c_double * cfg.nbins)()
     _chk(lib().qgx_update_levels(ctx.h, _ptr(v), K, C.c_size_t(d), C.byref(cfg), refit, _ptr(hist), host),
          "qgx_update_levels")
-    return [float(x) for x in host]
+    return host[:]
 
 
 # ---------------------------------------------------------------- the iteration

@@ -207,6 +207,7 @@ void qgx_destroy(qgx_ctx* c) {
     if (c->ws[i]) cudaFree(c->ws[i]);
   cudaFree(c->dstatus);
   cudaFreeHost(c->hstatus);
+  if (c->hist_pinned) cudaFreeHost(c->hist_pinned);
   delete c;
 }
 
@@ -405,8 +406,9 @@ namespace {
 struct BinnedCdf {
   int n;
   double width;
-  std::vector<double> mass, cum0, cum1;
-  BinnedCdf(const double* h, int nbins) : n(nbins), width(1.0 / nbins), mass(h, h + nbins), cum0(nbins + 1), cum1(nbins + 1) {
+  const double* mass;
+  std::vector<double> cum0, cum1;
+  BinnedCdf(const double* h, int nbins) : n(nbins), width(1.0 / nbins), mass(h), cum0(nbins + 1), cum1(nbins + 1) {
     cum0[0] = cum1[0] = 0.0;
     for (int j = 0; j < n; ++j) {
       const double mid = (j + 0.5) * width;              // centroid of a uniform bin
@@ -428,15 +430,30 @@ struct BinnedCdf {
     const double lo = j * width;
     return cum1[j] + mass[j] / width * 0.5 * (x - lo) * (x + lo);
   }
-  // smallest x with m0(x) >= target
-  double inverse(double target) const {
+  // smallest x with m0(x) >= target; the search begins near x = guess
+  double inverse(double target, double guess = 0.5) const {
     if (target <= 0.0) return 0.0;
     if (target >= cum0[n]) {
       int j = n;
       while (j > 0 && cum0[j - 1] >= cum0[n]) --j;       // right edge of the last bin that holds mass
       return j * width;
     }
-    const int j = (int)(std::lower_bound(cum0.begin() + 1, cum0.end(), target) - (cum0.begin() + 1));
+    // the first bin j with cum0[j + 1] >= target: 0 <= lo <= j <= hi <= n - 1, narrowed in doubling steps, then halved
+    int lo = 0, hi = n - 1, at = bin_of(guess);
+    for (int step = 1; lo < hi; step *= 2) {
+      if (cum0[at + 1] >= target) {
+        hi = std::min(hi, at);
+        if (at - step < lo) break;
+        at -= step;
+        if (cum0[at + 1] < target) { lo = at + 1; break; }
+      } else {
+        lo = std::max(lo, at + 1);
+        if (at + step > hi) break;
+        at += step;
+        if (cum0[at + 1] >= target) { hi = at; break; }
+      }
+    }
+    const int j = (int)(std::lower_bound(cum0.begin() + 1 + lo, cum0.begin() + 1 + hi, target) - (cum0.begin() + 1));
     if (!(mass[j] > 0.0)) return j * width;
     return j * width + (target - cum0[j]) / mass[j] * width;
   }
@@ -501,7 +518,7 @@ qgx_status qgx_fit_levels(const double* hist, int nbins, float* levels, int nlev
   const double min_gap = std::ldexp(1.0, -20);
   double l[QGX_MAX_LEVELS];
   if (first_fit) {
-    for (int j = 0; j < nlev; ++j) l[j] = F.inverse(total * j / (double)(nlev - 1));
+    for (int j = 0; j < nlev; ++j) l[j] = F.inverse(total * j / (double)(nlev - 1), j ? l[j - 1] : 0.0);
     l[0] = 0.0;
     l[nlev - 1] = 1.0;
   } else {
@@ -511,19 +528,23 @@ qgx_status qgx_fit_levels(const double* hist, int nbins, float* levels, int nlev
   for (int j = 1; j <= nlev - 2; ++j) l[j] = std::max(l[j], l[j - 1] + min_gap);
   for (int j = nlev - 2; j >= 1; --j) l[j] = std::min(l[j], l[j + 1] - min_gap);
   if (total > 0.0) {
+    double f0[QGX_MAX_LEVELS], f1[QGX_MAX_LEVELS];       // the cdf and the first moment up to each level
+    for (int j = 0; j < nlev; ++j) { f0[j] = F.m0(l[j]); f1[j] = F.m1(l[j]); }
     for (int sweep = 0; sweep < 32; ++sweep) {
       double moved = 0.0;
       for (int j = 1; j <= nlev - 2; ++j) {
         const double a = l[j - 1], c = l[j + 1];
-        const double Fa = F.m0(a), Fc = F.m0(c);
+        const double Fa = f0[j - 1], Fc = f0[j + 1];
         if (!(Fc - Fa > 0.0)) continue;
         // d/dl of the (QAda) objective is (c - a) F(l) - [c F(c) - a F(a) - (M1(c) - M1(a))]:
         // the coordinate minimiser is where the cdf reaches this value
-        const double target = (c * Fc - a * Fa - (F.m1(c) - F.m1(a))) / (c - a);
-        double x = F.inverse(target);
+        const double target = (c * Fc - a * Fa - (f1[j + 1] - f1[j - 1])) / (c - a);
+        double x = F.inverse(target, l[j]);
         x = std::min(std::max(x, a + min_gap), c - min_gap);
         moved = std::max(moved, std::fabs(x - l[j]));
         l[j] = x;
+        f0[j] = F.m0(x);
+        f1[j] = F.m1(x);
       }
       if (moved < 1e-7) break;
     }

@@ -49,6 +49,7 @@ struct qgx_ctx {
   float sym_levels[QGX_MAX_LEVELS];
   int decode_split;                      // QGX_SPLIT_AUTO / NEVER / ALWAYS: see qgx_set_decode_split
   int encode_path;                       // QGX_ENCODE_AUTO / REGISTERS: see qgx_set_encode_path
+  double* hist_pinned;                   // host side of the refit's histogram (page-locked, allocated at the first refit)
   int num_sms;                           // multiprocessors that this context's persistent kernels are launched for
   int all_sms;                           // multiprocessors of the device
   // host-side cache of the fused calls: tables derived from a quantizer configuration (with their device copies)
