@@ -211,7 +211,7 @@ def run_ours(args):
     enc_ms = ms_enc / max(n_enc, 1)
     achieved = enc_bytes / (enc_ms * 1e-3) / 1e9 if n_enc else None
     # DRAM bytes per launch of that kernel: counted by ncu on a smaller case of the same kernel (see
-    # profiles/exchange_kernels_K8_d16M.txt: 655.2 MB read + written for K * d = 2^27 coordinates) and scaled by
+    # profiles/exchange_kernels_K8_d16M.txt: K * d = 2^27 coordinates) and scaled by
     # the coordinates of a launch, which the traffic is proportional to.  Set to None when the kernel changes.
     dram_per_coord, instr_per_coord = profile_constants()
     traffic = args.traffic_bytes
@@ -226,7 +226,7 @@ def run_ours(args):
         alu_peak = 148 * 128 * sm_mhz * 1e6 / 1e12
         alu_ach = instr_per_coord * K * d / (enc_ms * 1e-3) / 1e12
         alu = {"achieved": alu_ach, "peak": alu_peak, "unit": "T thread-instructions/s", "frac": alu_ach / alu_peak}
-    roofline = {"bound": "hbm", "kernel": "k_exchange_encode", "achieved": achieved, "peak": peak, "unit": "GB/s",
+    roofline = {"bound": "hbm", "kernel": "k_encode_pipeline", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": (achieved / peak) if achieved else None, "peak_kind": "of " + peak_kind,
                 "traffic": traffic, "ms_per_launch": enc_ms, "alu": alu,
                 "kernels_ms_per_step": {"encode": ms_enc / args.steps, "decode": ms_dec / args.steps,
