@@ -368,6 +368,7 @@ struct UnpackArgs {
   size_t nb;
   const uint16_t* lut;                   // [1 << maxlen]: level | codeword length << 8
   int store;                             // bytes per symbol store: 16, 4 or 1
+  int spread;                            // lanes per bucket without sub-blocks (one of them walks)
   float* norms;
   uint8_t* sym;
   DevStatus* st;
@@ -387,7 +388,7 @@ __global__ void __launch_bounds__(128) k_unpack(const __grid_constant__ UnpackAr
   const int lane = threadIdx.x & 31;
   const uint32_t mask = (uint32_t)tab_n - 1u;
   const int G = ct.G, spb = ct.has_header ? (a.bucket + G - 1) / G : 1;         // sub-blocks of a whole bucket
-  int group = 1;                                                                // lanes per bucket
+  int group = ct.has_header ? 1 : a.spread;                                     // lanes per bucket
   while (group < spb && group < 32) group <<= 1;
   const int rows = (spb + 31) / 32, per_warp = 32 / group;                      // warps per bucket, or buckets per warp
   const size_t buckets = a.nb * (size_t)a.K;
@@ -607,6 +608,11 @@ qgx_status qgx_decode(qgx_ctx* c, const uint32_t* stream, size_t cap_words, cons
   const size_t spb = ct->has_header ? (size_t)((bucket + ct->G - 1) / ct->G) : 1;
   size_t lanes = 1;
   while (lanes < spb && lanes < 32) lanes *= 2;
+  // Without sub-blocks a bucket is one lane's walk, and lanes that fetch their next words at different symbols make the whole
+  // warp wait for memory at nearly every symbol: as few walks in a warp as leave up to 16 warps per SM (68 buckets of 512
+  // coordinates: walked 66 -> 45 us by a decode; 8 x 2^20 coordinates 540 -> 45).
+  while (!ct->has_header && lanes < 32 && nb * (size_t)K * lanes * 2 <= (size_t)c->num_sms * 16u * 32u) lanes *= 2;
+  a.spread = (int)lanes;
   const size_t warps = spb > 32 ? nb * (size_t)K * ((spb + 31) / 32) : (nb * (size_t)K * lanes + 31) / 32;
   const size_t smem = sizeof(uint16_t) * ((size_t)2 << ct->maxlen);
   const unsigned grid = (unsigned)std::max<size_t>(1, std::min<size_t>((warps + 3) / 4, (size_t)c->num_sms * 12u));

@@ -11,7 +11,7 @@
 // What bounds it: instruction issue and latency.  A quantizer's core alone (data already in shared memory, 16 warps) takes
 // 0.40 cycles per coordinate and SM: 33 instructions at 65 % issue, with the ALU, the integer multiplier (the generator's
 // wide products run at a quarter of the rate) and the shared-memory pipe each 55-60 % busy.  With copies, norms and
-// placing it is 65 instructions at about 57 %.  Shared memory (two stages and two to four images per quantizer) sets the
+// placing it is 60 instructions at 62 %.  Shared memory (two stages and two to four images per quantizer) sets the
 // number of warps.  Measured per 2^27 coordinates against the bucket-in-registers kernel, whose CTAs load, norm, round
 // and write one after the other with three CTA barriers per bucket: buckets of 16384 395 us (433), 8192 392 us (508),
 // 4096 390 us (480), 1024 379 us (883); rows that are not 16-byte aligned, 16 x 10^6 coordinates, 69 us (234), since

@@ -74,3 +74,18 @@ def test_steps_match_oracle(K, d, bucket, nlev, sub, roomy):
             assert qgx.qgx_sync_status(ctx, check=False) == qgx.QGX_ERR_CORRUPT
     finally:
         qgx.qgx_destroy(ctx)
+
+
+@pytest.mark.parametrize("K,d,bucket", [(2, 37 * 64, 64), (1, 148 * 16 * 32 * 4, 4), (1, 148 * 16 * 16 * 4 + 4, 4), (3, 148 * 16 * 4 * 16 + 13, 16)])
+def test_decode_without_sub_blocks_spreads_its_walks(K, d, bucket):
+    """One walk per bucket, from one to thirty-two buckets in a warp: on both sides of the counts where that changes."""
+    import paper_2308_09187_b200 as qgx
+    ctx = qgx.qgx_create(0)
+    v = torch.randn((K, d), device="cuda", generator=torch.Generator("cuda").manual_seed(d))
+    cb = qgx.qgx_build_codebook_elias(9, 0)
+    norms, sym = qgx.qgx_quantize(ctx, v, bucket, [j / 8 for j in range(9)], qgx.QGX_NORM_L2, 5, 1)
+    stream, bits, _ = qgx.qgx_encode(ctx, norms, sym, bucket, cb)
+    got_norms, got_sym = qgx.qgx_decode(ctx, stream, bits, d, bucket, cb)
+    qgx.qgx_sync_status(ctx)
+    assert torch.equal(got_norms, norms) and torch.equal(got_sym, sym)
+    qgx.qgx_destroy(ctx)
