@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(128) k_unpack(const __grid_constant__ UnpackAr
       }
     };
     int i = 0;
-    if (a.store == 16) {
+    if (a.store >= 4) {
       for (; i + 16 <= count; i += 16) {
         uint32_t wd[4];
 #pragma unroll
@@ -490,7 +490,12 @@ __global__ void __launch_bounds__(128) k_unpack(const __grid_constant__ UnpackAr
           x |= symbol() << 24;
           wd[q] = x;
         }
-        *reinterpret_cast<uint4*>(out + i) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+        if (a.store == 16) {
+          *reinterpret_cast<uint4*>(out + i) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) *reinterpret_cast<uint32_t*>(out + i + 4 * q) = wd[q];
+        }
       }
     }
     for (; i < count; i += kQuad) {
@@ -610,7 +615,7 @@ qgx_status qgx_decode(qgx_ctx* c, const uint32_t* stream, size_t cap_words, cons
   while (lanes < spb && lanes < 32) lanes *= 2;
   // Without sub-blocks a bucket is one lane's walk, and lanes that fetch their next words at different symbols make the whole
   // warp wait for memory at nearly every symbol: as few walks in a warp as leave up to 16 warps per SM (68 buckets of 512
-  // coordinates: walked 66 -> 45 us by a decode; 8 x 2^20 coordinates 540 -> 45).
+  // coordinates: 66 -> 45 us for a decode; 8 x 2^20 coordinates 540 -> 45).
   while (!ct->has_header && lanes < 32 && nb * (size_t)K * lanes * 2 <= (size_t)c->num_sms * 16u * 32u) lanes *= 2;
   a.spread = (int)lanes;
   const size_t warps = spb > 32 ? nb * (size_t)K * ((spb + 31) / 32) : (nb * (size_t)K * lanes + 31) / 32;
