@@ -199,8 +199,9 @@ __device__ __forceinline__ void fill_bin_table(float4* bin, const RoundTable& rt
     const uint32_t b = (uint32_t)(i >> rep_log);
     const float lo = __uint_as_float(kKeyBase + (b << rt.key_shift));
     const float hi = __uint_as_float(kKeyBase + ((b + 1u) << rt.key_shift) - 1u);
-    int t0 = 0;
-    for (int j = 1; j <= rt.nlev - 2; ++j) t0 = (rt.knot[j] <= lo) ? j : t0;
+    int t0 = 0;                            // the last interior level whose knot is not above lo (the knots rise)
+    for (int step = QGX_MAX_LEVELS / 2; step > 0; step >>= 1)
+      if (t0 + step <= rt.nlev - 2 && rt.knot[t0 + step] <= lo) t0 += step;
     const bool straddle = (t0 + 1 <= rt.nlev - 2) && (rt.knot[t0 + 1] <= hi);
     const float icpt = kind == BinKind::kFixed ? rt.afix[t0] : rt.a16[t0];
     bin[i] = make_float4(icpt, rt.b[t0] * scale, straddle ? rt.knot[t0 + 1] : 4.0f, straddle ? rt.db[t0 + 1] * scale : 0.0f);

@@ -9,15 +9,15 @@
 
 namespace qgx {
 
-// ---- what the separate calls derive from their levels and codes, kept between calls ---------------
-// Building the rounding table costs the host some 50 us, the decoder table a copy to the device: a program calls with a
-// handful of tables, so a context keeps the last few (compared in full on a hit).
+// ---- the rounding table of a level table, kept between calls on the host --------------------------
+// Building one takes the host some 50 us (four bin widths, up to 1025 bins, all levels), and a program calls with a handful of
+// level tables, so a context keeps the last few (compared in full on a hit).  It goes to the kernel by value: the call
+// allocates nothing, and a launch recorded in a stream capture keeps the table that it was recorded with.
+constexpr int kStepSlots = 8;
 struct StepLevels {
-  bool valid;
-  int nlev;
+  int nlev;                              // 0: empty
   float lev[QGX_MAX_LEVELS];
   RoundTable rt;
-  float4* bins;                          // [dev] the fixed-point map's bin table, owned
 };
 struct StepCode {
   bool valid;
@@ -26,15 +26,11 @@ struct StepCode {
   CodeTable ct;
   uint16_t* lut;                         // [dev] decoder table, owned
 };
-constexpr int kStepSlots = 8;
 struct StepCache {
   StepLevels lev[kStepSlots];
+  int oldest;                            // of the level tables: the next to be replaced
   StepCode code[kStepSlots];
 };
-
-__global__ void __launch_bounds__(512) k_build_bins(const __grid_constant__ RoundTable rt, float4* out) {
-  fill_bin_table(out, rt, BinKind::kFixed);
-}
 
 static StepCache* step_cache(qgx_ctx* c) {
   if (!c->step_cache) c->step_cache = new (std::nothrow) StepCache();          // value-initialized: all zero
@@ -43,10 +39,8 @@ static StepCache* step_cache(qgx_ctx* c) {
 void free_step_cache(qgx_ctx* c) {
   StepCache* sc = (StepCache*)c->step_cache;
   if (!sc) return;
-  for (int i = 0; i < kStepSlots; ++i) {
-    if (sc->lev[i].bins) cudaFree(sc->lev[i].bins);
+  for (int i = 0; i < kStepSlots; ++i)
     if (sc->code[i].lut) cudaFree(sc->code[i].lut);
-  }
   delete sc;
   c->step_cache = nullptr;
 }
@@ -56,27 +50,18 @@ static uint32_t mix_bytes(uint32_t h, const void* p, size_t n) {
   return h;
 }
 
-static qgx_status step_levels(qgx_ctx* c, const float* lev, int nlev, const StepLevels** out) {
+static const RoundTable* step_round_table(qgx_ctx* c, const float* lev, int nlev) {
   StepCache* sc = step_cache(c);
-  if (!sc) return QGX_ERR_CUDA;
-  StepLevels* e = &sc->lev[mix_bytes(2166136261u, lev, sizeof(float) * (size_t)nlev) % kStepSlots];
-  if (!(e->valid && e->nlev == nlev && std::memcmp(e->lev, lev, sizeof(float) * (size_t)nlev) == 0)) {
-    e->valid = false;
-    make_round_table(lev, nlev, &e->rt);
-    if (!e->bins && cudaMalloc((void**)&e->bins, sizeof(float4) * kBinEntries) != cudaSuccess) {
-      cudaGetLastError();
-      e->bins = nullptr;
-      return QGX_ERR_CUDA;
-    }
-    k_build_bins<<<1, 512, 0, c->stream>>>(e->rt, e->bins);           // ordered after the kernels that still read the old one
-    count_launch(c);
-    if (cudaGetLastError() != cudaSuccess) return QGX_ERR_CUDA;
-    e->nlev = nlev;
-    std::memcpy(e->lev, lev, sizeof(float) * (size_t)nlev);
-    e->valid = true;
-  }
-  *out = e;
-  return QGX_OK;
+  if (!sc) return nullptr;
+  const size_t bytes = sizeof(float) * (size_t)nlev;
+  for (const StepLevels& e : sc->lev)
+    if (e.nlev == nlev && std::memcmp(e.lev, lev, bytes) == 0) return &e.rt;
+  StepLevels* e = &sc->lev[sc->oldest];
+  sc->oldest = (sc->oldest + 1) % kStepSlots;
+  make_round_table(lev, nlev, &e->rt);
+  e->nlev = nlev;
+  std::memcpy(e->lev, lev, bytes);
+  return &e->rt;
 }
 
 qgx_status step_code(qgx_ctx* c, const qgx_codebook* cb, int bucket, const CodeTable** ct, const uint16_t** lut) {
@@ -119,7 +104,6 @@ struct QuantizeArgs {
   uint32_t xid;
   bool vec_ok;                           // 16-byte loads
   int store;                             // bytes per symbol store: 8, 4 or 1
-  const float4* bins;
   float* norms;
   uint8_t* sym;
   DevStatus* st;
@@ -127,8 +111,10 @@ struct QuantizeArgs {
 
 // Persistent CTAs, one bucket at a time held in registers between the norm and the rounding (v is read from HBM once); a
 // thread works on P octets of consecutive coordinates.  What bounds it: instruction issue -- about 26 instructions per
-// coordinate are the generator and the rounding map.  The map's table comes ready made from global memory, once per CTA:
-// built by every CTA for its one bucket, as before, it cost more than a small bucket.
+// coordinate are the generator and the rounding map.  Every CTA builds the map's table in shared memory from the launch's
+// parameters, once for all of its buckets: a table kept in device memory measured the same (quantize + encode of 8 x 2^22
+// coordinates 154.8 us with it, 154.7 so; four calls on 4 x 8200, 51.1 and 51.7, runs 5 % apart) but needs an allocation and
+// changes under a recorded launch.
 template <int P>
 __global__ void __launch_bounds__(P == 1 ? 256 : 512, P == 1 ? 4 : 2)
 k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ LevelTable lt, const __grid_constant__ PhiloxKey key,
@@ -136,7 +122,7 @@ k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ Level
   __shared__ __align__(128) float4 s_bin[kBinEntries];
   __shared__ float s_lev[QGX_MAX_LEVELS];
   __shared__ double s_red[2][32];
-  for (int i = threadIdx.x; i < kBinEntries; i += blockDim.x) s_bin[i] = __ldg(a.bins + i);
+  fill_bin_table(s_bin, rt, BinKind::kFixed);
   if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -310,9 +296,8 @@ static bool all_aligned16(std::initializer_list<const void*> ps) {
 qgx_status launch_quantize(qgx_ctx* c, DualSource src, int K, size_t d, int bucket, const LevelTable& lt, int norm_type,
                            uint64_t seed, uint32_t xid, int norms_supplied, float* norms, uint8_t* sym) {
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
-  const StepLevels* tables = nullptr;
-  const qgx_status rc = step_levels(c, lt.lev, lt.nlev, &tables);
-  if (rc != QGX_OK) return rc;
+  const RoundTable* rt = step_round_table(c, lt.lev, lt.nlev);
+  if (!rt) return QGX_ERR_CUDA;
   const PhiloxKey key = make_philox_key(seed);
   QuantizeArgs a;
   a.src = src; a.d = d; a.bucket = bucket; a.nb = nb; a.total = nb * (size_t)K;
@@ -320,7 +305,7 @@ qgx_status launch_quantize(qgx_ctx* c, DualSource src, int K, size_t d, int buck
   a.vec_ok = (d % kQuad == 0) && all_aligned16({src.v, src.a});
   const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
   a.store = (d % 8 == 0 && bucket % 8 == 0 && (at & 7u) == 0) ? 8 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
-  a.bins = tables->bins; a.norms = norms; a.sym = sym; a.st = c->dstatus;
+  a.norms = norms; a.sym = sym; a.st = c->dstatus;
   // octets per thread so that CTAs have at most 256 / 512 / 512 threads; as many CTAs as an SM holds (registers: 1024
   // threads; shared memory: 12 tables of 17 KB)
   const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
@@ -328,9 +313,9 @@ qgx_status launch_quantize(qgx_ctx* c, DualSource src, int K, size_t d, int buck
   const unsigned per_sm = (unsigned)std::min(12, std::max(2, 1024 / threads));
   const unsigned grid = (unsigned)std::min<size_t>(a.total, (size_t)c->num_sms * per_sm);
   switch (pp) {
-    case 1: k_quantize<1><<<grid, threads, 0, c->stream>>>(a, lt, key, tables->rt); break;
-    case 2: k_quantize<2><<<grid, threads, 0, c->stream>>>(a, lt, key, tables->rt); break;
-    default: k_quantize<4><<<grid, threads, 0, c->stream>>>(a, lt, key, tables->rt); break;
+    case 1: k_quantize<1><<<grid, threads, 0, c->stream>>>(a, lt, key, *rt); break;
+    case 2: k_quantize<2><<<grid, threads, 0, c->stream>>>(a, lt, key, *rt); break;
+    default: k_quantize<4><<<grid, threads, 0, c->stream>>>(a, lt, key, *rt); break;
   }
   count_launch(c);
   return cuda_status(cudaGetLastError());
