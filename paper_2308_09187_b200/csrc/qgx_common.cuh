@@ -189,22 +189,35 @@ struct RoundTable {
   uint32_t thrfix;                       // distances below this go to the exact routine (2^16: all of them)
 };
 
-// one entry per bin and copy: {a16 or afix, b, knot, db} of the interval of the bin's lowest value
+// one entry per bin and copy: {a16 or afix, b, knot, db} of the interval of the bin's lowest value.  A thread writes a run of
+// entries (an odd number of them, so that neighbouring threads' stores go to different banks) and fetches an interval's
+// numbers when its run reaches the interval: one bin at a time, each with its own search, took a CTA of two warps 2 us more.
 enum class BinKind { kOctet, kFixed };
 __device__ __forceinline__ void fill_bin_table(float4* bin, const RoundTable& rt, BinKind kind) {
   const float scale = kind == BinKind::kFixed ? rt.fix_scale : 1.0f;
   const int rep_log = rt.key_shift - kKeyShiftMin;
-  const int nbins = (int)((kKeyTop - kKeyBase) >> rt.key_shift) + 1;
-  for (int i = threadIdx.x; i < (nbins << rep_log); i += blockDim.x) {
-    const uint32_t b = (uint32_t)(i >> rep_log);
-    const float lo = __uint_as_float(kKeyBase + (b << rt.key_shift));
-    const float hi = __uint_as_float(kKeyBase + ((b + 1u) << rt.key_shift) - 1u);
-    int t0 = 0;                            // the last interior level whose knot is not above lo (the knots rise)
-    for (int step = QGX_MAX_LEVELS / 2; step > 0; step >>= 1)
-      if (t0 + step <= rt.nlev - 2 && rt.knot[t0 + step] <= lo) t0 += step;
-    const bool straddle = (t0 + 1 <= rt.nlev - 2) && (rt.knot[t0 + 1] <= hi);
-    const float icpt = kind == BinKind::kFixed ? rt.afix[t0] : rt.a16[t0];
-    bin[i] = make_float4(icpt, rt.b[t0] * scale, straddle ? rt.knot[t0 + 1] : 4.0f, straddle ? rt.db[t0 + 1] * scale : 0.0f);
+  const int n = ((int)((kKeyTop - kKeyBase) >> rt.key_shift) + 1) << rep_log;
+  const int run = ((n + (int)blockDim.x - 1) / (int)blockDim.x) | 1;
+  const auto lowest = [&](int i) { return __uint_as_float(kKeyBase + ((uint32_t)(i >> rep_log) << rt.key_shift)); };
+  int i = (int)threadIdx.x * run;
+  const int end = min(n, i + run);
+  if (i >= end) return;
+  int t0 = 0;                              // the last interior level whose knot is not above the bin's lowest value (the knots rise)
+  for (int step = QGX_MAX_LEVELS / 2; step > 0; step >>= 1)
+    if (t0 + step <= rt.nlev - 2 && rt.knot[t0 + step] <= lowest(i)) t0 += step;
+  float icpt, slope, knot, db;             // of that interval, and of the level above it (knot 4 where there is none)
+  const auto fetch = [&]() {
+    icpt = kind == BinKind::kFixed ? rt.afix[t0] : rt.a16[t0];
+    slope = rt.b[t0] * scale;
+    knot = rt.knot[t0 + 1];
+    db = rt.db[t0 + 1] * scale;
+  };
+  fetch();
+  for (; i < end; ++i) {
+    const float lo = lowest(i), hi = __uint_as_float(__float_as_uint(lo) + (1u << rt.key_shift) - 1u);
+    while (knot <= lo) { ++t0; fetch(); }
+    const bool straddle = knot <= hi;
+    bin[i] = make_float4(icpt, slope, straddle ? knot : 4.0f, straddle ? db : 0.0f);
   }
 }
 

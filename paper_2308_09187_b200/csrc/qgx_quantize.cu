@@ -112,9 +112,9 @@ struct QuantizeArgs {
 // Persistent CTAs, one bucket at a time held in registers between the norm and the rounding (v is read from HBM once); a
 // thread works on P octets of consecutive coordinates.  What bounds it: instruction issue -- about 26 instructions per
 // coordinate are the generator and the rounding map.  Every CTA builds the map's table in shared memory from the launch's
-// parameters, once for all of its buckets: a table kept in device memory measured the same (quantize + encode of 8 x 2^22
-// coordinates 154.8 us with it, 154.7 so; four calls on 4 x 8200, 51.1 and 51.7, runs 5 % apart) but needs an allocation and
-// changes under a recorded launch.
+// parameters, once for all of its buckets: a table kept in device memory measured the same (4 x 8200 coordinates 6.2 us a
+// call with it, 6.4 so; quantize + encode of 8 x 2^22, 155.0 and 154.6) but needs an allocation and changes under a recorded
+// launch.
 template <int P>
 __global__ void __launch_bounds__(P == 1 ? 256 : 512, P == 1 ? 4 : 2)
 k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ LevelTable lt, const __grid_constant__ PhiloxKey key,
