@@ -18,8 +18,9 @@
  *  - the library allocates device memory only inside qgx_create and when a call needs a larger
  *    workspace than any call before it (qgx_encode, qgx_decode, the fused calls and qgx_update_levels);
  *    the fused calls also keep device tables of the up to 32 configurations they have met.  qgx_quantize,
- *    qgx_average and qgx_encode_noalloc allocate nothing and may be recorded into a stream capture: what they
- *    derive from their level table or code goes with the launch, so a replay uses what was recorded.
+ *    qgx_average and qgx_encode_noalloc allocate nothing and may be recorded into a stream capture, qgx_decode once
+ *    its workspace has the size (after a call on as many buckets): what they derive from their level table or code
+ *    goes with the launch, so a replay uses what was recorded.
  *
  * Symbol byte: bits 0..4 level index, bit 7 sign (set only when the level index is nonzero).
  * Stream: 32-bit words, bit p of a stream is bit (p & 31) of word (p >> 5).

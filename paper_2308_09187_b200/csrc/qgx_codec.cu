@@ -5,7 +5,6 @@
 
 #include <algorithm>
 #include <mutex>
-#include <vector>
 
 namespace qgx {
 
@@ -68,13 +67,45 @@ __global__ void __launch_bounds__(512) k_bucket_bits(const uint8_t* __restrict__
   }
 }
 
+// The decoder's table: index = the next maxlen + 1 stream bits, entry = symbol byte | bits consumed << 8, 0 where no codeword
+// starts like the index.  By the threads of one CTA: codewords of up to six bits by way of a table of 64, so that neighbouring
+// threads write neighbouring entries, then the few entries of the longer ones.
+constexpr int kUnpackTableMax = 2 << QGX_MAX_CODE_LEN;
+__device__ __forceinline__ void build_unpack_table(const CodeTable& ct, uint16_t* table /* [2 << maxlen] */) {
+  __shared__ uint16_t s_short[64];       // level | length << 8
+  const int tab_n = 2 << ct.maxlen;
+  if (threadIdx.x < 64) {
+    uint32_t e = 0;
+    for (int j = 0; j < ct.nlev; ++j)
+      if (ct.len[j] <= 6 && (threadIdx.x & ((1u << ct.len[j]) - 1u)) == ct.rev[j]) e = (uint32_t)j | ((uint32_t)ct.len[j] << 8);
+    s_short[threadIdx.x] = (uint16_t)e;
+  }
+  __syncthreads();
+  const auto entry = [](uint32_t level, uint32_t L, uint32_t sign) { return (uint16_t)(level == 0 ? L << 8 : ((L + 1u) << 8) | level | (sign << 7)); };
+  for (int i = threadIdx.x; i < tab_n; i += blockDim.x) {
+    const uint32_t x = s_short[i & 63], L = x >> 8;
+    table[i] = x == 0 ? (uint16_t)0 : entry(x & 0xffu, L, ((uint32_t)i >> L) & 1u);
+  }
+  __syncthreads();
+  for (int j = 0; j < ct.nlev; ++j) {
+    const int L = ct.len[j];
+    if (L <= 6) continue;
+    for (int i = threadIdx.x; i < (tab_n >> L); i += blockDim.x) table[ct.rev[j] | (i << L)] = entry((uint32_t)j, (uint32_t)L, (uint32_t)i & 1u);
+  }
+}
+
 // One CTA per worker: off[k][b] = sum_{b' < b} ceil(bits[k][b'] / 32); total_bits[k]; a worker whose
 // words exceed cap_words is flagged (flags[k] = 1) and err_code is latched.  4096 buckets per turn of the loop: a worker's
-// lengths are a serial chain of turns, each a few barriers long.
+// lengths are a serial chain of turns, each a few barriers long.  Before a decode one CTA more (the K-th) builds the
+// decoder's table, afresh in every call: nothing is kept that a later call could change under a recorded one, and no launch
+// is added (decode + average of 8 x 2^22 coordinates 69.3 us with a table kept per code and widened by every CTA of the
+// decoder, 67.7 so; every CTA building it from the code, 71.5).
 constexpr int kScanThreads = 1024, kScanEach = 4;
 __global__ void __launch_bounds__(kScanThreads) k_scan_offsets(const uint32_t* __restrict__ bucket_bits, size_t nb, size_t cap_words,
                                                                uint64_t* __restrict__ off, uint64_t* __restrict__ total_bits,
-                                                               uint32_t* __restrict__ flags, unsigned int err_code, DevStatus* st) {
+                                                               uint32_t* __restrict__ flags, unsigned int err_code, DevStatus* st,
+                                                               int K, const __grid_constant__ CodeTable ct, uint16_t* table) {
+  if (blockIdx.x == (unsigned)K) { build_unpack_table(ct, table); return; }
   __shared__ uint64_t s_words[2][32], s_bits[2][32];
   const size_t k = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -363,10 +394,10 @@ struct UnpackArgs {
   const uint32_t* bucket_bits;
   const uint64_t* off;
   const uint32_t* flags;
+  const uint16_t* table;                 // see build_unpack_table
   size_t d;
   int bucket, K;
   size_t nb;
-  const uint16_t* lut;                   // [1 << maxlen]: level | codeword length << 8
   int store;                             // bytes per symbol store: 16, 4 or 1
   int spread;                            // lanes per bucket without sub-blocks (one of them walks)
   float* norms;
@@ -375,15 +406,12 @@ struct UnpackArgs {
 };
 
 // One thread per sub-block (per bucket without sub-blocks), a warp on consecutive ones of one bucket or of several small
-// buckets; persistent CTAs, so that the table is built once per CTA and not once per bucket.  Every read is bounded by the
+// buckets; persistent CTAs, so that the table is copied once per CTA and not once per bucket.  Every read is bounded by the
 // bucket's words.  A serial walk per thread: latency-bound with few sub-blocks, instruction-bound (14 per symbol) with many.
 __global__ void __launch_bounds__(128) k_unpack(const __grid_constant__ UnpackArgs a, const __grid_constant__ CodeTable ct) {
-  extern __shared__ uint16_t s_tab[];    // [2 << maxlen]: the next maxlen + 1 bits -> symbol byte | bits consumed << 8, 0: none
+  extern __shared__ __align__(16) uint16_t s_tab[];  // [2 << maxlen], see build_unpack_table
   const int tab_n = 2 << ct.maxlen;
-  for (int i = threadIdx.x; i < tab_n; i += blockDim.x) {
-    const uint32_t w = a.lut[i & ((tab_n >> 1) - 1)], L = w >> 8, idx = w & 0xffu;
-    s_tab[i] = (uint16_t)(L == 0 ? 0u : (idx == 0 ? L << 8 : ((L + 1u) << 8) | idx | ((((uint32_t)i >> L) & 1u) << 7)));
-  }
+  for (int i = threadIdx.x; i < (tab_n + 7) / 8; i += blockDim.x) reinterpret_cast<uint4*>(s_tab)[i] = __ldg(reinterpret_cast<const uint4*>(a.table) + i);
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const uint32_t mask = (uint32_t)tab_n - 1u;
@@ -573,7 +601,7 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
   const int threads = bucket_threads(bucket, v4);
   const dim3 grid((unsigned)nb, (unsigned)K);
   k_bucket_bits<<<grid, threads, 0, c->stream>>>(sym, d, bucket, ct, vec_ok, bucket_bits, c->dstatus);
-  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus);
+  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus, K, ct, nullptr);
   const size_t smem = sizeof(uint32_t) * (img_words + (size_t)(bucket / ct.G) + 2);
 #define QGX_LAUNCH_S(V)                                                                                         \
   do {                                                                                                          \
@@ -596,32 +624,32 @@ qgx_status qgx_decode(qgx_ctx* c, const uint32_t* stream, size_t cap_words, cons
                       int bucket, const qgx_codebook* cb, float* norms, uint8_t* sym) {
   if (!codec_args_ok(c, K, d, bucket) || !norms || !sym || !stream || !bucket_bits) return QGX_ERR_INVALID_ARG;
   if (cudaSetDevice(c->device) != cudaSuccess) return QGX_ERR_CUDA;
-  const CodeTable* ct = nullptr;
-  const uint16_t* lut = nullptr;
-  const qgx_status rc = step_code(c, cb, bucket, &ct, &lut);
+  CodeTable ct;
+  const qgx_status rc = make_code_table(cb, bucket, &ct);
   if (rc != QGX_OK) return rc;
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
   uint64_t* off = (uint64_t*)ws_get(c, 0, sizeof(uint64_t) * (size_t)K * nb);
   uint32_t* flags = (uint32_t*)ws_get(c, 1, sizeof(uint32_t) * (size_t)K);
-  if (!off || !flags) return QGX_ERR_CUDA;
-  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, nullptr, flags, QGX_ERR_CORRUPT, c->dstatus);
+  uint16_t* table = (uint16_t*)ws_get(c, 2, sizeof(uint16_t) * kUnpackTableMax);
+  if (!off || !flags || !table) return QGX_ERR_CUDA;
+  k_scan_offsets<<<K + 1, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, nullptr, flags, QGX_ERR_CORRUPT, c->dstatus, K, ct, table);
   UnpackArgs a;
-  a.stream = stream; a.cap_words = cap_words; a.bucket_bits = bucket_bits; a.off = off; a.flags = flags; a.d = d; a.bucket = bucket;
-  a.K = K; a.nb = nb; a.lut = lut; a.norms = norms; a.sym = sym; a.st = c->dstatus;
+  a.stream = stream; a.cap_words = cap_words; a.bucket_bits = bucket_bits; a.off = off; a.flags = flags; a.table = table; a.d = d;
+  a.bucket = bucket; a.K = K; a.nb = nb; a.norms = norms; a.sym = sym; a.st = c->dstatus;
   const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
-  a.store = (d % 16 == 0 && bucket % 16 == 0 && ct->G % 16 == 0 && (at & 15u) == 0) ? 16 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
-  const size_t spb = ct->has_header ? (size_t)((bucket + ct->G - 1) / ct->G) : 1;
+  a.store = (d % 16 == 0 && bucket % 16 == 0 && ct.G % 16 == 0 && (at & 15u) == 0) ? 16 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
+  const size_t spb = ct.has_header ? (size_t)((bucket + ct.G - 1) / ct.G) : 1;
   size_t lanes = 1;
   while (lanes < spb && lanes < 32) lanes *= 2;
   // Without sub-blocks a bucket is one lane's walk, and lanes that fetch their next words at different symbols make the whole
   // warp wait for memory at nearly every symbol: as few walks in a warp as leave up to 16 warps per SM (68 buckets of 512
   // coordinates: 66 -> 45 us for a decode; 8 x 2^20 coordinates 540 -> 45).
-  while (!ct->has_header && lanes < 32 && nb * (size_t)K * lanes * 2 <= (size_t)c->num_sms * 16u * 32u) lanes *= 2;
+  while (!ct.has_header && lanes < 32 && nb * (size_t)K * lanes * 2 <= (size_t)c->num_sms * 16u * 32u) lanes *= 2;
   a.spread = (int)lanes;
   const size_t warps = spb > 32 ? nb * (size_t)K * ((spb + 31) / 32) : (nb * (size_t)K * lanes + 31) / 32;
-  const size_t smem = sizeof(uint16_t) * ((size_t)2 << ct->maxlen);
+  const size_t smem = std::max<size_t>(16, sizeof(uint16_t) * ((size_t)2 << ct.maxlen));
   const unsigned grid = (unsigned)std::max<size_t>(1, std::min<size_t>((warps + 3) / 4, (size_t)c->num_sms * 12u));
-  k_unpack<<<grid, 128, smem, c->stream>>>(a, *ct);
+  k_unpack<<<grid, 128, smem, c->stream>>>(a, ct);
   count_launch(c, 2);
   return cuda_status(cudaGetLastError());
 }
@@ -669,7 +697,7 @@ qgx_status qgx_encode_noalloc(qgx_ctx* c, const float* norms, const uint8_t* sym
   const int threads = bucket_threads(bucket, v4);
   const dim3 grid((unsigned)nb, (unsigned)K);
   k_bucket_bits<<<grid, threads, 0, c->stream>>>(sym, d, bucket, ct, vec_ok, bucket_bits, c->dstatus);
-  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus);
+  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus, K, ct, nullptr);
   const size_t img_words = (((size_t)bucket * (ct.maxlen + 1) + 16u * (bucket / ct.G + 1) + kNormBits + 31u) >> 5) + 4;
   const size_t smem = sizeof(uint32_t) * (img_words + (size_t)(bucket / ct.G) + 2);
 #define QGX_LAUNCH_S(V)                                                                                         \

@@ -55,7 +55,7 @@ struct qgx_ctx {
   // host-side cache of the fused calls: tables derived from a quantizer configuration (with their device copies)
   // and launch shapes; owned by qgx_exchange.cu
   void* table_cache;
-  void* step_cache;                      // the same for the separate calls; owned by qgx_quantize.cu
+  void* step_cache;                      // host-side rounding tables of qgx_quantize; owned by qgx_quantize.cu
   // helper contexts (own streams and workspaces) that run the tensors of a layer-wise exchange side by side;
   // owned by qgx_exchange.cu
   void* seg_children;
@@ -455,7 +455,6 @@ void make_round_table(const float* lev, int nlev, RoundTable* out);
 void* ws_get(qgx_ctx* c, int which, size_t bytes);          // nullptr on failure
 void free_table_cache(qgx_ctx* c);
 void free_step_cache(qgx_ctx* c);
-qgx_status step_code(qgx_ctx* c, const qgx_codebook* cb, int bucket, const CodeTable** ct, const uint16_t** lut /*[dev]*/);
 void free_seg_children(qgx_ctx* c);
 uint64_t seg_children_launches(const qgx_ctx* c);
 qgx_status cuda_status(cudaError_t e);

@@ -5,7 +5,6 @@
 #include <algorithm>
 #include <cstring>
 #include <new>
-#include <vector>
 
 namespace qgx {
 
@@ -19,17 +18,9 @@ struct StepLevels {
   float lev[QGX_MAX_LEVELS];
   RoundTable rt;
 };
-struct StepCode {
-  bool valid;
-  int bucket;
-  qgx_codebook cb;
-  CodeTable ct;
-  uint16_t* lut;                         // [dev] decoder table, owned
-};
 struct StepCache {
   StepLevels lev[kStepSlots];
-  int oldest;                            // of the level tables: the next to be replaced
-  StepCode code[kStepSlots];
+  int oldest;                            // the next to be replaced
 };
 
 static StepCache* step_cache(qgx_ctx* c) {
@@ -37,17 +28,8 @@ static StepCache* step_cache(qgx_ctx* c) {
   return (StepCache*)c->step_cache;
 }
 void free_step_cache(qgx_ctx* c) {
-  StepCache* sc = (StepCache*)c->step_cache;
-  if (!sc) return;
-  for (int i = 0; i < kStepSlots; ++i)
-    if (sc->code[i].lut) cudaFree(sc->code[i].lut);
-  delete sc;
+  delete (StepCache*)c->step_cache;
   c->step_cache = nullptr;
-}
-static uint32_t mix_bytes(uint32_t h, const void* p, size_t n) {
-  const unsigned char* b = (const unsigned char*)p;
-  for (size_t i = 0; i < n; ++i) { h ^= b[i]; h *= 16777619u; }
-  return h;
 }
 
 static const RoundTable* step_round_table(qgx_ctx* c, const float* lev, int nlev) {
@@ -62,37 +44,6 @@ static const RoundTable* step_round_table(qgx_ctx* c, const float* lev, int nlev
   e->nlev = nlev;
   std::memcpy(e->lev, lev, bytes);
   return &e->rt;
-}
-
-qgx_status step_code(qgx_ctx* c, const qgx_codebook* cb, int bucket, const CodeTable** ct, const uint16_t** lut) {
-  StepCache* sc = step_cache(c);
-  if (!sc) return QGX_ERR_CUDA;
-  if (cb == nullptr || cb->nlev < 2 || cb->nlev > QGX_MAX_LEVELS) return QGX_ERR_INVALID_ARG;
-  uint32_t h = mix_bytes(2166136261u, cb->len, (size_t)cb->nlev);
-  h = mix_bytes(mix_bytes(h, &cb->subblock, sizeof(int)), &bucket, sizeof(int));
-  StepCode* e = &sc->code[h % kStepSlots];
-  if (!(e->valid && e->bucket == bucket && e->cb.nlev == cb->nlev && e->cb.subblock == cb->subblock &&
-        std::memcmp(e->cb.len, cb->len, (size_t)cb->nlev) == 0 && std::memcmp(e->cb.code, cb->code, sizeof(uint32_t) * (size_t)cb->nlev) == 0)) {
-    e->valid = false;
-    const qgx_status rc = make_code_table(cb, bucket, &e->ct);
-    if (rc != QGX_OK) return rc;
-    if (!e->lut && cudaMalloc((void**)&e->lut, sizeof(uint16_t) << QGX_MAX_CODE_LEN) != cudaSuccess) {
-      cudaGetLastError();
-      e->lut = nullptr;
-      return QGX_ERR_CUDA;
-    }
-    std::vector<uint16_t> table((size_t)1 << e->ct.maxlen);
-    build_dec_lut_host(e->ct, table.data());
-    // pageable source: the runtime stages it before returning, so the vector may go out of scope
-    if (cudaMemcpyAsync(e->lut, table.data(), table.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
-      return QGX_ERR_CUDA;
-    e->bucket = bucket;
-    e->cb = *cb;
-    e->valid = true;
-  }
-  *ct = &e->ct;
-  *lut = e->lut;
-  return QGX_OK;
 }
 
 struct QuantizeArgs {

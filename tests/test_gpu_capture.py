@@ -57,3 +57,35 @@ def test_recorded_quantize_and_encode_keep_their_levels(K, d, bucket, nlev, sub)
         del graph
         qgx.qgx_destroy(ctx)
         qgx.qgx_destroy(warm)
+
+
+@pytest.mark.parametrize("K,d,bucket,nlev,sub", [(2, 3001, 512, 9, 0), (3, 2 * 8192 + 4, 8192, 32, 128)])
+def test_recorded_decode_keeps_its_code(K, d, bucket, nlev, sub):
+    import paper_2308_09187_b200 as qgx
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ctx = qgx.qgx_create(0)
+        rng = np.random.default_rng(d)
+        v = gen.gaussian_mixture((K, d), seed=d, device="cuda")
+        codes = [qgx.qgx_build_codebook_huffman(list(rng.dirichlet(np.ones(nlev) * 0.5)), sub) for _ in range(24)]
+        norms, sym = qgx.qgx_quantize(ctx, v, bucket, _levels(rng, nlev), qgx.QGX_NORM_L2, 5, 2)
+        sent = [qgx.qgx_encode(ctx, norms, sym, bucket, cb)[:2] for cb in codes]
+        got_norms, got_sym = torch.empty_like(norms), torch.empty_like(sym)
+        qgx.qgx_decode(ctx, *sent[1], d, bucket, codes[1], norms=got_norms, sym=got_sym)   # the workspace has its size
+        qgx.qgx_sync_status(ctx)
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin()
+        try:
+            qgx.qgx_decode(ctx, *sent[0], d, bucket, codes[0], norms=got_norms, sym=got_sym)
+        finally:
+            graph.capture_end()
+        for at, cb in zip(sent[1:], codes[1:]):
+            _, other = qgx.qgx_decode(ctx, *at, d, bucket, cb)
+            assert torch.equal(other, sym)
+        got_norms.zero_()
+        got_sym.zero_()
+        graph.replay()
+        qgx.qgx_sync_status(ctx)
+        assert torch.equal(got_norms, norms) and torch.equal(got_sym, sym)
+        del graph
+        qgx.qgx_destroy(ctx)
