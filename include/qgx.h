@@ -188,7 +188,8 @@ qgx_status qgx_quantize(qgx_ctx *ctx, const float *v, int K, size_t d, int bucke
  * bucket_bits [dev] uint32[K][nb] receives each bucket's length in bits, total_bits [dev]
  * uint64[K] their sum.  Words the buckets do not use up to each worker's end are left untouched.
  * Device-side errors: QGX_ERR_CAPACITY (nothing is written for that worker), QGX_ERR_CORRUPT
- * for a level index >= nlev in sym. */
+ * for a level index >= nlev in sym, QGX_ERR_TIMEOUT (a bounded wait between CTAs ran out: only where cap_words is
+ * the worst case, see qgx_stream_capacity_words, for then one pass suffices). */
 qgx_status qgx_encode(qgx_ctx *ctx, const float *norms, const uint8_t *sym, int K, size_t d,
                       int bucket, const qgx_codebook *cb /*[host]*/, uint32_t *stream,
                       size_t cap_words, uint32_t *bucket_bits, uint64_t *total_bits);
@@ -201,8 +202,8 @@ qgx_status qgx_encode(qgx_ctx *ctx, const float *norms, const uint8_t *sym, int 
  * word offsets and per-worker overflow flags in a workspace that it grows with cudaMalloc; this entry
  * point keeps them in a fixed array inside the library image instead (about 516 KB, present on every GPU
  * that loads the library until the process ends) and calls no cudaMalloc, cudaFree or other allocating
- * routine.  Arguments, stream layout, outputs and device-side errors are those of qgx_encode; the results
- * are identical.
+ * routine.  Arguments, stream layout, outputs and device-side errors (but for QGX_ERR_TIMEOUT: nothing waits
+ * here) are those of qgx_encode; the results are identical.
  *  - Limits: K <= 1024 and K * nb <= 65536 buckets; beyond that the call returns QGX_ERR_TOO_LARGE and
  *    launches nothing.
  *  - The first call on each device looks up the array's device address (cudaGetSymbolAddress, with that
@@ -279,8 +280,8 @@ qgx_status qgx_exchange_decode(qgx_ctx *ctx, int K, size_t d, const qgx_quant_cf
 /* How many times a device-side wait (one bucket waiting for the word count of an earlier bucket of its worker)
  * polls before it gives up with QGX_ERR_TIMEOUT; the default, 2^22, is seconds.  No counterpart in the paper. */
 qgx_status qgx_set_wait_limit(qgx_ctx *ctx, int polls);
-/* Diagnostic (no counterpart in the paper): the next fused exchange on this context leaves the first `buckets`
- * buckets of every worker unencoded, so that the buckets after them wait for word counts that never come.  With a
+/* Diagnostic (no counterpart in the paper): the next fused exchange or one-pass qgx_encode on this context leaves the first
+ * `buckets` buckets of every worker unencoded, so that the buckets after them wait for word counts that never come.  With a
  * small wait limit this shows the bounded wait at work: the waiting buckets give up, QGX_ERR_TIMEOUT is latched,
  * nothing is written for them, the kernel ends, and the context stays usable. */
 qgx_status qgx_debug_skip_buckets(qgx_ctx *ctx, size_t buckets);

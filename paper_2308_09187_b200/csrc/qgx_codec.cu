@@ -246,7 +246,8 @@ struct PackArgs {
   uint64_t* total_bits;
   unsigned long long* status;            // [K][nb], zeroed before the launch
   unsigned int* ticket;                  // zeroed before the launch
-  int spin_limit;
+  size_t b_first;                        // first bucket of every worker to encode (0 but for the diagnostic)
+  int spin_limit;                        // polls of a wait for another bucket's words before it gives up
   DevStatus* st;
 };
 
@@ -279,15 +280,15 @@ k_pack(const __grid_constant__ PackArgs a, const __grid_constant__ CodeTable ct)
   __syncthreads();
   const uint32_t pair_sa = smem_addr(s_pair), weights = 4u | ((uint32_t)(8 * nlev) << 16);
   const uint32_t limit4 = (uint32_t)(128 - nlev) * 0x01010101u;        // carries into bit 7 of a byte >= nlev
-  const unsigned long long total = (unsigned long long)a.nb * (unsigned long long)a.K;
+  const unsigned long long total = (unsigned long long)(a.nb - a.b_first) * (unsigned long long)a.K;
   const int seg = ct.has_header ? ct.G / 8 : 32;                       // lanes per sub-block
   uint32_t used_words[2] = {0u, 0u};
   bool bad = false;
   for (int par = 0;; par ^= 1) {
     const unsigned long long t = s_ticket[par];
     if (t >= total) break;
-    const size_t b = total <= 0xffffffffull ? (size_t)((uint32_t)t / (uint32_t)a.K) : (size_t)(t / (unsigned long long)a.K);
-    const size_t k = (size_t)(t - (unsigned long long)b * (unsigned long long)a.K);
+    const size_t turn = total <= 0xffffffffull ? (size_t)((uint32_t)t / (uint32_t)a.K) : (size_t)(t / (unsigned long long)a.K);
+    const size_t k = (size_t)(t - (unsigned long long)turn * (unsigned long long)a.K), b = a.b_first + turn;
     const size_t lo = b * (size_t)a.bucket;
     const int len = (int)min((size_t)a.bucket, a.d - lo);
     uint32_t* s_img = s_dyn + par * img_words;
@@ -573,14 +574,16 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
     PackArgs a;
     a.norms = norms; a.sym = sym; a.d = d; a.bucket = bucket; a.K = K; a.nb = nb; a.stream = stream; a.cap_words = cap_words;
     a.bucket_bits = bucket_bits; a.total_bits = total_bits; a.status = status + 2; a.ticket = reinterpret_cast<unsigned int*>(status);
-    a.spin_limit = kSpinLimit; a.st = c->dstatus;
+    a.b_first = std::min(c->skip_buckets, nb); a.spin_limit = c->wait_limit; a.st = c->dstatus;
+    c->skip_buckets = 0;
+    if (a.b_first == nb) return QGX_OK;
     const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
     a.load = (d % 8 == 0 && bucket % 8 == 0 && (at & 7u) == 0) ? 8 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
     const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
     const int threads = bucket_threads(bucket, 2 * pp);
     const size_t smem = sizeof(uint32_t) * (2 * ((img_words + 3) & ~(size_t)3) + (size_t)(4 * ct.nlev * ct.nlev));
     const unsigned fit = (unsigned)std::max<size_t>(1, std::min<size_t>((size_t)(1024 / threads), (220u * 1024u) / (smem + 2048u)));
-    const unsigned grid = (unsigned)std::min<unsigned long long>((unsigned long long)nb * (unsigned long long)K, (unsigned long long)c->num_sms * fit);
+    const unsigned grid = (unsigned)std::min<unsigned long long>((unsigned long long)(nb - a.b_first) * (unsigned long long)K, (unsigned long long)c->num_sms * fit);
 #define QGX_LAUNCH_K(V)                                              \
   do {                                                               \
     allow_max_dynamic_smem((const void*)k_pack<V>, c->device);       \

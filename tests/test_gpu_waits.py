@@ -1,0 +1,35 @@
+"""Every bounded wait between CTAs can be made to run out: buckets left unencoded on purpose and a small limit.  The call
+ends by itself, QGX_ERR_TIMEOUT is latched, and the next call on the context is exact."""
+import time
+
+import numpy as np
+import pytest
+import torch
+
+import qgx_inputs as gen
+
+pytestmark = pytest.mark.gpu
+
+LEVELS = np.linspace(0, 1, 9, dtype=np.float32)
+DEFAULT_LIMIT = 1 << 22
+
+
+@pytest.mark.parametrize("sub", [0, 64])
+def test_one_pass_encode_wait_runs_out(sub):
+    import paper_2308_09187_b200 as qgx
+    ctx = qgx.qgx_create(0)
+    K, d, bucket = 3, 12 * 1024 + 40, 1024
+    v, cb = gen.gaussian((K, d), seed=4, device="cuda"), qgx.qgx_build_codebook_fixed(9, sub)
+    norms, sym = qgx.qgx_quantize(ctx, v, bucket, LEVELS, qgx.QGX_NORM_L2, 3, 1)
+    want = [t.clone() for t in qgx.qgx_encode(ctx, norms, sym, bucket, cb)]
+    qgx.qgx_sync_status(ctx)
+    qgx.qgx_set_wait_limit(ctx, 50)
+    for skip in (2, 13):                                     # the second leaves out everything: nobody waits
+        qgx.qgx_debug_skip_buckets(ctx, skip)
+        qgx.qgx_encode(ctx, norms, sym, bucket, cb)
+        assert qgx.qgx_sync_status(ctx, check=False) == (qgx.QGX_ERR_TIMEOUT if skip == 2 else qgx.QGX_OK)
+    qgx.qgx_set_wait_limit(ctx, DEFAULT_LIMIT)
+    got = qgx.qgx_encode(ctx, norms, sym, bucket, cb)
+    qgx.qgx_sync_status(ctx)
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+    qgx.qgx_destroy(ctx)
