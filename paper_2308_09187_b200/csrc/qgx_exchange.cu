@@ -1102,7 +1102,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   const RoundTable& qt = tables->rt;
   if (!ct.has_header || bucket % ct.G != 0 || (ct.G != 32 && ct.G != 64 && ct.G != 128)) return QGX_ERR_INVALID_ARG;
   // small vectors: everything in one launch (the other ways are there when a caller asks for one of them)
-  if (do_encode && c->skip_buckets == 0 && c->encode_path == QGX_ENCODE_AUTO && c->decode_split == QGX_SPLIT_AUTO &&
+  if (do_encode && c->skip_buckets < nb && c->encode_path == QGX_ENCODE_AUTO && c->decode_split == QGX_SPLIT_AUTO &&
       small_exchange_fits(c, K, nb, bucket)) {
     const size_t had = c->ws_bytes[WS_SMALL];
     unsigned long long* words = (unsigned long long*)ws_get(c, WS_SMALL, sizeof(uint64_t) * ((size_t)K * nb + 2));
@@ -1111,7 +1111,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     EncodeArgs es = ea;
     es.status = words + 2;                              // zero between launches: the kernel sees to it
     es.ticket = reinterpret_cast<unsigned int*>(words);
-    es.b_first = 0;
+    es.b_first = c->skip_buckets;                       // 0 but for the diagnostic
     es.spin_limit = c->wait_limit;
     SmallArgs sm;
     std::memset(&sm, 0, sizeof(sm));
@@ -1122,7 +1122,10 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     sm.sum_sq = sum_sq; sm.square = (sym_mode & 4) ? 1 : 0; sm.total_out = total_bits_out;
     ScopedKernelTimer timer(c, QGX_KERNEL_ENCODE);
     const qgx_status done = launch_exchange_small(c, es, sm, lt, lt_kept, ct, key, qt);
-    if (done != QGX_ERR_TOO_LARGE) return done;
+    if (done != QGX_ERR_TOO_LARGE) {
+      c->skip_buckets = 0;
+      return done;
+    }
   }
   // octets per thread chosen so that CTAs have at most 256 / 512 / 512 threads
   const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);

@@ -74,7 +74,7 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
   if (k == 0 && tid == 0)
     for (int i = 0; i < K; ++i) *cluster.map_shared_rank(&s_bucket, i) = ticket;
   cluster.sync();
-  const size_t b = s_bucket, lo = b * (size_t)a.bucket;
+  const size_t b = a.b_first + s_bucket, lo = b * (size_t)a.bucket;
   const int len = (int)min((size_t)a.bucket, a.d - lo);
 
   // ---- load, norm ----
@@ -284,7 +284,7 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
     __shared__ bool s_last;
     if (tid == 0) {
       __threadfence();
-      s_last = atomicAdd(a.ticket + 1, 1u) == (unsigned)(a.nb - 1);
+      s_last = atomicAdd(a.ticket + 1, 1u) == (unsigned)(a.nb - a.b_first - 1);
     }
     __syncthreads();
     if (s_last) {
@@ -347,7 +347,7 @@ qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, 
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)ea.K;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)(ea.nb * (size_t)ea.K));
+  cfg.gridDim = dim3((unsigned)((ea.nb - ea.b_first) * (size_t)ea.K));
   cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = c->stream;

@@ -33,3 +33,26 @@ def test_one_pass_encode_wait_runs_out(sub):
     qgx.qgx_sync_status(ctx)
     assert all(torch.equal(a, b) for a, b in zip(got, want))
     qgx.qgx_destroy(ctx)
+
+
+@pytest.mark.parametrize("K,bucket", [(3, 1024), (12, 512), (1, 128)])
+def test_one_launch_exchange_wait_runs_out(K, bucket):
+    import paper_2308_09187_b200 as qgx
+    ctx = qgx.qgx_create(0)
+    d = 12 * bucket + 40
+    v = gen.gaussian((K, d), seed=4, device="cuda")
+    cfg = qgx.make_quant_cfg(LEVELS, bucket, qgx.qgx_build_codebook_fixed(9, 32), 3)
+    want = [t.clone() for t in qgx.qgx_exchange(ctx, v, cfg, 1)]
+    qgx.qgx_sync_status(ctx)
+    qgx.qgx_set_wait_limit(ctx, 50)
+    qgx.qgx_debug_skip_buckets(ctx, 2)
+    before = qgx.qgx_launch_count(ctx)
+    qgx.qgx_exchange(ctx, v, cfg, 1)
+    assert qgx.qgx_launch_count(ctx) == before + 1           # it is the one launch that waited
+    assert qgx.qgx_sync_status(ctx, check=False) == qgx.QGX_ERR_TIMEOUT
+    qgx.qgx_set_wait_limit(ctx, DEFAULT_LIMIT)
+    for _ in range(2):                                       # the scan's words were left as they were found
+        got = qgx.qgx_exchange(ctx, v, cfg, 1)
+        qgx.qgx_sync_status(ctx)
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+    qgx.qgx_destroy(ctx)
