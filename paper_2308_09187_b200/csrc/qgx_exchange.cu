@@ -1371,10 +1371,7 @@ static SegChildren* seg_children(qgx_ctx* c) {
     std::memset(h, 0, sizeof(*h));
     h->device = c->device;
     h->sym_slot = -1;
-    h->wait_limit = c->wait_limit;
-    h->decode_split = c->decode_split;
-    h->encode_path = c->encode_path;
-    h->num_sms = c->num_sms;
+    h->num_sms = c->num_sms;                            // (this and the context's modes are set again for every exchange)
     h->all_sms = c->all_sms;
     h->dstatus = c->dstatus;                            // errors latch into the parent's status block
     if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1482,6 +1479,7 @@ qgx_status qgx_exchange_segments(qgx_ctx* c, const float* v, int K, size_t d, co
     for (int i = 0; i < lanes; ++i) {
       sc->ctx[i]->decode_split = c->decode_split;
       sc->ctx[i]->encode_path = c->encode_path;
+      sc->ctx[i]->wait_limit = c->wait_limit;
       sc->ctx[i]->num_sms = shares ? std::max(1, (int)(c->num_sms * part[i] / all)) : c->num_sms;
       if (cudaStreamWaitEvent(sc->ctx[i]->stream, sc->fork, 0) != cudaSuccess) return QGX_ERR_CUDA;
     }
@@ -1496,6 +1494,7 @@ qgx_status qgx_exchange_segments(qgx_ctx* c, const float* v, int K, size_t d, co
       if (!seg_bits) { rc = QGX_ERR_CUDA; break; }
     }
     DualSource src{v + segs[s].offset, nullptr, d, 0};
+    if (sc) h->skip_buckets = c->skip_buckets;          // the diagnostic: of every tensor
     const qgx_status mine = exchange_impl(h, src, K, segs[s].length, segs[s].cfg, exchange_id, 0, mean_out + segs[s].offset, seg_bits,
                                           nullptr, 0, nullptr, segs[s].offset);
     if (mine == QGX_OK && total_bits) {
@@ -1504,7 +1503,9 @@ qgx_status qgx_exchange_segments(qgx_ctx* c, const float* v, int K, size_t d, co
       count_launch(h);
     }
     if (mine != QGX_OK && s < rc_seg) { rc = mine; rc_seg = s; }
+    if (sc) h->skip_buckets = 0;                        // (left over where the call refused its arguments)
   }
+  if (sc) c->skip_buckets = 0;
   if (sc) {                                             // join, also after an error: the caller's stream waits for the helpers
     for (int i = 0; i < lanes; ++i)
       if (cudaEventRecord(sc->join[i], sc->ctx[i]->stream) != cudaSuccess ||

@@ -56,3 +56,25 @@ def test_one_launch_exchange_wait_runs_out(K, bucket):
         qgx.qgx_sync_status(ctx)
         assert all(torch.equal(a, b) for a, b in zip(got, want))
     qgx.qgx_destroy(ctx)
+
+
+def test_layer_wise_exchange_waits_follow_the_context():
+    """The tensors run on helper contexts, made at the first such exchange: a limit set after that holds for them too."""
+    import paper_2308_09187_b200 as qgx
+    ctx = qgx.qgx_create(0)
+    K, bucket, sizes = 2, 1024, [8 * 1024, 700 * 1024, 3 * 1024]     # one launch, the large kernels, one launch
+    v = gen.gaussian((K, sum(sizes)), seed=4, device="cuda")
+    cfgs = [qgx.make_quant_cfg(LEVELS, bucket, qgx.qgx_build_codebook_fixed(9, 32), 3 + s) for s in range(len(sizes))]
+    want = [t.clone() for t in qgx.qgx_exchange_segments(ctx, v, sizes, cfgs, 1)]
+    qgx.qgx_sync_status(ctx)
+    qgx.qgx_set_wait_limit(ctx, 50)
+    qgx.qgx_debug_skip_buckets(ctx, 2)
+    start = time.perf_counter()
+    qgx.qgx_exchange_segments(ctx, v, sizes, cfgs, 1)
+    assert qgx.qgx_sync_status(ctx, check=False) == qgx.QGX_ERR_TIMEOUT
+    assert time.perf_counter() - start < 1.0                 # (with the default limit: seconds)
+    qgx.qgx_set_wait_limit(ctx, DEFAULT_LIMIT)
+    got = qgx.qgx_exchange_segments(ctx, v, sizes, cfgs, 1)
+    qgx.qgx_sync_status(ctx)
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+    qgx.qgx_destroy(ctx)
