@@ -278,7 +278,9 @@ qgx_status qgx_set_encode_path(qgx_ctx *ctx, int mode);
  * the slot's buffers). */
 qgx_status qgx_exchange_decode(qgx_ctx *ctx, int K, size_t d, const qgx_quant_cfg *cfg, int slot, float *mean_out);
 /* How many times a device-side wait (one bucket waiting for the word count of an earlier bucket of its worker)
- * polls before it gives up with QGX_ERR_TIMEOUT; the default, 2^22, is seconds.  No counterpart in the paper. */
+ * polls before it gives up with QGX_ERR_TIMEOUT; the default, 2^22, is seconds.  It holds for qgx_encode, the fused calls
+ * and every tensor of a layer-wise exchange; the waits of an encode kernel's warps for one another follow it (up to
+ * 80 ms longer).  No counterpart in the paper. */
 qgx_status qgx_set_wait_limit(qgx_ctx *ctx, int polls);
 /* Diagnostic (no counterpart in the paper): the next fused exchange or one-pass qgx_encode on this context leaves the first
  * `buckets` buckets of every worker unencoded, so that the buckets after them wait for word counts that never come.  With a

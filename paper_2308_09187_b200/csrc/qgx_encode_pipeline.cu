@@ -99,6 +99,7 @@ struct PipeShape {
   uint32_t bin_mask, bin_copy;                           // of the rounding table: see RoundFix; bytes of a bin's copies less 16
   size_t units;                                          // per worker
   size_t status_ld, status_first;                        // status words per worker, the first one used (the diagnostic leaves some unpublished)
+  int bar_looks;                                         // looks at a barrier before its wait gives up
 };
 // ---- mbarriers by 32-bit shared address ----
 __device__ __forceinline__ void bar_init(uint32_t bar, unsigned count) {
@@ -112,10 +113,10 @@ __device__ __forceinline__ void bar_arrive_n(uint32_t bar, unsigned n) {
 }
 // Waits for the phase of the given parity; called by whole warps.  False if the bounded wait ran out or another warp of
 // the CTA gave up (*quit, shared memory).  The warp is suspended between its looks (at most 20 us each): polls would take
-// issue slots from the warps that compute.
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* quit) {
+// issue slots from the warps that compute.  The number of looks follows the limit on polls (kBarLooksPolls).
+__device__ __forceinline__ bool bar_wait_looks(uint32_t bar, uint32_t parity, volatile int* quit, int looks) {
   unsigned done = 0;
-  for (int i = 0; i < kSpinLimit; ++i) {
+  for (int i = 0; i < looks; ++i) {
     asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p; }"
                  : "=r"(done) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
     if (done) break;
@@ -123,6 +124,10 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile
   }
   return __all_sync(0xffffffffu, done != 0);
 }
+
+// A poll of the look-back is about a microsecond, a look up to twenty: one for every sixteen polls, plus 80 ms, so that a
+// wait for a warp that waits for another CTA rarely ends before that warp's own does.  The default limit is some 5 s.
+constexpr int kBarLooksBase = 4096, kBarLooksPolls = 16;
 
 // 16 (4) bytes from global to shared memory without passing through registers; `bytes` of them are read, the rest is zero
 __device__ __forceinline__ void copy_async16(uint32_t dst, const float* src, int bytes) {
@@ -292,6 +297,7 @@ k_encode_pipeline(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
   if (threadIdx.x < kTurnRing) bar_init(turned + 8u * threadIdx.x, kQuantizers);
   __syncthreads();
   volatile int* quit = &s_quit;
+  const auto bar_wait = [&](uint32_t bar, uint32_t parity, volatile int* q) { return bar_wait_looks(bar, parity, q, h.bar_looks); };
   // a wait that ran out: everybody gives up, the launch ends and reports it
   auto give_up = [&]() {
     if (lane == 0) {
@@ -711,6 +717,7 @@ qgx_status launch_encode_pipeline(qgx_ctx* c, const EncodeArgs& ea, const LevelT
   ps.units = plan.units;
   ps.status_first = plan.status_first;
   ps.status_ld = plan.status_ld;
+  ps.bar_looks = kBarLooksBase + ea.spin_limit / kBarLooksPolls;
   ps.image_turns = kMaxImageTurns;
   while (ps.image_turns > 2 && pipe_smem(ct.nlev, ct.maxlen, ps.image_turns).bytes > kPipeSmemMax) --ps.image_turns;
   ps.smem = pipe_smem(ct.nlev, ct.maxlen, ps.image_turns);

@@ -78,3 +78,28 @@ def test_layer_wise_exchange_waits_follow_the_context():
     qgx.qgx_sync_status(ctx)
     assert all(torch.equal(a, b) for a, b in zip(got, want))
     qgx.qgx_destroy(ctx)
+
+
+@pytest.mark.parametrize("limit", [50, 1 << 15])
+def test_pipelined_encode_ends_when_many_waits_run_out(limit):
+    """Every worker's first unit is missing, so the scanners' waits run out one after the other while the other warps of
+    their CTAs wait for them at barriers: whichever gives up first, the launch ends soon and says so."""
+    import paper_2308_09187_b200 as qgx
+    ctx = qgx.qgx_create(0)
+    qgx.qgx_set_encode_path(ctx, qgx.QGX_ENCODE_STAGED)
+    K, bucket, d = 64, 1024, 300 * 1024 + 5
+    v = gen.gaussian((K, d), seed=4, device="cuda")
+    cfg = qgx.make_quant_cfg(LEVELS, bucket, qgx.qgx_build_codebook_fixed(9, 32), 3)
+    want = [t.clone() for t in qgx.qgx_exchange(ctx, v, cfg, 1)]
+    qgx.qgx_sync_status(ctx)
+    qgx.qgx_set_wait_limit(ctx, limit)
+    qgx.qgx_debug_skip_buckets(ctx, 4)
+    start = time.perf_counter()
+    qgx.qgx_exchange(ctx, v, cfg, 1)
+    assert qgx.qgx_sync_status(ctx, check=False) == qgx.QGX_ERR_TIMEOUT
+    assert time.perf_counter() - start < 2.0
+    qgx.qgx_set_wait_limit(ctx, DEFAULT_LIMIT)
+    got = qgx.qgx_exchange(ctx, v, cfg, 1)
+    qgx.qgx_sync_status(ctx)
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+    qgx.qgx_destroy(ctx)
