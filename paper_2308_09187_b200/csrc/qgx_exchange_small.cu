@@ -64,7 +64,8 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
     const uint32_t e = __ldg(r.lut_len + 2 * i);                       // bits 0..4 bits consumed, 8..15 the symbol byte
     s_tab[i] = (uint16_t)(((e & 31u) << 8) | ((e >> 8) & 0xffu));
   }
-  for (int i = tid; i < 2 * QGX_MAX_LEVELS; i += blockDim.x) s_lut.e[i] = __ldg(a.tables->lut.e + i);   // (a bucket of 128 has one warp)
+  if (tid < 2 * QGX_MAX_LEVELS) s_lut.e[tid] = __ldg(a.tables->lut.e + tid);
+  if (blockDim.x == kWarp) s_lut.e[QGX_MAX_LEVELS + tid] = __ldg(a.tables->lut.e + QGX_MAX_LEVELS + tid);   // a bucket of 128 has one warp
   if (tid < QGX_MAX_LEVELS) {
     s_lev[tid] = tid < lt.nlev ? lt.lev[tid] : 1.0f;
     s_lev_kept[tid] = tid < lt_kept.nlev ? lt_kept.lev[tid] : 0.0f;
