@@ -1103,7 +1103,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   if (!ct.has_header || bucket % ct.G != 0 || (ct.G != 32 && ct.G != 64 && ct.G != 128)) return QGX_ERR_INVALID_ARG;
   // small vectors: everything in one launch (the other ways are there when a caller asks for one of them)
   if (do_encode && c->skip_buckets < nb && c->encode_path == QGX_ENCODE_AUTO && c->decode_split == QGX_SPLIT_AUTO &&
-      small_exchange_fits(c, K, nb, bucket)) {
+      small_exchange_fits(c, K, nb, bucket, ct, qt, ea.vec_ok && ea.quad_base % 2 == 0)) {
     const size_t had = c->ws_bytes[WS_SMALL];
     unsigned long long* words = (unsigned long long*)ws_get(c, WS_SMALL, sizeof(uint64_t) * ((size_t)K * nb + 2));
     if (!words) return QGX_ERR_CUDA;
@@ -1121,11 +1121,8 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     sm.sym_out = sym_out; sm.sym_prev = sym_prev; sm.sym_ld = sym_ld; sm.norms_prev = norms_prev;
     sm.sum_sq = sum_sq; sm.square = (sym_mode & 4) ? 1 : 0; sm.total_out = total_bits_out;
     ScopedKernelTimer timer(c, QGX_KERNEL_ENCODE);
-    const qgx_status done = launch_exchange_small(c, es, sm, lt, lt_kept, ct, key, qt);
-    if (done != QGX_ERR_TOO_LARGE) {
-      c->skip_buckets = 0;
-      return done;
-    }
+    c->skip_buckets = 0;
+    return launch_exchange_small(c, es, sm, lt, lt_kept, ct, key, qt);
   }
   // octets per thread chosen so that CTAs have at most 256 / 512 / 512 threads
   const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
@@ -1469,7 +1466,7 @@ qgx_status qgx_exchange_segments(qgx_ctx* c, const float* v, int K, size_t d, co
       const int l = (int)(std::min_element(load, load + lanes) - load);
       const double w = (double)K * (double)segs[s].length;
       const size_t bucket = (size_t)std::max(segs[s].cfg->bucket, 1);
-      const bool one_launch = small_exchange_fits(c, K, (segs[s].length + bucket - 1) / bucket, (int)bucket);
+      const bool one_launch = small_exchange_size(c, K, (segs[s].length + bucket - 1) / bucket, (int)bucket);
       lane_of[(size_t)s] = l;
       load[l] += w + kSegFixed;
       part[l] += one_launch ? w : w + kSegFixed;        // (a tensor done in one launch takes the SMs that it finds)

@@ -13,7 +13,6 @@
 #include <cooperative_groups.h>
 #include <cstring>
 #include <mutex>
-#include <vector>
 
 namespace cg = cooperative_groups;
 
@@ -295,83 +294,113 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
   }
 }
 
-// Whether `workers` CTAs of this shape fit into a cluster (more than eight: not on every part), asked once per shape.
-static bool cluster_fits(const void* fn, int device, int workers, int threads, size_t smem) {
-  if (workers <= 8) return true;
-  struct Seen { const void* fn; int device, workers, threads; size_t smem; bool fits; };
-  static std::vector<Seen> seen;
-  static std::mutex guard;
-  std::lock_guard<std::mutex> lock(guard);
-  for (const Seen& x : seen)
-    if (x.fn == fn && x.device == device && x.workers == workers && x.threads == threads && x.smem == smem) return x.fits;
-  cudaLaunchConfig_t cfg;
-  std::memset(&cfg, 0, sizeof(cfg));
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)workers;
-  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)workers);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  const bool fits = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                    cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) == cudaSuccess && clusters >= 4;
-  if (!fits) cudaGetLastError();
-  seen.push_back(Seen{fn, device, workers, threads, smem, fits});
-  return fits;
+// What a launch for these buckets and tables looks like.
+struct SmallShape {
+  const void* fn;
+  int threads, entries;                  // entries: of the tables that every CTA brings in
+  uint32_t img_words, off_img, off_sym, off_tab;
+  size_t smem;
+};
+static SmallShape small_shape(int bucket, const CodeTable& ct, const RoundTable& rt) {
+  SmallShape s;
+  const int Q = bucket <= 2048 ? 1 : (bucket <= 4096 ? 2 : 4);
+  const size_t nbins = ((kKeyTop - kKeyBase) >> rt.key_shift) + 1;
+  s.threads = ((bucket / kQuad + Q - 1) / Q + 31) / 32 * 32;
+  s.entries = (int)nbins + (2 << ct.maxlen);
+  s.img_words = (uint32_t)(((size_t)bucket * (ct.maxlen + 1) + 16u * (bucket / ct.G + 1) + kNormBits + 31u) / 32u + 4u);
+  s.off_img = (uint32_t)((nbins * sizeof(float4) + 127) & ~(size_t)127);
+  s.off_sym = (uint32_t)((s.off_img + s.img_words * 4u + 15u) & ~15u);
+  s.off_tab = (uint32_t)((s.off_sym + (uint32_t)bucket + 15u) & ~15u);
+  s.smem = s.off_tab + (sizeof(uint16_t) << (ct.maxlen + 1));
+#define QGX_SMALL_G(QQ) (ct.G == 32 ? (const void*)k_exchange_small<QQ, 32> : (ct.G == 64 ? (const void*)k_exchange_small<QQ, 64> : (const void*)k_exchange_small<QQ, 128>))
+  s.fn = Q == 1 ? QGX_SMALL_G(1) : (Q == 2 ? QGX_SMALL_G(2) : QGX_SMALL_G(4));
+#undef QGX_SMALL_G
+  return s;
 }
 
-// One bucket per CTA, so the launch takes ever more turns as the vector grows, while the large kernels' time hardly moves
-// until theirs are full.  Measured (us, this way against the other): 4 x 10^4 coordinates of bucket 1024 12.3 : 28.7,
-// 4 x 10^5 16.7 : 28.6, 8 x 10^5 22.1 : 31.8, 1.2 x 10^6 32.4 : 31.7; of bucket 4096 1.2 x 10^6 24.5 : 31.3, 2.4 x 10^6 38.5 : 38.8;
-// of bucket 16384 1.6 x 10^6 24.6 : 34.9.
-bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket) {
+static void small_config(const SmallShape& s, int workers, size_t clusters, cudaStream_t stream, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
+  std::memset(cfg, 0, sizeof(*cfg));
+  std::memset(attr, 0, sizeof(*attr));
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)workers;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cfg->gridDim = dim3((unsigned)(clusters * (size_t)workers));
+  cfg->blockDim = dim3((unsigned)s.threads);
+  cfg->dynamicSmemBytes = s.smem;
+  cfg->stream = stream;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+}
+
+// How many clusters of `workers` CTAs, and how many CTAs of an SM, are resident at a time (0: none, as for more than eight
+// CTAs on a part without larger clusters).  Asked once per shape; the last kSeen shapes are remembered.
+struct SmallResidency { int clusters, per_sm; };
+static SmallResidency small_residency(const SmallShape& s, int device, int workers) {
+  struct Seen { const void* fn; int device, workers, threads; size_t smem; SmallResidency r; };
+  constexpr int kSeen = 64;
+  static Seen seen[kSeen];
+  static int used = 0, oldest = 0;
+  static std::mutex guard;                              // contexts may be driven from different host threads
+  std::lock_guard<std::mutex> lock(guard);
+  for (int i = 0; i < used; ++i)
+    if (seen[i].fn == s.fn && seen[i].device == device && seen[i].workers == workers && seen[i].threads == s.threads && seen[i].smem == s.smem) return seen[i].r;
+  allow_max_dynamic_smem(s.fn, device);
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  small_config(s, workers, 1, nullptr, &cfg, &attr);
+  SmallResidency r{0, 0};
+  if ((workers > 8 && cudaFuncSetAttribute(s.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+      cudaOccupancyMaxActiveClusters(&r.clusters, s.fn, &cfg) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r.per_sm, s.fn, s.threads, s.smem) != cudaSuccess) {
+    cudaGetLastError();
+    r = SmallResidency{0, 0};
+  }
+  const int at = used < kSeen ? used++ : oldest;
+  if (used == kSeen) oldest = (at + 1) % kSeen;
+  seen[at] = Seen{s.fn, device, workers, s.threads, s.smem, r};
+  return r;
+}
+
+// The most work for which one launch has been seen to be the faster way.
+bool small_exchange_size(const qgx_ctx* c, int K, size_t nb, int bucket) {
   if (K > kSmallMaxWorkers || bucket < 128 || bucket % 128 != 0 || nb > 65536) return false;
   return nb * (size_t)K * (size_t)bucket <= (size_t)c->all_sms * (bucket >= 4096 ? 12288 : 7168);
 }
 
+// One launch, or the large kernels?  Both sides' times in us, fitted to 13420 measurements on B200 (1 to 16 workers, 14
+// bucket sizes from 128 to 16384, 512 to 16384 coordinates per SM, five pairs of levels and code).  One launch takes a turn
+// for every time that the resident clusters are full, and each costs what its CTAs do before and for their bucket: tables
+// (0.18 us per entry and thread), load, walk, sums.  The large kernels' time hardly moves until theirs are full; codes of
+// many bits cost them larger tables, buckets that are not the pipelined encoder's a step each, and a longer one where their
+// encoder goes coordinate by coordinate (`octets` false: rows or counters off the grid of eight).  Within 11 % (one launch) and
+// 9 %, so the large kernels get a start of 1 us.  Up to the size limit above, which alone decided before, 877 of the
+// measured shapes were slower in one launch by more than 8 % (16 workers, 129 buckets of 512, 17 fitted levels, 82 us
+// against 53; 12 workers, 9 buckets of 16384, 9 uniform levels, 47 against 37); now 90 are, 1.40 times at most, and 15 lose
+// 8 to 13 %.  Where it holds, 9 uniform levels: 4 workers, 18 buckets of 1024, 13 : 28; 8 workers, 129 of 512, 21 : 33, 16 of
+// 4096, 21 : 27, and 27 of 8192, 25 : 34; 16 workers, 9 of 4096, 23 : 27.
+bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct, const RoundTable& rt, bool octets) {
+  if (!small_exchange_size(c, K, nb, bucket)) return false;
+  const SmallShape s = small_shape(bucket, ct, rt);
+  const SmallResidency r = small_residency(s, c->device, K);
+  if (r.clusters < 1) return false;
+  const double kilo = 1e-3 * bucket, buckets = (double)nb * K / c->all_sms;              // of an SM
+  const double turns = (double)((nb + (size_t)r.clusters - 1) / (size_t)r.clusters);
+  const double one = 3.5 + turns * (12.0 + 0.18 * s.entries / s.threads + (0.45 + 0.085 * r.per_sm) * kilo + 0.13 * K);
+  const bool pipelined = bucket % kChunk == 0 && (bucket & (bucket - 1)) == 0;
+  const bool whole = octets && bucket % (256 * (bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4))) == 0;   // else coordinate by coordinate
+  const double other = 23.0 + 1.2 * ct.maxlen + 0.65 * buckets * kilo + (pipelined ? 0.03 * buckets : (whole ? 0.8 * buckets : 1.5 * buckets + 4.0));
+  return one <= other + 1.0;
+}
+
 qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, const LevelTable& lt, const LevelTable& lt_kept,
                                  const CodeTable& ct, const PhiloxKey& key, const RoundTable& rt) {
-  const int Q = ea.bucket <= 2048 ? 1 : (ea.bucket <= 4096 ? 2 : 4);
-  const int threads = ((ea.bucket / kQuad + Q - 1) / Q + 31) / 32 * 32;
-  const size_t nbins = ((kKeyTop - kKeyBase) >> rt.key_shift) + 1;
-  r.img_words = (uint32_t)(((size_t)ea.bucket * (ct.maxlen + 1) + 16u * (ea.bucket / ct.G + 1) + kNormBits + 31u) / 32u + 4u);
-  r.off_img = (uint32_t)((nbins * sizeof(float4) + 127) & ~(size_t)127);
-  r.off_sym = (uint32_t)((r.off_img + r.img_words * 4u + 15u) & ~15u);
-  r.off_tab = (uint32_t)((r.off_sym + (uint32_t)ea.bucket + 15u) & ~15u);
-  const size_t smem = r.off_tab + (sizeof(uint16_t) << (ct.maxlen + 1));
+  const SmallShape s = small_shape(ea.bucket, ct, rt);
+  r.img_words = s.img_words; r.off_img = s.off_img; r.off_sym = s.off_sym; r.off_tab = s.off_tab;
   cudaLaunchConfig_t cfg;
-  std::memset(&cfg, 0, sizeof(cfg));
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)ea.K;
-  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)((ea.nb - ea.b_first) * (size_t)ea.K));
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = c->stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t err = cudaSuccess;
-#define QGX_SMALL(QQ, GG)                                                                    \
-  do {                                                                                       \
-    allow_max_dynamic_smem((const void*)k_exchange_small<QQ, GG>, c->device);                \
-    if (!cluster_fits((const void*)k_exchange_small<QQ, GG>, c->device, ea.K, threads, smem)) return QGX_ERR_TOO_LARGE; \
-    err = cudaLaunchKernelEx(&cfg, k_exchange_small<QQ, GG>, ea, r, lt, lt_kept, ct, key, rt); \
-  } while (0)
-#define QGX_SMALL_G(QQ)                          \
-  do {                                           \
-    if (ct.G == 32) QGX_SMALL(QQ, 32);           \
-    else if (ct.G == 64) QGX_SMALL(QQ, 64);      \
-    else QGX_SMALL(QQ, 128);                     \
-  } while (0)
-  if (Q == 1) QGX_SMALL_G(1);
-  else if (Q == 2) QGX_SMALL_G(2);
-  else QGX_SMALL_G(4);
-#undef QGX_SMALL_G
-#undef QGX_SMALL
+  cudaLaunchAttribute attr;
+  small_config(s, ea.K, ea.nb - ea.b_first, c->stream, &cfg, &attr);
+  void* args[] = {(void*)&ea, (void*)&r, (void*)&lt, (void*)&lt_kept, (void*)&ct, (void*)&key, (void*)&rt};
+  const cudaError_t err = cudaLaunchKernelExC(&cfg, s.fn, args);
   count_launch(c);
   return cuda_status(err != cudaSuccess ? err : cudaGetLastError());
 }

@@ -24,9 +24,9 @@ struct SmallArgs {
   uint32_t img_words, off_img, off_sym, off_tab;
 };
 
-bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket);
-// ea.status [K][nb] and ea.ticket [2] are zero before the launch and again after it.  QGX_ERR_TOO_LARGE: nothing was
-// launched, the device has no clusters of that many CTAs.
+bool small_exchange_size(const qgx_ctx* c, int K, size_t nb, int bucket);   // necessary, without the tables
+bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct, const RoundTable& rt, bool octets);
+// After small_exchange_fits.  ea.status [K][nb] and ea.ticket [2] are zero before the launch and again after it.
 qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, const LevelTable& lt, const LevelTable& lt_kept,
                                  const CodeTable& ct, const PhiloxKey& key, const RoundTable& rt);
 
