@@ -99,7 +99,6 @@ struct PipeShape {
   uint32_t bin_mask, bin_copy;                           // of the rounding table: see RoundFix; bytes of a bin's copies less 16
   size_t units;                                          // per worker
   size_t status_ld, status_first;                        // status words per worker, the first one used (the diagnostic leaves some unpublished)
-  int bar_looks;                                         // looks at a barrier before its wait gives up
 };
 // ---- mbarriers by 32-bit shared address ----
 __device__ __forceinline__ void bar_init(uint32_t bar, unsigned count) {
@@ -111,16 +110,17 @@ __device__ __forceinline__ void bar_arrive(uint32_t bar) {
 __device__ __forceinline__ void bar_arrive_n(uint32_t bar, unsigned n) {
   asm volatile("{ .reg .b64 st; mbarrier.arrive.shared::cta.b64 st, [%0], %1; }" ::"r"(bar), "r"(n) : "memory");
 }
-// Waits for the phase of the given parity; called by whole warps.  False if the bounded wait ran out or another warp of
-// the CTA gave up (*quit, shared memory).  The warp is suspended between its looks (at most 20 us each): polls would take
-// issue slots from the warps that compute.  The number of looks follows the limit on polls (kBarLooksPolls).
-__device__ __forceinline__ bool bar_wait_looks(uint32_t bar, uint32_t parity, volatile int* quit, int looks) {
+// Waits for the phase of the given parity; called by whole warps.  False if the bounded wait ran out (after quit[1] looks,
+// see kBarLooksPolls) or another warp of the CTA gave up (quit[0]).  The warp is suspended between its looks (at most 20 us
+// each): polls would take issue slots from the warps that compute.  Both words are in shared memory and read every sixteen
+// looks only: with the limit as an operand of every look an exchange of 8 x 2^24 coordinates took 540 us, not 530.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* quit) {
   unsigned done = 0;
-  for (int i = 0; i < looks; ++i) {
+  for (int i = 1;; ++i) {
     asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3; selp.u32 %0, 1, 0, p; }"
                  : "=r"(done) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
     if (done) break;
-    if ((i & 15) == 15 && *quit) break;
+    if ((i & 15) == 0 && (quit[0] || i >= quit[1])) break;
   }
   return __all_sync(0xffffffffu, done != 0);
 }
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
 k_encode_pipeline(const __grid_constant__ EncodeArgs a, const __grid_constant__ PipeShape h, const __grid_constant__ LevelTable lt, const __grid_constant__ CodeTable ct,
                   const __grid_constant__ PhiloxKey key, const __grid_constant__ RoundTable rt) {
   extern __shared__ __align__(1024) unsigned char s_pipe[];
-  __shared__ int s_quit;
+  __shared__ int s_quit[2];                              // somebody gave up; looks at a barrier before its wait gives up
   const PipeSmem& L = h.smem;
   const uint32_t sa = smem_addr(s_pipe);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -293,11 +293,10 @@ k_encode_pipeline(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
     bar_init(placed + 8u * threadIdx.x, 1);
     bar_init(written + 8u * threadIdx.x, kCopiers);
   }
-  if (threadIdx.x == 0) s_quit = 0;
+  if (threadIdx.x == 0) { s_quit[0] = 0; s_quit[1] = kBarLooksBase + a.spin_limit / kBarLooksPolls; }
   if (threadIdx.x < kTurnRing) bar_init(turned + 8u * threadIdx.x, kQuantizers);
   __syncthreads();
-  volatile int* quit = &s_quit;
-  const auto bar_wait = [&](uint32_t bar, uint32_t parity, volatile int* q) { return bar_wait_looks(bar, parity, q, h.bar_looks); };
+  volatile int* quit = s_quit;
   // a wait that ran out: everybody gives up, the launch ends and reports it
   auto give_up = [&]() {
     if (lane == 0) {
@@ -717,7 +716,6 @@ qgx_status launch_encode_pipeline(qgx_ctx* c, const EncodeArgs& ea, const LevelT
   ps.units = plan.units;
   ps.status_first = plan.status_first;
   ps.status_ld = plan.status_ld;
-  ps.bar_looks = kBarLooksBase + ea.spin_limit / kBarLooksPolls;
   ps.image_turns = kMaxImageTurns;
   while (ps.image_turns > 2 && pipe_smem(ct.nlev, ct.maxlen, ps.image_turns).bytes > kPipeSmemMax) --ps.image_turns;
   ps.smem = pipe_smem(ct.nlev, ct.maxlen, ps.image_turns);
