@@ -1,6 +1,6 @@
 // Device pieces of the prefix codec (Sec. 3.2 / App. J) shared by the stand-alone and the fused
-// kernels: packing a quad's codewords, placing bits into a shared-memory image of a bucket, and a
-// bounded bit reader with a table-driven decoder.
+// kernels: packing a quad's codewords, placing bits into a shared-memory image of a bucket, and the
+// chained scan of the buckets' lengths.
 #pragma once
 
 #include "qgx_common.cuh"
@@ -101,47 +101,6 @@ __device__ __forceinline__ void put_bits2(uint32_t* img, uint32_t pos, uint64_t 
 // Decoder table: index = next `maxlen` stream bits, entry = level | codeword length << 8 (0 = no
 // codeword starts with these bits).
 constexpr int kDecLutMax = 1 << QGX_MAX_CODE_LEN;
-
-// Reads a bucket's words with every access bounded by nwords.
-struct BitReader {
-  const uint32_t* w;
-  uint32_t nwords;
-  uint32_t next;          // index of the next word to fetch
-  uint64_t buf;           // bits not yet consumed, next bit at bit 0
-  int avail;
-  __device__ __forceinline__ uint32_t fetch(uint32_t i) const { return i < nwords ? w[i] : 0u; }
-  __device__ __forceinline__ void seek(uint32_t bitpos) {
-    next = bitpos >> 5;
-    const uint32_t sh = bitpos & 31u;
-    buf = (uint64_t)(fetch(next) >> sh);
-    avail = 32 - (int)sh;
-    ++next;
-    refill();
-  }
-  __device__ __forceinline__ void refill() {
-    if (avail <= 32) {
-      buf |= (uint64_t)fetch(next) << avail;
-      avail += 32;
-      ++next;
-    }
-  }
-  __device__ __forceinline__ void skip(int n) { buf >>= n; avail -= n; }
-};
-
-// decodes one symbol; returns false on an unassigned pattern.  *used accumulates consumed bits.
-__device__ __forceinline__ bool decode_symbol(BitReader& br, const uint16_t* lut, uint32_t mask, uint32_t* sym, uint32_t* used) {
-  br.refill();
-  const uint32_t e = lut[(uint32_t)br.buf & mask];
-  const int L = (int)(e >> 8);
-  if (L == 0) return false;
-  const uint32_t idx = e & 0xffu;
-  br.skip(L);
-  uint32_t neg = 0;
-  if (idx != 0) { neg = (uint32_t)br.buf & 1u; br.skip(1); }
-  *sym = idx | (neg << 7);
-  *used += (uint32_t)L + (idx != 0 ? 1u : 0u);
-  return true;
-}
 
 // ---- chained scan of bucket lengths ("decoupled look-back") ----------------------------------
 // status word of bucket (k, b): bits 62..63 state, bits 0..61 a word count.

@@ -25,7 +25,7 @@ struct EncodeArgs {
   float* norms;                 // [K][nb] (kept for the caller; the streams carry them too)
   unsigned long long* status;   // [K][nb], zeroed before the launch
   unsigned int* ticket;         // zeroed before the launch
-  const struct EncodeTables* tables;   // the shared-memory tables of the configuration, built once (null: every CTA builds them)
+  const struct EncodeTables* tables;   // the shared-memory tables of the configuration, built once
   DevStatus* st;
   size_t b_first;               // first bucket of every worker to encode (0 but for the diagnostic)
   int spin_limit;               // polls of a wait for another bucket's count before it gives up

@@ -107,9 +107,6 @@ __device__ __forceinline__ void bar_init(uint32_t bar, unsigned count) {
 __device__ __forceinline__ void bar_arrive(uint32_t bar) {
   asm volatile("{ .reg .b64 st; mbarrier.arrive.shared::cta.b64 st, [%0]; }" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void bar_arrive_n(uint32_t bar, unsigned n) {
-  asm volatile("{ .reg .b64 st; mbarrier.arrive.shared::cta.b64 st, [%0], %1; }" ::"r"(bar), "r"(n) : "memory");
-}
 // Waits for the phase of the given parity; called by whole warps.  False if the bounded wait ran out (after quit[1] looks,
 // see kBarLooksPolls) or another warp of the CTA gave up (quit[0]).  The warp is suspended between its looks (at most 20 us
 // each): polls would take issue slots from the warps that compute.  Both words are in shared memory and read every sixteen

@@ -124,7 +124,7 @@ k_exchange_encode(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
   constexpr int kSegLanes = G / kOctet;                 // lanes per sub-block within a row of 256 coordinates
   constexpr int kSegs = 32 / kSegLanes;                 // sub-blocks per row
 
-  if (a.tables) {
+  {
     const uint4* gb = reinterpret_cast<const uint4*>(a.tables->bin);
     const uint4* gp = reinterpret_cast<const uint4*>(a.tables->pair);
     uint4* sb = reinterpret_cast<uint4*>(s_bin);
@@ -132,15 +132,10 @@ k_exchange_encode(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
     for (int i = threadIdx.x; i < kBinEntries; i += blockDim.x) sb[i] = __ldg(gb + i);
     for (int i = threadIdx.x; i < kPairLutSize / 4; i += blockDim.x) sp[i] = __ldg(gp + i);
     for (int i = threadIdx.x; i < 2 * QGX_MAX_LEVELS; i += blockDim.x) s_lut.e[i] = __ldg(a.tables->lut.e + i);
-  } else {
-    fill_enc_lut(&s_lut, ct);
-    fill_bin_table(s_bin, rt, BinKind::kOctet);
   }
   if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
   if (threadIdx.x == 0) s_ticket[0] = atomicAdd(a.ticket, 1u);
   for (int i = threadIdx.x; i < 2 * img_words; i += blockDim.x) s_dyn[i] = 0;
-  __syncthreads();
-  if (!a.tables) fill_pair_lut_signed(s_pair, &s_lut);
   __syncthreads();
   const int nlev = lt.nlev;
   const uint32_t pair_sa = smem_addr(s_pair);
@@ -337,7 +332,6 @@ struct DecodeArgs {
 };
 
 constexpr int kDecThreads = 128;
-constexpr bool kTwoPassByDefault = false;   // large vectors decode in two passes (walk, then sums) unless told otherwise
 constexpr uint32_t kBadSymbol = 0x40u;      // symbol byte of an index that no codeword starts like (no level has bit 6)
 
 // Bits not yet consumed of one sub-block: a 64-bit window refilled 32 bits at a time.  The streams
@@ -904,8 +898,8 @@ __global__ void __launch_bounds__(256) k_sum_workers(const float* __restrict__ v
   }
 }
 
-qgx_status launch_decode_average(qgx_ctx* c, const DecodeArgs& args, const CodeTable& ct, const LevelTable& lt, int sym_mode,
-                                 bool walk_only = false);
+qgx_status launch_decode_average(qgx_ctx* c, const DecodeArgs& args, const CodeTable& ct, const LevelTable& lt, int sym_mode);
+qgx_status launch_decode_walk(qgx_ctx* c, const DecodeArgs& args, const CodeTable& ct, const LevelTable& lt);
 
 // ---- what a call derives from a quantizer configuration, kept between calls --------------------
 // Building the rounding table, the code table and the decoder table and copying the latter to the device costs
@@ -927,7 +921,7 @@ struct TableCache {
   CachedTables e[kTableCacheSlots];
   LaunchShape enc[3][3];                // [octets per thread 1, 2, 4][sub-block 32, 64, 128]
   LaunchShape dec[3][6];                // [sub-block][symbol mode]
-  LaunchShape dec_walk[3][6];           // the walk alone
+  LaunchShape dec_walk[3];              // the walk alone
 };
 
 // Lets a kernel use all the dynamic shared memory that the device allows, once per kernel and device.  (The
@@ -1206,17 +1200,16 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     da.values = (float*)ws_get(c, WS_VALUES, sizeof(float) * (size_t)K * d);
     if (!da.values) return QGX_ERR_CUDA;
   }
-  // Large vectors: the walk alone with one worker per thread (twice the warps of the one-pass kernel, whose 64 running
+  // On request: the walk alone with one worker per thread (twice the warps of the one-pass kernel, whose 64 running
   // sums per thread fill the register file), every worker's symbol bytes kept, and the ordered sums from those.
   da.norms_out = nullptr;
   const bool in_place = (sym_mode & 3) == 3;             // compares with the kept symbols and overwrites them: one pass
-  const bool two_pass = K > 1 && !da.values && !in_place &&
-                        (c->decode_split == QGX_SPLIT_SYMBOLS || (c->decode_split == QGX_SPLIT_AUTO && !small && kTwoPassByDefault));
+  const bool two_pass = K > 1 && !da.values && !in_place && c->decode_split == QGX_SPLIT_SYMBOLS;
   if (two_pass) {
     if (!da.sym_out) da.sym_out = (uint8_t*)ws_get(c, WS_SYMTMP, (size_t)K * sym_ld);
     da.norms_out = (float*)ws_get(c, WS_NORMSDEC, sizeof(float) * (size_t)K * nb);
     if (!da.sym_out || !da.norms_out) return QGX_ERR_CUDA;
-    rc = launch_decode_average(c, da, ct, lt_kept, 0, true);
+    rc = launch_decode_walk(c, da, ct, lt_kept);
     if (rc != QGX_OK) return rc;
     MeanArgs ma;
     ma.sym = da.sym_out; ma.sym_ld = sym_ld; ma.norms = da.norms_out; ma.sym_prev = da.sym_prev; ma.norms_prev = da.norms_prev;
@@ -1266,7 +1259,8 @@ static qgx_status launch_decode_gs(qgx_ctx* c, const DecodeArgs& da, const CodeT
     ScopedKernelTimer timer(c, QGX_KERNEL_DECODE);
     allow_max_dynamic_smem((const void*)k_exchange_decode<G, SYM, VAL>, c->device);
     TableCache* tc = table_cache(c);
-    LaunchShape& shape = (VAL ? tc->dec : tc->dec_walk)[G == 32 ? 0 : (G == 64 ? 1 : 2)][SYM];
+    constexpr int g = G == 32 ? 0 : (G == 64 ? 1 : 2);
+    LaunchShape& shape = VAL ? tc->dec[g][SYM] : tc->dec_walk[g];
     if (shape.smem != lut_bytes + 1) {                       // occupancy asked once per shape, not per call
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_exchange_decode<G, SYM, VAL>, kDecThreads, lut_bytes);
       shape.smem = lut_bytes + 1;
@@ -1280,33 +1274,34 @@ static qgx_status launch_decode_gs(qgx_ctx* c, const DecodeArgs& da, const CodeT
   return cuda_status(cudaGetLastError());
 }
 
-template <int G, bool VAL>
+template <int G>
 static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, int sym_mode) {
   switch (sym_mode) {
-    case 1: return launch_decode_gs<G, 1, VAL>(c, da, ct, lt);
-    case 2: return launch_decode_gs<G, 2, VAL>(c, da, ct, lt);
-    case 3: return launch_decode_gs<G, 3, VAL>(c, da, ct, lt);
-    case 4: return launch_decode_gs<G, 4, VAL>(c, da, ct, lt);
-    case 5: return launch_decode_gs<G, 5, VAL>(c, da, ct, lt);
-    default: return launch_decode_gs<G, 0, VAL>(c, da, ct, lt);
+    case 1: return launch_decode_gs<G, 1, true>(c, da, ct, lt);
+    case 2: return launch_decode_gs<G, 2, true>(c, da, ct, lt);
+    case 3: return launch_decode_gs<G, 3, true>(c, da, ct, lt);
+    case 4: return launch_decode_gs<G, 4, true>(c, da, ct, lt);
+    case 5: return launch_decode_gs<G, 5, true>(c, da, ct, lt);
+    default: return launch_decode_gs<G, 0, true>(c, da, ct, lt);
   }
 }
 
-qgx_status launch_decode_average(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, int sym_mode,
-                                 bool walk_only) {
+qgx_status launch_decode_average(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, int sym_mode) {
   if (!ct.has_header || da.bucket % ct.G != 0) return QGX_ERR_INVALID_ARG;
-  if (walk_only) {
-    switch (ct.G) {
-      case 32: return launch_decode_g<32, false>(c, da, ct, lt, sym_mode);
-      case 64: return launch_decode_g<64, false>(c, da, ct, lt, sym_mode);
-      case 128: return launch_decode_g<128, false>(c, da, ct, lt, sym_mode);
-      default: return QGX_ERR_INVALID_ARG;
-    }
-  }
   switch (ct.G) {
-    case 32: return launch_decode_g<32, true>(c, da, ct, lt, sym_mode);
-    case 64: return launch_decode_g<64, true>(c, da, ct, lt, sym_mode);
-    case 128: return launch_decode_g<128, true>(c, da, ct, lt, sym_mode);
+    case 32: return launch_decode_g<32>(c, da, ct, lt, sym_mode);
+    case 64: return launch_decode_g<64>(c, da, ct, lt, sym_mode);
+    case 128: return launch_decode_g<128>(c, da, ct, lt, sym_mode);
+    default: return QGX_ERR_INVALID_ARG;
+  }
+}
+
+qgx_status launch_decode_walk(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt) {
+  if (!ct.has_header || da.bucket % ct.G != 0) return QGX_ERR_INVALID_ARG;
+  switch (ct.G) {
+    case 32: return launch_decode_gs<32, 0, false>(c, da, ct, lt);
+    case 64: return launch_decode_gs<64, 0, false>(c, da, ct, lt);
+    case 128: return launch_decode_gs<128, 0, false>(c, da, ct, lt);
     default: return QGX_ERR_INVALID_ARG;
   }
 }
