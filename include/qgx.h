@@ -17,7 +17,9 @@
  *    qgx_sync_status, which synchronizes the stream.  No call aborts, traps or prints;
  *  - the library allocates device memory only inside qgx_create and when a call needs a larger
  *    workspace than any call before it (qgx_encode, qgx_decode, the fused calls and qgx_update_levels);
- *    the fused calls also keep device tables of the up to 32 configurations they have met.  qgx_quantize,
+ *    the fused calls also keep device tables of the up to 32 configurations they have met, where a fused call
+ *    recorded into a stream capture reads them: other configurations used on the context before a replay may
+ *    have taken their place.  qgx_quantize,
  *    qgx_average and qgx_encode_noalloc allocate nothing and may be recorded into a stream capture, qgx_decode once
  *    its workspace has the size (after a call on as many buckets): what they derive from their level table or code
  *    goes with the launch, so a replay uses what was recorded.
@@ -229,8 +231,8 @@ qgx_status qgx_average(qgx_ctx *ctx, const float *norms, const uint8_t *sym, int
 
 /* ---- fused exchange ------------------------------------------------------------------------ */
 
-/* quantize -> encode -> decode -> average in two kernels, same streams and same mean as the four
- * calls above in sequence.  v [dev] float[K][d]; mean_out [dev] float[d]; total_bits [dev]
+/* quantize -> encode -> decode -> average in one to three kernels, same streams and same mean as the
+ * four calls above in sequence.  v [dev] float[K][d]; mean_out [dev] float[d]; total_bits [dev]
  * uint64[K] (may be NULL).  The streams live in the context's workspace (slot 0 or 1, so that
  * the two exchanges of one iteration can both be kept); the workspace grows on first use (cudaMalloc) and is
  * freed by qgx_destroy.  The code must have sub-blocks of 32, 64 or 128 coordinates that divide the bucket
@@ -253,9 +255,10 @@ typedef struct {
 } qgx_segment;
 qgx_status qgx_exchange_segments(qgx_ctx *ctx, const float *v, int K, size_t d, const qgx_segment *segs /*[host]*/,
                                  int nseg, uint32_t exchange_id, float *mean_out, uint64_t *total_bits);
-/* How the decode pass of the fused calls spreads its work.  By default (QGX_SPLIT_AUTO) vectors with few
- * sub-blocks are decoded one worker per thread, followed by a kernel that adds the workers' values in worker
- * order (same results, K times more threads, K * d floats of workspace, at most 256 MB); large vectors are decoded
+/* How the decode pass of the fused calls spreads its work (where the exchange is not one launch, see
+ * qgx_set_encode_path).  By default (QGX_SPLIT_AUTO) vectors with few sub-blocks are decoded one worker per
+ * thread, followed by a kernel that adds the workers' values in worker order (same results, K times more
+ * threads, K * d floats of workspace, at most 256 MB); large vectors are decoded
  * by one thread per sub-block over all workers.  QGX_SPLIT_NEVER / QGX_SPLIT_ALWAYS force one way (ALWAYS still
  * falls back when the workspace would exceed 256 MB).  QGX_SPLIT_SYMBOLS decodes in two passes: the walk alone, one
  * worker per thread, writes every worker's symbol bytes (K * d bytes of workspace unless the exchange keeps its
@@ -268,7 +271,8 @@ qgx_status qgx_set_decode_split(qgx_ctx *ctx, int mode);
  * rounding.  QGX_ENCODE_STAGED: buckets of 1024, 2048, 4096, 8192 or 16384 coordinates (whatever the alignment and the
  * length of the vectors) are staged in shared memory by asynchronous copies and packed 32 coordinates per lane by warps
  * that do not wait for one another's buckets; other bucket sizes still go through the first kernel.  QGX_ENCODE_AUTO
- * (the default) takes the kernel that measured faster on B200. */
+ * (the default) takes what measured faster on B200: with QGX_SPLIT_AUTO, short vectors of up to 16 workers (buckets a multiple
+ * of 128) go out in one launch that encodes, decodes and averages; otherwise one of the two kernels. */
 enum { QGX_ENCODE_AUTO = 0, QGX_ENCODE_REGISTERS = 1, QGX_ENCODE_STAGED = 2 };
 qgx_status qgx_set_encode_path(qgx_ctx *ctx, int mode);
 /* The receiving side alone (Algorithm 1: decode, aggregate): decodes the streams that the last qgx_exchange with

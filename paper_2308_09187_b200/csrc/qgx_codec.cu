@@ -1,5 +1,7 @@
-// qgx_encode and qgx_decode as separate steps: bucket bit lengths -> exclusive scan of the
-// word-aligned lengths (offsets) -> bit scatter; and offsets -> bit gather.
+// qgx_encode and qgx_decode as separate steps.  Encoding takes one pass (k_pack: pack a bucket, find its place by look-back,
+// copy it out) where the capacity fits any outcome and the sub-blocks are a warp's, else three kernels: bucket bit lengths ->
+// exclusive scan of the word-aligned lengths (offsets) -> bit scatter; qgx_encode_noalloc takes the three always.  Decoding:
+// offsets (k_scan_offsets, which also builds the decoder's table) -> k_unpack.
 #include "qgx_bucket.cuh"
 #include "qgx_codec.cuh"
 

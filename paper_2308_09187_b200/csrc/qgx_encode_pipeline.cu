@@ -12,12 +12,12 @@
 // 0.40 cycles per coordinate and SM: 33 instructions at 65 % issue, with the ALU, the integer multiplier (the generator's
 // wide products run at a quarter of the rate) and the shared-memory pipe each 55-60 % busy.  With copies, norms and
 // placing it is 60 instructions at 62 %.  Shared memory (two stages and two to four images per quantizer) sets the
-// number of warps.  Measured per 2^27 coordinates against the bucket-in-registers kernel, whose CTAs load, norm, round
-// and write one after the other with three CTA barriers per bucket: buckets of 16384 395 us (433), 8192 392 us (508),
-// 4096 390 us (480), 1024 379 us (883); rows that are not 16-byte aligned, 16 x 10^6 coordinates, 69 us (234), since
-// there the rounding map serves, too, and a row costs four-byte instead of 16-byte copies.
-// Tried: loaders as warps of their own (they share the issue slots of one warp each and fall behind), and quantizers that
-// copy their own bits out (fewer warps to hide latency behind): 5-30 % slower.
+// number of warps.  Measured per 2^27 Gaussian coordinates, 17 fitted levels, against the bucket-in-registers kernel, whose
+// CTAs load, norm, round and write one after the other with three CTA barriers per bucket: buckets of 16384 362 us (407),
+// 8192 359 us (482), 4096 361 us (487), 2048 362 us (680), 1024 353 us (858); rows that are not 16-byte aligned, 16 x 10^6
+// coordinates, 66 us (210), since there the rounding map serves, too, and a row costs four-byte instead of 16-byte copies.
+// Tried: loaders as warps of their own (they share the issue slots of one warp each and fall behind), 4.1 to 6.5 ps per
+// coordinate against 2.8, and quantizers that copy their own bits out (fewer warps to hide latency behind), 3.1 to 3.3.
 //
 // In a translation unit of its own: the quantizers' loop runs at the register limit.
 #include "qgx_encode.cuh"

@@ -1145,8 +1145,10 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     else QGX_LAUNCH_E(V, 128);                             \
   } while (0)
   // Buckets of 1024 * 2^j coordinates go through the pipelined kernel, other sizes through the bucket-in-registers kernel.
-  // (So do a few hundred buckets of 4096, which that kernel holds all at once: 36864 coordinates of 16 workers 15 us
-  // against 17 us; from some 600 buckets on the pipeline is ahead.)
+  // So do up to four buckets of 4096 per SM, which that kernel holds all at once (they come here with more than 16 workers, or
+  // when they are too many for one launch).  Whole exchanges, that kernel : the pipeline, 9 uniform levels: 32 x 9 buckets
+  // 31.1 us : 34.3, 8 x 56 33.5 : 37.4, 16 x 36 36.1 : 39.9, 128 x 2 39.1 : 42.0; 17 levels with codewords of up to 12 bits:
+  // 8 x 37 43.6 : 45.2, 8 x 74 56.0 : 58.6, 8 x 92 65.0 : 63.8, 8 x 222 98.0 : 95.2.
   const bool pipelined = bucket % kChunk == 0 && (bucket & (bucket - 1)) == 0 && c->encode_path != QGX_ENCODE_REGISTERS &&
                          (unsigned long long)nb * (unsigned long long)K < (1ull << 31) &&
                          (bucket != 4 * kChunk || c->encode_path == QGX_ENCODE_STAGED || nb * (size_t)K >= 4 * (size_t)c->num_sms);
@@ -1313,9 +1315,19 @@ qgx_status launch_decode_walk(qgx_ctx* c, const DecodeArgs& da, const CodeTable&
 // Each tensor is still a chain of launches with gaps, ends that not all SMs reach together and a start that fills slowly,
 // and the persistent kernels of two streams do not share an SM.  So, once there is enough work to fill the GPU, every
 // stream runs on the SMs of its share of the work: the chains then run side by side and a gap in one idles only its SMs.
-// 16 tensors of 1728 to 2.4 * 10^6 coordinates, 16 workers, bucket 4096: 905 us on 4 streams over all SMs, 766 on 4 with
-// shares, 706 on 8; 24 tensors of 10^3 to 1.3 * 10^6, 8 workers: 485, 440, 370.  Below kSegSplitCoords there is
-// nothing to share out and each further stream costs two events (8 tensors, 60 * 10^3 coordinates: 59 us on 4, 62 on 8).
+// us on 1 stream / 4 over all SMs / 4 with shares / 8 over all / 8 with shares:
+//   16 tensors of 1728 to 2.4 * 10^6, 16 workers, bucket 4096:  1135 / 878 / 753 / 884 / 670
+//   24 of 4000 to 1.3 * 10^6, 16 workers, bucket 8192:          1054 / 652 / 575 / 630 / 517
+//   6 of 4 * 10^6, 4 workers, bucket 8192:                      562 / 466 / 446 / 464 / 431
+//   3 of 5 * 10^5 to 3 * 10^6, 16 workers, bucket 8192:         407 / 351 / 328 / 351 / 328
+//   24 of 1000 to 2.6 * 10^5, 8 workers, bucket 1024:           497 / 221 / 215 / 185 / 182
+//   12 of 4000 to 6.4 * 10^5, 2 workers, bucket 1024:           260 / 129 / 118 / 111 / 100
+//   20 of 10^5, 8 workers, bucket 4096:                         451 / 200 / 200 / 197 / 197
+//   50 of 2 * 10^4, 8 workers, bucket 1024:                     855 / 316 / 315 / 312 / 305
+//   10 of 500 to 2.4 * 10^5, 3 workers, bucket 4096:            194 / 81 / 76 / 75 / 75      (18263 coordinates per SM)
+//   24 of 2500, 4 workers, bucket 1024:                         348 / 157 / 156 / 158 / 158  (1621)
+// Below kSegSplitCoordsPerSm there is nothing to share out and each further stream costs two events.  kSegFixed of 0.3 and
+// 4 * 10^6 instead of 10^6: 669 and 693 for the first, 543 and 532 for the second, the others within 3 %.
 constexpr int kSegStreams = 8;
 constexpr int kSegStreamsSmall = 4;
 constexpr double kSegSplitCoordsPerSm = 16384.0;        // workers * coordinates per SM

@@ -9,9 +9,10 @@
 namespace qgx {
 
 // ---- the rounding table of a level table, kept between calls on the host --------------------------
-// Building one takes the host some 50 us (four bin widths, up to 1025 bins, all levels), and a program calls with a handful of
-// level tables, so a context keeps the last few (compared in full on a hit).  It goes to the kernel by value: the call
-// allocates nothing, and a launch recorded in a stream capture keeps the table that it was recorded with.
+// Building one takes the host some 20 us for 17 levels (four bin widths, up to 1025 bins, all levels; a first call with a table
+// 39 us, another 17), and a program calls with a handful of level tables, so a context keeps the last few (compared in full
+// on a hit).  It goes to the kernel by value: the call allocates nothing, and a launch recorded in a stream capture keeps the
+// table that it was recorded with.
 constexpr int kStepSlots = 8;
 struct StepLevels {
   int nlev;                              // 0: empty
