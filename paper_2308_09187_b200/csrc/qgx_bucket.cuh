@@ -126,11 +126,12 @@ __device__ __forceinline__ float bucket_norm(const BucketRegs<V4>& r, int norm_t
   return (float)red[32];
 }
 
-// Norm of the bucket held by the CTA, one barrier: per-warp partials go to shared memory and every
-// warp then reduces them in the same order (so all warps hold the same value).
-template <int V4>
-__device__ __forceinline__ float bucket_norm_all(const BucketRegs<V4>& r, int norm_type, double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+// Norm of the bucket held by `nwarps` warps, one barrier of theirs (`sync`): per-warp partials go to shared memory and
+// every warp then reduces them in the same order (so all warps hold the same value).
+template <int V4, typename Sync>
+__device__ __forceinline__ float bucket_norm_team(const BucketRegs<V4>& r, int norm_type, double* red, int warp, int nwarps,
+                                                  Sync sync) {
+  const int lane = threadIdx.x & 31;
   double acc = 0.0;
   if (norm_type == QGX_NORM_L2) {
 #pragma unroll
@@ -152,22 +153,28 @@ __device__ __forceinline__ float bucket_norm_all(const BucketRegs<V4>& r, int no
     acc = __any_sync(0xffffffffu, bad) ? (double)__int_as_float(0x7fc00000) : (double)m;
   }
   if (lane == 0) red[warp] = acc;
-  __syncthreads();
+  sync();
   double t = lane < nwarps ? red[lane] : 0.0;
   if (norm_type == QGX_NORM_L2) return (float)sqrt(warp_sum(t));
   const bool bad = __any_sync(0xffffffffu, t != t);
   const float m = warp_max((float)t);
   return bad ? __int_as_float(0x7fc00000) : m;
 }
+// ... by the CTA
+template <int V4>
+__device__ __forceinline__ float bucket_norm_all(const BucketRegs<V4>& r, int norm_type, double* red) {
+  return bucket_norm_team<V4>(r, norm_type, red, (int)(threadIdx.x >> 5), (int)(blockDim.x >> 5),
+                              [] { __syncthreads(); });
+}
 
-// Loads bucket [lo, lo + len) of worker k: warp w holds coordinates [w * 256 * P, (w + 1) * 256 * P), row j of
-// them 32 octets (8 consecutive coordinates: two quads), lane l the l-th octet of the row.
+// Loads bucket [lo, lo + len) of worker k into `nwarps` warps: warp w holds coordinates [w * 256 * P, (w + 1) * 256 * P),
+// row j of them 32 octets (8 consecutive coordinates: two quads), lane l the l-th octet of the row.
 template <int P>
 __device__ __forceinline__ void load_bucket_octets(BucketRegs<2 * P>& r, const DualSource& s, size_t k, size_t d,
-                                                   size_t lo, int len, bool vec_ok) {
+                                                   size_t lo, int len, bool vec_ok, int warp, int nwarps) {
   const size_t ld = s.ld ? s.ld : d;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (vec_ok && len == 256 * P * (int)(blockDim.x >> 5)) {
+  const int lane = threadIdx.x & 31;
+  if (vec_ok && len == 256 * P * nwarps) {
     // every lane holds full octets: the kind of source is decided once, not per quad
     const float4* pv = s.v ? reinterpret_cast<const float4*>(s.v + k * ld + lo) + ((warp * P * 32 + lane) << 1) : nullptr;
     const float4* pa = s.a ? reinterpret_cast<const float4*>(s.a + lo) + ((warp * P * 32 + lane) << 1) : nullptr;

@@ -151,7 +151,7 @@ k_exchange_encode(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
     uint32_t* s_img = s_dyn + par * img_words;
 
     BucketRegs<2 * P> r;
-    load_bucket_octets<P>(r, a.src, k, a.d, lo, len, a.vec_ok);
+    load_bucket_octets<P>(r, a.src, k, a.d, lo, len, a.vec_ok, warp, nwarps);
     {
       // this image was last read by the copy-out two buckets ago; two barriers have passed since
       uint4* z = reinterpret_cast<uint4*>(s_img);

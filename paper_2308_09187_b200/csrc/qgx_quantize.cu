@@ -54,6 +54,7 @@ struct QuantizeArgs {
   size_t nb, total;                      // buckets per worker, of all workers
   int norm_type, norms_supplied;
   uint32_t xid;
+  int team, teams;                       // threads per bucket, buckets that a CTA works on side by side
   bool vec_ok;                           // 16-byte loads
   int store;                             // bytes per symbol store: 8, 4 or 1
   float* norms;
@@ -61,12 +62,13 @@ struct QuantizeArgs {
   DevStatus* st;
 };
 
-// Persistent CTAs, one bucket at a time held in registers between the norm and the rounding (v is read from HBM once); a
-// thread works on P octets of consecutive coordinates.  What bounds it: instruction issue -- about 26 instructions per
-// coordinate are the generator and the rounding map.  Every CTA builds the map's table in shared memory from the launch's
-// parameters, once for all of its buckets: a table kept in device memory measured the same (4 x 8200 coordinates 6.2 us a
-// call with it, 6.4 so; quantize + encode of 8 x 2^22, 155.0 and 154.6) but needs an allocation and changes under a recorded
-// launch.
+// Persistent CTAs; a bucket is held in registers between the norm and the rounding (v is read from HBM once), a thread works
+// on P octets of consecutive coordinates.  What bounds it: instruction issue -- about 26 instructions per coordinate are the
+// generator and the rounding map.  Every CTA builds the map's table in shared memory from the launch's parameters, once for
+// all of its buckets: a table kept in device memory would need an allocation and change under a recorded launch.  Buckets of
+// up to 1024 coordinates are worked on side by side by teams of one to four warps that share a CTA and its table: with a
+// table for every one of them, 8 x 10^6 coordinates in buckets of 256 took 37.1 us, of 512 28.8 (a table from device memory
+// 35.3 and 27.4; teams 26.6 and 26.7), 4 x 2000 in buckets of 256 8.6 us (7.2; 7.1).
 template <int P>
 __global__ void __launch_bounds__(P == 1 ? 256 : 512, P == 1 ? 4 : 2)
 k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ LevelTable lt, const __grid_constant__ PhiloxKey key,
@@ -77,29 +79,39 @@ k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ Level
   fill_bin_table(s_bin, rt, BinKind::kFixed);
   if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr bool kTeams = P == 1;
+  const int lane = threadIdx.x & 31;
+  const int threads = kTeams ? a.team : (int)blockDim.x, nwarps = threads >> 5;
+  const int teams = kTeams ? a.teams : 1, team = kTeams ? (int)threadIdx.x / threads : 0;
+  const int warp = ((int)threadIdx.x - team * threads) >> 5;
+  if (kTeams && team >= teams) return;   // only here to fill the table; no barrier of the whole CTA follows
+  const auto sync = [&]() {
+    if constexpr (!kTeams) __syncthreads();
+    else if (nwarps == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(threads) : "memory");
+  };
   const uint32_t lev_sa = smem_addr(s_lev);
   RoundFix rc;
   const uint32_t copies = 16u << (rt.key_shift - kKeyShiftMin);
   rc.mask = ~(copies - 1u);
   rc.base = smem_addr(s_bin) - kBinAddrBase + (((uint32_t)lane << 4) & (copies - 1u));
   int par = 0;
-  for (size_t t = blockIdx.x; t < a.total; t += gridDim.x, par ^= 1) {
+  for (size_t t = (size_t)blockIdx.x * teams + team; t < a.total; t += (size_t)gridDim.x * teams, par ^= 1) {
     const size_t k = a.total <= 0xffffffffull ? (size_t)((uint32_t)t / (uint32_t)a.nb) : t / a.nb;
     const uint32_t ku = (uint32_t)k;
     const size_t lo = (t - k * a.nb) * (size_t)a.bucket;
     const int len = (int)min((size_t)a.bucket, a.d - lo);
     BucketRegs<2 * P> r;
-    load_bucket_octets<P>(r, a.src, k, a.d, lo, len, a.vec_ok);
+    load_bucket_octets<P>(r, a.src, k, a.d, lo, len, a.vec_ok, warp, nwarps);
     float norm;
     if (a.norms_supplied) {
       norm = a.norms[t];
     } else {
-      norm = bucket_norm_all<2 * P>(r, a.norm_type, s_red[par]);
-      if (threadIdx.x == 0) a.norms[t] = norm;
+      norm = bucket_norm_team<2 * P>(r, a.norm_type, s_red[par] + team * nwarps, warp, nwarps, sync);
+      if (warp == 0 && lane == 0) a.norms[t] = norm;
     }
     const bool finite = (norm - norm) == 0.0f;
-    if (!finite && threadIdx.x == 0) latch_error(a.st, QGX_ERR_NONFINITE);
+    if (!finite && warp == 0 && lane == 0) latch_error(a.st, QGX_ERR_NONFINITE);
     const bool live = finite && norm != 0.0f;
     const bool fast = rt.usable && norm > 7.9e-31f && norm < 1.2e30f;
     rc.rn = fast ? __frcp_rn(norm) : 0.0f;
@@ -258,12 +270,16 @@ qgx_status launch_quantize(qgx_ctx* c, DualSource src, int K, size_t d, int buck
   const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
   a.store = (d % 8 == 0 && bucket % 8 == 0 && (at & 7u) == 0) ? 8 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
   a.norms = norms; a.sym = sym; a.st = c->dstatus;
-  // octets per thread so that CTAs have at most 256 / 512 / 512 threads; as many CTAs as an SM holds (registers: 1024
-  // threads; shared memory: 12 tables of 17 KB)
+  // Octets per thread so that a bucket has at most 256 / 512 / 512 threads.  CTAs of 256 threads take as many buckets of up
+  // to 1024 coordinates side by side as they have warps for, unless that would leave SMs without any: the time of a few
+  // buckets is that of one, whatever shares its SM.  (Buckets of 1024, where a table per bucket cost least, 8 x 10^6
+  // coordinates: 27.1 us with a table each, 27.0 with two to a CTA.)
   const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
-  const int threads = bucket_threads(bucket, 2 * pp);
-  const unsigned per_sm = (unsigned)std::min(12, std::max(2, 1024 / threads));
-  const unsigned grid = (unsigned)std::min<size_t>(a.total, (size_t)c->num_sms * per_sm);
+  a.team = bucket_threads(bucket, 2 * pp);
+  a.teams = pp == 1 ? (int)std::max<size_t>(1, std::min<size_t>((size_t)(256 / a.team), a.total / (size_t)c->num_sms)) : 1;
+  const int threads = pp == 1 ? 256 : a.team;
+  const unsigned per_sm = (unsigned)std::max(2, 1024 / threads);      // registers: 1024 threads
+  const unsigned grid = (unsigned)std::min<size_t>((a.total + (size_t)a.teams - 1) / (size_t)a.teams, (size_t)c->num_sms * per_sm);
   switch (pp) {
     case 1: k_quantize<1><<<grid, threads, 0, c->stream>>>(a, lt, key, *rt); break;
     case 2: k_quantize<2><<<grid, threads, 0, c->stream>>>(a, lt, key, *rt); break;

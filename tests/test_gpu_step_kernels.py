@@ -89,3 +89,29 @@ def test_decode_without_sub_blocks_spreads_its_walks(K, d, bucket):
     qgx.qgx_sync_status(ctx)
     assert torch.equal(got_norms, norms) and torch.equal(got_sym, sym)
     qgx.qgx_destroy(ctx)
+
+
+@pytest.mark.parametrize("bucket", [4, 256, 260, 512, 516, 768, 1024, 1028, 2048])
+@pytest.mark.parametrize("nb", [1, 147, 2 * 148 + 1, 9 * 148 + 5])
+def test_quantize_buckets_side_by_side(bucket, nb):
+    """Buckets of one to eight warps, one to eight of them in a CTA, with warps left over and not: on both sides of the
+    counts where that changes.  The last bucket of every worker is short, one bucket is zero, one not finite."""
+    import paper_2308_09187_b200 as qgx
+    K, d = (1, nb * bucket - 3) if nb % 3 else (3, nb // 3 * bucket - 3)
+    nb = o.nbuckets(d, bucket)
+    ctx = qgx.qgx_create(0)
+    v = torch.randn((K, d), device="cuda", generator=torch.Generator("cuda").manual_seed(d))
+    v[K - 1, : min(bucket, d)] = 0.0
+    lev = [0.0, 0.01, 0.02, 0.1, 0.3, 0.6, 1.0]
+    for norm_type in (qgx.QGX_NORM_L2, qgx.QGX_NORM_LINF):
+        norms, sym = qgx.qgx_quantize(ctx, v, bucket, lev, norm_type, 5, 2)
+        qgx.qgx_sync_status(ctx)
+        n, x = norms.cpu().numpy(), v.cpu().numpy()
+        assert np.all(np.abs(n - o.bucket_norms(x, bucket, norm_type)) <= np.spacing(n))
+        assert np.array_equal(sym.cpu().numpy(), o.quantize(x, bucket, lev, n, 5, 2))
+    v[0, d - 1] = float("inf")
+    _, sym2 = qgx.qgx_quantize(ctx, v, bucket, lev, qgx.QGX_NORM_LINF, 5, 2)
+    assert qgx.qgx_sync_status(ctx, check=False) == qgx.QGX_ERR_NONFINITE
+    last = (nb - 1) * bucket
+    assert not sym2[0, last:].any() and torch.equal(sym2[0, :last], sym[0, :last]) and torch.equal(sym2[1:], sym[1:])
+    qgx.qgx_destroy(ctx)
