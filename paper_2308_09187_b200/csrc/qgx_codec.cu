@@ -70,30 +70,32 @@ __global__ void __launch_bounds__(512) k_bucket_bits(const uint8_t* __restrict__
 }
 
 // The decoder's table: index = the next maxlen + 1 stream bits, entry = symbol byte | bits consumed << 8, 0 where no codeword
-// starts like the index.  By the threads of one CTA: codewords of up to six bits by way of a table of 64, so that neighbouring
-// threads write neighbouring entries, then the few entries of the longer ones.
+// starts like the index.  By the 32 warps of one CTA, a level each: codewords of up to six bits by way of a table of 64, so
+// that neighbouring threads write neighbouring entries, then the few entries of the longer ones.  It is on the way of every
+// decode, whatever its size: with a loop over the levels in every thread 4 x 2000 coordinates in buckets of 256 took 16.0 us,
+// 15.0 so.
 constexpr int kUnpackTableMax = 2 << QGX_MAX_CODE_LEN;
+constexpr int kScanThreads = 1024, kScanEach = 4;
 __device__ __forceinline__ void build_unpack_table(const CodeTable& ct, uint16_t* table /* [2 << maxlen] */) {
+  static_assert(kScanThreads == 32 * QGX_MAX_LEVELS, "a warp per level");
   __shared__ uint16_t s_short[64];       // level | length << 8
-  const int tab_n = 2 << ct.maxlen;
-  if (threadIdx.x < 64) {
-    uint32_t e = 0;
-    for (int j = 0; j < ct.nlev; ++j)
-      if (ct.len[j] <= 6 && (threadIdx.x & ((1u << ct.len[j]) - 1u)) == ct.rev[j]) e = (uint32_t)j | ((uint32_t)ct.len[j] << 8);
-    s_short[threadIdx.x] = (uint16_t)e;
+  const int tab_n = 2 << ct.maxlen, lane = threadIdx.x & 31, level = threadIdx.x >> 5;
+  if (threadIdx.x < 64) s_short[threadIdx.x] = 0;
+  const int L = ct.len[level];           // 0 beyond the last level
+  const uint32_t rev = ct.rev[level];
+  __syncthreads();
+  if (L >= 1 && L <= 6 && lane < (64 >> L)) s_short[rev | ((uint32_t)lane << L)] = (uint16_t)(level | (L << 8));
+  __syncthreads();
+  const auto entry = [](uint32_t j, uint32_t len, uint32_t sign) {
+    return (uint16_t)(j == 0 ? len << 8 : ((len + 1u) << 8) | j | (sign << 7));
+  };
+  for (int i = threadIdx.x; i < tab_n; i += kScanThreads) {
+    const uint32_t x = s_short[i & 63], len = x >> 8;
+    table[i] = x == 0 ? (uint16_t)0 : entry(x & 0xffu, len, ((uint32_t)i >> len) & 1u);
   }
   __syncthreads();
-  const auto entry = [](uint32_t level, uint32_t L, uint32_t sign) { return (uint16_t)(level == 0 ? L << 8 : ((L + 1u) << 8) | level | (sign << 7)); };
-  for (int i = threadIdx.x; i < tab_n; i += blockDim.x) {
-    const uint32_t x = s_short[i & 63], L = x >> 8;
-    table[i] = x == 0 ? (uint16_t)0 : entry(x & 0xffu, L, ((uint32_t)i >> L) & 1u);
-  }
-  __syncthreads();
-  for (int j = 0; j < ct.nlev; ++j) {
-    const int L = ct.len[j];
-    if (L <= 6) continue;
-    for (int i = threadIdx.x; i < (tab_n >> L); i += blockDim.x) table[ct.rev[j] | (i << L)] = entry((uint32_t)j, (uint32_t)L, (uint32_t)i & 1u);
-  }
+  if (L > 6)
+    for (int i = lane; i < (tab_n >> L); i += 32) table[rev | ((uint32_t)i << L)] = entry((uint32_t)level, (uint32_t)L, (uint32_t)i & 1u);
 }
 
 // One CTA per worker: off[k][b] = sum_{b' < b} ceil(bits[k][b'] / 32); total_bits[k]; a worker whose
@@ -102,7 +104,6 @@ __device__ __forceinline__ void build_unpack_table(const CodeTable& ct, uint16_t
 // decoder's table, afresh in every call: nothing is kept that a later call could change under a recorded one, and no launch
 // is added (decode + average of 8 x 2^22 coordinates 69.3 us with a table kept per code and widened by every CTA of the
 // decoder, 67.7 so; every CTA building it from the code, 71.5).
-constexpr int kScanThreads = 1024, kScanEach = 4;
 __global__ void __launch_bounds__(kScanThreads) k_scan_offsets(const uint32_t* __restrict__ bucket_bits, size_t nb, size_t cap_words,
                                                                uint64_t* __restrict__ off, uint64_t* __restrict__ total_bits,
                                                                uint32_t* __restrict__ flags, unsigned int err_code, DevStatus* st,

@@ -115,3 +115,33 @@ def test_quantize_buckets_side_by_side(bucket, nb):
     last = (nb - 1) * bucket
     assert not sym2[0, last:].any() and torch.equal(sym2[0, :last], sym[0, :last]) and torch.equal(sym2[1:], sym[1:])
     qgx.qgx_destroy(ctx)
+
+
+@pytest.mark.parametrize("lengths", [[1, 1], list(range(1, 13)) + [12], [5] * 32, [1] + [6] * 31, [2, 7, 7] + [3] * 5, [12] * 8])
+@pytest.mark.parametrize("sub", [0, 32])
+def test_decoder_table_of_every_length(lengths, sub):
+    """The decoder's table: codewords below, at and above the six bits of its first half, alone and mixed; codes that use
+    all their codewords and codes that leave some over."""
+    import paper_2308_09187_b200 as qgx
+    nlev, K, d, bucket = len(lengths), 3, 5003, 512
+    order = sorted(range(nlev), key=lambda j: (lengths[j], j))
+    code, words, prev = 0, [0] * nlev, lengths[order[0]]
+    for j in order:                                                  # canonical: consecutive codewords, shorter ones first
+        code <<= lengths[j] - prev
+        words[j], prev, code = code, lengths[j], code + 1
+    cb = qgx.qgx_build_codebook_fixed(nlev, sub)
+    for j in range(nlev):
+        cb.len[j], cb.code[j] = lengths[j], words[j]
+    cb.maxlen = max(lengths)
+    rng = np.random.default_rng(nlev)
+    s = rng.integers(0, nlev, size=(K, d)).astype(np.uint8)
+    s |= (rng.integers(0, 2, size=s.shape).astype(np.uint8) << 7) * (s > 0)
+    n = rng.uniform(0.5, 2.0, size=(K, o.nbuckets(d, bucket))).astype(np.float32)
+    cbo = o.codebook_from(cb.lengths(), cb.codes(), subblock=sub)
+    st_ref, bb_ref, _ = o.encode(n, s, bucket, cbo)
+    ctx = qgx.qgx_create(0)
+    stream, bits = torch.from_numpy(st_ref.view(np.int32)).cuda(), torch.from_numpy(bb_ref.view(np.int32)).cuda()
+    norms, sym = qgx.qgx_decode(ctx, stream, bits, d, bucket, cb)
+    qgx.qgx_sync_status(ctx)
+    assert np.array_equal(norms.cpu().numpy(), n) and np.array_equal(sym.cpu().numpy(), s)
+    qgx.qgx_destroy(ctx)
