@@ -249,7 +249,7 @@ struct PackArgs {
   uint64_t* total_bits;
   unsigned long long* status;            // [K][nb], zeroed before the launch
   unsigned int* ticket;                  // zeroed before the launch
-  size_t b_first;                        // first bucket of every worker to encode (0 but for the diagnostic)
+  unsigned int first_ticket;             // K times the first bucket of every worker to encode (0 but for the diagnostic)
   int spin_limit;                        // polls of a wait for another bucket's words before it gives up
   DevStatus* st;
 };
@@ -272,7 +272,7 @@ k_pack(const __grid_constant__ PackArgs a, const __grid_constant__ CodeTable ct)
   const int img_words = (int)((((((uint32_t)a.bucket * (uint32_t)(ct.maxlen + 1) + 16u * (uint32_t)(a.bucket / ct.G + 1) + kNormBits + 31u) >> 5) + 4) + 3u) & ~3u);
   uint32_t* s_pair = s_dyn + 2 * img_words;
   fill_enc_lut(&s_lut, ct);
-  if (threadIdx.x == 0) s_ticket[0] = atomicAdd(a.ticket, 1u);
+  if (threadIdx.x == 0) s_ticket[0] = a.first_ticket + atomicAdd(a.ticket, 1u);
   for (int i = threadIdx.x; i < 2 * img_words; i += blockDim.x) s_dyn[i] = 0;
   __syncthreads();
   for (int i = threadIdx.x; i < n2 * n2; i += blockDim.x) {            // (first, second): a level, plus nlev for a negative one
@@ -283,15 +283,15 @@ k_pack(const __grid_constant__ PackArgs a, const __grid_constant__ CodeTable ct)
   __syncthreads();
   const uint32_t pair_sa = smem_addr(s_pair), weights = 4u | ((uint32_t)(8 * nlev) << 16);
   const uint32_t limit4 = (uint32_t)(128 - nlev) * 0x01010101u;        // carries into bit 7 of a byte >= nlev
-  const unsigned long long total = (unsigned long long)(a.nb - a.b_first) * (unsigned long long)a.K;
+  const unsigned long long total = (unsigned long long)a.nb * (unsigned long long)a.K;
   const int seg = ct.has_header ? ct.G / 8 : 32;                       // lanes per sub-block
   uint32_t used_words[2] = {0u, 0u};
   bool bad = false;
   for (int par = 0;; par ^= 1) {
     const unsigned long long t = s_ticket[par];
     if (t >= total) break;
-    const size_t turn = total <= 0xffffffffull ? (size_t)((uint32_t)t / (uint32_t)a.K) : (size_t)(t / (unsigned long long)a.K);
-    const size_t k = (size_t)(t - (unsigned long long)turn * (unsigned long long)a.K), b = a.b_first + turn;
+    const size_t b = total <= 0xffffffffull ? (size_t)((uint32_t)t / (uint32_t)a.K) : (size_t)(t / (unsigned long long)a.K);
+    const size_t k = (size_t)(t - (unsigned long long)b * (unsigned long long)a.K);
     const size_t lo = b * (size_t)a.bucket;
     const int len = (int)min((size_t)a.bucket, a.d - lo);
     uint32_t* s_img = s_dyn + par * img_words;
@@ -379,7 +379,7 @@ k_pack(const __grid_constant__ PackArgs a, const __grid_constant__ CodeTable ct)
         if (b + 1 == a.nb) a.total_bits[k] = 32ull * words - (incl >> kPadShift);
         s_prefix[par] = excl & ((1ull << kPadShift) - 1ull);
         s_skip[par] = timed_out || words > (unsigned long long)a.cap_words ? 1 : 0;
-        s_ticket[par ^ 1] = atomicAdd(a.ticket, 1u);
+        s_ticket[par ^ 1] = a.first_ticket + atomicAdd(a.ticket, 1u);
       }
     }
     __syncthreads();
@@ -577,16 +577,17 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
     PackArgs a;
     a.norms = norms; a.sym = sym; a.d = d; a.bucket = bucket; a.K = K; a.nb = nb; a.stream = stream; a.cap_words = cap_words;
     a.bucket_bits = bucket_bits; a.total_bits = total_bits; a.status = status + 2; a.ticket = reinterpret_cast<unsigned int*>(status);
-    a.b_first = std::min(c->skip_buckets, nb); a.spin_limit = c->wait_limit; a.st = c->dstatus;
+    const size_t todo = (nb - std::min(c->skip_buckets, nb)) * (size_t)K;
+    a.first_ticket = (unsigned int)(nb * (size_t)K - todo); a.spin_limit = c->wait_limit; a.st = c->dstatus;
     c->skip_buckets = 0;
-    if (a.b_first == nb) return QGX_OK;
+    if (todo == 0) return QGX_OK;
     const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
     a.load = (d % 8 == 0 && bucket % 8 == 0 && (at & 7u) == 0) ? 8 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
     const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
     const int threads = bucket_threads(bucket, 2 * pp);
     const size_t smem = sizeof(uint32_t) * (2 * ((img_words + 3) & ~(size_t)3) + (size_t)(4 * ct.nlev * ct.nlev));
     const unsigned fit = (unsigned)std::max<size_t>(1, std::min<size_t>((size_t)(1024 / threads), (220u * 1024u) / (smem + 2048u)));
-    const unsigned grid = (unsigned)std::min<unsigned long long>((unsigned long long)(nb - a.b_first) * (unsigned long long)K, (unsigned long long)c->num_sms * fit);
+    const unsigned grid = (unsigned)std::min<size_t>(todo, (size_t)c->num_sms * fit);
 #define QGX_LAUNCH_K(V)                                              \
   do {                                                               \
     allow_max_dynamic_smem((const void*)k_pack<V>, c->device);       \
