@@ -255,15 +255,9 @@ typedef struct {
 } qgx_segment;
 qgx_status qgx_exchange_segments(qgx_ctx *ctx, const float *v, int K, size_t d, const qgx_segment *segs /*[host]*/,
                                  int nseg, uint32_t exchange_id, float *mean_out, uint64_t *total_bits);
-/* How the decode pass of the fused calls spreads its work (where the exchange is not one launch, see
- * qgx_set_encode_path).  By default (QGX_SPLIT_AUTO) vectors with few sub-blocks are decoded one worker per
- * thread, followed by a kernel that adds the workers' values in worker order (same results, K times more
- * threads, K * d floats of workspace, at most 256 MB); large vectors are decoded
- * by one thread per sub-block over all workers.  QGX_SPLIT_NEVER / QGX_SPLIT_ALWAYS force one way (ALWAYS still
- * falls back when the workspace would exceed 256 MB).  QGX_SPLIT_SYMBOLS decodes in two passes: the walk alone, one
- * worker per thread, writes every worker's symbol bytes (K * d bytes of workspace unless the exchange keeps its
- * symbols anyway), and a second kernel forms the ordered sums, the squared differences and the state update from
- * them -- same results; exchanges that compare with and overwrite the kept symbols in one go stay in one pass. */
+/* Whether the fused calls may use the one launch of short vectors (see qgx_set_encode_path): QGX_SPLIT_AUTO, the default,
+ * lets them; the other values always take the separate encode and decode kernels.  (The values named three ways of
+ * spreading the decode pass over threads; one kernel now serves every size, with the same results.) */
 enum { QGX_SPLIT_AUTO = 0, QGX_SPLIT_NEVER = 1, QGX_SPLIT_ALWAYS = 2, QGX_SPLIT_SYMBOLS = 3 };
 qgx_status qgx_set_decode_split(qgx_ctx *ctx, int mode);
 /* Which kernel the encode pass of the fused calls uses (no counterpart in the paper; the streams are the same bit

@@ -18,15 +18,6 @@ constexpr size_t kNoAllocMaxWorkers = 1024;             // K
 constexpr size_t kNoAllocBytes = kNoAllocMaxBuckets * sizeof(uint64_t) + kNoAllocMaxWorkers * sizeof(uint32_t);
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
-void build_dec_lut_host(const CodeTable& ct, uint16_t* lut) {
-  const int n = 1 << ct.maxlen;
-  for (int i = 0; i < n; ++i) lut[i] = 0;
-  for (int j = 0; j < ct.nlev; ++j) {
-    const int L = ct.len[j];
-    for (int hi = 0; hi < (1 << (ct.maxlen - L)); ++hi) lut[ct.rev[j] | (hi << L)] = (uint16_t)(j | (L << 8));
-  }
-}
-
 __device__ __forceinline__ uint32_t load_quad_syms(const uint8_t* p, int nvalid, bool vec_ok) {
   if (nvalid == kQuad && vec_ok) return *reinterpret_cast<const uint32_t*>(p);
   uint32_t x = 0;

@@ -98,10 +98,6 @@ __device__ __forceinline__ void put_bits2(uint32_t* img, uint32_t pos, uint64_t 
   }
 }
 
-// Decoder table: index = next `maxlen` stream bits, entry = level | codeword length << 8 (0 = no
-// codeword starts with these bits).
-constexpr int kDecLutMax = 1 << QGX_MAX_CODE_LEN;
-
 // ---- chained scan of bucket lengths ("decoupled look-back") ----------------------------------
 // status word of bucket (k, b): bits 62..63 state, bits 0..61 a word count.
 constexpr unsigned long long kStEmpty = 0ull, kStAggregate = 1ull << 62, kStPrefix = 2ull << 62;
@@ -149,7 +145,5 @@ __device__ __forceinline__ unsigned long long lookback_prefix(unsigned long long
   *timed_out = fail;
   return prefix;
 }
-
-void build_dec_lut_host(const CodeTable& ct, uint16_t* lut /*[1 << maxlen]*/);
 
 }  // namespace qgx

@@ -1,0 +1,590 @@
+// The decode pass of the fused exchange: the streams of K workers -> their mean (and the state update, the kept symbols, the
+// squared differences).
+//
+// A team of warps takes a row of 32 consecutive sub-blocks.  Each warp walks the row of one worker, a lane per sub-block, and
+// leaves the symbols, a byte each, in shared memory; then the team's threads add the workers' values in worker order, four
+// consecutive coordinates each.  Four teams share a CTA and its tables: while one walks, another adds.  What a row's turn needs
+// from global memory is asked for one turn (header words) or two (bucket lengths and offsets) ahead, its stream words are
+// copied while the turn before is added up.
+//
+// What bounds it: instructions and the shared-memory pipe (22 executed instructions per symbol at 60-75 % issue; 24 M
+// wavefronts per 2^27 symbols, 58 %).  The kernel before this one walked and added in the same thread, one look-up per symbol and
+// 64 sums in registers: 16 warps per SM (12 when comparing) that waited for one another's look-ups, 32 % issue.  A look-up of
+// two symbols halves the chain, and without the sums a thread has 64 registers, 32 warps per SM.  Per 2^27 symbols, 8 workers,
+// 17 fitted levels: kept symbols 281 -> 148 us, compared 359 -> 213.  Vectors with few sub-blocks had a walk that wrote every
+// value (4 bytes per symbol, in pieces of four bytes when the length was odd) and a kernel that added them: 16 workers of
+// 1000003 coordinates 120 -> 34 us.
+#include "qgx_decode.cuh"
+
+#include <algorithm>
+#include <type_traits>
+
+namespace qgx {
+
+// ---- tables -----------------------------------------------------------------------------------
+struct NextSymbol { uint32_t sym, bits; bool known; };
+// the symbol that `bits` (the stream's next ones, first at bit 0) start with
+__device__ __forceinline__ NextSymbol next_symbol(uint32_t bits, const CodeTable& ct) {
+  NextSymbol s{bad_symbol(ct.nlev), 1u, false};
+  for (int j = 0; j < ct.nlev; ++j) {
+    const uint32_t L = ct.len[j];
+    if ((bits & ((1u << L) - 1u)) != ct.rev[j]) continue;
+    s.known = true;
+    s.sym = (uint32_t)j + (j != 0 && ((bits >> L) & 1u) ? (uint32_t)ct.nlev : 0u);
+    s.bits = L + (j != 0 ? 1u : 0u);
+  }
+  return s;
+}
+__global__ void __launch_bounds__(256) k_build_decode_tables(const __grid_constant__ CodeTable ct, DecodeTables* out) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  const NextSymbol a = next_symbol(i, ct);
+  if (i < (2u << ct.maxlen)) out->single[i] = (uint16_t)(a.sym | (a.bits << 8));
+  const uint32_t P = (uint32_t)pair_bits(ct.maxlen);
+  if (i >= (1u << P)) return;
+  const NextSymbol b = next_symbol(i >> a.bits, ct);
+  // the second symbol counts where the index holds all its bits (or all that could tell that there is none)
+  const bool both = a.bits + (b.known ? b.bits : (uint32_t)ct.maxlen + 1u) <= P;
+  out->pair[i] = (both ? (a.bits + b.bits) | (b.sym << 24) : a.bits | kPairEscape) | (a.bits << 8) | (a.sym << 16);
+}
+void launch_build_decode_tables(const CodeTable& ct, DecodeTables* out, cudaStream_t stream) {
+  const int n = 1 << std::max(ct.maxlen + 1, pair_bits(ct.maxlen));
+  k_build_decode_tables<<<(n + 255) / 256, 256, 0, stream>>>(ct, out);
+}
+
+// ---- the walk ---------------------------------------------------------------------------------
+// Words that a lane may read past the one that holds its sub-block's first bit: G symbols of at most 13 bits, the partial
+// first word and the word fetched ahead.
+template <int G>
+struct WalkReach { static constexpr int kWords = (G * 13) / 32 + 4; };
+
+// Position in a stream: the lowest five bits of `pos` are the place in w0, bit 5 says whether that has been left; what is above
+// is junk (entries of the pair table are added as they are).  The two bits before the next symbol lie in the window, too, so
+// that an index comes out as a byte offset.  SH: the words are in shared memory (32-bit addresses).
+template <bool SH> struct WordAt { using Addr = uint32_t; };
+template <> struct WordAt<false> { using Addr = const uint32_t*; };
+template <bool SH>
+struct Walk {
+  typename WordAt<SH>::Addr next;        // of the word after w1
+  uint32_t w0, w1, pos, old;             // old: pos when w0 was last checked
+  static __device__ __forceinline__ uint32_t word(uint32_t a) { return lds32(a); }
+  static __device__ __forceinline__ uint32_t word(const uint32_t* a) { return *a; }
+  static __device__ __forceinline__ uint32_t step(uint32_t a, int words) { return a + 4u * (uint32_t)words; }
+  static __device__ __forceinline__ const uint32_t* step(const uint32_t* a, int words) { return a + words; }
+  static __device__ __forceinline__ uint32_t words_from(uint32_t a, uint32_t b) { return (a - b) >> 2; }
+  static __device__ __forceinline__ uint32_t words_from(const uint32_t* a, const uint32_t* b) { return (uint32_t)(a - b); }
+  // p = the word that holds the bit two before the first, sh = that bit's place in it
+  __device__ __forceinline__ void open(typename WordAt<SH>::Addr p, uint32_t sh) {
+    w0 = word(p);
+    w1 = word(step(p, 1));
+    next = step(p, 2);
+    pos = old = sh;
+  }
+  __device__ __forceinline__ uint32_t window() const { return __funnelshift_r(w0, w1, pos); }
+  // after at most 32 bits: moves on a word where the position has left w0
+  __device__ __forceinline__ void settle() {
+    if ((pos ^ old) & 32u) {
+      w0 = w1;
+      w1 = word(next);
+      next = step(next, 1);
+    }
+    old = pos;
+  }
+  // bits taken since open(p, sh)
+  __device__ __forceinline__ uint32_t taken(typename WordAt<SH>::Addr p, uint32_t sh) const { return 32u * (words_from(next, p) - 2u) + (pos & 31u) - sh; }
+};
+
+struct WalkTable {
+  uint32_t pair;                         // shared address of the pair table, its mask for byte offsets
+  uint32_t mask;
+  __device__ __forceinline__ uint32_t entry(uint32_t window) const { return lds_table32(pair + (window & mask)); }
+};
+__device__ __forceinline__ uint32_t first_bits(uint32_t entry) { return (entry >> 8) & 31u; }
+
+// G symbols of one sub-block to row[0 .. G / 4) (shared address), four to a word.  A window holds 30 bits to come, so two
+// entries of at most 13; where an entry stands for one symbol only the second is looked up on its own, its bits taken at once
+// and the entry's own cleared.
+template <int G, bool SH>
+__device__ __forceinline__ void walk_whole(Walk<SH>& w, uint32_t row, const WalkTable& t) {
+#pragma unroll
+  for (int i = 0; i < G; i += 4) {
+    uint32_t win = w.window();
+    uint32_t e = t.entry(win);
+    if (e & kPairEscape) {
+      const uint32_t f = t.entry(__funnelshift_r(win, 0u, e));
+      w.pos += (e & 31u) + first_bits(f);
+      w.settle();
+      win = w.window();
+      e = prmt(prmt(e, f, 0x6200u), 0u, 0x3244u);                      // the two symbols, nothing taken
+    }
+    w.pos += e;
+    win = __funnelshift_r(win, 0u, e);
+    uint32_t f = t.entry(win);
+    if (f & kPairEscape) {
+      w.settle();
+      w.pos += f & 31u;
+      w.settle();
+      const uint32_t g = t.entry(w.window());
+      w.pos += first_bits(g);
+      f = prmt(prmt(f, g, 0x6200u), 0u, 0x3244u);
+    }
+    w.pos += f;
+    w.settle();
+    sts32(row + (uint32_t)i, prmt(e, f, 0x7632u));
+  }
+}
+// the same, one symbol at a time, for `count` symbols (the vector's last sub-block)
+template <bool SH>
+__device__ __forceinline__ void walk_some(Walk<SH>& w, int count, uint32_t row, const WalkTable& t) {
+#pragma unroll 1
+  for (int i = 0; i < count; i += 4) {
+    uint32_t word = 0;
+#pragma unroll 1
+    for (int q = 0; q < 4 && i + q < count; ++q) {
+      const uint32_t e = t.entry(w.window());
+      w.pos += first_bits(e);
+      w.settle();
+      word |= ((e >> 16) & 0xffu) << (8 * q);
+    }
+    sts32(row + (uint32_t)i, word);
+  }
+}
+
+// ---- where a lane's sub-block lies ------------------------------------------------------------
+struct DecodeShape {
+  uint64_t minus_zero;                   // two fp32 -0: see mul2
+  int team_warps;                        // warps of a team: 8, 16 or 32
+  int teams;                             // of a CTA
+  int rows;                              // rows that a team works on side by side (more than one: all workers at once)
+  int groups;                            // turns over the workers
+  uint32_t total_rows, units;            // units: turns of `rows` rows
+  uint32_t spb, spb_mul, spb_shift;      // sub-blocks per bucket; n / spb = (n * spb_mul >> 32) >> spb_shift
+  uint32_t whole_subs, last_count;       // sub-blocks of G coordinates, and the coordinates of the one after them
+  uint32_t hdr_bits, hdr_bits_last;      // of a bucket, of the last bucket
+  uint32_t pair_mask;                    // of byte offsets into the pair table
+  uint32_t row_words;                    // room for a warp's stream words, a multiple of 4
+  uint32_t off_val, off_kept, off_norm, off_norm_kept, off_sym, off_row;   // bytes of dynamic shared memory
+};
+
+// Row r of a worker: its sub-blocks 32 r .. 32 r + 31, of one bucket or of several in a row.
+struct RowPlace {
+  uint32_t b, s;                         // the lane's bucket, the sub-block's number in it
+  int count;                             // its coordinates, 0 beyond the end
+};
+template <int G>
+__device__ __forceinline__ RowPlace row_place(const DecodeArgs& a, const DecodeShape& h, uint32_t row, int lane) {
+  const uint32_t gs = row * 32u + (uint32_t)lane;
+  RowPlace p;
+  p.count = gs < h.whole_subs ? G : (gs == h.whole_subs ? (int)h.last_count : 0);
+  const uint32_t in = p.count > 0 ? gs : 0u;                           // beyond the end: the first bucket's first, to have some
+  p.b = __umulhi(in, h.spb_mul) >> h.spb_shift;
+  p.s = in - p.b * h.spb;
+  return p;
+}
+
+struct SubBlockAt {
+  const uint32_t* p;                     // the word that holds the bit two before its first one ...
+  uint32_t staged;                       // ... and that word's shared address where all of its words are staged, else 0
+  uint32_t sh;
+  uint32_t want;                         // bits of the sub-block
+  float norm;
+  int count;
+  bool ok;
+};
+
+// What is asked for ahead of a row's turn: two turns ahead the bucket's numbers, one turn ahead what its header says.
+struct BucketAhead { uint32_t nbits, off; };
+constexpr int kAheadWords = 4;           // header words per lane that are fetched ahead: 256 sub-blocks before the row's
+struct HeaderAhead {
+  float norm;
+  uint32_t field, before[kAheadWords];
+  bool ok;                               // the bucket's numbers agree
+};
+
+// The header words of the row's lanes, and those of lane 0's bucket before them
+template <int G>
+__device__ __forceinline__ HeaderAhead ask_header(const DecodeArgs& a, const DecodeShape& h, uint32_t row, int k, const BucketAhead& n, int lane) {
+  const RowPlace rp = row_place<G>(a, h, row, lane);
+  const uint32_t hdr = rp.b + 1u == a.nb ? h.hdr_bits_last : h.hdr_bits;
+  const uint32_t* base = a.stream + (size_t)k * a.cap_words;
+  HeaderAhead r;
+  r.ok = n.nbits >= hdr && n.nbits < (1u << 18) && (size_t)n.off + ((n.nbits + 31u) >> 5) <= a.cap_words;
+  r.norm = 0.0f;
+  r.field = 0u;
+  if (r.ok && rp.count > 0) {
+    const uint32_t* w = base + n.off;
+    r.norm = __uint_as_float(w[0]);
+    r.field = w[1 + (rp.s >> 1)];
+  }
+  const uint32_t s_first = __shfl_sync(0xffffffffu, r.ok ? rp.s : 0u, 0);
+  const uint32_t* w0 = base + __shfl_sync(0xffffffffu, n.off, 0) + 1u + (uint32_t)lane;
+#pragma unroll
+  for (int t = 0; t < kAheadWords; ++t) r.before[t] = (uint32_t)lane * 2u + 64u * (uint32_t)t < s_first ? w0[32 * t] : 0u;
+  return r;
+}
+
+// Finds worker k's sub-blocks of a row and starts the asynchronous copy of their stream words into `row_sa` (h.row_words
+// words, the warp's own).
+template <int G>
+__device__ __forceinline__ SubBlockAt find_row(const DecodeArgs& a, const DecodeShape& h, uint32_t row, int k, const BucketAhead& n,
+                                               const HeaderAhead& ha, int lane, uint32_t row_sa) {
+  const RowPlace rp = row_place<G>(a, h, row, lane);
+  const uint32_t hdr = rp.b + 1u == a.nb ? h.hdr_bits_last : h.hdr_bits;
+  const uint32_t* base = a.stream + (size_t)k * a.cap_words;
+  SubBlockAt r;
+  r.count = rp.count;
+  r.norm = ha.norm;
+  const uint32_t len = (ha.field >> (16u * (rp.s & 1u))) & 0xffffu;
+  // bits of lane 0's bucket before lane 0's sub-block
+  const uint32_t s_first = __shfl_sync(0xffffffffu, ha.ok ? rp.s : 0u, 0);
+  uint32_t before = 0;
+  if (s_first != 0u) {
+    const uint32_t half = s_first >> 1;                                // an odd number: the last word counts by its low half
+#pragma unroll
+    for (int t = 0; t < kAheadWords; ++t) before = __dp2a_lo(ha.before[t], (uint32_t)(lane + 32 * t) == half ? 0x0001u : 0x0101u, before);
+    if (s_first > 64u * kAheadWords) {
+      const uint32_t* w0 = base + __shfl_sync(0xffffffffu, n.off, 0) + 1u;
+      for (uint32_t i = (uint32_t)lane + 32u * kAheadWords; 2u * i < s_first; i += 32u) before = __dp2a_lo(w0[i], i == half ? 0x0001u : 0x0101u, before);
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+  }
+  const uint32_t excl = warp_incl_scan(len, lane) - len;
+  const uint32_t excl0 = __shfl_sync(0xffffffffu, excl, rp.s <= (uint32_t)lane ? lane - (int)rp.s : 0);   // at the bucket's first lane
+  uint32_t start = hdr + (excl - excl0) + (rp.s > (uint32_t)lane ? before : 0u);
+  r.ok = rp.count > 0 && ha.ok && start + len <= n.nbits && len < (1u << 14);
+  // A bucket whose numbers disagree is reported, and its walk reads the start of the worker's stream instead (in range
+  // whatever the offsets say).
+  r.want = len;
+  uint32_t off = n.off;
+  if (!r.ok) { start = 2u; r.want = 0u; r.norm = 0.0f; off = 0u; }
+  const uint32_t mine = off + ((start - 2u) >> 5);                     // of the worker's words: rows start on 16 bytes
+  r.p = base + mine;
+  r.sh = (start - 2u) & 31u;
+  r.staged = 0u;
+  const unsigned live = __ballot_sync(0xffffffffu, rp.count > 0);
+  if (__any_sync(0xffffffffu, rp.count > 0 && !r.ok)) return r;
+  const uint32_t first = __shfl_sync(0xffffffffu, mine, 0) & ~3u;
+  const uint32_t last = __shfl_sync(0xffffffffu, off + ((start + len + 31u) >> 5), 31 - __clz((int)live)) + WalkReach<G>::kWords;   // the buffer ends 64 words after the streams
+  if (last <= first) return r;                                         // (buckets out of order)
+  const uint32_t n4 = min(h.row_words, (last - first + 3u) & ~3u) >> 2;
+  const uint32_t* from = base + first;
+  for (uint32_t c = (uint32_t)lane; c < n4; c += 32u)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(row_sa + 16u * c), "l"(from + 4u * c) : "memory");
+  if (mine >= first && mine - first + WalkReach<G>::kWords <= 4u * n4) r.staged = row_sa + 4u * (mine - first);
+  if (rp.count <= 0) r.staged = row_sa;                                // walks nothing
+  return r;
+}
+
+// ---- two fp32 numbers at a time ---------------------------------------------------------------
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float* lo, float* hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(*lo), "=f"(*hi) : "l"(v)); }
+// Products rounded on their own.  The assembler fuses mul.rn.f32x2 with the sum it feeds (which it may not do with scalar
+// mul.rn): the product plus -0, which is the product, is what it leaves alone as long as it cannot see that number.
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b, uint64_t minus_zero) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(minus_zero));
+  return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {     // a - b as (-1) b + a
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// ---- the kernel -------------------------------------------------------------------------------
+template <int G> constexpr int kDecodeWarps = G == 128 ? 24 : 32;       // of a CTA: what its shared memory and registers hold
+template <int G>
+__host__ __device__ constexpr uint32_t sym_row_bytes() { return 32u * (uint32_t)(G / 4 + 1) * 4u; }   // a word more than needed: no bank conflicts
+
+template <int G, int SYM>
+__global__ void __launch_bounds__(kDecodeWarps<G> * 32, 1)
+k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeShape h, const __grid_constant__ LevelTable lt,
+                  const __grid_constant__ LevelTable lt_kept) {
+  constexpr bool kStore = (SYM & 1) != 0, kCompare = (SYM & 2) != 0, kSquare = (SYM & 4) != 0;
+  constexpr int kWords = G / 4, kStride = kWords + 1;                  // words of a sub-block, and from one to the next
+  constexpr int kQuads = 8 * G;                                        // quads of a row
+  constexpr int kTurn = kCompare && G > 32 ? 4 : 8;                              // workers that a thread adds in one go
+  constexpr int QT = G / 32;                                           // of them per thread of a team of eight warps
+  extern __shared__ __align__(128) unsigned char s_raw[];
+  const uint32_t sa = smem_addr(s_raw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int W = h.team_warps, team = warp / W, tw = warp - team * W;
+  const int team_threads = 32 * W, tt = (int)threadIdx.x - team * team_threads;
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(a.tables->pair);
+    uint4* dst = reinterpret_cast<uint4*>(s_raw);
+    const int n = (int)((h.pair_mask + 4u) >> 4);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = __ldg(src + i);
+    fill_signed_values(reinterpret_cast<float*>(s_raw + h.off_val), lt);
+    if (kCompare) fill_signed_values(reinterpret_cast<float*>(s_raw + h.off_kept), lt_kept);
+  }
+  __syncthreads();
+  const WalkTable wt{sa, h.pair_mask};
+  const uint32_t val_sa = sa + h.off_val, kept_sa = sa + h.off_kept;
+  const uint32_t my_sym = sa + h.off_sym + (uint32_t)warp * sym_row_bytes<G>() + (uint32_t)lane * (uint32_t)(kStride * 4);
+  const uint32_t team_sym = sa + h.off_sym + (uint32_t)(team * W) * sym_row_bytes<G>();
+  const uint32_t row_sa = sa + h.off_row + (uint32_t)warp * h.row_words * 4u;
+  float* s_norm = reinterpret_cast<float*>(s_raw + h.off_norm) + 32 * (team * W);
+  float* s_norm_kept = reinterpret_cast<float*>(s_raw + h.off_norm_kept) + 32 * (team * W);
+  const int K = a.K;
+  const float Kf = (float)K, Kinv = 1.0f / Kf;
+  const bool k_pow2 = (K & (K - 1)) == 0;                              // then the product with 1 / K is the same number
+  const float gam = a.update == 1 ? (float)a.scalars[1] : 1.0f;        // update 2 subtracts the mean itself (1 * m is exact)
+  auto team_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "r"(team_threads) : "memory"); };
+
+  // The turns of a team: (unit, g) for g = 0 .. groups - 1, unit after unit.  This warp walks worker g W + k_of of row `row_of`
+  // of the unit's rows, where there is one.
+  const int row_of = h.rows > 1 ? tw / K : 0, k_of = h.rows > 1 ? tw - row_of * K : tw;
+  const uint32_t stride = gridDim.x * (uint32_t)h.teams;
+  struct Turn { uint32_t unit; int g; };
+  auto after = [&](Turn t) {
+    if (++t.g == h.groups) { t.g = 0; t.unit += stride; }
+    return t;
+  };
+  auto row_at = [&](Turn t) { return t.unit * (uint32_t)h.rows + (uint32_t)row_of; };
+  auto works = [&](Turn t) { return t.unit < h.units && t.g * W + k_of < K && row_of < h.rows && row_at(t) < h.total_rows; };
+  auto ask_bucket = [&](Turn t) {
+    BucketAhead n{0u, 0u};
+    if (works(t)) {
+      const size_t kb = (size_t)(t.g * W + k_of) * a.nb + row_place<G>(a, h, row_at(t), lane).b;
+      n.nbits = a.bucket_bits[kb];
+      n.off = a.offsets[kb];
+    }
+    return n;
+  };
+  auto ask = [&](Turn t, const BucketAhead& n) {
+    HeaderAhead r{};
+    if (works(t)) r = ask_header<G>(a, h, row_at(t), t.g * W + k_of, n, lane);
+    return r;
+  };
+  Turn now{blockIdx.x + gridDim.x * (uint32_t)team, 0};
+  SubBlockAt at{};
+  BucketAhead next_bucket = ask_bucket(after(now));
+  {
+    const BucketAhead n = ask_bucket(now);
+    const HeaderAhead ha = ask(now, n);
+    if (works(now)) at = find_row<G>(a, h, row_at(now), now.g * W + k_of, n, ha, lane, row_sa);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  // this thread's quads of a row: q = tt + j team_threads, of sub-block q / kWords
+  const uint32_t sub0 = (uint32_t)tt / (uint32_t)kWords, sub_step = (uint32_t)team_threads / (uint32_t)kWords;
+  const uint32_t quads_at = team_sym + 4u * ((uint32_t)tt + sub0);     // a sub-block's words are followed by one that is not used
+  bool bad = false;
+  double sq0 = 0.0, sq1 = 0.0;
+  uint64_t acc[QT][2];
+  while (now.unit < h.units) {
+    const Turn next = after(now);
+    const HeaderAhead next_header = ask(next, next_bucket);
+    const BucketAhead later_bucket = ask_bucket(after(next));
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    if (works(now)) {
+      uint32_t used = 0;
+      auto walk = [&](auto w, auto p) {
+        w.open(p, at.sh);
+        if (at.count == G) walk_whole<G>(w, my_sym, wt);
+        else walk_some(w, at.count, my_sym, wt);
+        used = w.taken(p, at.sh);
+      };
+      if (__all_sync(0xffffffffu, at.staged != 0u)) walk(Walk<true>(), at.staged);
+      else walk(Walk<false>(), at.p);
+      if (at.count > 0) bad = bad || !at.ok || used != at.want;         // every sub-block uses exactly its length
+      s_norm[32 * tw + lane] = at.norm;
+      if (kCompare) s_norm_kept[32 * tw + lane] = a.norms_prev[(size_t)(now.g * W + k_of) * a.nb + row_place<G>(a, h, row_at(now), lane).b];
+      __syncwarp();                                                    // the staged words are no longer read
+    }
+    if (works(next)) at = find_row<G>(a, h, row_at(next), next.g * W + k_of, next_bucket, next_header, lane, row_sa);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    next_bucket = later_bucket;
+    team_sync();
+
+    // the ordered sums of this turn's workers
+    const int nk = min(K - now.g * W, h.rows > 1 ? K : W);
+    for (int r = 0; r < h.rows; ++r) {
+      const uint32_t row = now.unit * (uint32_t)h.rows + (uint32_t)r;
+      if (row >= h.total_rows) break;
+#pragma unroll
+      for (int j = 0; j < QT; ++j) {
+        const uint32_t q = (uint32_t)(j * team_threads + tt);
+        const size_t e0 = (size_t)row * (size_t)(32 * G) + 4u * q;
+        if (q >= (uint32_t)kQuads || e0 >= a.d) continue;
+        const int nv = a.d - e0 >= 4 ? 4 : (int)(a.d - e0);
+        if (now.g == 0) acc[j][0] = acc[j][1] = 0ull;
+        const uint32_t sub = sub0 + (uint32_t)j * sub_step;
+        const uint32_t sym_at = quads_at + (uint32_t)(r * K) * sym_row_bytes<G>() + 4u * (uint32_t)j * ((uint32_t)team_threads + sub_step);
+        const float* norm = s_norm + 32 * (r * K) + sub;
+        const float* norm_kept = s_norm_kept + 32 * (r * K) + sub;
+        const size_t kept_at = (size_t)(now.g * W) * a.sym_ld + e0;
+        const uint32_t valid = nv == 4 ? 0xffffffffu : (1u << (8 * nv)) - 1u;   // symbol 0 is the value 0, in both vectors
+        auto add = [&](uint32_t word, uint32_t was, int kk) {          // worker g W + kk
+          const float nrm = norm[32 * kk];
+          const uint64_t n2 = pack2(nrm, nrm);
+          auto value = [&](uint32_t w, int i, uint32_t base) { return __uint_as_float(lds_table32(__dp4a(w, 4u << (8 * i), base))); };
+          const uint64_t v01 = mul2(pack2(value(word, 0, val_sa), value(word, 1, val_sa)), n2, h.minus_zero);
+          const uint64_t v23 = mul2(pack2(value(word, 2, val_sa), value(word, 3, val_sa)), n2, h.minus_zero);
+          acc[j][0] = add2(acc[j][0], v01);
+          acc[j][1] = add2(acc[j][1], v23);
+          if (kCompare || kSquare) {
+            float dlt[4];
+            if (kCompare) {
+              const float nrm_kept = norm_kept[32 * kk];
+              const uint64_t m2 = pack2(nrm_kept, nrm_kept);
+              const uint64_t p01 = mul2(pack2(value(was, 0, kept_sa), value(was, 1, kept_sa)), m2, h.minus_zero);
+              const uint64_t p23 = mul2(pack2(value(was, 2, kept_sa), value(was, 3, kept_sa)), m2, h.minus_zero);
+              unpack2(sub2(p01, v01), &dlt[0], &dlt[1]);
+              unpack2(sub2(p23, v23), &dlt[2], &dlt[3]);
+            } else {
+              unpack2(v01, &dlt[0], &dlt[1]);
+              unpack2(v23, &dlt[2], &dlt[3]);
+            }
+            sq0 = fma((double)dlt[0], (double)dlt[0], sq0);
+            sq1 = fma((double)dlt[1], (double)dlt[1], sq1);
+            sq0 = fma((double)dlt[2], (double)dlt[2], sq0);
+            sq1 = fma((double)dlt[3], (double)dlt[3], sq1);
+          }
+        };
+#pragma unroll 1
+        for (int k0 = 0; k0 < nk; k0 += kTurn) {
+          const uint32_t at_k0 = sym_at + (uint32_t)k0 * sym_row_bytes<G>();
+          const uint8_t* was_at = kCompare ? a.sym_prev + kept_at + (size_t)k0 * a.sym_ld : nullptr;
+          uint8_t* out = kStore ? a.sym_out + kept_at + (size_t)k0 * a.sym_ld : nullptr;
+          auto turn = [&](auto whole_tag) {                            // of kTurn workers, or of what is left
+            constexpr bool kWhole = decltype(whole_tag)::value;
+            uint32_t was[kTurn];
+#pragma unroll
+            for (int u = 0; u < kTurn; ++u) {
+              was[u] = 0u;
+              if (kCompare && (kWhole || k0 + u < nk)) was[u] = *reinterpret_cast<const uint32_t*>(was_at + (size_t)u * a.sym_ld) & valid;
+            }
+#pragma unroll
+            for (int u = 0; u < kTurn; ++u) {
+              if (!kWhole && k0 + u >= nk) break;
+              uint32_t word = lds32(at_k0 + (uint32_t)u * sym_row_bytes<G>());
+              if (kCompare || kSquare) word &= valid;
+              add(word, was[u], k0 + u);
+              if (kStore) *reinterpret_cast<uint32_t*>(out + (size_t)u * a.sym_ld) = word;
+            }
+          };
+          if (nk - k0 >= kTurn) turn(std::true_type());
+          else turn(std::false_type());
+        }
+        if (now.g + 1 < h.groups) continue;
+        float m[4];
+        unpack2(acc[j][0], &m[0], &m[1]);
+        unpack2(acc[j][1], &m[2], &m[3]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          m[i] = k_pow2 ? __fmul_rn(m[i], Kinv) : __fdiv_rn(m[i], Kf);
+          // bits that no codeword starts like left a NaN in their coordinate's sum (as a norm that is not finite does)
+          bad = bad || (i < nv && m[i] != m[i]);
+        }
+        if (nv == 4 && a.vec_out) {
+          *reinterpret_cast<float4*>(a.mean + e0) = make_float4(m[0], m[1], m[2], m[3]);
+          if (a.update != 0) {
+            const float4 x = *reinterpret_cast<const float4*>(a.xin + e0);
+            *reinterpret_cast<float4*>(a.xout + e0) = make_float4(__fsub_rn(x.x, __fmul_rn(gam, m[0])), __fsub_rn(x.y, __fmul_rn(gam, m[1])),
+                                                                  __fsub_rn(x.z, __fmul_rn(gam, m[2])), __fsub_rn(x.w, __fmul_rn(gam, m[3])));
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (i < nv) {
+              a.mean[e0 + i] = m[i];
+              if (a.update != 0) a.xout[e0 + i] = __fsub_rn(a.xin[e0 + i], __fmul_rn(gam, m[i]));
+            }
+          }
+        }
+      }
+    }
+    now = next;
+    team_sync();                                                       // the symbols may be overwritten
+  }
+  if (kCompare || kSquare) {
+    const double sq = warp_sum(sq0 + sq1);
+    if (lane == 0 && sq != 0.0) atomicAdd(a.sum_sq, sq);
+  }
+  if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
+}
+
+// ---- launch -----------------------------------------------------------------------------------
+template <int G>
+static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, const LevelTable& lt_kept, int sym_mode) {
+  DecodeShape h;
+  h.minus_zero = 0x8000000080000000ull;
+  h.spb = (uint32_t)(da.bucket / G);
+  const size_t subs = (da.d + G - 1) / G;
+  if (subs >= (1ull << 31)) return QGX_ERR_INVALID_ARG;
+  // n / spb for n < 2^31: with 2^(L - 1) < spb <= 2^L the multiplier, 2^(31 + L) / spb rounded up, is below 2^32 and off by at
+  // most spb / 2^(31 + L) of itself
+  int log2up = 1;
+  while ((1u << log2up) < h.spb) ++log2up;
+  h.spb_mul = (uint32_t)((1ull << (31 + log2up)) / h.spb + 1u);
+  h.spb_shift = (uint32_t)log2up - 1u;
+  h.whole_subs = (uint32_t)(da.d / G);
+  h.last_count = (uint32_t)(da.d % G);
+  h.hdr_bits = (uint32_t)kNormBits + 16u * h.spb;
+  h.hdr_bits_last = (uint32_t)kNormBits + 16u * (uint32_t)(subs - (da.nb - 1) * (size_t)h.spb);
+  h.total_rows = (uint32_t)((subs + 31) / 32);
+  // Shared memory: the pair table, small tables, then per warp the symbols of a row and room for its stream words: as many as
+  // any code can need, or what is left.
+  const int max_warps = kDecodeWarps<G>;
+  h.team_warps = 8;
+  h.rows = std::max(1, h.team_warps / da.K);
+  while (2 * h.team_warps <= max_warps && h.team_warps < da.K && (size_t)h.total_rows * 2 * (size_t)h.team_warps <= (size_t)c->num_sms * (size_t)max_warps) h.team_warps *= 2;
+  h.teams = max_warps / h.team_warps;
+  h.groups = (da.K + h.team_warps - 1) / h.team_warps;
+  h.units = (h.total_rows + (uint32_t)h.rows - 1u) / (uint32_t)h.rows;
+  const int warps = h.teams * h.team_warps;
+  h.pair_mask = (4u << pair_bits(ct.maxlen)) - 4u;
+  uint32_t at = 4u << pair_bits(ct.maxlen);
+  auto take = [&](uint32_t bytes) { const uint32_t was = at; at += (bytes + 15u) & ~15u; return was; };
+  h.off_val = take(4u * kSignedValues);
+  h.off_kept = take(4u * kSignedValues);
+  h.off_norm = take((uint32_t)warps * 128u);
+  h.off_norm_kept = take((uint32_t)warps * 128u);
+  h.off_sym = take((uint32_t)warps * sym_row_bytes<G>());
+  h.off_row = at;
+  const uint32_t worst = (uint32_t)(G * (ct.maxlen + 1) + 3 * 32 + WalkReach<G>::kWords + 8) & ~3u;
+  const uint32_t room = (224u * 1024u - at) / (uint32_t)(4 * warps) & ~3u;
+  h.row_words = std::min(worst, room);
+  const size_t smem = at + (size_t)warps * h.row_words * 4u;
+  const unsigned grid = (unsigned)std::min<size_t>((size_t)c->num_sms, h.units);
+  ScopedKernelTimer timer(c, QGX_KERNEL_DECODE);
+#define QGX_LAUNCH_D(SS)                                                                                  \
+  do {                                                                                                    \
+    allow_max_dynamic_smem((const void*)k_exchange_decode<G, SS>, c->device);                             \
+    k_exchange_decode<G, SS><<<grid, 32 * warps, smem, c->stream>>>(da, h, lt, lt_kept);                  \
+  } while (0)
+  switch (sym_mode) {
+    case 1: QGX_LAUNCH_D(1); break;
+    case 2: QGX_LAUNCH_D(2); break;
+    case 3: QGX_LAUNCH_D(3); break;
+    case 4: QGX_LAUNCH_D(4); break;
+    case 5: QGX_LAUNCH_D(5); break;
+    default: QGX_LAUNCH_D(0); break;
+  }
+#undef QGX_LAUNCH_D
+  count_launch(c);
+  return cuda_status(cudaGetLastError());
+}
+
+qgx_status launch_exchange_decode(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, const LevelTable& lt_kept,
+                                  int sym_mode) {
+  if (!ct.has_header || da.bucket % ct.G != 0) return QGX_ERR_INVALID_ARG;
+  switch (ct.G) {
+    case 32: return launch_decode_g<32>(c, da, ct, lt, lt_kept, sym_mode);
+    case 64: return launch_decode_g<64>(c, da, ct, lt, lt_kept, sym_mode);
+    case 128: return launch_decode_g<128>(c, da, ct, lt, lt_kept, sym_mode);
+    default: return QGX_ERR_INVALID_ARG;
+  }
+}
+
+}  // namespace qgx

@@ -1,6 +1,7 @@
 // Fused exchange: one pass over the dual vectors writes the compact streams (quantize + encode),
 // one pass over the streams writes the mean (decode + average).  Same streams, bit for bit, and
 // the same mean as qgx_quantize -> qgx_encode -> qgx_decode -> qgx_average.
+#include "qgx_decode.cuh"
 #include "qgx_encode.cuh"
 #include "qgx_small.cuh"
 
@@ -283,623 +284,12 @@ k_exchange_encode(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
 }  // namespace qgx
 
 
-namespace qgx {
-
-// ---- decode + average ------------------------------------------------------------------------
-// Decoder table of the fused path: index = the next maxlen + 1 stream bits (codeword, then the sign
-// bit of a nonzero level); entry = the signed level value and, in `len`, the bits consumed (bits 0..4) and the
-// symbol byte (bits 8..15).  Where no codeword starts like the index the value is NaN -- it stays in the running
-// sum of its coordinate, where the kernel looks for it -- and one bit is consumed so that the walk goes on.
-struct DecEntry {
-  float val;
-  uint32_t len;
-};
-
-struct DecodeArgs {
-  const uint32_t* stream;       // [K][cap_words]
-  size_t cap_words;
-  const uint32_t* bucket_bits;  // [K][nb]
-  const uint32_t* offsets;      // [K][nb]
-  size_t d;
-  int bucket;
-  int K;
-  size_t nb;
-  const DecEntry* lut;          // decoder table in global memory, 1 << (maxlen + 1) entries
-  float* mean;                  // [d]
-  // optional fused state update (the two axpy of Eq. Q-GenX)
-  int update;                   // 0 none, 1: xout = xin - gamma * mean, 2: xout = xin - mean
-  const float* xin;
-  float* xout;
-  const double* scalars;        // scalars[1] = gamma_t
-  bool vec_out;                 // d % 4 == 0 and mean, xin, xout 16-byte aligned: 128-bit stores
-  // small vectors: a thread decodes its sub-block of ONE worker and stores the values to values[K][d]; the
-  // ordered sum over the workers, the division and the state update follow in k_sum_workers
-  float* values;                // [K][d] or null
-  // large vectors: the walk alone (one worker per thread, VAL = false) writes every worker's symbol bytes to sym_out
-  // and the norms it read from the streams to norms_out; k_symbols_mean forms the ordered sums from them
-  float* norms_out;             // [K][nb] or null
-  // optional: keep the decoded symbols (1 byte per coordinate and worker) ...
-  // Symbol bytes are kept transposed, so that a warp's accesses coalesce: worker k, sub-block gs, coordinate i of the
-  // sub-block -> byte k * sym_ld + (gs / 32) * 32 * G + (i / 4) * 128 + (gs % 32) * 4 + i % 4.
-  uint8_t* sym_out;             // [K][sym_ld] or null
-  // ... or compare with the symbols and norms kept by the other exchange of the iteration:
-  // *sum_sq += sum_k ||vhat_k of that exchange - vhat_k of this one||^2 (fp32 differences, fp64 sum)
-  const uint8_t* sym_prev;      // [K][sym_ld] or null
-  size_t sym_ld;
-  const float* norms_prev;      // [K][nb]
-  double* sum_sq;
-  DevStatus* st;
-};
-
-constexpr int kDecThreads = 128;
-constexpr uint32_t kBadSymbol = 0x40u;      // symbol byte of an index that no codeword starts like (no level has bit 6)
-
-// Bits not yet consumed of one sub-block: a 64-bit window refilled 32 bits at a time.  The streams
-// of the fused path lie in the context's workspace, which extends past every bucket, so a read a
-// few words beyond a (corrupt) sub-block stays inside allocated memory.  SH: the words are read from the warp's
-// staged row by shared-memory loads (the address is a 32-bit shared address); otherwise from wherever p points.
-template <bool SH>
-struct Window {
-  using Addr = typename std::conditional<SH, uint32_t, const uint32_t*>::type;
-  Addr next;              // address of `ahead`
-  Addr first;             // address of the word that held the first bit
-  uint32_t lo, hi;
-  uint32_t ahead;         // the word after the window, fetched one refill early
-  int avail;
-  uint32_t sh0;
-  static __device__ __forceinline__ uint32_t word(uint32_t a) { return lds32(a); }
-  static __device__ __forceinline__ uint32_t word(const uint32_t* a) { return *a; }
-  static __device__ __forceinline__ Addr at(const uint32_t* p, std::true_type) { return smem_addr(p); }
-  static __device__ __forceinline__ Addr at(const uint32_t* p, std::false_type) { return p; }
-  static __device__ __forceinline__ uint32_t step(uint32_t a, int words) { return a + 4u * (uint32_t)words; }
-  static __device__ __forceinline__ const uint32_t* step(const uint32_t* a, int words) { return a + words; }
-  // p = address of the word that holds the first bit, sh = first bit within it
-  __device__ __forceinline__ void open(const uint32_t* p, uint32_t sh) {
-    first = at(p, std::integral_constant<bool, SH>());
-    const uint32_t w0 = word(first), w1 = word(step(first, 1)), w2 = word(step(first, 2));
-    lo = __funnelshift_r(w0, w1, sh);
-    hi = w1 >> sh;
-    avail = 64 - (int)sh;                               // the window ends on a word boundary
-    sh0 = sh;
-    ahead = w2;
-    next = step(first, 2);
-  }
-  __device__ __forceinline__ void refill() {            // needs avail <= 32
-    const uint32_t w = ahead;
-    next = step(next, 1);
-    ahead = word(next);                                 // not needed before the next refill
-    lo |= __funnelshift_lc(0u, w, (uint32_t)avail);     // w << avail, nothing when avail == 32
-    hi |= __funnelshift_lc(w, 0u, (uint32_t)avail);     // the bits of w that do not fit the low word
-    avail += 32;
-  }
-  __device__ __forceinline__ void skip(uint32_t n) {    // n < 32
-    lo = __funnelshift_r(lo, hi, n);
-    hi >>= n;
-    avail -= (int)n;
-  }
-  static __device__ __forceinline__ uint32_t words_from(uint32_t a, uint32_t b) { return (a - b) >> 2; }
-  static __device__ __forceinline__ uint32_t words_from(const uint32_t* a, const uint32_t* b) { return (uint32_t)(a - b); }
-  // bits consumed since open(): the words taken in so far, less what is still in the window
-  __device__ __forceinline__ uint32_t used() const { return 32u * words_from(next, first) - sh0 - (uint32_t)avail; }
-};
-
-// start of sub-block `s` (bits after the header) = sum of the 16-bit lengths before it; all lanes of
-// the warp share the bucket and hold consecutive sub-blocks
-__device__ __forceinline__ uint32_t header_sum_before_warp(const uint32_t* w, uint32_t warp_first, int lane) {
-  uint32_t before = 0;
-  for (uint32_t i = (uint32_t)lane; i < warp_first; i += 32) {
-    const uint32_t bit = kNormBits + 16u * i;
-    before += (w[bit >> 5] >> (bit & 31u)) & 0xffffu;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-  return before;
-}
-
-// where sub-block s of bucket (k, b) starts and how long it is; false if the bucket's numbers disagree
-__device__ __forceinline__ bool locate_subblock(const uint32_t* stream, size_t cap_words, const uint32_t* bucket_bits,
-                                                const uint32_t* offsets, size_t kb, uint32_t hdr_bits, uint32_t s,
-                                                bool exists, bool uniform, int lane, const uint32_t** words, float* norm,
-                                                uint32_t* start, uint32_t* want, uint32_t* row_before, uint32_t* row_bits) {
-  const uint32_t nbits = bucket_bits[kb];
-  const uint32_t off = offsets[kb];
-  const uint32_t* w = stream + off;
-  *words = w;
-  const bool ok = nbits >= hdr_bits && (size_t)off + ((nbits + 31) >> 5) <= cap_words;
-  uint32_t st = 0, len = 0;
-  float nm = 0.0f;
-  *row_before = 0;
-  *row_bits = 0;
-  if (ok) {
-    nm = __uint_as_float(w[0]);
-    if (uniform) {
-      const uint32_t bit = kNormBits + 16u * s;
-      len = exists ? ((w[bit >> 5] >> (bit & 31u)) & 0xffffu) : 0u;
-      const uint32_t incl = warp_incl_scan(len, lane);
-      const uint32_t before = header_sum_before_warp(w, s - (uint32_t)lane, lane);
-      st = before + incl - len;
-      *row_before = before;
-      *row_bits = __shfl_sync(0xffffffffu, incl, 31);
-    } else if (exists) {
-      for (uint32_t i = 0; i <= s; ++i) {
-        const uint32_t bit = kNormBits + 16u * i;
-        const uint32_t L = (w[bit >> 5] >> (bit & 31u)) & 0xffffu;
-        if (i < s) st += L; else len = L;
-      }
-    }
-  }
-  *norm = nm;
-  *start = hdr_bits + st;
-  *want = len;
-  return ok && (!exists || (hdr_bits + st + len <= nbits && nbits < (1u << 18) && len < (1u << 14)));
-}
-
-// One thread per sub-block, workers in the outer loop: the thread keeps all G running sums of its
-// sub-block in registers (fixed k order, so the mean is bit-identical to a sequential sum) and reads each
-// worker's sub-block once, front to back, so that every fetched sector is used up at once.  The next
-// worker's sub-block is located while the current one is decoded.
-struct SubBlockAt {
-  const uint32_t* p;      // word that holds the first bit: in the warp's staged row (shared memory) or in the stream
-  uint32_t sh;            // first bit within that word
-  uint32_t want;          // bits of the sub-block
-  float norm;
-  float norm_prev;        // norm of the same bucket in the other exchange (when comparing)
-  bool ok;
-  bool staged;            // p points into the warp's staged row
-};
-
-// Words that a thread may read past the first word of its sub-block: G symbols of at most 13 bits, the
-// partial first word and the two words fetched ahead.
-template <int G>
-struct DecodeReach { static constexpr int kWords = (G * 13) / 32 + 4; };
-
-// Locates sub-block s of bucket (k, b) and starts the asynchronous copy of the warp's row -- the stream words
-// of its 32 consecutive sub-blocks plus what a thread may read past them -- into `row` (shared memory, row_words
-// words).  A thread whose reads would leave the staged words reads the stream itself.  The copies belong to the
-// caller's next commit group.
-template <int G>
-__device__ __forceinline__ SubBlockAt find_subblock(const DecodeArgs& a, int k, size_t b, uint32_t hdr_bits, uint32_t s,
-                                                    bool exists, bool uniform, int lane, uint32_t* row, int row_words) {
-  SubBlockAt r;
-  const uint32_t* w;
-  uint32_t st, row_before, row_bits;
-  r.ok = locate_subblock(a.stream + (size_t)k * a.cap_words, a.cap_words, a.bucket_bits, a.offsets, (size_t)k * a.nb + b,
-                         hdr_bits, s, exists, uniform, lane, &w, &r.norm, &st, &r.want, &row_before, &row_bits);
-  // a bucket whose numbers disagree is reported, and its walk reads the start of the worker's stream instead
-  // (in range whatever the offsets say)
-  if (!r.ok) { st = 0; r.want = 0; r.norm = 0.0f; w = a.stream + (size_t)k * a.cap_words; }
-  r.p = w + (st >> 5);
-  r.sh = st & 31u;
-  // bucket-level validity is the same for all lanes; the lengths are bounded, so the row is at most 2^19 bits
-  const bool stage = uniform && __all_sync(0xffffffffu, r.ok) && row_bits < (1u << 19);
-  r.staged = false;
-  if (stage) {
-    const size_t first = (size_t)(w - a.stream) + ((hdr_bits + row_before) >> 5);       // word index in the whole buffer
-    const size_t first_al = first & ~(size_t)3;                                          // 16-byte aligned
-    const size_t last = (size_t)(w - a.stream) + ((hdr_bits + row_before + row_bits + 31u) >> 5) + DecodeReach<G>::kWords;
-    const int nwords = (int)min((size_t)row_words, ((last - first_al) + 3) & ~(size_t)3);   // the buffer ends 64 words after the streams
-    for (int c = lane; c < nwords / 4; c += 32) {
-      const unsigned sa = (unsigned)__cvta_generic_to_shared(row + 4 * c);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(a.stream + first_al + 4 * (size_t)c) : "memory");
-    }
-    const size_t mine = (size_t)(r.p - a.stream) - first_al;
-    if (mine + DecodeReach<G>::kWords <= (size_t)nwords) { r.p = row + mine; r.staged = true; }
-  }
-  r.norm_prev = a.norms_prev ? a.norms_prev[(size_t)k * a.nb + b] : 0.0f;
-  return r;
-}
-
-// Copies one row of kept symbol words (kWords words, contiguous, 16-byte aligned) into shared memory without
-// waiting; the copies belong to the caller's next commit group.
-template <int kWords>
-__device__ __forceinline__ void stage_symbol_row(uint32_t* dst, const uint8_t* src, int lane) {
-#pragma unroll
-  for (int c = lane; c < kWords / 4; c += 32) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + 4 * c);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(src + 16 * (size_t)c) : "memory");
-  }
-}
-
-// shared memory of the decode kernel after its table: per warp two stream rows and (when comparing) two symbol rows --
-// one of each when a thread walks a single worker and nothing is fetched a worker ahead (VAL = false)
-template <int G, int SYM, bool VAL>
-struct DecodeSmem {
-  static constexpr int kStreamRow = 9 * G + 64;         // words, a multiple of 4
-  static constexpr int kBufs = VAL ? 2 : 1;
-  static constexpr size_t kBytes = sizeof(uint32_t) * kBufs * (128 / 32) * (size_t)(kStreamRow + ((SYM & 2) ? G * 8 : 0));
-};
-
-// SYM, a set of bits: 1 keeps the decoded symbols; 2 adds the squared differences between the vectors kept by an
-// earlier exchange (whose level table is `lt`) and the ones decoded now to *sum_sq; 4 adds the squared decoded values
-// themselves (an earlier vector of zero).  1 | 2 compares first and then overwrites the kept symbols in place.
-// VAL = false: the walk alone, one worker per thread -- no running sums, so half the registers and twice the warps;
-// symbols always go to a.sym_out, the norms read from the streams to a.norms_out.
-template <int G, int SYM, bool VAL>
-__global__ void __launch_bounds__(kDecThreads, VAL ? (G == 128 ? 3 : (G == 64 ? 4 : 6)) : 10) k_exchange_decode(const __grid_constant__ DecodeArgs a,
-                                                                      const __grid_constant__ CodeTable ct,
-                                                                      const __grid_constant__ LevelTable lt) {
-  constexpr bool kStore = (SYM & 1) != 0 || !VAL, kCompare = VAL && (SYM & 2) != 0, kSquare = VAL && (SYM & 4) != 0;
-  constexpr int kBufs = DecodeSmem<G, SYM, VAL>::kBufs;
-  extern __shared__ __align__(16) unsigned char s_raw[];
-  __shared__ float s_lev[QGX_MAX_LEVELS];            // the table of the kept symbols (comparing)
-  // comparing: the kept symbol words of the warp's 32 sub-blocks, one worker ahead (asynchronous copies)
-  constexpr int kRowWords = G * 8;                      // 32 sub-blocks x G bytes
-  // the stream words of the warp's 32 sub-blocks, one worker ahead (asynchronous copies): room for 8 bits per
-  // symbol and sign on average; longer rows are partly read from the stream itself
-  constexpr int kStreamRow = DecodeSmem<G, SYM, VAL>::kStreamRow;
-  const int lut_n = 2 << ct.maxlen;
-  // dynamic shared memory: table, stream rows, symbol rows.  The walk alone needs only the entries' second word
-  // (bits consumed, symbol byte).
-  DecEntry* s_lut = reinterpret_cast<DecEntry*>(s_raw);
-  uint32_t* s_len = reinterpret_cast<uint32_t*>(s_raw);
-  uint32_t* s_rows = reinterpret_cast<uint32_t*>(s_raw + (VAL ? sizeof(DecEntry) : sizeof(uint32_t)) * (size_t)lut_n);
-  uint32_t* s_prev = s_rows + kBufs * (kDecThreads / 32) * kStreamRow;
-  {
-    const uint2* src = reinterpret_cast<const uint2*>(a.lut);
-    uint2* dst = reinterpret_cast<uint2*>(s_lut);
-    for (int i = threadIdx.x; i < lut_n; i += blockDim.x) {
-      if constexpr (VAL) dst[i] = src[i];
-      else s_len[i] = src[i].y;
-    }
-  }
-  if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 0.0f;
-  __syncthreads();
-  const uint32_t mask = (uint32_t)lut_n - 1u;
-  const int lane = threadIdx.x & 31, tid = threadIdx.x;
-  const size_t spb = (size_t)a.bucket / G;
-  const size_t total_sub = a.nb * spb;
-  const bool uniform = (spb % 32 == 0);
-  const float Kf = (float)a.K;
-  // the mean is sum / K, one fp32 division; for K a power of two the product with 1 / K is the same number
-  const bool k_pow2 = (a.K & (a.K - 1)) == 0;
-  const float Kinv = 1.0f / Kf;
-  bool bad = false;
-  double sq = 0.0;
-
-  const bool wide = !VAL || a.values != nullptr;
-  const size_t sub_pad = (total_sub + 31) & ~(size_t)31;                // whole warps per worker
-  const size_t items = wide ? sub_pad * (size_t)a.K : total_sub;
-  for (size_t item = (size_t)blockIdx.x * blockDim.x + tid; item - lane < items; item += (size_t)gridDim.x * blockDim.x) {
-    const size_t gs = wide ? item % sub_pad : item;                      // the sub-block
-    const int kbeg = wide ? (int)(item / sub_pad) : 0, kend = wide ? kbeg + 1 : a.K;
-    const bool live = gs < total_sub;
-    const size_t b = live ? gs / spb : a.nb - 1;
-    const uint32_t s = live ? (uint32_t)(gs % spb) : 0u;
-    const size_t lo = b * (size_t)a.bucket;
-    const int len = (int)min((size_t)a.bucket, a.d - lo);
-    const int first = (int)s * G;
-    const int count = live ? max(0, min(G, len - first)) : 0;
-    const uint32_t nsub = (uint32_t)((len + G - 1) / G);
-    const uint32_t hdr_bits = kNormBits + 16u * nsub;
-    if (!__any_sync(0xffffffffu, count > 0)) continue;   // beyond the end of a short last bucket
-    const size_t e0 = lo + (size_t)first;
-    const size_t sbase = (gs >> 5) * (size_t)(32 * G) + (size_t)(gs & 31) * 4;   // see DecodeArgs::sym_out
-
-    float acc[VAL ? G : 1];
-#pragma unroll
-    for (int i = 0; i < (VAL ? G : 1); ++i) acc[i] = 0.0f;
-    uint32_t* my_rows = s_prev + (kCompare ? (tid >> 5) * kBufs * kRowWords : 0);
-    uint32_t* my_stream = s_rows + (tid >> 5) * kBufs * kStreamRow;
-    __syncwarp();                                         // the previous sub-block's rows are no longer read
-    SubBlockAt nxt = find_subblock<G>(a, kbeg, b, hdr_bits, s, count > 0, uniform, lane, my_stream + (kbeg & (kBufs - 1)) * kStreamRow, kStreamRow);
-    if (kCompare)
-      stage_symbol_row<kRowWords>(my_rows + (kbeg & (kBufs - 1)) * kRowWords, a.sym_prev + (size_t)kbeg * a.sym_ld + (gs >> 5) * (size_t)(32 * G), lane);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    for (int k = kbeg; k < kend; ++k) {
-      const SubBlockAt cur = nxt;
-      const uint32_t* prev_row = my_rows + (k & (kBufs - 1)) * kRowWords + lane;
-      __syncwarp();                                       // every lane is done with the rows that are overwritten next
-      if (k + 1 < kend) {
-        nxt = find_subblock<G>(a, k + 1, b, hdr_bits, s, count > 0, uniform, lane, my_stream + ((k + 1) & (kBufs - 1)) * kStreamRow, kStreamRow);
-        if (kCompare)
-          stage_symbol_row<kRowWords>(my_rows + ((k + 1) & (kBufs - 1)) * kRowWords,
-                                      a.sym_prev + (size_t)(k + 1) * a.sym_ld + (gs >> 5) * (size_t)(32 * G), lane);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");       // one group per worker, empty after the last
-      asm volatile("cp.async.wait_group 1;" ::: "memory");       // worker k's rows have landed
-      __syncwarp();
-      bad = bad || !cur.ok;
-      uint32_t used = 0;
-      // the walk over the sub-block's symbols, with the window's words read from the staged row (every lane's
-      // words are there) or from wherever they are
-      auto walk = [&](auto shared_tag) {
-        Window<decltype(shared_tag)::value> win;
-        win.open(cur.p, cur.sh);
-        if (count == G) {
-          uint32_t pack = 0, prev4 = 0;
-#pragma unroll
-          for (int i = 0; i < G; ++i) {
-            if ((i & 1) == 0) {                              // two symbols use at most 26 bits
-              if (win.avail <= 32) win.refill();
-            }
-            if (kCompare && (i & 3) == 0) prev4 = prev_row[(i >> 2) * 32];
-            DecEntry e;
-            if constexpr (VAL) e = s_lut[win.lo & mask];
-            else { e.len = s_len[win.lo & mask]; e.val = 0.0f; }
-            win.skip(e.len & 31u);
-            const float val = __fmul_rn(cur.norm, e.val);
-            if constexpr (VAL) acc[i] = __fadd_rn(acc[i], val);
-            if (kCompare) {
-              const float dlt = __fsub_rn(dequantize_symbol((prev4 >> (8 * (i & 3))) & 0xffu, cur.norm_prev, s_lev), val);
-              sq = fma((double)dlt, (double)dlt, sq);
-            }
-            if (kSquare) sq = fma((double)val, (double)val, sq);
-            if (kStore) {
-              // byte 1 of e.len, the symbol byte, becomes byte i % 4 of the word
-              pack = prmt(pack, e.len, (i & 3) == 0 ? 0x3215u : ((i & 3) == 1 ? 0x3250u : ((i & 3) == 2 ? 0x3510u : 0x5210u)));
-              if ((i & 3) == 3) *reinterpret_cast<uint32_t*>(a.sym_out + (size_t)k * a.sym_ld + sbase + (i >> 2) * 128) = pack;
-            }
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < G; ++i) {
-            if ((i & 1) == 0) {
-              if (win.avail <= 32) win.refill();
-            }
-            if (i < count) {
-              DecEntry e;
-              if constexpr (VAL) e = s_lut[win.lo & mask];
-              else { e.len = s_len[win.lo & mask]; e.val = 0.0f; }
-              win.skip(e.len & 31u);
-              const float val = __fmul_rn(cur.norm, e.val);
-              if constexpr (VAL) acc[i] = __fadd_rn(acc[i], val);
-              if (kCompare) {
-                const float dlt = __fsub_rn(dequantize_symbol(a.sym_prev[(size_t)k * a.sym_ld + sbase + (i >> 2) * 128 + (i & 3)], cur.norm_prev, s_lev), val);
-                sq = fma((double)dlt, (double)dlt, sq);
-              }
-              if (kSquare) sq = fma((double)val, (double)val, sq);
-              if (kStore) a.sym_out[(size_t)k * a.sym_ld + sbase + (i >> 2) * 128 + (i & 3)] = (uint8_t)((e.len >> 8) & 0xffu);
-            }
-          }
-        }
-        used = win.used();
-      };
-      if (__all_sync(0xffffffffu, cur.staged)) walk(std::true_type());
-      else walk(std::false_type());
-      bad = bad || (count > 0 && used != cur.want);          // every sub-block uses exactly its length
-    }
-    if (count <= 0) continue;
-    if constexpr (!VAL) {
-      if (s == 0) a.norms_out[(size_t)kbeg * a.nb + b] = nxt.norm;       // the bucket's norm as the stream gives it
-    } else {
-    {
-      // an index that no codeword starts like left a NaN in its coordinate's sum (as a norm that is not finite does)
-      bool marked = false;
-#pragma unroll
-      for (int i = 0; i < G; ++i) marked = marked || (acc[i] != acc[i]);
-      bad = bad || marked;
-    }
-    if (wide) {                                         // the worker's values; summed by k_sum_workers
-      float* out = a.values + (size_t)kbeg * a.d + e0;
-      if (count == G && a.vec_out) {
-#pragma unroll
-        for (int i = 0; i < G; i += 4) *reinterpret_cast<float4*>(out + i) = make_float4(acc[i], acc[i + 1], acc[i + 2], acc[i + 3]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < G; ++i)
-          if (i < count) out[i] = acc[i];
-      }
-      continue;
-    }
-
-    float gam = 1.0f;
-    if (a.update == 1) gam = (float)a.scalars[1];
-    if (count == G && a.vec_out) {
-      auto emit = [&](auto pow2_tag) {
-        auto mean_of = [&](float sum) { return decltype(pow2_tag)::value ? __fmul_rn(sum, Kinv) : __fdiv_rn(sum, Kf); };
-#pragma unroll
-        for (int i = 0; i < G; i += 4) {
-          const float4 m = make_float4(mean_of(acc[i]), mean_of(acc[i + 1]), mean_of(acc[i + 2]), mean_of(acc[i + 3]));
-          *reinterpret_cast<float4*>(a.mean + e0 + i) = m;
-          if (a.update != 0) {
-            const float4 x = *reinterpret_cast<const float4*>(a.xin + e0 + i);
-            const float g = a.update == 1 ? gam : 1.0f;      // update 2 subtracts the mean itself (1 * m is exact)
-            *reinterpret_cast<float4*>(a.xout + e0 + i) =
-                make_float4(__fsub_rn(x.x, __fmul_rn(g, m.x)), __fsub_rn(x.y, __fmul_rn(g, m.y)),
-                            __fsub_rn(x.z, __fmul_rn(g, m.z)), __fsub_rn(x.w, __fmul_rn(g, m.w)));
-          }
-        }
-      };
-      if (k_pow2) emit(std::true_type());
-      else emit(std::false_type());
-    } else {
-#pragma unroll
-      for (int i = 0; i < G; ++i) {
-        if (i < count) {
-          const float m = __fdiv_rn(acc[i], Kf);
-          a.mean[e0 + i] = m;
-          if (a.update == 1) a.xout[e0 + i] = __fsub_rn(a.xin[e0 + i], __fmul_rn(gam, m));
-          if (a.update == 2) a.xout[e0 + i] = __fsub_rn(a.xin[e0 + i], m);
-        }
-      }
-    }
-    }   // VAL
-  }
-  if (kCompare || kSquare) {
-    sq = warp_sum(sq);
-    if (lane == 0 && sq != 0.0) atomicAdd(a.sum_sq, sq);
-  }
-  if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
-}
-
-// The ordered sums of the two-pass decode: worker k's quantized coordinate is norm_k * (signed level of its symbol
-// byte), added in the order k = 0..K-1, divided by K, and the state update applied -- the same operations in the same
-// order as the one-pass kernel's.  A thread takes 16 consecutive coordinates of one sub-block (four symbol words per
-// worker; the transposed layout makes a warp's loads of one word index contiguous).  The signed level values sit in
-// shared memory once per lane (bank = lane), NaN for bytes that are no symbol: a NaN mean reports the stream.
-// SYM & 2: also adds sum_k ||vhat_k kept by the other exchange - vhat_k of this one||^2 to *sum_sq (fp32 differences,
-// fp64 sum; the kept symbols dequantized with their own table and norms); SYM & 4: sum_k ||vhat_k||^2 instead.
-struct MeanArgs {
-  const uint8_t* sym;           // [K][sym_ld], this exchange's symbol bytes (transposed layout of DecodeArgs::sym_out)
-  size_t sym_ld;
-  const float* norms;           // [K][nb], as the walk read them from the streams
-  const uint8_t* sym_prev;      // [K][sym_ld] or null
-  const float* norms_prev;      // [K][nb]
-  double* sum_sq;
-  int K;
-  size_t d;
-  int bucket;
-  size_t nb;
-  float* mean;
-  int update;
-  const float* xin;
-  float* xout;
-  const double* scalars;
-  bool vec_out;
-  DevStatus* st;
-};
-
-template <int G, int SYM>
-__global__ void __launch_bounds__(256) k_symbols_mean(const __grid_constant__ MeanArgs a, const __grid_constant__ LevelTable lt,
-                                                      const __grid_constant__ LevelTable lt_kept) {
-  constexpr bool kCompare = (SYM & 2) != 0, kSquare = (SYM & 4) != 0;
-  extern __shared__ __align__(16) float s_val[];                       // [256][32], then (comparing) the kept table [256]
-  for (int t = threadIdx.x; t < 256 * 32; t += blockDim.x) {
-    const int byte = t >> 5, idx = byte & 31;
-    const bool symbol = (byte & 0x60) == 0 && idx < lt.nlev && byte != 0x80;
-    s_val[t] = symbol ? ((byte & 0x80) ? -lt.lev[idx] : lt.lev[idx]) : __int_as_float(0x7fc00000);
-  }
-  if (kCompare) {
-    for (int t = threadIdx.x; t < 256; t += blockDim.x) {
-      const int idx = t & 31;
-      s_val[256 * 32 + t] = idx < lt_kept.nlev ? ((t & 0x80) ? -lt_kept.lev[idx] : lt_kept.lev[idx]) : 0.0f;
-    }
-  }
-  __syncthreads();
-  constexpr int kParts = G / 16;                                       // threads per sub-block
-  const uint32_t val_sa = smem_addr(s_val) + 4u * (threadIdx.x & 31u);
-  const uint32_t kept_sa = smem_addr(s_val + 256 * 32);
-  const size_t spb = (size_t)a.bucket / G, total_sub = a.nb * spb, rows = (total_sub + 31) / 32;
-  const int K = a.K;
-  const float Kf = (float)K, Kinv = 1.0f / Kf;
-  const bool k_pow2 = (K & (K - 1)) == 0;
-  const int lane = threadIdx.x & 31;
-  float gam = 1.0f;
-  if (a.update == 1) gam = (float)a.scalars[1];
-  bool bad = false;
-  double sq = 0.0;
-  const size_t ldw = a.sym_ld / 4;
-  const size_t items = rows * kParts * 32;
-  for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < items; t += (size_t)gridDim.x * blockDim.x) {
-    const size_t rest = t >> 5, row = rest / kParts;
-    const int part = (int)(rest % kParts);
-    const size_t gs = row * 32 + (size_t)lane;
-    if (gs >= total_sub) continue;
-    const size_t b = gs / spb, lo = b * (size_t)a.bucket;
-    const int len = (int)min((size_t)a.bucket, a.d - lo);
-    const int first = (int)(gs % spb) * G + 16 * part;                 // of this thread's coordinates, within the bucket
-    const int count = max(0, min(16, len - first));
-    if (count == 0) continue;
-    const size_t word0 = row * (size_t)(8 * G) + (size_t)(4 * part) * 32 + lane;
-    const uint32_t* words = reinterpret_cast<const uint32_t*>(a.sym) + word0;
-    const uint32_t* kept = kCompare ? reinterpret_cast<const uint32_t*>(a.sym_prev) + word0 : nullptr;
-    float acc[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
-    auto add = [&](const uint32_t (&w)[4], const uint32_t (&p)[4], float norm, float norm_kept) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint32_t byte = prmt(w[j], 0u, 0x4440u + (uint32_t)q);                 // byte q of the word
-          const float val = __fmul_rn(norm, __uint_as_float(lds_table32(val_sa + (byte << 7))));
-          acc[4 * j + q] = __fadd_rn(acc[4 * j + q], val);
-          if (kCompare) {
-            const uint32_t pbyte = prmt(p[j], 0u, 0x4440u + (uint32_t)q);
-            const float was = __fmul_rn(norm_kept, __uint_as_float(lds_table32(kept_sa + (pbyte << 2))));
-            const float dlt = __fsub_rn(was, val);
-            if (4 * j + q < count) sq = fma((double)dlt, (double)dlt, sq);
-          }
-          if (kSquare) { if (4 * j + q < count) sq = fma((double)val, (double)val, sq); }
-        }
-      }
-    };
-    // one worker's words and norms are asked for while the one before is added (k = K asks for nothing)
-    uint32_t w[4] = {0u, 0u, 0u, 0u}, p[4] = {0u, 0u, 0u, 0u};
-    float nrm = 0.0f, nrm_kept = 0.0f;
-    auto fetch = [&](int k, uint32_t (&fw)[4], uint32_t (&fp)[4], float* fn, float* fk) {
-      if (k >= K) return;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        fw[j] = __ldcs(words + (size_t)k * ldw + j * 32);
-        if (kCompare) fp[j] = __ldcs(kept + (size_t)k * ldw + j * 32);
-      }
-      *fn = a.norms[(size_t)k * a.nb + b];
-      if (kCompare) *fk = a.norms_prev[(size_t)k * a.nb + b];
-    };
-    fetch(0, w, p, &nrm, &nrm_kept);
-    for (int k = 0; k < K; k += 2) {
-      uint32_t w1[4] = {0u, 0u, 0u, 0u}, p1[4] = {0u, 0u, 0u, 0u};
-      float n1 = 0.0f, m1 = 0.0f;
-      fetch(k + 1, w1, p1, &n1, &m1);
-      add(w, p, nrm, nrm_kept);
-      fetch(k + 2, w, p, &nrm, &nrm_kept);
-      if (k + 1 < K) add(w1, p1, n1, m1);
-    }
-    const size_t e0 = lo + (size_t)first;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      float m[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        m[q] = k_pow2 ? __fmul_rn(acc[4 * j + q], Kinv) : __fdiv_rn(acc[4 * j + q], Kf);
-        bad = bad || (4 * j + q < count && m[q] != m[q]);
-      }
-      if (4 * j + 4 <= count && a.vec_out) {
-        *reinterpret_cast<float4*>(a.mean + e0 + 4 * j) = make_float4(m[0], m[1], m[2], m[3]);
-        if (a.update != 0) {
-          const float4 x = *reinterpret_cast<const float4*>(a.xin + e0 + 4 * j);
-          const float g = a.update == 1 ? gam : 1.0f;      // update 2 subtracts the mean itself (1 * m is exact)
-          *reinterpret_cast<float4*>(a.xout + e0 + 4 * j) =
-              make_float4(__fsub_rn(x.x, __fmul_rn(g, m[0])), __fsub_rn(x.y, __fmul_rn(g, m[1])),
-                          __fsub_rn(x.z, __fmul_rn(g, m[2])), __fsub_rn(x.w, __fmul_rn(g, m[3])));
-        }
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (4 * j + q < count) {
-            a.mean[e0 + 4 * j + q] = m[q];
-            if (a.update == 1) a.xout[e0 + 4 * j + q] = __fsub_rn(a.xin[e0 + 4 * j + q], __fmul_rn(gam, m[q]));
-            if (a.update == 2) a.xout[e0 + 4 * j + q] = __fsub_rn(a.xin[e0 + 4 * j + q], m[q]);
-          }
-        }
-      }
-    }
-  }
-  if (kCompare || kSquare) {
-    sq = warp_sum(sq);
-    if ((threadIdx.x & 31) == 0 && sq != 0.0) atomicAdd(a.sum_sq, sq);
-  }
-  if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
-}
-
-}  // namespace qgx
-
 // ---- host side ---------------------------------------------------------------------------------
 namespace qgx {
 
 // workspace slots of a context
 enum { WS_OFF64 = 0, WS_FLAGS = 1, WS_LUT = 2, WS_SLOT0 = 3 /* stream, bits, offsets, total: 3..6 and 7..10 */,
-       WS_NORMS = 12, WS_SYM = 13, WS_NORMS2 = 14, WS_OPVAL = 15, WS_MEAN = 16, WS_DLUT = 18, WS_SEGBITS = 19, WS_VALUES = 20, WS_SYMTMP = 21, WS_NORMSDEC = 22, WS_SMALL = 23 };
-
-// Small vectors, second part: mean_i = (((0 + v_{0,i}) + v_{1,i}) + ...) / K in worker order (the same sequential
-// sum as in the fused decode pass), then the optional state update.
-__global__ void __launch_bounds__(256) k_sum_workers(const float* __restrict__ values, int K, size_t d, float* __restrict__ mean,
-                                                     int update, const float* xin, float* xout, const double* scalars) {
-  const float Kf = (float)K;
-  const float gam = update == 1 ? (float)scalars[1] : 1.0f;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (size_t)gridDim.x * blockDim.x) {
-    float acc = 0.0f;
-    for (int k = 0; k < K; ++k) acc = __fadd_rn(acc, values[(size_t)k * d + i]);
-    const float m = __fdiv_rn(acc, Kf);
-    mean[i] = m;
-    if (update == 1) xout[i] = __fsub_rn(xin[i], __fmul_rn(gam, m));
-    if (update == 2) xout[i] = __fsub_rn(xin[i], m);
-  }
-}
-
-qgx_status launch_decode_average(qgx_ctx* c, const DecodeArgs& args, const CodeTable& ct, const LevelTable& lt, int sym_mode);
-qgx_status launch_decode_walk(qgx_ctx* c, const DecodeArgs& args, const CodeTable& ct, const LevelTable& lt);
+       WS_NORMS = 12, WS_SYM = 13, WS_NORMS2 = 14, WS_OPVAL = 15, WS_MEAN = 16, WS_SEGBITS = 19, WS_SMALL = 23 };
 
 // ---- what a call derives from a quantizer configuration, kept between calls --------------------
 // Building the rounding table, the code table and the decoder table and copying the latter to the device costs
@@ -912,7 +302,7 @@ struct CachedTables {
   qgx_codebook cb;
   CodeTable ct;
   RoundTable rt;
-  DecEntry* lut_dev;                    // 2 * kDecLutMax entries, owned
+  DecodeTables* dec_dev;                // owned; built by k_build_decode_tables
   EncodeTables* enc_dev;                // owned; built by k_build_encode_tables
 };
 constexpr int kTableCacheSlots = 32;
@@ -920,8 +310,6 @@ struct LaunchShape { size_t smem; int per_sm; };      // smem == 0: not asked ye
 struct TableCache {
   CachedTables e[kTableCacheSlots];
   LaunchShape enc[3][3];                // [octets per thread 1, 2, 4][sub-block 32, 64, 128]
-  LaunchShape dec[3][6];                // [sub-block][symbol mode]
-  LaunchShape dec_walk[3];              // the walk alone
 };
 
 // Lets a kernel use all the dynamic shared memory that the device allows, once per kernel and device.  (The
@@ -949,7 +337,7 @@ void free_table_cache(qgx_ctx* c) {
   TableCache* tc = (TableCache*)c->table_cache;
   if (!tc) return;
   for (int i = 0; i < kTableCacheSlots; ++i) {
-    if (tc->e[i].lut_dev) cudaFree(tc->e[i].lut_dev);
+    if (tc->e[i].dec_dev) cudaFree(tc->e[i].dec_dev);
     if (tc->e[i].enc_dev) cudaFree(tc->e[i].enc_dev);
   }
   delete tc;
@@ -983,30 +371,14 @@ static qgx_status cached_tables(qgx_ctx* c, const qgx_quant_cfg* cfg, const Cach
     qgx_status rc = make_code_table(&cfg->cb, cfg->bucket, &e->ct);
     if (rc != QGX_OK) return rc;
     make_round_table(cfg->levels, cfg->nlev, &e->rt);
-    if (!e->lut_dev && cudaMalloc((void**)&e->lut_dev, sizeof(DecEntry) * (size_t)(2 * kDecLutMax)) != cudaSuccess) {
+    // both sides' tables are built on the device, stream-ordered after the kernels that still read this slot's previous ones
+    if (!e->dec_dev && cudaMalloc((void**)&e->dec_dev, sizeof(DecodeTables)) != cudaSuccess) {
       cudaGetLastError();
-      e->lut_dev = nullptr;
+      e->dec_dev = nullptr;
       return QGX_ERR_CUDA;
     }
-    // decoder table: the next maxlen + 1 bits -> signed level value and bits consumed
-    const CodeTable& ct = e->ct;
-    std::vector<uint16_t> by_code((size_t)1 << ct.maxlen);
-    build_dec_lut_host(ct, by_code.data());
-    std::vector<DecEntry> h_lut((size_t)2 << ct.maxlen);
-    for (size_t i = 0; i < h_lut.size(); ++i) {
-      const uint16_t w = by_code[i & (((size_t)1 << ct.maxlen) - 1)];
-      const uint32_t L = w >> 8, idx = w & 0xffu;
-      if (L == 0) { h_lut[i].val = std::numeric_limits<float>::quiet_NaN(); h_lut[i].len = 1u | (kBadSymbol << 8); continue; }   // no codeword starts like this
-      if (idx == 0) { h_lut[i].val = 0.0f; h_lut[i].len = L; continue; }       // symbol byte 0
-      const bool neg = (i >> L) & 1u;
-      h_lut[i].val = neg ? -cfg->levels[idx] : cfg->levels[idx];
-      h_lut[i].len = (L + 1u) | ((idx | (neg ? 0x80u : 0u)) << 8);       // bits 8..15: the symbol byte
-    }
-    // stream-ordered after the kernels that still read this slot's previous table; the source is pageable, so
-    // the call returns once it has been staged
-    if (cudaMemcpyAsync(e->lut_dev, h_lut.data(), h_lut.size() * sizeof(DecEntry), cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
-      return QGX_ERR_CUDA;
-    // the encoder's tables, built on the device by the routines that the kernels would run themselves
+    launch_build_decode_tables(e->ct, e->dec_dev, c->stream);
+    count_launch(c);
     if (!e->enc_dev && cudaMalloc((void**)&e->enc_dev, sizeof(EncodeTables)) != cudaSuccess) {
       cudaGetLastError();
       e->enc_dev = nullptr;
@@ -1047,17 +419,17 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   for (int j = 0; j < QGX_MAX_LEVELS; ++j) lt.lev[j] = j < cfg->nlev ? cfg->levels[j] : 1.0f;
 
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
-  const size_t cap = qgx_stream_capacity_words(d, bucket, cfg->cb.subblock, QGX_MAX_CODE_LEN);   // fits any codebook
+  // fits any codebook; a worker's words start on 16 bytes
+  const size_t cap = (qgx_stream_capacity_words(d, bucket, cfg->cb.subblock, QGX_MAX_CODE_LEN) + 3) & ~(size_t)3;
   const int base = WS_SLOT0 + 4 * slot;
-  uint32_t* stream = (uint32_t*)ws_get(c, base + 0, sizeof(uint32_t) * ((size_t)K * cap + 64));   // slack: see Window
+  uint32_t* stream = (uint32_t*)ws_get(c, base + 0, sizeof(uint32_t) * ((size_t)K * cap + 64));   // slack: see WalkReach
   uint32_t* bbits = (uint32_t*)ws_get(c, base + 1, sizeof(uint32_t) * (size_t)K * nb);
   uint32_t* offs = (uint32_t*)ws_get(c, base + 2, sizeof(uint32_t) * (size_t)K * nb);
   // one block per slot, zeroed by one memset: the per-worker bit totals, the ticket counter, the status words of the scan
   unsigned long long* tot = (unsigned long long*)ws_get(c, base + 3, sizeof(uint64_t) * ((size_t)K + 2 + (size_t)K * (nb + 1)));
   unsigned long long* status = tot ? tot + K + 2 : nullptr;
   float* norms = (float*)ws_get(c, slot == 0 ? WS_NORMS : WS_NORMS2, sizeof(float) * (size_t)K * nb);
-  const DecEntry* lut = tables->lut_dev;
-  if (!stream || !bbits || !offs || !tot || !status || !norms || !lut) return QGX_ERR_CUDA;
+    if (!stream || !bbits || !offs || !tot || !status || !norms) return QGX_ERR_CUDA;
   c->slot_cap_words[slot] = cap;
   c->slot_K[slot] = K;
   c->slot_nb[slot] = nb;
@@ -1073,7 +445,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   ea.status = status; ea.ticket = reinterpret_cast<unsigned int*>(tot + K); ea.st = c->dstatus; ea.tables = tables->enc_dev;
   uint8_t* sym_out = nullptr;
   const uint8_t* sym_prev = nullptr;
-  const size_t sym_ld = ((nb * (size_t)(bucket / ct.G) + 31) / 32) * 32 * (size_t)ct.G;   // see DecodeArgs::sym_out
+  const size_t sym_ld = (d + 15) & ~(size_t)15;             // see DecodeArgs::sym_out
   const float* norms_prev = nullptr;
   if (sym_mode < 0 || sym_mode > 5) return QGX_ERR_INVALID_ARG;
   if ((sym_mode & 6) && !sum_sq) return QGX_ERR_INVALID_ARG;
@@ -1088,7 +460,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   if (sym_mode & 1) {
     sym_out = (uint8_t*)ws_get(c, WS_SYM, (size_t)K * sym_ld + 16);
     if (!sym_out) return QGX_ERR_CUDA;
-    c->sym_slot = slot; c->sym_K = K; c->sym_d = d; c->sym_ld = sym_ld; c->sym_bucket = bucket; c->sym_G = ct.G;
+    c->sym_slot = slot; c->sym_K = K; c->sym_d = d; c->sym_ld = sym_ld;
     c->sym_nlev = cfg->nlev;
     for (int j = 0; j < cfg->nlev; ++j) c->sym_levels[j] = cfg->levels[j];
   }
@@ -1109,7 +481,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     es.spin_limit = c->wait_limit;
     SmallArgs sm;
     std::memset(&sm, 0, sizeof(sm));
-    sm.lut_len = reinterpret_cast<const uint32_t*>(lut) + 1;
+    sm.tables = tables->dec_dev;
     sm.mean = mean_out;
     sm.update = upd ? upd->mode : 0; sm.xin = upd ? upd->xin : nullptr; sm.xout = upd ? upd->xout : nullptr; sm.scalars = upd ? upd->scalars : nullptr;
     sm.sym_out = sym_out; sm.sym_prev = sym_prev; sm.sym_ld = sym_ld; sm.norms_prev = norms_prev;
@@ -1187,125 +559,12 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   DecodeArgs da;
   da.stream = stream; da.cap_words = cap; da.bucket_bits = bbits; da.offsets = offs;
   da.sym_out = sym_out; da.sym_prev = sym_prev; da.sym_ld = sym_ld; da.norms_prev = norms_prev; da.sum_sq = sum_sq;
-  da.d = d; da.bucket = bucket; da.K = K; da.nb = nb; da.lut = lut; da.mean = mean_out;
+  da.d = d; da.bucket = bucket; da.K = K; da.nb = nb; da.tables = tables->dec_dev; da.mean = mean_out;
   da.update = upd ? upd->mode : 0; da.xin = upd ? upd->xin : nullptr; da.xout = upd ? upd->xout : nullptr;
   da.scalars = upd ? upd->scalars : nullptr; da.st = c->dstatus;
-  da.vec_out = (d % kQuad == 0) && ((reinterpret_cast<uintptr_t>(mean_out) & 15u) == 0) &&
-               ((reinterpret_cast<uintptr_t>(da.xin) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(da.xout) & 15u) == 0);
-  // Small vectors leave most of the GPU idle and make every thread walk all K workers one after the other: there
-  // the decode pass runs one worker per thread and a second kernel forms the ordered sums.
-  const size_t total_sub = nb * (size_t)(bucket / ct.G);
-  da.values = nullptr;
-  const bool fits = (size_t)K * d * sizeof(float) <= ((size_t)256 << 20);
-  const bool small = total_sub * 2 < (size_t)c->num_sms * kDecThreads * 4;
-  if (K > 1 && fits && c->decode_split != QGX_SPLIT_NEVER && c->decode_split != QGX_SPLIT_SYMBOLS && (small || c->decode_split == QGX_SPLIT_ALWAYS)) {
-    da.values = (float*)ws_get(c, WS_VALUES, sizeof(float) * (size_t)K * d);
-    if (!da.values) return QGX_ERR_CUDA;
-  }
-  // On request: the walk alone with one worker per thread (twice the warps of the one-pass kernel, whose 64 running
-  // sums per thread fill the register file), every worker's symbol bytes kept, and the ordered sums from those.
-  da.norms_out = nullptr;
-  const bool in_place = (sym_mode & 3) == 3;             // compares with the kept symbols and overwrites them: one pass
-  const bool two_pass = K > 1 && !da.values && !in_place && c->decode_split == QGX_SPLIT_SYMBOLS;
-  if (two_pass) {
-    if (!da.sym_out) da.sym_out = (uint8_t*)ws_get(c, WS_SYMTMP, (size_t)K * sym_ld);
-    da.norms_out = (float*)ws_get(c, WS_NORMSDEC, sizeof(float) * (size_t)K * nb);
-    if (!da.sym_out || !da.norms_out) return QGX_ERR_CUDA;
-    rc = launch_decode_walk(c, da, ct, lt_kept);
-    if (rc != QGX_OK) return rc;
-    MeanArgs ma;
-    ma.sym = da.sym_out; ma.sym_ld = sym_ld; ma.norms = da.norms_out; ma.sym_prev = da.sym_prev; ma.norms_prev = da.norms_prev;
-    ma.sum_sq = da.sum_sq; ma.K = K; ma.d = d; ma.bucket = bucket; ma.nb = nb; ma.mean = mean_out; ma.update = da.update;
-    ma.xin = da.xin; ma.xout = da.xout; ma.scalars = da.scalars; ma.vec_out = da.vec_out; ma.st = c->dstatus;
-    {
-      ScopedKernelTimer timer(c, QGX_KERNEL_DECODE);
-      const size_t rows = (total_sub + 31) / 32;
-      const size_t threads = rows * (size_t)(ct.G / 16) * 32;
-      const unsigned grid = (unsigned)std::max<size_t>(1, std::min<size_t>((threads + 255) / 256, (size_t)c->num_sms * 6));
-      const size_t smem = sizeof(float) * (256 * 32 + 256);
-#define QGX_LAUNCH_M(GG, SS) k_symbols_mean<GG, SS><<<grid, 256, smem, c->stream>>>(ma, lt, lt_kept)
-#define QGX_LAUNCH_MG(GG)                                  \
-  do {                                                     \
-    if (sym_mode & 2) QGX_LAUNCH_M(GG, 2);                 \
-    else if (sym_mode & 4) QGX_LAUNCH_M(GG, 4);            \
-    else QGX_LAUNCH_M(GG, 0);                              \
-  } while (0)
-      if (ct.G == 32) QGX_LAUNCH_MG(32);
-      else if (ct.G == 64) QGX_LAUNCH_MG(64);
-      else QGX_LAUNCH_MG(128);
-#undef QGX_LAUNCH_MG
-#undef QGX_LAUNCH_M
-    }
-    count_launch(c);
-    return cuda_status(cudaGetLastError());
-  }
-  rc = launch_decode_average(c, da, ct, lt_kept, sym_mode);
-  if (rc != QGX_OK || !da.values) return rc;
-  {
-    ScopedKernelTimer timer(c, QGX_KERNEL_DECODE);
-    const unsigned grid = (unsigned)std::max<size_t>(1, std::min<size_t>((d + 255) / 256, (size_t)c->num_sms * 8));
-    k_sum_workers<<<grid, 256, 0, c->stream>>>(da.values, K, d, mean_out, da.update, da.xin, da.xout, da.scalars);
-  }
-  count_launch(c);
-  return cuda_status(cudaGetLastError());
-}
-
-template <int G, int SYM, bool VAL>
-static qgx_status launch_decode_gs(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt) {
-  const size_t subs = da.nb * ((size_t)da.bucket / G);
-  const size_t total_sub = (!VAL || da.values) ? ((subs + 31) & ~(size_t)31) * (size_t)da.K : subs;   // threads wanted
-  const size_t lut_bytes = (VAL ? sizeof(DecEntry) : sizeof(uint32_t)) * ((size_t)2 << ct.maxlen) + DecodeSmem<G, SYM, VAL>::kBytes;   // table, then the rows
-  const size_t want = (total_sub + kDecThreads - 1) / kDecThreads;
-  int per_sm = 1;
-  {
-    ScopedKernelTimer timer(c, QGX_KERNEL_DECODE);
-    allow_max_dynamic_smem((const void*)k_exchange_decode<G, SYM, VAL>, c->device);
-    TableCache* tc = table_cache(c);
-    constexpr int g = G == 32 ? 0 : (G == 64 ? 1 : 2);
-    LaunchShape& shape = VAL ? tc->dec[g][SYM] : tc->dec_walk[g];
-    if (shape.smem != lut_bytes + 1) {                       // occupancy asked once per shape, not per call
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_exchange_decode<G, SYM, VAL>, kDecThreads, lut_bytes);
-      shape.smem = lut_bytes + 1;
-      shape.per_sm = per_sm < 1 ? 1 : per_sm;
-    }
-    per_sm = shape.per_sm;
-    const unsigned grid = (unsigned)std::max<size_t>(1, std::min<size_t>(want, (size_t)c->num_sms * per_sm));
-    k_exchange_decode<G, SYM, VAL><<<grid, kDecThreads, lut_bytes, c->stream>>>(da, ct, lt);
-  }
-  count_launch(c);
-  return cuda_status(cudaGetLastError());
-}
-
-template <int G>
-static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, int sym_mode) {
-  switch (sym_mode) {
-    case 1: return launch_decode_gs<G, 1, true>(c, da, ct, lt);
-    case 2: return launch_decode_gs<G, 2, true>(c, da, ct, lt);
-    case 3: return launch_decode_gs<G, 3, true>(c, da, ct, lt);
-    case 4: return launch_decode_gs<G, 4, true>(c, da, ct, lt);
-    case 5: return launch_decode_gs<G, 5, true>(c, da, ct, lt);
-    default: return launch_decode_gs<G, 0, true>(c, da, ct, lt);
-  }
-}
-
-qgx_status launch_decode_average(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, int sym_mode) {
-  if (!ct.has_header || da.bucket % ct.G != 0) return QGX_ERR_INVALID_ARG;
-  switch (ct.G) {
-    case 32: return launch_decode_g<32>(c, da, ct, lt, sym_mode);
-    case 64: return launch_decode_g<64>(c, da, ct, lt, sym_mode);
-    case 128: return launch_decode_g<128>(c, da, ct, lt, sym_mode);
-    default: return QGX_ERR_INVALID_ARG;
-  }
-}
-
-qgx_status launch_decode_walk(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt) {
-  if (!ct.has_header || da.bucket % ct.G != 0) return QGX_ERR_INVALID_ARG;
-  switch (ct.G) {
-    case 32: return launch_decode_gs<32, 0, false>(c, da, ct, lt);
-    case 64: return launch_decode_gs<64, 0, false>(c, da, ct, lt);
-    case 128: return launch_decode_gs<128, 0, false>(c, da, ct, lt);
-    default: return QGX_ERR_INVALID_ARG;
-  }
+  da.vec_out = ((reinterpret_cast<uintptr_t>(mean_out) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(da.xin) & 15u) == 0) &&
+               ((reinterpret_cast<uintptr_t>(da.xout) & 15u) == 0);
+  return launch_exchange_decode(c, da, ct, lt, lt_kept, sym_mode);
 }
 
 // ---- helper contexts of the layer-wise exchange -------------------------------------------------
@@ -1391,25 +650,21 @@ static SegChildren* seg_children(qgx_ctx* c) {
   return sc;
 }
 
-// counts[j] += coordinates of the kept symbols (layout: DecodeArgs::sym_out) that carry level j
-__global__ void __launch_bounds__(256) k_level_counts(const uint8_t* __restrict__ sym, int K, size_t d, size_t sym_ld, int bucket, int G,
+// counts[j] += coordinates of the kept symbols (see DecodeArgs::sym_out) that carry level j
+__global__ void __launch_bounds__(256) k_level_counts(const uint8_t* __restrict__ sym, int K, size_t d, size_t sym_ld, int nlev,
                                                       unsigned long long* counts) {
   __shared__ unsigned int s_cnt[8][QGX_MAX_LEVELS];                  // one set per warp
   const int warp = threadIdx.x >> 5;
   if ((threadIdx.x & 31) < QGX_MAX_LEVELS) s_cnt[warp][threadIdx.x & 31] = 0u;
   __syncwarp();
   const size_t wpw = sym_ld / 4;                                      // words per worker
-  const size_t spb = (size_t)(bucket / G);
-  const size_t total_sub = ((d + (size_t)bucket - 1) / (size_t)bucket) * spb;
   for (size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x; w < (size_t)K * wpw; w += (size_t)gridDim.x * blockDim.x) {
-    const size_t at = (w % wpw) * 4;                                  // byte inside the worker's symbols
-    const size_t gs = (at / (size_t)(32 * G)) * 32 + (at % 128) / 4;  // the sub-block
-    const size_t i0 = ((at % (size_t)(32 * G)) / 128) * 4;            // first of the word's four coordinates in it
-    if (gs >= total_sub) continue;
-    const size_t e0 = (gs / spb) * (size_t)bucket + (gs % spb) * (size_t)G + i0;
+    const size_t e0 = (w % wpw) * 4;
     const uint32_t four = *reinterpret_cast<const uint32_t*>(sym + w * 4);
-    for (int cc = 0; cc < 4; ++cc)
-      if (e0 + cc < d && e0 + cc < (gs / spb + 1) * (size_t)bucket) atomicAdd(&s_cnt[warp][(four >> (8 * cc)) & 31u], 1u);
+    for (int cc = 0; cc < 4; ++cc) {
+      const int s = (int)((four >> (8 * cc)) & 0xffu), level = s < nlev ? s : s - nlev;
+      if (e0 + cc < d && level < nlev) atomicAdd(&s_cnt[warp][level], 1u);
+    }
   }
   __syncwarp();
   const unsigned int mine = (threadIdx.x & 31) < QGX_MAX_LEVELS ? s_cnt[warp][threadIdx.x & 31] : 0u;
@@ -1550,12 +805,12 @@ qgx_status qgx_set_keep_symbols(qgx_ctx* c, int on) {
 }
 
 qgx_status qgx_level_counts(qgx_ctx* c, uint64_t* counts) {
-  if (!c || !counts || c->sym_slot < 0 || !c->ws[WS_SYM] || c->sym_G <= 0) return QGX_ERR_INVALID_ARG;
+  if (!c || !counts || c->sym_slot < 0 || !c->ws[WS_SYM]) return QGX_ERR_INVALID_ARG;
   if (cudaSetDevice(c->device) != cudaSuccess) return QGX_ERR_CUDA;
   if (cudaMemsetAsync(counts, 0, sizeof(uint64_t) * QGX_MAX_LEVELS, c->stream) != cudaSuccess) return QGX_ERR_CUDA;
   const size_t words = (size_t)c->sym_K * (c->sym_ld / 4);
   const unsigned grid = (unsigned)std::max<size_t>(1, std::min<size_t>((words + 255) / 256, (size_t)c->num_sms * 8));
-  k_level_counts<<<grid, 256, 0, c->stream>>>((const uint8_t*)c->ws[WS_SYM], c->sym_K, c->sym_d, c->sym_ld, c->sym_bucket, c->sym_G,
+  k_level_counts<<<grid, 256, 0, c->stream>>>((const uint8_t*)c->ws[WS_SYM], c->sym_K, c->sym_d, c->sym_ld, c->sym_nlev,
                                                reinterpret_cast<unsigned long long*>(counts));
   count_launch(c);
   return cuda_status(cudaGetLastError());

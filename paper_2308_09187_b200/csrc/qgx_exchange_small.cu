@@ -27,6 +27,13 @@ __device__ __forceinline__ uint32_t round_fixed_one(float x, uint32_t w, float r
   return __float_as_uint(z) - (w >> 16);
 }
 
+// The value of a decoded symbol (the low byte of `sym`, one that is a symbol; see qgx_walk.cuh).
+__device__ __forceinline__ float value_of(uint32_t sym, float norm, const float* lev, int nlev) {
+  const int s = (int)(sym & 0xffu), level = s < nlev ? s : s - nlev;
+  const float val = __fmul_rn(norm, lev[level & 31]);
+  return s < nlev ? val : -val;
+}
+
 constexpr int kPadShift = 33;            // status words carry the words (low) and the unused bits (high) of the buckets so far
 
 // Q quads per thread; G coordinates per sub-block.
@@ -50,8 +57,8 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
   const int K = a.K;
   float4* s_bin = reinterpret_cast<float4*>(s_raw);
   uint32_t* s_img = reinterpret_cast<uint32_t*>(s_raw + r.off_img);
-  uint32_t* s_sym = reinterpret_cast<uint32_t*>(s_raw + r.off_sym);    // the decoded symbols, four per word
-  uint16_t* s_tab = reinterpret_cast<uint16_t*>(s_raw + r.off_tab);    // the next maxlen + 1 bits -> symbol byte | bits << 8
+  uint32_t* s_sym = reinterpret_cast<uint32_t*>(s_raw + r.off_sym);    // the decoded symbols (see qgx_walk.cuh), four per word
+  uint16_t* s_tab = reinterpret_cast<uint16_t*>(s_raw + r.off_tab);    // see DecodeTables::single
 
   // which bucket: a ticket per cluster, so that the buckets a bucket looks back at are already under way
   unsigned ticket = 0;
@@ -59,10 +66,7 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
   asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
   const int rep = rt.key_shift - kKeyShiftMin, nbins = (int)((kKeyTop - kKeyBase) >> rt.key_shift) + 1;
   for (int i = tid; i < nbins; i += blockDim.x) s_bin[i] = __ldg(a.tables->bin_fix + (i << rep));
-  for (int i = tid; i < (2 << ct.maxlen); i += blockDim.x) {
-    const uint32_t e = __ldg(r.lut_len + 2 * i);                       // bits 0..4 bits consumed, 8..15 the symbol byte
-    s_tab[i] = (uint16_t)(((e & 31u) << 8) | ((e >> 8) & 0xffu));
-  }
+  for (int i = tid; i < (1 << ct.maxlen); i += blockDim.x) reinterpret_cast<uint32_t*>(s_tab)[i] = __ldg(reinterpret_cast<const uint32_t*>(r.tables->single) + i);
   if (tid < 2 * QGX_MAX_LEVELS) s_lut.e[tid] = __ldg(a.tables->lut.e + tid);
   if (blockDim.x == kWarp) s_lut.e[QGX_MAX_LEVELS + tid] = __ldg(a.tables->lut.e + QGX_MAX_LEVELS + tid);   // a bucket of 128 has one warp
   if (tid < QGX_MAX_LEVELS) {
@@ -194,7 +198,7 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
             buf >>= n;
             avail -= (int)n;
             left -= n;
-            bad = bad || (e & 0x40u) != 0u;                            // an index that no codeword starts like
+            bad = bad || (e & 0xffu) == bad_symbol(ct.nlev);            // bits that no codeword starts like
             word |= (e & 0xffu) << (8 * q);
           }
         }
@@ -236,12 +240,10 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
   __syncthreads();
   const float Kf = (float)K, gam = r.update == 1 ? (float)r.scalars[1] : 1.0f;
   const int quads = (len + kQuad - 1) / kQuad;
-  const size_t spb = (size_t)a.bucket / G;
   double sq = 0.0;
   for (int q = (int)k * blockDim.x + tid; q < quads; q += K * (int)blockDim.x) {
-    const int e = q * kQuad, nv = min(kQuad, len - e), i = e % G;
-    const size_t gs = b * spb + (size_t)(e / G);
-    const size_t sat = (gs >> 5) * (size_t)(32 * G) + (size_t)(i >> 2) * 128 + (size_t)(gs & 31) * 4;   // see DecodeArgs::sym_out
+    const int e = q * kQuad, nv = min(kQuad, len - e);
+    const size_t sat = lo + (size_t)e;                                 // see DecodeArgs::sym_out
     float acc[kQuad] = {0.f, 0.f, 0.f, 0.f};
     for (int kk = 0; kk < K; ++kk) {
       const uint32_t word = *cluster.map_shared_rank(s_sym + q, kk);
@@ -249,10 +251,10 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
       const uint32_t was = r.sym_prev ? *reinterpret_cast<const uint32_t*>(r.sym_prev + (size_t)kk * r.sym_ld + sat) : 0u;
 #pragma unroll
       for (int c = 0; c < kQuad; ++c) {
-        const float val = dequantize_symbol((word >> (8 * c)) & 0xffu, nrm, s_lev);
+        const float val = value_of(word >> (8 * c), nrm, s_lev, lt.nlev);
         acc[c] = __fadd_rn(acc[c], val);
         if (c < nv && r.sym_prev) {
-          const float dlt = __fsub_rn(dequantize_symbol((was >> (8 * c)) & 0xffu, s_norms_kept[kk], s_lev_kept), val);
+          const float dlt = __fsub_rn(value_of(was >> (8 * c), s_norms_kept[kk], s_lev_kept, lt_kept.nlev), val);
           sq = fma((double)dlt, (double)dlt, sq);
         } else if (c < nv && r.square) {
           sq = fma((double)val, (double)val, sq);

@@ -2,13 +2,14 @@
 #pragma once
 
 #include "qgx_encode.cuh"
+#include "qgx_walk.cuh"
 
 namespace qgx {
 
 constexpr int kSmallMaxWorkers = 16;     // the largest cluster (more than 8 where the device allows it)
 
 struct SmallArgs {
-  const uint32_t* lut_len;               // second words of the decoder table's entries, 8 bytes apart
+  const DecodeTables* tables;
   float* mean;
   int update;                            // as DecodeArgs
   const float* xin;

@@ -1,0 +1,57 @@
+"""The decode pass where its rows and teams change shape: rows of one bucket and of many, workers that do not fill a team or take
+several turns, codes whose pairs of symbols do not fit the look-up table, the vector's last sub-block.  Means bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import qgx_inputs as gen
+from oracle import qgx_oracle as o
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # K, d, bucket, nlev, sub, code
+    (1, 97, 96, 3, 32, "fixed"),                            # eight rows side by side, one of them there
+    (2, 3 * 96 * 40 + 1, 96, 9, 32, "steep"),               # three sub-blocks per bucket: a row of eleven buckets
+    (3, 33 * 1024 - 1, 1024, 17, 128, "steep"),             # two rows side by side, six of eight warps
+    (5, 2 * 16384 + 8192 + 31, 16384, 32, 32, "elias"),     # 512 sub-blocks: headers beyond what is fetched ahead; every pair escapes
+    (8, 70000, 8192, 17, 64, "gauss"),
+    (9, 3 * 4096 + 64, 4096, 9, 64, "elias"),               # few rows: teams of sixteen
+    (17, 5000, 1024, 32, 32, "steep"),                      # few rows: teams of thirty-two
+    (33, 2 * 16384 + 5, 16384, 17, 128, "steep"),           # more workers than a team has warps
+    (40, 600 * 1024, 1024, 5, 32, "fixed"),                 # teams of eight, five turns; many rows per team
+    (64, 128 * 7 + 3, 256, 2, 128, "fixed"),
+]
+
+
+@pytest.mark.parametrize("K,d,bucket,nlev,sub,code", CASES)
+def test_decode_pass_matches_oracle(K, d, bucket, nlev, sub, code):
+    import paper_2308_09187_b200 as qgx
+    ctx = qgx.qgx_create(0)
+    try:
+        qgx.qgx_set_decode_split(ctx, qgx.QGX_SPLIT_NEVER)  # not in one launch
+        qgx.qgx_set_keep_symbols(ctx, True)
+        rng = np.random.default_rng(d)
+        v = gen.gaussian_mixture((K, d), seed=d + 1, device="cuda")
+        top = 0.6 if code == "elias" else 0.05              # high levels are rare, but for the code that pays for them
+        lev = np.r_[0.0, np.sort(rng.uniform(1e-3, top, size=nlev - 2)), 1.0].astype(np.float32)
+        if code == "fixed":
+            cb = qgx.qgx_build_codebook_fixed(nlev, sub)
+        elif code == "elias":
+            cb = qgx.qgx_build_codebook_elias(nlev, sub)
+        else:                                               # codewords of one to twelve bits; of the order that the levels have
+            p = 2.0 ** -np.arange(1, nlev + 1) if code == "steep" else 1.0 / np.arange(1, nlev + 1)
+            cb = qgx.qgx_build_codebook_huffman(list(p / p.sum()), sub)
+        cfg = qgx.make_quant_cfg(lev, bucket, cb, 77)
+        mean, _ = qgx.qgx_exchange(ctx, v, cfg, 5)
+        qgx.qgx_sync_status(ctx)
+        norms, _ = qgx.qgx_quantize(ctx, v, bucket, lev, qgx.QGX_NORM_L2, 77, 5)
+        n = norms.cpu().numpy()
+        sym = o.quantize(v.cpu().numpy(), bucket, lev, n, 77, 5)
+        assert np.array_equal(mean.cpu().numpy(), o.average(n, sym, bucket, lev))
+        counts = qgx.qgx_level_counts(ctx).cpu().numpy()
+        assert np.array_equal(counts, np.bincount((sym & 31).ravel(), minlength=32))
+        assert torch.equal(qgx.qgx_exchange_decode(ctx, K, d, cfg), mean)
+        qgx.qgx_sync_status(ctx)
+    finally:
+        qgx.qgx_destroy(ctx)
