@@ -217,8 +217,8 @@ qgx_status qgx_encode_noalloc(qgx_ctx *ctx, const float *norms, const uint8_t *s
                               int bucket, const qgx_codebook *cb /*[host]*/, uint32_t *stream,
                               size_t cap_words, uint32_t *bucket_bits, uint64_t *total_bits);
 
-/* DEQ o CODE: the exact inverse of qgx_encode, driven by bucket_bits.  Every read is bounded by
- * the bucket's length; a codeword that runs past it, an unassigned bit pattern, a sub-block whose
+/* DEQ o CODE: the exact inverse of qgx_encode, driven by bucket_bits.  Every read stays inside
+ * the stream buffer; a codeword that runs past it, an unassigned bit pattern, a sub-block whose
  * length disagrees with its header, or lengths that exceed cap_words latch QGX_ERR_CORRUPT. */
 qgx_status qgx_decode(qgx_ctx *ctx, const uint32_t *stream, size_t cap_words,
                       const uint32_t *bucket_bits, int K, size_t d, int bucket,

@@ -1,9 +1,10 @@
 // qgx_encode and qgx_decode as separate steps.  Encoding takes one pass (k_pack: pack a bucket, find its place by look-back,
 // copy it out) where the capacity fits any outcome and the sub-blocks are a warp's, else three kernels: bucket bit lengths ->
 // exclusive scan of the word-aligned lengths (offsets) -> bit scatter; qgx_encode_noalloc takes the three always.  Decoding:
-// offsets (k_scan_offsets, which also builds the decoder's table) -> k_unpack.
+// offsets (k_scan_offsets, which also builds the decoder's table) -> k_unpack_rows or k_unpack.
 #include "qgx_bucket.cuh"
 #include "qgx_codec.cuh"
+#include "qgx_unpack.cuh"
 
 #include <algorithm>
 #include <mutex>
@@ -67,6 +68,7 @@ __global__ void __launch_bounds__(512) k_bucket_bits(const uint8_t* __restrict__
 // 15.0 so.
 constexpr int kUnpackTableMax = 2 << QGX_MAX_CODE_LEN;
 constexpr int kScanThreads = 1024, kScanEach = 4;
+constexpr unsigned kPairBuilders = 8;    // CTAs that build a pair table: an entry per thread
 __device__ __forceinline__ void build_unpack_table(const CodeTable& ct, uint16_t* table /* [2 << maxlen] */) {
   static_assert(kScanThreads == 32 * QGX_MAX_LEVELS, "a warp per level");
   __shared__ uint16_t s_short[64];       // level | length << 8
@@ -98,8 +100,12 @@ __device__ __forceinline__ void build_unpack_table(const CodeTable& ct, uint16_t
 __global__ void __launch_bounds__(kScanThreads) k_scan_offsets(const uint32_t* __restrict__ bucket_bits, size_t nb, size_t cap_words,
                                                                uint64_t* __restrict__ off, uint64_t* __restrict__ total_bits,
                                                                uint32_t* __restrict__ flags, unsigned int err_code, DevStatus* st,
-                                                               int K, const __grid_constant__ CodeTable ct, uint16_t* table) {
-  if (blockIdx.x == (unsigned)K) { build_unpack_table(ct, table); return; }
+                                                               int K, const __grid_constant__ CodeTable ct, uint16_t* table, uint32_t* pair) {
+  if (blockIdx.x >= (unsigned)K) {
+    if (pair) build_unpack_pairs(ct, pair, (blockIdx.x - (unsigned)K) * kScanThreads + threadIdx.x, kPairBuilders * kScanThreads);
+    else build_unpack_table(ct, table);
+    return;
+  }
   __shared__ uint64_t s_words[2][32], s_bits[2][32];
   const size_t k = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -401,8 +407,8 @@ struct UnpackArgs {
 };
 
 // One thread per sub-block (per bucket without sub-blocks), a warp on consecutive ones of one bucket or of several small
-// buckets; persistent CTAs, so that the table is copied once per CTA and not once per bucket.  Every read is bounded by the
-// bucket's words.  A serial walk per thread: latency-bound with few sub-blocks, instruction-bound (14 per symbol) with many.
+// buckets; persistent CTAs, so that the table is copied once per CTA and not once per bucket.  For what k_unpack_rows does not
+// take: sub-blocks of other lengths, or none.  Every read is bounded by the bucket's words.  A serial walk per thread: latency-bound with few sub-blocks, instruction-bound (14 per symbol) with many.
 __global__ void __launch_bounds__(128) k_unpack(const __grid_constant__ UnpackArgs a, const __grid_constant__ CodeTable ct) {
   extern __shared__ __align__(16) uint16_t s_tab[];  // [2 << maxlen], see build_unpack_table
   const int tab_n = 2 << ct.maxlen;
@@ -599,7 +605,7 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
   const int threads = bucket_threads(bucket, v4);
   const dim3 grid((unsigned)nb, (unsigned)K);
   k_bucket_bits<<<grid, threads, 0, c->stream>>>(sym, d, bucket, ct, vec_ok, bucket_bits, c->dstatus);
-  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus, K, ct, nullptr);
+  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus, K, ct, nullptr, nullptr);
   const size_t smem = sizeof(uint32_t) * (img_words + (size_t)(bucket / ct.G) + 2);
 #define QGX_LAUNCH_S(V)                                                                                         \
   do {                                                                                                          \
@@ -628,11 +634,18 @@ qgx_status qgx_decode(qgx_ctx* c, const uint32_t* stream, size_t cap_words, cons
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
   uint64_t* off = (uint64_t*)ws_get(c, 0, sizeof(uint64_t) * (size_t)K * nb);
   uint32_t* flags = (uint32_t*)ws_get(c, 1, sizeof(uint32_t) * (size_t)K);
-  uint16_t* table = (uint16_t*)ws_get(c, 2, sizeof(uint16_t) * kUnpackTableMax);
+  const bool rows = unpack_rows_fits(K, d, bucket, ct);
+  void* table = ws_get(c, 2, std::max(sizeof(uint16_t) * (size_t)kUnpackTableMax, sizeof(uint32_t) << kPairBitsMax));
   if (!off || !flags || !table) return QGX_ERR_CUDA;
-  k_scan_offsets<<<K + 1, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, nullptr, flags, QGX_ERR_CORRUPT, c->dstatus, K, ct, table);
+  k_scan_offsets<<<K + (rows ? kPairBuilders : 1u), kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, nullptr, flags, QGX_ERR_CORRUPT,
+                                                                                  c->dstatus, K, ct, (uint16_t*)table, rows ? (uint32_t*)table : nullptr);
+  if (rows) {
+    count_launch(c);
+    const UnpackRowsArgs r{stream, cap_words, bucket_bits, off, flags, (const uint32_t*)table, d, K, nb, norms, sym, c->dstatus};
+    return launch_unpack_rows(c, r, bucket, ct);
+  }
   UnpackArgs a;
-  a.stream = stream; a.cap_words = cap_words; a.bucket_bits = bucket_bits; a.off = off; a.flags = flags; a.table = table; a.d = d;
+  a.stream = stream; a.cap_words = cap_words; a.bucket_bits = bucket_bits; a.off = off; a.flags = flags; a.table = (const uint16_t*)table; a.d = d;
   a.bucket = bucket; a.K = K; a.nb = nb; a.norms = norms; a.sym = sym; a.st = c->dstatus;
   const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
   a.store = (d % 16 == 0 && bucket % 16 == 0 && ct.G % 16 == 0 && (at & 15u) == 0) ? 16 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
@@ -695,7 +708,7 @@ qgx_status qgx_encode_noalloc(qgx_ctx* c, const float* norms, const uint8_t* sym
   const int threads = bucket_threads(bucket, v4);
   const dim3 grid((unsigned)nb, (unsigned)K);
   k_bucket_bits<<<grid, threads, 0, c->stream>>>(sym, d, bucket, ct, vec_ok, bucket_bits, c->dstatus);
-  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus, K, ct, nullptr);
+  k_scan_offsets<<<K, kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, total_bits, flags, QGX_ERR_CAPACITY, c->dstatus, K, ct, nullptr, nullptr);
   const size_t img_words = (((size_t)bucket * (ct.maxlen + 1) + 16u * (bucket / ct.G + 1) + kNormBits + 31u) >> 5) + 4;
   const size_t smem = sizeof(uint32_t) * (img_words + (size_t)(bucket / ct.G) + 2);
 #define QGX_LAUNCH_S(V)                                                                                         \

@@ -419,6 +419,33 @@ __device__ __forceinline__ float dequantize_symbol(uint32_t sym, float norm, con
   return __uint_as_float(__float_as_uint(val) ^ ((sym & 0x80u) << 24));
 }
 
+// ---- two fp32 numbers at a time ---------------------------------------------------------------
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float* lo, float* hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(*lo), "=f"(*hi) : "l"(v)); }
+// Products rounded on their own.  The assembler fuses mul.rn.f32x2 with the sum it feeds (which it may not do with scalar
+// mul.rn): the product plus -0, which is the product, is what it leaves alone as long as it cannot see that number:
+// kernels take it as an argument (kMinusZero2).
+constexpr uint64_t kMinusZero2 = 0x8000000080000000ull;
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b, uint64_t minus_zero) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(minus_zero));
+  return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {     // a - b as (-1) b + a
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // ---- reductions ------------------------------------------------------------------------------
 __device__ __forceinline__ double warp_sum(double x) {
 #pragma unroll

@@ -22,131 +22,19 @@
 namespace qgx {
 
 // ---- tables -----------------------------------------------------------------------------------
-struct NextSymbol { uint32_t sym, bits; bool known; };
-// the symbol that `bits` (the stream's next ones, first at bit 0) start with
-__device__ __forceinline__ NextSymbol next_symbol(uint32_t bits, const CodeTable& ct) {
-  NextSymbol s{bad_symbol(ct.nlev), 1u, false};
-  for (int j = 0; j < ct.nlev; ++j) {
-    const uint32_t L = ct.len[j];
-    if ((bits & ((1u << L) - 1u)) != ct.rev[j]) continue;
-    s.known = true;
-    s.sym = (uint32_t)j + (j != 0 && ((bits >> L) & 1u) ? (uint32_t)ct.nlev : 0u);
-    s.bits = L + (j != 0 ? 1u : 0u);
-  }
-  return s;
-}
 __global__ void __launch_bounds__(256) k_build_decode_tables(const __grid_constant__ CodeTable ct, DecodeTables* out) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  const NextSymbol a = next_symbol(i, ct);
-  if (i < (2u << ct.maxlen)) out->single[i] = (uint16_t)(a.sym | (a.bits << 8));
-  const uint32_t P = (uint32_t)pair_bits(ct.maxlen);
-  if (i >= (1u << P)) return;
-  const NextSymbol b = next_symbol(i >> a.bits, ct);
-  // the second symbol counts where the index holds all its bits (or all that could tell that there is none)
-  const bool both = a.bits + (b.known ? b.bits : (uint32_t)ct.maxlen + 1u) <= P;
-  out->pair[i] = (both ? (a.bits + b.bits) | (b.sym << 24) : a.bits | kPairEscape) | (a.bits << 8) | (a.sym << 16);
+  const auto symbol = [&](const NextSymbol& s) { return s.known ? s.level + (s.negative ? (uint32_t)ct.nlev : 0u) : bad_symbol(ct.nlev); };
+  if (i < (2u << ct.maxlen)) {
+    const NextSymbol a = next_symbol(i, ct);
+    out->single[i] = (uint16_t)(symbol(a) | (a.bits << 8));
+  }
+  if (i < (1u << pair_bits(ct.maxlen)))
+    out->pair[i] = pair_entry_of(i, ct, symbol);
 }
 void launch_build_decode_tables(const CodeTable& ct, DecodeTables* out, cudaStream_t stream) {
   const int n = 1 << std::max(ct.maxlen + 1, pair_bits(ct.maxlen));
   k_build_decode_tables<<<(n + 255) / 256, 256, 0, stream>>>(ct, out);
-}
-
-// ---- the walk ---------------------------------------------------------------------------------
-// Words that a lane may read past the one that holds its sub-block's first bit: G symbols of at most 13 bits, the partial
-// first word and the word fetched ahead.
-template <int G>
-struct WalkReach { static constexpr int kWords = (G * 13) / 32 + 4; };
-
-// Position in a stream: the lowest five bits of `pos` are the place in w0, bit 5 says whether that has been left; what is above
-// is junk (entries of the pair table are added as they are).  The two bits before the next symbol lie in the window, too, so
-// that an index comes out as a byte offset.  SH: the words are in shared memory (32-bit addresses).
-template <bool SH> struct WordAt { using Addr = uint32_t; };
-template <> struct WordAt<false> { using Addr = const uint32_t*; };
-template <bool SH>
-struct Walk {
-  typename WordAt<SH>::Addr next;        // of the word after w1
-  uint32_t w0, w1, pos, old;             // old: pos when w0 was last checked
-  static __device__ __forceinline__ uint32_t word(uint32_t a) { return lds32(a); }
-  static __device__ __forceinline__ uint32_t word(const uint32_t* a) { return *a; }
-  static __device__ __forceinline__ uint32_t step(uint32_t a, int words) { return a + 4u * (uint32_t)words; }
-  static __device__ __forceinline__ const uint32_t* step(const uint32_t* a, int words) { return a + words; }
-  static __device__ __forceinline__ uint32_t words_from(uint32_t a, uint32_t b) { return (a - b) >> 2; }
-  static __device__ __forceinline__ uint32_t words_from(const uint32_t* a, const uint32_t* b) { return (uint32_t)(a - b); }
-  // p = the word that holds the bit two before the first, sh = that bit's place in it
-  __device__ __forceinline__ void open(typename WordAt<SH>::Addr p, uint32_t sh) {
-    w0 = word(p);
-    w1 = word(step(p, 1));
-    next = step(p, 2);
-    pos = old = sh;
-  }
-  __device__ __forceinline__ uint32_t window() const { return __funnelshift_r(w0, w1, pos); }
-  // after at most 32 bits: moves on a word where the position has left w0
-  __device__ __forceinline__ void settle() {
-    if ((pos ^ old) & 32u) {
-      w0 = w1;
-      w1 = word(next);
-      next = step(next, 1);
-    }
-    old = pos;
-  }
-  // bits taken since open(p, sh)
-  __device__ __forceinline__ uint32_t taken(typename WordAt<SH>::Addr p, uint32_t sh) const { return 32u * (words_from(next, p) - 2u) + (pos & 31u) - sh; }
-};
-
-struct WalkTable {
-  uint32_t pair;                         // shared address of the pair table, its mask for byte offsets
-  uint32_t mask;
-  __device__ __forceinline__ uint32_t entry(uint32_t window) const { return lds_table32(pair + (window & mask)); }
-};
-__device__ __forceinline__ uint32_t first_bits(uint32_t entry) { return (entry >> 8) & 31u; }
-
-// G symbols of one sub-block to row[0 .. G / 4) (shared address), four to a word.  A window holds 30 bits to come, so two
-// entries of at most 13; where an entry stands for one symbol only the second is looked up on its own, its bits taken at once
-// and the entry's own cleared.
-template <int G, bool SH>
-__device__ __forceinline__ void walk_whole(Walk<SH>& w, uint32_t row, const WalkTable& t) {
-#pragma unroll
-  for (int i = 0; i < G; i += 4) {
-    uint32_t win = w.window();
-    uint32_t e = t.entry(win);
-    if (e & kPairEscape) {
-      const uint32_t f = t.entry(__funnelshift_r(win, 0u, e));
-      w.pos += (e & 31u) + first_bits(f);
-      w.settle();
-      win = w.window();
-      e = prmt(prmt(e, f, 0x6200u), 0u, 0x3244u);                      // the two symbols, nothing taken
-    }
-    w.pos += e;
-    win = __funnelshift_r(win, 0u, e);
-    uint32_t f = t.entry(win);
-    if (f & kPairEscape) {
-      w.settle();
-      w.pos += f & 31u;
-      w.settle();
-      const uint32_t g = t.entry(w.window());
-      w.pos += first_bits(g);
-      f = prmt(prmt(f, g, 0x6200u), 0u, 0x3244u);
-    }
-    w.pos += f;
-    w.settle();
-    sts32(row + (uint32_t)i, prmt(e, f, 0x7632u));
-  }
-}
-// the same, one symbol at a time, for `count` symbols (the vector's last sub-block)
-template <bool SH>
-__device__ __forceinline__ void walk_some(Walk<SH>& w, int count, uint32_t row, const WalkTable& t) {
-#pragma unroll 1
-  for (int i = 0; i < count; i += 4) {
-    uint32_t word = 0;
-#pragma unroll 1
-    for (int q = 0; q < 4 && i + q < count; ++q) {
-      const uint32_t e = t.entry(w.window());
-      w.pos += first_bits(e);
-      w.settle();
-      word |= ((e >> 16) & 0xffu) << (8 * q);
-    }
-    sts32(row + (uint32_t)i, word);
-  }
 }
 
 // ---- where a lane's sub-block lies ------------------------------------------------------------
@@ -156,30 +44,12 @@ struct DecodeShape {
   int teams;                             // of a CTA
   int rows;                              // rows that a team works on side by side (more than one: all workers at once)
   int groups;                            // turns over the workers
-  uint32_t total_rows, units;            // units: turns of `rows` rows
-  uint32_t spb, spb_mul, spb_shift;      // sub-blocks per bucket; n / spb = (n * spb_mul >> 32) >> spb_shift
-  uint32_t whole_subs, last_count;       // sub-blocks of G coordinates, and the coordinates of the one after them
-  uint32_t hdr_bits, hdr_bits_last;      // of a bucket, of the last bucket
+  RowShape row;
+  uint32_t units;                        // turns of `rows` rows
   uint32_t pair_mask;                    // of byte offsets into the pair table
   uint32_t row_words;                    // room for a warp's stream words, a multiple of 4
   uint32_t off_val, off_kept, off_norm, off_norm_kept, off_sym, off_row;   // bytes of dynamic shared memory
 };
-
-// Row r of a worker: its sub-blocks 32 r .. 32 r + 31, of one bucket or of several in a row.
-struct RowPlace {
-  uint32_t b, s;                         // the lane's bucket, the sub-block's number in it
-  int count;                             // its coordinates, 0 beyond the end
-};
-template <int G>
-__device__ __forceinline__ RowPlace row_place(const DecodeArgs& a, const DecodeShape& h, uint32_t row, int lane) {
-  const uint32_t gs = row * 32u + (uint32_t)lane;
-  RowPlace p;
-  p.count = gs < h.whole_subs ? G : (gs == h.whole_subs ? (int)h.last_count : 0);
-  const uint32_t in = p.count > 0 ? gs : 0u;                           // beyond the end: the first bucket's first, to have some
-  p.b = __umulhi(in, h.spb_mul) >> h.spb_shift;
-  p.s = in - p.b * h.spb;
-  return p;
-}
 
 struct SubBlockAt {
   const uint32_t* p;                     // the word that holds the bit two before its first one ...
@@ -203,8 +73,8 @@ struct HeaderAhead {
 // The header words of the row's lanes, and those of lane 0's bucket before them
 template <int G>
 __device__ __forceinline__ HeaderAhead ask_header(const DecodeArgs& a, const DecodeShape& h, uint32_t row, int k, const BucketAhead& n, int lane) {
-  const RowPlace rp = row_place<G>(a, h, row, lane);
-  const uint32_t hdr = rp.b + 1u == a.nb ? h.hdr_bits_last : h.hdr_bits;
+  const RowPlace rp = row_place<G>(h.row, row, lane);
+  const uint32_t hdr = rp.b + 1u == a.nb ? h.row.hdr_bits_last : h.row.hdr_bits;
   const uint32_t* base = a.stream + (size_t)k * a.cap_words;
   HeaderAhead r;
   r.ok = n.nbits >= hdr && n.nbits < (1u << 18) && (size_t)n.off + ((n.nbits + 31u) >> 5) <= a.cap_words;
@@ -227,8 +97,8 @@ __device__ __forceinline__ HeaderAhead ask_header(const DecodeArgs& a, const Dec
 template <int G>
 __device__ __forceinline__ SubBlockAt find_row(const DecodeArgs& a, const DecodeShape& h, uint32_t row, int k, const BucketAhead& n,
                                                const HeaderAhead& ha, int lane, uint32_t row_sa) {
-  const RowPlace rp = row_place<G>(a, h, row, lane);
-  const uint32_t hdr = rp.b + 1u == a.nb ? h.hdr_bits_last : h.hdr_bits;
+  const RowPlace rp = row_place<G>(h.row, row, lane);
+  const uint32_t hdr = rp.b + 1u == a.nb ? h.row.hdr_bits_last : h.row.hdr_bits;
   const uint32_t* base = a.stream + (size_t)k * a.cap_words;
   SubBlockAt r;
   r.count = rp.count;
@@ -274,36 +144,8 @@ __device__ __forceinline__ SubBlockAt find_row(const DecodeArgs& a, const Decode
   return r;
 }
 
-// ---- two fp32 numbers at a time ---------------------------------------------------------------
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float* lo, float* hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(*lo), "=f"(*hi) : "l"(v)); }
-// Products rounded on their own.  The assembler fuses mul.rn.f32x2 with the sum it feeds (which it may not do with scalar
-// mul.rn): the product plus -0, which is the product, is what it leaves alone as long as it cannot see that number.
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b, uint64_t minus_zero) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(minus_zero));
-  return r;
-}
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {     // a - b as (-1) b + a
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
 // ---- the kernel -------------------------------------------------------------------------------
 template <int G> constexpr int kDecodeWarps = G == 128 ? 24 : 32;       // of a CTA: what its shared memory and registers hold
-template <int G>
-__host__ __device__ constexpr uint32_t sym_row_bytes() { return 32u * (uint32_t)(G / 4 + 1) * 4u; }   // a word more than needed: no bank conflicts
-
 template <int G, int SYM>
 __global__ void __launch_bounds__(kDecodeWarps<G> * 32, 1)
 k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeShape h, const __grid_constant__ LevelTable lt,
@@ -350,11 +192,11 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     return t;
   };
   auto row_at = [&](Turn t) { return t.unit * (uint32_t)h.rows + (uint32_t)row_of; };
-  auto works = [&](Turn t) { return t.unit < h.units && t.g * W + k_of < K && row_of < h.rows && row_at(t) < h.total_rows; };
+  auto works = [&](Turn t) { return t.unit < h.units && t.g * W + k_of < K && row_of < h.rows && row_at(t) < h.row.rows; };
   auto ask_bucket = [&](Turn t) {
     BucketAhead n{0u, 0u};
     if (works(t)) {
-      const size_t kb = (size_t)(t.g * W + k_of) * a.nb + row_place<G>(a, h, row_at(t), lane).b;
+      const size_t kb = (size_t)(t.g * W + k_of) * a.nb + row_place<G>(h.row, row_at(t), lane).b;
       n.nbits = a.bucket_bits[kb];
       n.off = a.offsets[kb];
     }
@@ -398,7 +240,7 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
       else walk(Walk<false>(), at.p);
       if (at.count > 0) bad = bad || !at.ok || used != at.want;         // every sub-block uses exactly its length
       s_norm[32 * tw + lane] = at.norm;
-      if (kCompare) s_norm_kept[32 * tw + lane] = a.norms_prev[(size_t)(now.g * W + k_of) * a.nb + row_place<G>(a, h, row_at(now), lane).b];
+      if (kCompare) s_norm_kept[32 * tw + lane] = a.norms_prev[(size_t)(now.g * W + k_of) * a.nb + row_place<G>(h.row, row_at(now), lane).b];
       __syncwarp();                                                    // the staged words are no longer read
     }
     if (works(next)) at = find_row<G>(a, h, row_at(next), next.g * W + k_of, next_bucket, next_header, lane, row_sa);
@@ -410,7 +252,7 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     const int nk = min(K - now.g * W, h.rows > 1 ? K : W);
     for (int r = 0; r < h.rows; ++r) {
       const uint32_t row = now.unit * (uint32_t)h.rows + (uint32_t)r;
-      if (row >= h.total_rows) break;
+      if (row >= h.row.rows) break;
 #pragma unroll
       for (int j = 0; j < QT; ++j) {
         const uint32_t q = (uint32_t)(j * team_threads + tt);
@@ -518,30 +360,17 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
 template <int G>
 static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, const LevelTable& lt_kept, int sym_mode) {
   DecodeShape h;
-  h.minus_zero = 0x8000000080000000ull;
-  h.spb = (uint32_t)(da.bucket / G);
-  const size_t subs = (da.d + G - 1) / G;
-  if (subs >= (1ull << 31)) return QGX_ERR_INVALID_ARG;
-  // n / spb for n < 2^31: with 2^(L - 1) < spb <= 2^L the multiplier, 2^(31 + L) / spb rounded up, is below 2^32 and off by at
-  // most spb / 2^(31 + L) of itself
-  int log2up = 1;
-  while ((1u << log2up) < h.spb) ++log2up;
-  h.spb_mul = (uint32_t)((1ull << (31 + log2up)) / h.spb + 1u);
-  h.spb_shift = (uint32_t)log2up - 1u;
-  h.whole_subs = (uint32_t)(da.d / G);
-  h.last_count = (uint32_t)(da.d % G);
-  h.hdr_bits = (uint32_t)kNormBits + 16u * h.spb;
-  h.hdr_bits_last = (uint32_t)kNormBits + 16u * (uint32_t)(subs - (da.nb - 1) * (size_t)h.spb);
-  h.total_rows = (uint32_t)((subs + 31) / 32);
+  h.minus_zero = kMinusZero2;
+  if (!make_row_shape(da.d, da.bucket, G, da.nb, &h.row)) return QGX_ERR_INVALID_ARG;
   // Shared memory: the pair table, small tables, then per warp the symbols of a row and room for its stream words: as many as
   // any code can need, or what is left.
   const int max_warps = kDecodeWarps<G>;
   h.team_warps = 8;
   h.rows = std::max(1, h.team_warps / da.K);
-  while (2 * h.team_warps <= max_warps && h.team_warps < da.K && (size_t)h.total_rows * 2 * (size_t)h.team_warps <= (size_t)c->num_sms * (size_t)max_warps) h.team_warps *= 2;
+  while (2 * h.team_warps <= max_warps && h.team_warps < da.K && (size_t)h.row.rows * 2 * (size_t)h.team_warps <= (size_t)c->num_sms * (size_t)max_warps) h.team_warps *= 2;
   h.teams = max_warps / h.team_warps;
   h.groups = (da.K + h.team_warps - 1) / h.team_warps;
-  h.units = (h.total_rows + (uint32_t)h.rows - 1u) / (uint32_t)h.rows;
+  h.units = (h.row.rows + (uint32_t)h.rows - 1u) / (uint32_t)h.rows;
   const int warps = h.teams * h.team_warps;
   h.pair_mask = (4u << pair_bits(ct.maxlen)) - 4u;
   uint32_t at = 4u << pair_bits(ct.maxlen);
@@ -552,9 +381,8 @@ static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTa
   h.off_norm_kept = take((uint32_t)warps * 128u);
   h.off_sym = take((uint32_t)warps * sym_row_bytes<G>());
   h.off_row = at;
-  const uint32_t worst = (uint32_t)(G * (ct.maxlen + 1) + 3 * 32 + WalkReach<G>::kWords + 8) & ~3u;
   const uint32_t room = (224u * 1024u - at) / (uint32_t)(4 * warps) & ~3u;
-  h.row_words = std::min(worst, room);
+  h.row_words = std::min(row_words_worst(G, ct.maxlen), room);
   const size_t smem = at + (size_t)warps * h.row_words * 4u;
   const unsigned grid = (unsigned)std::min<size_t>((size_t)c->num_sms, h.units);
   ScopedKernelTimer timer(c, QGX_KERNEL_DECODE);

@@ -1,0 +1,225 @@
+// qgx_decode for codes with sub-blocks of 32, 64 or 128 coordinates: a warp takes a row of 32 consecutive sub-blocks of one
+// worker, copies its stream words to shared memory, walks them a lane per sub-block, two symbols per look-up, and copies the
+// symbols out.  The next row's numbers and header are asked for while this one is walked.
+// What bounds it: instructions, 17 per symbol at 64 % issue.  A thread per sub-block with its own window on global memory, one
+// symbol per look-up (k_unpack, which still serves other sub-block lengths and none) takes 45.7 us for 8 x 2^22 symbols of 17
+// fitted levels, this 27.5.
+#include "qgx_unpack.cuh"
+
+#include <algorithm>
+
+namespace qgx {
+
+struct UnpackShape {
+  RowShape row;
+  uint32_t items;                        // rows of all workers
+  uint32_t pair_mask;                    // of byte offsets into the pair table
+  uint32_t max_bits;                     // of a sub-block
+  uint32_t row_words, off_sym, off_row;
+  bool wide;                             // the stream buffer is 16-byte aligned
+};
+
+template <int G>
+__global__ void __launch_bounds__(1024, 1) k_unpack_rows(const __grid_constant__ UnpackRowsArgs a, const __grid_constant__ UnpackShape h) {
+  constexpr int kWords = G / 4, kStride = kWords + 1;
+  constexpr int kAhead = 4;              // header words per lane that are fetched ahead: 256 sub-blocks before the row's
+  extern __shared__ __align__(128) unsigned char s_raw[];
+  const uint32_t sa = smem_addr(s_raw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t stride = gridDim.x * (blockDim.x >> 5);
+  const uint32_t row_sa = sa + h.off_row + (uint32_t)warp * h.row_words * 4u;
+  const uint32_t sym_sa = sa + h.off_sym + (uint32_t)warp * sym_row_bytes<G>();
+  const uint32_t my_sym = sym_sa + (uint32_t)lane * (uint32_t)(kStride * 4);
+
+  struct Item { uint32_t k, row; };
+  auto item_of = [&](uint32_t it) { const uint32_t k = it / h.row.rows; return Item{k, it - k * h.row.rows}; };
+  struct Bucket { uint32_t nbits; uint64_t off; bool dead; };
+  struct Header { float norm; uint32_t field, before[kAhead]; bool sound; };
+  auto hdr_of = [&](const RowPlace& rp) { return rp.b + 1u == a.nb ? h.row.hdr_bits_last : h.row.hdr_bits; };
+  auto ask_bucket = [&](uint32_t it) {
+    Bucket n{0u, 0ull, true};
+    if (it < h.items) {
+      const Item i = item_of(it);
+      const size_t kb = (size_t)i.k * a.nb + row_place<G>(h.row, i.row, lane).b;
+      n.nbits = a.bucket_bits[kb];
+      n.off = a.off[kb];
+      n.dead = a.flags[i.k] != 0u;       // the worker's lengths exceed its words: nothing is read
+    }
+    return n;
+  };
+  auto ask_header = [&](uint32_t it, const Bucket& n) {
+    Header r;
+    r.norm = 0.0f;
+    r.field = 0u;
+    r.sound = false;
+#pragma unroll
+    for (int t = 0; t < kAhead; ++t) r.before[t] = 0u;
+    if (it < h.items) {
+      const Item i = item_of(it);
+      const RowPlace rp = row_place<G>(h.row, i.row, lane);
+      r.sound = rp.count > 0 && !n.dead && n.nbits >= hdr_of(rp);
+      const uint32_t* w = a.stream + (size_t)i.k * a.cap_words + (r.sound ? n.off : 0ull);
+      if (r.sound) {
+        r.norm = __uint_as_float(w[0]);
+        r.field = w[1 + (rp.s >> 1)];
+      }
+      const uint32_t s_first = __shfl_sync(0xffffffffu, r.sound ? rp.s : 0u, 0);
+      const uint32_t* w0 = reinterpret_cast<const uint32_t*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(w), 0)) + 1 + lane;
+#pragma unroll
+      for (int t = 0; t < kAhead; ++t)
+        if ((uint32_t)lane * 2u + 64u * (uint32_t)t < s_first) r.before[t] = w0[32 * t];
+    }
+    return r;
+  };
+
+  uint32_t it = blockIdx.x + gridDim.x * (uint32_t)warp;
+  Bucket bucket = ask_bucket(it);
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(a.pair);
+    const int n = (int)((h.pair_mask + 4u) >> 4);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) reinterpret_cast<uint4*>(s_raw)[i] = __ldg(src + i);
+  }
+  __syncthreads();
+  const WalkTable wt{sa, h.pair_mask};
+  Header header = ask_header(it, bucket);
+  Bucket next_bucket = ask_bucket(it + stride);
+  bool bad = false;
+  for (; it < h.items; it += stride) {
+    const Item i = item_of(it);
+    const RowPlace rp = row_place<G>(h.row, i.row, lane);
+    const uint32_t hdr = hdr_of(rp), nsub = (hdr - (uint32_t)kNormBits) / 16u;
+    // where the lane's sub-block starts
+    const uint32_t len = (header.field >> (16u * (rp.s & 1u))) & 0xffffu;
+    const uint32_t s_first = __shfl_sync(0xffffffffu, header.sound ? rp.s : 0u, 0);
+    uint32_t before = 0;
+    if (s_first != 0u) {
+      const uint32_t half = s_first >> 1;                              // an odd number: the last word counts by its low half
+#pragma unroll
+      for (int t = 0; t < kAhead; ++t) before = __dp2a_lo(header.before[t], (uint32_t)(lane + 32 * t) == half ? 0x0001u : 0x0101u, before);
+      if (s_first > 64u * kAhead) {
+        const uint32_t* w0 = a.stream + (size_t)i.k * a.cap_words + __shfl_sync(0xffffffffu, (unsigned long long)bucket.off, 0) + 1;
+        for (uint32_t j = (uint32_t)lane + 32u * kAhead; 2u * j < s_first; j += 32u) before = __dp2a_lo(w0[j], j == half ? 0x0001u : 0x0101u, before);
+      }
+      before = __reduce_add_sync(0xffffffffu, before);
+    }
+    const uint32_t excl = warp_incl_scan(len, lane) - len;
+    const uint32_t excl0 = __shfl_sync(0xffffffffu, excl, rp.s <= (uint32_t)lane ? lane - (int)rp.s : 0);   // at the bucket's first lane
+    const uint32_t start = hdr + (excl - excl0) + (rp.s > (uint32_t)lane ? before : 0u);
+    bool ok = header.sound && len <= h.max_bits && start + len <= bucket.nbits && (rp.s + 1u < nsub || start + len == bucket.nbits);
+    // its words: from the buffer's 16-byte grid, the worker's first word being `mis` words past it
+    const uint32_t mis = h.wide ? (uint32_t)(((size_t)i.k * a.cap_words) & 3u) : 0u;
+    const uint32_t* base = a.stream + (size_t)i.k * a.cap_words - mis;
+    const unsigned long long limit = (unsigned long long)(a.K - (int)i.k) * a.cap_words + mis;      // words to the buffer's end
+    const unsigned long long mine = bucket.off + mis + ((start - 2u) >> 5);
+    const unsigned oks = __ballot_sync(0xffffffffu, ok);
+    uint32_t at = row_sa;
+    if (oks) {
+      const unsigned long long first = __shfl_sync(0xffffffffu, mine, __ffs((int)oks) - 1) & ~3ull;
+      const unsigned long long last = __shfl_sync(0xffffffffu, bucket.off + mis + ((start + len + 31u) >> 5), 31 - __clz((int)oks)) + WalkReach<G>::kWords;
+      const uint32_t n4 = (uint32_t)min((unsigned long long)h.row_words, last - first + 3ull) >> 2;
+      if (h.wide) {
+        for (uint32_t c = (uint32_t)lane; c < n4; c += 32u) {
+          const unsigned long long from = first + 4ull * c;
+          const int bytes = from >= limit ? 0 : (int)min(16ull, (limit - from) * 4ull);
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(row_sa + 16u * c), "l"(base + (bytes > 0 ? from : 0ull)), "r"(bytes) : "memory");
+        }
+      } else {
+        for (uint32_t c = (uint32_t)lane; c < 4u * n4; c += 32u) {
+          const unsigned long long from = first + c;
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(row_sa + 4u * c), "l"(base + (from < limit ? from : 0ull)), "r"(from < limit ? 4 : 0) : "memory");
+        }
+      }
+      ok = ok && mine - first + WalkReach<G>::kWords <= 4ull * n4;     // (not where lengths in between are absurd)
+      at = row_sa + 4u * (uint32_t)(ok ? mine - first : 0ull);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (rp.count > 0 && rp.s == 0u) a.norms[(size_t)i.k * a.nb + rp.b] = header.norm;
+    bad = bad || (rp.count > 0 && !ok && !bucket.dead);
+    const Header next_header = ask_header(it + stride, next_bucket);
+    const Bucket later_bucket = ask_bucket(it + 2u * stride);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    if (ok) {
+      Walk<true> w;
+      w.open(at, (start - 2u) & 31u);
+      if (rp.count == G) walk_whole<G>(w, my_sym, wt);
+      else walk_some(w, rp.count, my_sym, wt);
+      bad = bad || w.taken(at, (start - 2u) & 31u) != len;             // every sub-block uses exactly its length
+    } else {
+#pragma unroll 1
+      for (int q = 0; q < kWords; ++q) sts32(my_sym + 4u * (uint32_t)q, 0u);
+    }
+    __syncwarp();
+    // the row's symbols, a word per lane and store
+    const size_t e0 = (size_t)i.row * (size_t)(32 * G);
+    const uint32_t n = (uint32_t)min((size_t)(32 * G), a.d - e0);
+    uint8_t* out = a.sym + (size_t)i.k * a.d + e0;
+    const uint32_t shift = (uint32_t)(reinterpret_cast<uintptr_t>(out) & 3u);            // bytes past the word that `out` lies in
+    uint32_t marks = 0;
+    auto word = [&](uint32_t q) { return lds32(sym_sa + 4u * (q + q / (uint32_t)kWords)); };
+    if (shift == 0u) {
+      for (uint32_t q = (uint32_t)lane; q < n / 4u; q += 32u) {
+        const uint32_t x = word(q);
+        marks |= x;
+        reinterpret_cast<uint32_t*>(out)[q] = x & 0xbfbfbfbfu;
+      }
+    } else {
+      uint32_t* words = reinterpret_cast<uint32_t*>(out - shift);
+      for (uint32_t q = 1u + (uint32_t)lane; 4u * q + 4u <= n + shift; q += 32u) {
+        const uint32_t x = __funnelshift_l(word(q - 1u), word(q), 8u * shift);
+        marks |= x;
+        words[q] = x & 0xbfbfbfbfu;
+      }
+    }
+    // the bytes before the first whole word and after the last
+    const uint32_t head = shift == 0u ? 0u : min(4u - shift, n), tail = head == n ? n : n - ((n + shift) & 3u);
+    const uint32_t e = (uint32_t)lane < head ? (uint32_t)lane : tail + ((uint32_t)lane - head);
+    if (e < n) {
+      const uint32_t x = (word(e >> 2) >> (8u * (e & 3u))) & 0xffu;
+      marks |= x;
+      if ((uint32_t)lane < head || e - tail < 4u) out[e] = (uint8_t)(x & 0xbfu);
+    }
+    bad = bad || (marks & (kNoSymbol * 0x01010101u)) != 0u;
+    __syncwarp();
+    bucket = next_bucket;
+    header = next_header;
+    next_bucket = later_bucket;
+  }
+  if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
+}
+
+bool unpack_rows_fits(int K, size_t d, int bucket, const CodeTable& ct) {
+  return ct.has_header && (ct.G == 32 || ct.G == 64 || ct.G == 128) && bucket % ct.G == 0 &&
+         (unsigned long long)K * ((d + (size_t)ct.G * 32 - 1) / ((size_t)ct.G * 32)) < (1ull << 31);
+}
+
+template <int G>
+static qgx_status launch_unpack_g(qgx_ctx* c, const UnpackRowsArgs& a, int bucket, const CodeTable& ct) {
+  UnpackShape h;
+  if (!make_row_shape(a.d, bucket, G, a.nb, &h.row)) return QGX_ERR_INVALID_ARG;
+  h.items = h.row.rows * (uint32_t)a.K;
+  h.pair_mask = (4u << pair_bits(ct.maxlen)) - 4u;
+  h.max_bits = (uint32_t)(G * (ct.maxlen + 1));
+  h.wide = (reinterpret_cast<uintptr_t>(a.stream) & 15u) == 0;
+  h.row_words = row_words_worst(G, ct.maxlen);
+  // as many warps as the SM's shared memory holds rows of (at least 16), and as there are rows for
+  const uint32_t table = 4u << pair_bits(ct.maxlen), each = sym_row_bytes<G>() + 4u * h.row_words;
+  uint32_t warps = std::min(32u, (224u * 1024u - table) / each);
+  const uint32_t per_sm = (h.items + (uint32_t)c->num_sms - 1u) / (uint32_t)c->num_sms;
+  warps = std::max(1u, std::min(warps, per_sm));
+  h.off_sym = table;
+  h.off_row = table + warps * sym_row_bytes<G>();
+  const size_t smem = table + (size_t)warps * each;
+  const unsigned grid = std::min((uint32_t)c->num_sms, h.items);
+  allow_max_dynamic_smem((const void*)k_unpack_rows<G>, c->device);
+  k_unpack_rows<G><<<grid, 32 * warps, smem, c->stream>>>(a, h);
+  count_launch(c);
+  return cuda_status(cudaGetLastError());
+}
+qgx_status launch_unpack_rows(qgx_ctx* c, const UnpackRowsArgs& a, int bucket, const CodeTable& ct) {
+  if (ct.G == 32) return launch_unpack_g<32>(c, a, bucket, ct);
+  if (ct.G == 64) return launch_unpack_g<64>(c, a, bucket, ct);
+  return launch_unpack_g<128>(c, a, bucket, ct);
+}
+
+}  // namespace qgx

@@ -1,0 +1,34 @@
+// qgx_decode by rows of sub-blocks (qgx_unpack.cu).
+#pragma once
+
+#include "qgx_walk.cuh"
+
+namespace qgx {
+
+constexpr uint32_t kNoSymbol = 0x40u;    // the byte of bits that no codeword starts like (no symbol has bit 6)
+
+// The pair table of a code (see DecodeTables) with symbol bytes as qgx_encode takes them, by threads first, first + 1, ... of `stride`
+__device__ __forceinline__ void build_unpack_pairs(const CodeTable& ct, uint32_t* pair, uint32_t first, uint32_t stride) {
+  const auto symbol = [](const NextSymbol& s) { return s.known ? s.level | (s.negative ? 0x80u : 0u) : kNoSymbol; };
+  for (uint32_t i = first; i < (1u << pair_bits(ct.maxlen)); i += stride) pair[i] = pair_entry_of(i, ct, symbol);
+}
+
+struct UnpackRowsArgs {
+  const uint32_t* stream;                // [K][cap_words]
+  size_t cap_words;
+  const uint32_t* bucket_bits;           // [K][nb]
+  const uint64_t* off;                   // [K][nb], their words' sums
+  const uint32_t* flags;                 // [K], nonzero: the sums exceed cap_words
+  const uint32_t* pair;                  // see build_unpack_pairs
+  size_t d;
+  int K;
+  size_t nb;
+  float* norms;
+  uint8_t* sym;
+  DevStatus* st;
+};
+
+bool unpack_rows_fits(int K, size_t d, int bucket, const CodeTable& ct);
+qgx_status launch_unpack_rows(qgx_ctx* c, const UnpackRowsArgs& a, int bucket, const CodeTable& ct);
+
+}  // namespace qgx

@@ -55,3 +55,35 @@ def test_decode_pass_matches_oracle(K, d, bucket, nlev, sub, code):
         qgx.qgx_sync_status(ctx)
     finally:
         qgx.qgx_destroy(ctx)
+
+
+@pytest.mark.parametrize("shift", [0, 1])                   # words by which the stream buffer misses 16 bytes
+@pytest.mark.parametrize("K,d,bucket,nlev,sub,code", CASES + [(1, 2048 + 3, 2048, 9, 64, "fixed"), (3, 2, 128, 9, 32, "fixed"),
+                                                              (5, 4 * 1024 + 2, 1024, 17, 32, "steep")])
+def test_separate_decode_and_average(K, d, bucket, nlev, sub, code, shift):
+    """The four calls on the same shapes: decode inverts encode whatever the alignment of streams, symbols and rows."""
+    import paper_2308_09187_b200 as qgx
+    ctx = qgx.qgx_create(0)
+    try:
+        rng = np.random.default_rng(d)
+        v = gen.gaussian_mixture((K, d), seed=d + 2, device="cuda")
+        lev = np.r_[0.0, np.sort(rng.uniform(1e-3, 0.2, size=nlev - 2)), 1.0].astype(np.float32)
+        if code == "fixed":
+            cb = qgx.qgx_build_codebook_fixed(nlev, sub)
+        elif code == "elias":
+            cb = qgx.qgx_build_codebook_elias(nlev, sub)
+        else:
+            cb = qgx.qgx_build_codebook_huffman([2.0 ** -(j + 1) for j in range(nlev)], sub)
+        norms, sym = qgx.qgx_quantize(ctx, v, bucket, lev, qgx.QGX_NORM_L2, 3, 1)
+        _, bits, _ = qgx.qgx_encode(ctx, norms, sym, bucket, cb)
+        used = int(((bits.long() + 31) // 32).sum(dim=1).max())
+        room = torch.zeros(K * used + shift, dtype=torch.int32, device="cuda")     # no word to spare at its end
+        stream, bits, _ = qgx.qgx_encode(ctx, norms, sym, bucket, cb, stream=room[shift:].view(K, used), cap_words=used)
+        got_norms, got = qgx.qgx_decode(ctx, stream, bits, d, bucket, cb)
+        qgx.qgx_sync_status(ctx)
+        assert torch.equal(got_norms, norms) and torch.equal(got, sym)
+        mean = qgx.qgx_average(ctx, norms, sym, bucket, lev)
+        qgx.qgx_sync_status(ctx)
+        assert np.array_equal(mean.cpu().numpy(), o.average(norms.cpu().numpy(), sym.cpu().numpy(), bucket, lev))
+    finally:
+        qgx.qgx_destroy(ctx)
