@@ -43,6 +43,7 @@ struct qgx_ctx {
   int keep_symbols;                      // qgx_exchange keeps its decoded symbols too (qgx_set_keep_symbols)
   int wait_limit;                        // polls of a device-side wait before it gives up (qgx_set_wait_limit)
   size_t skip_buckets;                   // diagnostic: the next exchange leaves these first buckets unencoded
+  int add_totals;                        // set around the exchange of a tensor: its bits are added to the caller's totals
   int decode_only;                       // set around the decode-only entry point
   int sym_nlev;                          // the level table those symbols were quantized with
   float sym_levels[QGX_MAX_LEVELS];

@@ -168,6 +168,12 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     fill_signed_values(reinterpret_cast<float*>(s_raw + h.off_val), lt);
     if (kCompare) fill_signed_values(reinterpret_cast<float*>(s_raw + h.off_kept), lt_kept);
   }
+  if (blockIdx.x == 0 && a.total_out) {
+    for (int k = threadIdx.x; k < a.K; k += blockDim.x) {
+      if (a.total_add) atomicAdd(a.total_out + k, a.total_bits[k]);
+      else a.total_out[k] = a.total_bits[k];
+    }
+  }
   __syncthreads();
   const WalkTable wt{sa, h.pair_mask};
   const uint32_t val_sa = sa + h.off_val, kept_sa = sa + h.off_kept;

@@ -30,6 +30,9 @@ struct DecodeArgs {
   size_t sym_ld;                // a multiple of 4, at least d
   const float* norms_prev;      // [K][nb]
   double* sum_sq;
+  const unsigned long long* total_bits;   // [K], as the encode pass left them, and the caller's copy or null
+  unsigned long long* total_out;
+  int total_add;                // added to what is there
   DevStatus* st;
 };
 

@@ -289,14 +289,15 @@ namespace qgx {
 
 // workspace slots of a context
 enum { WS_OFF64 = 0, WS_FLAGS = 1, WS_LUT = 2, WS_SLOT0 = 3 /* stream, bits, offsets, total: 3..6 and 7..10 */,
-       WS_NORMS = 12, WS_SYM = 13, WS_NORMS2 = 14, WS_OPVAL = 15, WS_MEAN = 16, WS_SEGBITS = 19, WS_SMALL = 23 };
+       WS_NORMS = 12, WS_SYM = 13, WS_NORMS2 = 14, WS_OPVAL = 15, WS_MEAN = 16, WS_SMALL = 23 };
 
 // ---- what a call derives from a quantizer configuration, kept between calls --------------------
 // Building the rounding table, the code table and the decoder table and copying the latter to the device costs
 // more host time than a small exchange; iterations reuse a handful of configurations, so the results are kept,
-// keyed by the configuration's contents (compared in full on a hit).
+// keyed by the configuration's contents (compared in full on a hit); the one not used for longest makes room.  (With a
+// slot per hash two of sixteen tensors' tables collided and were built again in every layer-wise exchange.)
 struct CachedTables {
-  bool valid;
+  uint64_t hash, used;                  // of the contents; the cache's clock at the last use (0: empty)
   int nlev, bucket;
   float levels[QGX_MAX_LEVELS];
   qgx_codebook cb;
@@ -309,6 +310,7 @@ constexpr int kTableCacheSlots = 32;
 struct LaunchShape { size_t smem; int per_sm; };      // smem == 0: not asked yet
 struct TableCache {
   CachedTables e[kTableCacheSlots];
+  uint64_t clock;
   LaunchShape enc[3][3];                // [octets per thread 1, 2, 4][sub-block 32, 64, 128]
 };
 
@@ -354,20 +356,32 @@ static qgx_status cached_tables(qgx_ctx* c, const qgx_quant_cfg* cfg, const Cach
   TableCache* tc = table_cache(c);
   if (!tc) return QGX_ERR_CUDA;
   uint64_t h = 1469598103934665603ull;
-  auto mix = [&](const void* p, size_t n) {
-    const unsigned char* b = (const unsigned char*)p;
-    for (size_t i = 0; i < n; ++i) { h ^= b[i]; h *= 1099511628211ull; }
+  auto mix = [&](const void* p, size_t words) {
+    for (size_t i = 0; i < words; ++i) {
+      uint32_t w;
+      std::memcpy(&w, (const unsigned char*)p + 4 * i, 4);
+      h = (h ^ w) * 1099511628211ull;
+    }
   };
-  mix(&cfg->nlev, sizeof(int)); mix(&cfg->bucket, sizeof(int)); mix(cfg->levels, sizeof(float) * (size_t)cfg->nlev);
-  mix(&cfg->cb.subblock, sizeof(int)); mix(cfg->cb.len, (size_t)cfg->nlev); mix(cfg->cb.code, sizeof(uint32_t) * (size_t)cfg->nlev);
-  CachedTables* e = &tc->e[h % kTableCacheSlots];
-  const bool hit = e->valid && e->nlev == cfg->nlev && e->bucket == cfg->bucket && e->cb.nlev == cfg->cb.nlev &&
-                   e->cb.subblock == cfg->cb.subblock &&
-                   std::memcmp(e->levels, cfg->levels, sizeof(float) * (size_t)cfg->nlev) == 0 &&
-                   std::memcmp(e->cb.len, cfg->cb.len, (size_t)cfg->nlev) == 0 &&
-                   std::memcmp(e->cb.code, cfg->cb.code, sizeof(uint32_t) * (size_t)cfg->nlev) == 0;
+  mix(&cfg->nlev, 1); mix(&cfg->bucket, 1); mix(&cfg->cb.subblock, 1);
+  mix(cfg->levels, (size_t)cfg->nlev); mix(cfg->cb.code, (size_t)cfg->nlev);
+  h ^= h >> 32;
+  CachedTables* e = nullptr;
+  for (CachedTables& t : tc->e)
+    if (t.used && t.hash == h && t.nlev == cfg->nlev && t.bucket == cfg->bucket && t.cb.nlev == cfg->cb.nlev && t.cb.subblock == cfg->cb.subblock &&
+        std::memcmp(t.levels, cfg->levels, sizeof(float) * (size_t)cfg->nlev) == 0 && std::memcmp(t.cb.len, cfg->cb.len, (size_t)cfg->nlev) == 0 &&
+        std::memcmp(t.cb.code, cfg->cb.code, sizeof(uint32_t) * (size_t)cfg->nlev) == 0) {
+      e = &t;
+      break;
+    }
+  const bool hit = e != nullptr;
   if (!hit) {
-    e->valid = false;
+    e = &tc->e[0];
+    for (CachedTables& t : tc->e)
+      if (t.used < e->used) e = &t;
+  }
+  if (!hit) {
+    e->used = 0;
     qgx_status rc = make_code_table(&cfg->cb, cfg->bucket, &e->ct);
     if (rc != QGX_OK) return rc;
     make_round_table(cfg->levels, cfg->nlev, &e->rt);
@@ -391,8 +405,9 @@ static qgx_status cached_tables(qgx_ctx* c, const qgx_quant_cfg* cfg, const Cach
     e->bucket = cfg->bucket;
     std::memcpy(e->levels, cfg->levels, sizeof(e->levels));
     e->cb = cfg->cb;
-    e->valid = true;
+    e->hash = h;
   }
+  e->used = ++tc->clock;
   *out = e;
   return QGX_OK;
 }
@@ -485,7 +500,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     sm.mean = mean_out;
     sm.update = upd ? upd->mode : 0; sm.xin = upd ? upd->xin : nullptr; sm.xout = upd ? upd->xout : nullptr; sm.scalars = upd ? upd->scalars : nullptr;
     sm.sym_out = sym_out; sm.sym_prev = sym_prev; sm.sym_ld = sym_ld; sm.norms_prev = norms_prev;
-    sm.sum_sq = sum_sq; sm.square = (sym_mode & 4) ? 1 : 0; sm.total_out = total_bits_out;
+    sm.sum_sq = sum_sq; sm.square = (sym_mode & 4) ? 1 : 0; sm.total_out = (unsigned long long*)total_bits_out; sm.total_add = c->add_totals;
     ScopedKernelTimer timer(c, QGX_KERNEL_ENCODE);
     c->skip_buckets = 0;
     return launch_exchange_small(c, es, sm, lt, lt_kept, ct, key, qt);
@@ -552,16 +567,13 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
 #undef QGX_LAUNCH_EG
 #undef QGX_LAUNCH_E
   if (cudaGetLastError() != cudaSuccess) return QGX_ERR_CUDA;
-  if (total_bits_out &&
-      cudaMemcpyAsync(total_bits_out, tot, sizeof(uint64_t) * (size_t)K, cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)
-    return QGX_ERR_CUDA;
-
   DecodeArgs da;
   da.stream = stream; da.cap_words = cap; da.bucket_bits = bbits; da.offsets = offs;
   da.sym_out = sym_out; da.sym_prev = sym_prev; da.sym_ld = sym_ld; da.norms_prev = norms_prev; da.sum_sq = sum_sq;
   da.d = d; da.bucket = bucket; da.K = K; da.nb = nb; da.tables = tables->dec_dev; da.mean = mean_out;
   da.update = upd ? upd->mode : 0; da.xin = upd ? upd->xin : nullptr; da.xout = upd ? upd->xout : nullptr;
   da.scalars = upd ? upd->scalars : nullptr; da.st = c->dstatus;
+  da.total_bits = tot; da.total_out = (unsigned long long*)total_bits_out; da.total_add = c->add_totals;
   da.vec_out = ((reinterpret_cast<uintptr_t>(mean_out) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(da.xin) & 15u) == 0) &&
                ((reinterpret_cast<uintptr_t>(da.xout) & 15u) == 0);
   return launch_exchange_decode(c, da, ct, lt, lt_kept, sym_mode);
@@ -671,12 +683,6 @@ __global__ void __launch_bounds__(256) k_level_counts(const uint8_t* __restrict_
   if (mine) atomicAdd(counts + (threadIdx.x & 31), (unsigned long long)mine);
 }
 
-// acc[i] += x[i]; several streams may add into the same totals
-__global__ void k_add_u64_atomic(unsigned long long* acc, const unsigned long long* x, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) atomicAdd(acc + i, x[i]);
-}
-
 }  // namespace qgx
 
 using namespace qgx;
@@ -747,20 +753,12 @@ qgx_status qgx_exchange_segments(qgx_ctx* c, const float* v, int K, size_t d, co
   int rc_seg = nseg;                                    // the first segment that failed decides the status
   for (int s : order) {
     qgx_ctx* h = sc ? sc->ctx[lane_of[(size_t)s]] : c;
-    uint64_t* seg_bits = nullptr;
-    if (total_bits) {
-      seg_bits = (uint64_t*)ws_get(h, WS_SEGBITS, sizeof(uint64_t) * (size_t)K);
-      if (!seg_bits) { rc = QGX_ERR_CUDA; break; }
-    }
     DualSource src{v + segs[s].offset, nullptr, d, 0};
     if (sc) h->skip_buckets = c->skip_buckets;          // the diagnostic: of every tensor
-    const qgx_status mine = exchange_impl(h, src, K, segs[s].length, segs[s].cfg, exchange_id, 0, mean_out + segs[s].offset, seg_bits,
+    h->add_totals = 1;                                  // several streams add into the same totals
+    const qgx_status mine = exchange_impl(h, src, K, segs[s].length, segs[s].cfg, exchange_id, 0, mean_out + segs[s].offset, total_bits,
                                           nullptr, 0, nullptr, segs[s].offset);
-    if (mine == QGX_OK && total_bits) {
-      k_add_u64_atomic<<<(K + 255) / 256, 256, 0, h->stream>>>(reinterpret_cast<unsigned long long*>(total_bits),
-                                                               reinterpret_cast<const unsigned long long*>(seg_bits), K);
-      count_launch(h);
-    }
+    h->add_totals = 0;
     if (mine != QGX_OK && s < rc_seg) { rc = mine; rc_seg = s; }
     if (sc) h->skip_buckets = 0;                        // (left over where the call refused its arguments)
   }

@@ -220,7 +220,10 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
       if (b + 1 == a.nb) {
         const unsigned long long bits = 32ull * words - (incl >> kPadShift);
         a.total_bits[k] = bits;
-        if (r.total_out) r.total_out[k] = bits;
+        if (r.total_out) {
+          if (r.total_add) atomicAdd(r.total_out + k, bits);
+          else r.total_out[k] = bits;
+        }
       }
       s_prefix = at;
       s_skip = timed_out || over ? 1 : 0;

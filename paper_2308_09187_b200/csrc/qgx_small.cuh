@@ -21,7 +21,8 @@ struct SmallArgs {
   const float* norms_prev;
   double* sum_sq;
   int square;                            // add the squared values themselves
-  uint64_t* total_out;                   // the caller's copy of the totals, or null
+  unsigned long long* total_out;         // the caller's copy of the totals, or null
+  int total_add;                         // added to what is there
   uint32_t img_words, off_img, off_sym, off_tab;
 };
 
