@@ -101,6 +101,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_offsets(const uint32_t* _
                                                                uint64_t* __restrict__ off, uint64_t* __restrict__ total_bits,
                                                                uint32_t* __restrict__ flags, unsigned int err_code, DevStatus* st,
                                                                int K, const __grid_constant__ CodeTable ct, uint16_t* table, uint32_t* pair) {
+  start_next();
+  await_previous();
   if (blockIdx.x >= (unsigned)K) {
     if (pair) build_unpack_pairs(ct, pair, (blockIdx.x - (unsigned)K) * kScanThreads + threadIdx.x, kPairBuilders * kScanThreads);
     else build_unpack_table(ct, table);
@@ -411,6 +413,8 @@ struct UnpackArgs {
 // take: sub-blocks of other lengths, or none.  Every read is bounded by the bucket's words.  A serial walk per thread: latency-bound with few sub-blocks, instruction-bound (14 per symbol) with many.
 __global__ void __launch_bounds__(128) k_unpack(const __grid_constant__ UnpackArgs a, const __grid_constant__ CodeTable ct) {
   extern __shared__ __align__(16) uint16_t s_tab[];  // [2 << maxlen], see build_unpack_table
+  start_next();
+  await_previous();
   const int tab_n = 2 << ct.maxlen;
   for (int i = threadIdx.x; i < (tab_n + 7) / 8; i += blockDim.x) reinterpret_cast<uint4*>(s_tab)[i] = __ldg(reinterpret_cast<const uint4*>(a.table) + i);
   __syncthreads();
@@ -637,8 +641,8 @@ qgx_status qgx_decode(qgx_ctx* c, const uint32_t* stream, size_t cap_words, cons
   const bool rows = unpack_rows_fits(K, d, bucket, ct);
   void* table = ws_get(c, 2, std::max(sizeof(uint16_t) * (size_t)kUnpackTableMax, sizeof(uint32_t) << kPairBitsMax));
   if (!off || !flags || !table) return QGX_ERR_CUDA;
-  k_scan_offsets<<<K + (rows ? kPairBuilders : 1u), kScanThreads, 0, c->stream>>>(bucket_bits, nb, cap_words, off, nullptr, flags, QGX_ERR_CORRUPT,
-                                                                                  c->dstatus, K, ct, (uint16_t*)table, rows ? (uint32_t*)table : nullptr);
+  launch_next(true, k_scan_offsets, K + (rows ? kPairBuilders : 1u), kScanThreads, 0, c->stream, bucket_bits, nb, cap_words, off, nullptr, flags,
+              QGX_ERR_CORRUPT, c->dstatus, K, ct, (uint16_t*)table, rows ? (uint32_t*)table : nullptr);
   if (rows) {
     count_launch(c);
     const UnpackRowsArgs r{stream, cap_words, bucket_bits, off, flags, (const uint32_t*)table, d, K, nb, norms, sym, c->dstatus};
@@ -660,7 +664,7 @@ qgx_status qgx_decode(qgx_ctx* c, const uint32_t* stream, size_t cap_words, cons
   const size_t warps = spb > 32 ? nb * (size_t)K * ((spb + 31) / 32) : (nb * (size_t)K * lanes + 31) / 32;
   const size_t smem = std::max<size_t>(16, sizeof(uint16_t) * ((size_t)2 << ct.maxlen));
   const unsigned grid = (unsigned)std::max<size_t>(1, std::min<size_t>((warps + 3) / 4, (size_t)c->num_sms * 12u));
-  k_unpack<<<grid, 128, smem, c->stream>>>(a, ct);
+  launch_next(true, k_unpack, grid, 128, smem, c->stream, a, ct);
   count_launch(c, 2);
   return cuda_status(cudaGetLastError());
 }

@@ -35,6 +35,7 @@ struct qgx_ctx {
   size_t slot_cap_words[2];
   int slot_K[2];
   size_t slot_nb[2];
+  int scan_dirty[2];                     // the slot's sums and scan words are not known to be zero
   // which exchange slot last kept its symbols in the workspace (-1: none), and for what shape
   int sym_slot;
   int sym_K;
@@ -43,6 +44,7 @@ struct qgx_ctx {
   int keep_symbols;                      // qgx_exchange keeps its decoded symbols too (qgx_set_keep_symbols)
   int wait_limit;                        // polls of a device-side wait before it gives up (qgx_set_wait_limit)
   size_t skip_buckets;                   // diagnostic: the next exchange leaves these first buckets unencoded
+  int helper;                            // runs a tensor of a layer-wise exchange: no CTA waits on an SM that another stream could use
   int add_totals;                        // set around the exchange of a tensor: its bits are added to the caller's totals
   int decode_only;                       // set around the decode-only entry point
   int sym_nlev;                          // the level table those symbols were quantized with
@@ -68,6 +70,29 @@ struct qgx_ctx {
 };
 
 namespace qgx {
+
+// ---- kernels that start while the one before them in the stream ends ---------------------------
+// The kernels of an iteration or an exchange follow one another without anything in between, many of them short.  Launched by
+// launch_next, a kernel's CTAs may start as soon as all CTAs of the kernel before have called start_next (or are gone): they
+// bring in their tables and then wait in await_previous, in every thread that goes on, before they touch anything that a
+// kernel before them writes, reads or leaves behind; all of its stores are visible then, and by the same rule those of the
+// kernels before it.  Tables that a call builds itself are not brought in early: see `fresh` in qgx_exchange.cu.
+__device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void await_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch_next(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
 
 // ---- level table and code tables handed to kernels by value ---------------------------------
 struct LevelTable {

@@ -168,13 +168,22 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     fill_signed_values(reinterpret_cast<float*>(s_raw + h.off_val), lt);
     if (kCompare) fill_signed_values(reinterpret_cast<float*>(s_raw + h.off_kept), lt_kept);
   }
-  if (blockIdx.x == 0 && a.total_out) {
+  __syncthreads();
+  start_next();
+  await_previous();
+  // for the next exchange's scan and totals; nobody reads them after the encode pass
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.scan_words; i += (size_t)gridDim.x * blockDim.x) a.scan[i] = 0ull;
+  if (blockIdx.x == 0 && a.sums) {
     for (int k = threadIdx.x; k < a.K; k += blockDim.x) {
-      if (a.total_add) atomicAdd(a.total_out + k, a.total_bits[k]);
-      else a.total_out[k] = a.total_bits[k];
+      const unsigned long long bits = a.sums[k];
+      a.sums[k] = 0ull;
+      a.total_bits[k] = bits;
+      if (a.total_out) {
+        if (a.total_add) atomicAdd(a.total_out + k, bits);
+        else a.total_out[k] = bits;
+      }
     }
   }
-  __syncthreads();
   const WalkTable wt{sa, h.pair_mask};
   const uint32_t val_sa = sa + h.off_val, kept_sa = sa + h.off_kept;
   const uint32_t my_sym = sa + h.off_sym + (uint32_t)warp * sym_row_bytes<G>() + (uint32_t)lane * (uint32_t)(kStride * 4);
@@ -364,7 +373,7 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
 
 // ---- launch -----------------------------------------------------------------------------------
 template <int G>
-static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, const LevelTable& lt_kept, int sym_mode) {
+static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, const LevelTable& lt_kept, int sym_mode, bool early) {
   DecodeShape h;
   h.minus_zero = kMinusZero2;
   if (!make_row_shape(da.d, da.bucket, G, da.nb, &h.row)) return QGX_ERR_INVALID_ARG;
@@ -395,7 +404,7 @@ static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTa
 #define QGX_LAUNCH_D(SS)                                                                                  \
   do {                                                                                                    \
     allow_max_dynamic_smem((const void*)k_exchange_decode<G, SS>, c->device);                             \
-    k_exchange_decode<G, SS><<<grid, 32 * warps, smem, c->stream>>>(da, h, lt, lt_kept);                  \
+    launch_next(early, k_exchange_decode<G, SS>, grid, 32 * warps, smem, c->stream, da, h, lt, lt_kept);  \
   } while (0)
   switch (sym_mode) {
     case 1: QGX_LAUNCH_D(1); break;
@@ -411,12 +420,12 @@ static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTa
 }
 
 qgx_status launch_exchange_decode(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, const LevelTable& lt_kept,
-                                  int sym_mode) {
+                                  int sym_mode, bool early) {
   if (!ct.has_header || da.bucket % ct.G != 0) return QGX_ERR_INVALID_ARG;
   switch (ct.G) {
-    case 32: return launch_decode_g<32>(c, da, ct, lt, lt_kept, sym_mode);
-    case 64: return launch_decode_g<64>(c, da, ct, lt, lt_kept, sym_mode);
-    case 128: return launch_decode_g<128>(c, da, ct, lt, lt_kept, sym_mode);
+    case 32: return launch_decode_g<32>(c, da, ct, lt, lt_kept, sym_mode, early);
+    case 64: return launch_decode_g<64>(c, da, ct, lt, lt_kept, sym_mode, early);
+    case 128: return launch_decode_g<128>(c, da, ct, lt, lt_kept, sym_mode, early);
     default: return QGX_ERR_INVALID_ARG;
   }
 }

@@ -30,17 +30,22 @@ struct DecodeArgs {
   size_t sym_ld;                // a multiple of 4, at least d
   const float* norms_prev;      // [K][nb]
   double* sum_sq;
-  const unsigned long long* total_bits;   // [K], as the encode pass left them, and the caller's copy or null
+  // what the encode pass summed up, [K], or null; cleared here, as its scan's words are, for the next exchange
+  unsigned long long* sums;
+  unsigned long long* total_bits;   // [K], where the sums go, and the caller's copy of them or null
   unsigned long long* total_out;
   int total_add;                // added to what is there
+  unsigned long long* scan;
+  size_t scan_words;
   DevStatus* st;
 };
 
 // sym_mode, a set of bits: 1 keeps the decoded symbols; 2 adds the squared differences between the vectors kept by an
 // earlier exchange (whose level table is `lt_kept`) and the ones decoded now to *sum_sq; 4 adds the squared decoded values
-// themselves (an earlier vector of zero).  1 | 2 compares first and then overwrites the kept symbols in place.
+// themselves (an earlier vector of zero).  1 | 2 compares first and then overwrites the kept symbols in place.  early: see
+// launch_next.
 qgx_status launch_exchange_decode(qgx_ctx* c, const DecodeArgs& da, const CodeTable& ct, const LevelTable& lt, const LevelTable& lt_kept,
-                                  int sym_mode);
+                                  int sym_mode, bool early);
 void launch_build_decode_tables(const CodeTable& ct, DecodeTables* out, cudaStream_t stream);
 
 }  // namespace qgx

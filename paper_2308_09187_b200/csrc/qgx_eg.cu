@@ -51,6 +51,8 @@ __device__ __forceinline__ double gemv_row(const float* __restrict__ m, size_t n
 __global__ void __launch_bounds__(256) k_gemv_rows(const float* __restrict__ mat, size_t nrows, size_t ncols,
                                                    const float* __restrict__ x, const float* __restrict__ bias,
                                                    float* __restrict__ out, bool vec_ok) {
+  start_next();
+  await_previous();
   const int lane = threadIdx.x & 31;
   const size_t warp = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const size_t nwarps = ((size_t)gridDim.x * blockDim.x) >> 5;
@@ -66,6 +68,8 @@ __global__ void __launch_bounds__(256) k_gemv_rows(const float* __restrict__ mat
 __global__ void __launch_bounds__(1024) k_bilinear(const float* __restrict__ mat, size_t n, const float* __restrict__ z,
                                                    float* __restrict__ out_all, bool vec_ok) {
   __shared__ double s_part[32][33];
+  start_next();
+  await_previous();
   const int cx = threadIdx.x, ry = threadIdx.y;
   const size_t col_blocks = (n + 31) / 32;
   if (blockIdx.x >= col_blocks) {
@@ -105,6 +109,8 @@ __global__ void __launch_bounds__(1024) k_bilinear(const float* __restrict__ mat
 }
 
 __global__ void __launch_bounds__(256) k_diag(const float* __restrict__ D, const float* __restrict__ x, float* __restrict__ out, size_t d) {
+  start_next();
+  await_previous();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (size_t)gridDim.x * blockDim.x)
     out[i] = __fmul_rn(D[i], x[i]);
 }
@@ -122,6 +128,8 @@ __global__ void __launch_bounds__(256) k_eg_init(float* X, float* Y, float* Xbar
 __global__ void __launch_bounds__(256) k_eg_finish(float* __restrict__ X, const float* __restrict__ Y, float* __restrict__ Xbar,
                                                    const float* __restrict__ Xhalf, const float* __restrict__ anchor,
                                                    double* scalars, size_t d, int K, int t) {
+  start_next();
+  await_previous();
   const float gamma = (float)((double)K / sqrt(1.0 + scalars[0]));
   const float tf = (float)t;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (size_t)gridDim.x * blockDim.x) {
@@ -136,6 +144,8 @@ __global__ void __launch_bounds__(256) k_eg_finish(float* __restrict__ X, const 
 // X_{t+1/2} = X_t - gamma_t * m (optimistic dual averaging: m is the mean of the previous iteration's quantized vectors)
 __global__ void __launch_bounds__(256) k_half_from_mean(const float* __restrict__ X, const float* __restrict__ m,
                                                         const double* __restrict__ scalars, float* __restrict__ Xhalf, size_t d) {
+  start_next();
+  await_previous();
   const float gamma = (float)scalars[1];
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (size_t)gridDim.x * blockDim.x)
     Xhalf[i] = __fsub_rn(X[i], __fmul_rn(gamma, m[i]));
@@ -151,16 +161,16 @@ qgx_status apply_operator_impl(qgx_ctx* c, const qgx_operator* op, const float* 
   ScopedKernelTimer timer(c, QGX_KERNEL_OPERATOR);
   if (op->kind == QGX_OP_DENSE_AFFINE) {
     const bool vec_ok = (d % 4 == 0) && ((reinterpret_cast<uintptr_t>(op->mat) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(x) & 15u) == 0);
-    k_gemv_rows<<<grid_for(c, d * 32, 256), 256, 0, c->stream>>>(op->mat, d, d, x, op->bias, out, vec_ok);
+    launch_next(true, k_gemv_rows, grid_for(c, d * 32, 256), 256, 0, c->stream, op->mat, d, d, x, op->bias, out, vec_ok);
     count_launch(c);
   } else if (op->kind == QGX_OP_BILINEAR) {
     if (d % 2) return QGX_ERR_INVALID_ARG;
     const size_t n = d / 2;
     const bool vec_ok = (n % 4 == 0) && ((reinterpret_cast<uintptr_t>(op->mat) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(x + n) & 15u) == 0);
-    k_bilinear<<<(unsigned)(2 * ((n + 31) / 32)), dim3(32, 32), 0, c->stream>>>(op->mat, n, x, out, vec_ok);
+    launch_next(true, k_bilinear, (unsigned)(2 * ((n + 31) / 32)), dim3(32, 32), 0, c->stream, op->mat, n, x, out, vec_ok);
     count_launch(c);
   } else if (op->kind == QGX_OP_DIAGONAL) {
-    k_diag<<<grid_for(c, d, 256), 256, 0, c->stream>>>(op->mat, x, out, d);
+    launch_next(true, k_diag, grid_for(c, d, 256), 256, 0, c->stream, op->mat, x, out, d);
     count_launch(c);
   } else {
     return QGX_ERR_INVALID_ARG;
@@ -231,7 +241,7 @@ static qgx_status eg_step_impl(qgx_ctx* c, qgx_eg_state* st, const qgx_operator*
   if (rc != QGX_OK) return rc;
   {
     ScopedKernelTimer timer(c, QGX_KERNEL_FINISH);
-    k_eg_finish<<<grid_for(c, d, 256), 256, 0, c->stream>>>(st->X, st->Y, st->Xbar, st->Xhalf, st->anchor, st->scalars, d, K, st->t);
+    launch_next(true, k_eg_finish, grid_for(c, d, 256), 256, 0, c->stream, st->X, st->Y, st->Xbar, st->Xhalf, st->anchor, st->scalars, d, K, st->t);
   }
   count_launch(c);
   st->t += 1;
@@ -269,7 +279,7 @@ qgx_status qgx_family_step(qgx_ctx* c, qgx_eg_state* st, int method, const qgx_o
 
   if (method == QGX_METHOD_OPTDA && st->t > 1) {
     ScopedKernelTimer timer(c, QGX_KERNEL_FINISH);
-    k_half_from_mean<<<grid_for(c, d, 256), 256, 0, c->stream>>>(st->X, mean_prev, st->scalars, st->Xhalf, d);   // g_{k,t-1/2}
+    launch_next(true, k_half_from_mean, grid_for(c, d, 256), 256, 0, c->stream, st->X, mean_prev, st->scalars, st->Xhalf, d);   // g_{k,t-1/2}
     count_launch(c);
   } else {                                                                       // no earlier feedback: X_{t+1/2} = X_t
     if (cudaMemcpyAsync(st->Xhalf, st->X, sizeof(float) * d, cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess)
@@ -293,7 +303,7 @@ qgx_status qgx_family_step(qgx_ctx* c, qgx_eg_state* st, int method, const qgx_o
   if (rc != QGX_OK) return rc;
   {
     ScopedKernelTimer timer(c, QGX_KERNEL_FINISH);
-    k_eg_finish<<<grid_for(c, d, 256), 256, 0, c->stream>>>(st->X, st->Y, st->Xbar, st->Xhalf, st->anchor, st->scalars, d, K, st->t);
+    launch_next(true, k_eg_finish, grid_for(c, d, 256), 256, 0, c->stream, st->X, st->Y, st->Xbar, st->Xhalf, st->anchor, st->scalars, d, K, st->t);
   }
   count_launch(c);
   st->t += 1;

@@ -21,10 +21,10 @@ struct EncodeArgs {
   size_t cap_words;
   uint32_t* bucket_bits;        // [K][nb]
   uint32_t* offsets;            // [K][nb] word offset of each bucket
-  unsigned long long* total_bits;   // [K], zeroed before the launch
+  unsigned long long* total_bits;   // [K], zero before the launch
   float* norms;                 // [K][nb] (kept for the caller; the streams carry them too)
-  unsigned long long* status;   // [K][nb], zeroed before the launch
-  unsigned int* ticket;         // zeroed before the launch
+  unsigned long long* status;   // [K][nb], zero before the launch
+  unsigned int* ticket;         // zero before the launch
   const struct EncodeTables* tables;   // the shared-memory tables of the configuration, built once
   DevStatus* st;
   size_t b_first;               // first bucket of every worker to encode (0 but for the diagnostic)
@@ -45,7 +45,7 @@ static_assert(sizeof(EncodeTables) % 16 == 0, "copied in 16-byte pieces");
 
 struct PipePlan;
 qgx_status launch_encode_pipeline(qgx_ctx* c, const EncodeArgs& ea, const LevelTable& lt, const CodeTable& ct, const PhiloxKey& key,
-                                  const RoundTable& rt, const PipePlan& plan);
+                                  const RoundTable& rt, const PipePlan& plan, bool early);
 
 // The cut of a launch's work (see the kernel): chunks of kChunk coordinates, `unit` of them per unit of work, `units` units
 // per worker; a unit has one status word, `status_ld` per worker of which the first `status_first` are never published

@@ -293,6 +293,8 @@ k_encode_pipeline(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
   if (threadIdx.x == 0) { s_quit[0] = 0; s_quit[1] = kBarLooksBase + a.spin_limit / kBarLooksPolls; }
   if (threadIdx.x < kTurnRing) bar_init(turned + 8u * threadIdx.x, kQuantizers);
   __syncthreads();
+  start_next();
+  await_previous();
   volatile int* quit = s_quit;
   // a wait that ran out: everybody gives up, the launch ends and reports it
   auto give_up = [&]() {
@@ -701,7 +703,7 @@ PipePlan plan_encode_pipeline(const qgx_ctx* c, int bucket, size_t nb, size_t b_
 }
 
 qgx_status launch_encode_pipeline(qgx_ctx* c, const EncodeArgs& ea, const LevelTable& lt, const CodeTable& ct, const PhiloxKey& key,
-                                  const RoundTable& rt, const PipePlan& plan) {
+                                  const RoundTable& rt, const PipePlan& plan, bool early) {
   PipeShape ps;
   std::memset(&ps, 0, sizeof(ps));
   ps.b_log = 31 - __builtin_clz((unsigned)ea.bucket);
@@ -727,7 +729,7 @@ qgx_status launch_encode_pipeline(qgx_ctx* c, const EncodeArgs& ea, const LevelT
 #define QGX_LAUNCH_P(GG)                                                                              \
   do {                                                                                                \
     allow_max_dynamic_smem((const void*)k_encode_pipeline<GG>, c->device);                            \
-    k_encode_pipeline<GG><<<grid, kPipeThreads, ps.smem.bytes, c->stream>>>(ea, ps, lt, ct, key, rt); \
+    launch_next(early, k_encode_pipeline<GG>, grid, kPipeThreads, ps.smem.bytes, c->stream, ea, ps, lt, ct, key, rt); \
   } while (0)
   if (ct.G == 32) QGX_LAUNCH_P(32);
   else if (ct.G == 64) QGX_LAUNCH_P(64);

@@ -135,8 +135,10 @@ k_exchange_encode(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
     for (int i = threadIdx.x; i < 2 * QGX_MAX_LEVELS; i += blockDim.x) s_lut.e[i] = __ldg(a.tables->lut.e + i);
   }
   if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
-  if (threadIdx.x == 0) s_ticket[0] = atomicAdd(a.ticket, 1u);
   for (int i = threadIdx.x; i < 2 * img_words; i += blockDim.x) s_dyn[i] = 0;
+  start_next();
+  await_previous();
+  if (threadIdx.x == 0) s_ticket[0] = atomicAdd(a.ticket, 1u);
   __syncthreads();
   const int nlev = lt.nlev;
   const uint32_t pair_sa = smem_addr(s_pair);
@@ -289,7 +291,7 @@ namespace qgx {
 
 // workspace slots of a context
 enum { WS_OFF64 = 0, WS_FLAGS = 1, WS_LUT = 2, WS_SLOT0 = 3 /* stream, bits, offsets, total: 3..6 and 7..10 */,
-       WS_NORMS = 12, WS_SYM = 13, WS_NORMS2 = 14, WS_OPVAL = 15, WS_MEAN = 16, WS_SMALL = 23 };
+       WS_NORMS = 12, WS_SYM = 13, WS_NORMS2 = 14, WS_OPVAL = 15, WS_MEAN = 16, WS_TOTALS = 18 /* and 19 */, WS_SMALL = 23 };
 
 // ---- what a call derives from a quantizer configuration, kept between calls --------------------
 // Building the rounding table, the code table and the decoder table and copying the latter to the device costs
@@ -352,7 +354,9 @@ static TableCache* table_cache(qgx_ctx* c) {
 }
 
 // tables of cfg (built, and the decoder table copied to the device, on a miss)
-static qgx_status cached_tables(qgx_ctx* c, const qgx_quant_cfg* cfg, const CachedTables** out) {
+// *fresh: built by this call.  The kernel that uses them first is launched behind the ones that build them, not early; the
+// kernels after it may bring them in before they wait.
+static qgx_status cached_tables(qgx_ctx* c, const qgx_quant_cfg* cfg, const CachedTables** out, bool* fresh) {
   TableCache* tc = table_cache(c);
   if (!tc) return QGX_ERR_CUDA;
   uint64_t h = 1469598103934665603ull;
@@ -409,6 +413,7 @@ static qgx_status cached_tables(qgx_ctx* c, const qgx_quant_cfg* cfg, const Cach
   }
   e->used = ++tc->clock;
   *out = e;
+  *fresh = !hit;
   return QGX_OK;
 }
 
@@ -426,7 +431,8 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   if (cfg->cb.nlev != cfg->nlev) return QGX_ERR_INVALID_ARG;
   if (cudaSetDevice(c->device) != cudaSuccess) return QGX_ERR_CUDA;
   const CachedTables* tables = nullptr;
-  qgx_status rc = cached_tables(c, cfg, &tables);
+  bool fresh = false;
+  qgx_status rc = cached_tables(c, cfg, &tables, &fresh);
   if (rc != QGX_OK) return rc;
   const CodeTable& ct = tables->ct;
   LevelTable lt;
@@ -440,11 +446,15 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   uint32_t* stream = (uint32_t*)ws_get(c, base + 0, sizeof(uint32_t) * ((size_t)K * cap + 64));   // slack: see WalkReach
   uint32_t* bbits = (uint32_t*)ws_get(c, base + 1, sizeof(uint32_t) * (size_t)K * nb);
   uint32_t* offs = (uint32_t*)ws_get(c, base + 2, sizeof(uint32_t) * (size_t)K * nb);
-  // one block per slot, zeroed by one memset: the per-worker bit totals, the ticket counter, the status words of the scan
-  unsigned long long* tot = (unsigned long long*)ws_get(c, base + 3, sizeof(uint64_t) * ((size_t)K + 2 + (size_t)K * (nb + 1)));
-  unsigned long long* status = tot ? tot + K + 2 : nullptr;
+  // One block per slot, zero between exchanges (the decode pass sees to it): the per-worker sums of bits, the ticket counter, the
+  // status words of the scan.
+  const size_t had = c->ws_bytes[base + 3];
+  unsigned long long* sums = (unsigned long long*)ws_get(c, base + 3, sizeof(uint64_t) * ((size_t)K + 2 + (size_t)K * (nb + 1)));
+  if (c->ws_bytes[base + 3] != had) c->scan_dirty[slot] = 1;
+  unsigned long long* status = sums ? sums + K + 2 : nullptr;
+  unsigned long long* tot = (unsigned long long*)ws_get(c, WS_TOTALS + slot, sizeof(uint64_t) * (size_t)K);
   float* norms = (float*)ws_get(c, slot == 0 ? WS_NORMS : WS_NORMS2, sizeof(float) * (size_t)K * nb);
-    if (!stream || !bbits || !offs || !tot || !status || !norms) return QGX_ERR_CUDA;
+    if (!stream || !bbits || !offs || !tot || !sums || !norms) return QGX_ERR_CUDA;
   c->slot_cap_words[slot] = cap;
   c->slot_K[slot] = K;
   c->slot_nb[slot] = nb;
@@ -456,8 +466,8 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   ea.vec_ok = (d % kQuad == 0) && (src.ld % kQuad == 0) && ((reinterpret_cast<uintptr_t>(src.v) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(src.a) & 15u) == 0);
   ea.v_vec = (reinterpret_cast<uintptr_t>(src.v ? src.v : src.a) & 15u) == 0 && (!src.v || K == 1 || (src.ld ? src.ld : d) % kQuad == 0);
   ea.a_vec = (reinterpret_cast<uintptr_t>(src.a) & 15u) == 0;
-  ea.stream = stream; ea.cap_words = cap; ea.bucket_bits = bbits; ea.offsets = offs; ea.total_bits = tot; ea.norms = norms;
-  ea.status = status; ea.ticket = reinterpret_cast<unsigned int*>(tot + K); ea.st = c->dstatus; ea.tables = tables->enc_dev;
+  ea.stream = stream; ea.cap_words = cap; ea.bucket_bits = bbits; ea.offsets = offs; ea.total_bits = sums; ea.norms = norms;
+  ea.status = status; ea.ticket = reinterpret_cast<unsigned int*>(sums + K); ea.st = c->dstatus; ea.tables = tables->enc_dev;
   uint8_t* sym_out = nullptr;
   const uint8_t* sym_prev = nullptr;
   const size_t sym_ld = (d + 15) & ~(size_t)15;             // see DecodeArgs::sym_out
@@ -485,14 +495,15 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   // small vectors: everything in one launch (the other ways are there when a caller asks for one of them)
   if (do_encode && c->skip_buckets < nb && c->encode_path == QGX_ENCODE_AUTO && c->decode_split == QGX_SPLIT_AUTO &&
       small_exchange_fits(c, K, nb, bucket, ct, qt, ea.vec_ok && ea.quad_base % 2 == 0)) {
-    const size_t had = c->ws_bytes[WS_SMALL];
+    const size_t had_words = c->ws_bytes[WS_SMALL];
     unsigned long long* words = (unsigned long long*)ws_get(c, WS_SMALL, sizeof(uint64_t) * ((size_t)K * nb + 2));
     if (!words) return QGX_ERR_CUDA;
-    if (c->ws_bytes[WS_SMALL] != had && cudaMemsetAsync(words, 0, c->ws_bytes[WS_SMALL], c->stream) != cudaSuccess) return QGX_ERR_CUDA;
+    if (c->ws_bytes[WS_SMALL] != had_words && cudaMemsetAsync(words, 0, c->ws_bytes[WS_SMALL], c->stream) != cudaSuccess) return QGX_ERR_CUDA;
     EncodeArgs es = ea;
     es.status = words + 2;                              // zero between launches: the kernel sees to it
     es.ticket = reinterpret_cast<unsigned int*>(words);
     es.b_first = c->skip_buckets;                       // 0 but for the diagnostic
+    es.total_bits = tot;                                // written by the last bucket, not summed
     es.spin_limit = c->wait_limit;
     SmallArgs sm;
     std::memset(&sm, 0, sizeof(sm));
@@ -503,7 +514,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     sm.sum_sq = sum_sq; sm.square = (sym_mode & 4) ? 1 : 0; sm.total_out = (unsigned long long*)total_bits_out; sm.total_add = c->add_totals;
     ScopedKernelTimer timer(c, QGX_KERNEL_ENCODE);
     c->skip_buckets = 0;
-    return launch_exchange_small(c, es, sm, lt, lt_kept, ct, key, qt);
+    return launch_exchange_small(c, es, sm, lt, lt_kept, ct, key, qt, !fresh && !c->helper);
   }
   // octets per thread chosen so that CTAs have at most 256 / 512 / 512 threads
   const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
@@ -523,7 +534,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     per_sm = shape.per_sm;                                                                                     \
     const unsigned long long want = (unsigned long long)(nb - ea.b_first) * (unsigned long long)K;             \
     const unsigned grid = (unsigned)std::min<unsigned long long>(want, (unsigned long long)c->num_sms * (unsigned long long)per_sm);   \
-    k_exchange_encode<V, GG><<<grid, threads, smem, c->stream>>>(ea, lt, ct, key, qt);                         \
+    launch_next(!fresh && !c->helper, k_exchange_encode<V, GG>, grid, threads, smem, c->stream, ea, lt, ct, key, qt); \
   } while (0)
 #define QGX_LAUNCH_EG(V)                                   \
   do {                                                     \
@@ -547,13 +558,17 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
     plan = plan_encode_pipeline(c, bucket, nb, ea.b_first, K);
     status_ld = plan.status_ld;
   }
-  if (do_encode && cudaMemsetAsync(tot, 0, sizeof(uint64_t) * ((size_t)K + 2 + (size_t)K * status_ld), c->stream) != cudaSuccess) return QGX_ERR_CUDA;
+  if (do_encode) {
+    // (the whole block: what an exchange that went wrong left of it may be of another shape)
+    if (c->scan_dirty[slot] && cudaMemsetAsync(sums, 0, c->ws_bytes[base + 3], c->stream) != cudaSuccess) return QGX_ERR_CUDA;
+    c->scan_dirty[slot] = 1;
+  }
   c->skip_buckets = 0;
   ea.spin_limit = c->wait_limit;
   if (do_encode && ea.b_first < nb) {
     ScopedKernelTimer timer(c, QGX_KERNEL_ENCODE);
     if (pipelined) {
-      rc = launch_encode_pipeline(c, ea, lt, ct, key, qt, plan);
+      rc = launch_encode_pipeline(c, ea, lt, ct, key, qt, plan, !fresh && !c->helper);
       if (rc != QGX_OK) return rc;
     } else {
       switch (pp) {
@@ -573,10 +588,13 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   da.d = d; da.bucket = bucket; da.K = K; da.nb = nb; da.tables = tables->dec_dev; da.mean = mean_out;
   da.update = upd ? upd->mode : 0; da.xin = upd ? upd->xin : nullptr; da.xout = upd ? upd->xout : nullptr;
   da.scalars = upd ? upd->scalars : nullptr; da.st = c->dstatus;
-  da.total_bits = tot; da.total_out = (unsigned long long*)total_bits_out; da.total_add = c->add_totals;
+  da.sums = do_encode ? sums : nullptr; da.total_bits = tot; da.total_out = (unsigned long long*)total_bits_out; da.total_add = c->add_totals;
+  da.scan = sums + K; da.scan_words = do_encode ? 2 + (size_t)K * status_ld : 0;
   da.vec_out = ((reinterpret_cast<uintptr_t>(mean_out) & 15u) == 0) && ((reinterpret_cast<uintptr_t>(da.xin) & 15u) == 0) &&
                ((reinterpret_cast<uintptr_t>(da.xout) & 15u) == 0);
-  return launch_exchange_decode(c, da, ct, lt, lt_kept, sym_mode);
+  rc = launch_exchange_decode(c, da, ct, lt, lt_kept, sym_mode, !c->helper && (!fresh || (do_encode && ea.b_first < nb)));
+  if (rc == QGX_OK && do_encode) c->scan_dirty[slot] = 0;
+  return rc;
 }
 
 // ---- helper contexts of the layer-wise exchange -------------------------------------------------
@@ -648,6 +666,7 @@ static SegChildren* seg_children(qgx_ctx* c) {
     h->sym_slot = -1;
     h->num_sms = c->num_sms;                            // (this and the context's modes are set again for every exchange)
     h->all_sms = c->all_sms;
+    h->helper = 1;
     h->dstatus = c->dstatus;                            // errors latch into the parent's status block
     if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&sc->join[i], cudaEventDisableTiming) != cudaSuccess) {
@@ -821,7 +840,7 @@ qgx_status qgx_exchange_streams(qgx_ctx* c, int slot, const uint32_t** stream, s
   if (stream) *stream = (const uint32_t*)c->ws[base + 0];
   if (cap_words) *cap_words = c->slot_cap_words[slot];
   if (bucket_bits) *bucket_bits = (const uint32_t*)c->ws[base + 1];
-  if (total_bits) *total_bits = (const uint64_t*)c->ws[base + 3];
+  if (total_bits) *total_bits = (const uint64_t*)c->ws[WS_TOTALS + slot];
   return QGX_OK;
 }
 

@@ -60,9 +60,6 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
   uint32_t* s_sym = reinterpret_cast<uint32_t*>(s_raw + r.off_sym);    // the decoded symbols (see qgx_walk.cuh), four per word
   uint16_t* s_tab = reinterpret_cast<uint16_t*>(s_raw + r.off_tab);    // see DecodeTables::single
 
-  // which bucket: a ticket per cluster, so that the buckets a bucket looks back at are already under way
-  unsigned ticket = 0;
-  if (k == 0 && tid == 0) ticket = atomicAdd(a.ticket, 1u);
   asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
   const int rep = rt.key_shift - kKeyShiftMin, nbins = (int)((kKeyTop - kKeyBase) >> rt.key_shift) + 1;
   for (int i = tid; i < nbins; i += blockDim.x) s_bin[i] = __ldg(a.tables->bin_fix + (i << rep));
@@ -74,6 +71,11 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
     s_lev_kept[tid] = tid < lt_kept.nlev ? lt_kept.lev[tid] : 0.0f;
   }
   for (uint32_t i = (uint32_t)tid; i < r.img_words; i += blockDim.x) s_img[i] = 0u;
+  start_next();
+  await_previous();
+  // which bucket: a ticket per cluster, so that the buckets a bucket looks back at are already under way
+  unsigned ticket = 0;
+  if (k == 0 && tid == 0) ticket = atomicAdd(a.ticket, 1u);
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");          // the cluster's CTAs are there: their memory can be written
   if (k == 0 && tid == 0)
     for (int i = 0; i < K; ++i) *cluster.map_shared_rank(&s_bucket, i) = ticket;
@@ -398,12 +400,16 @@ bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const C
 }
 
 qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, const LevelTable& lt, const LevelTable& lt_kept,
-                                 const CodeTable& ct, const PhiloxKey& key, const RoundTable& rt) {
+                                 const CodeTable& ct, const PhiloxKey& key, const RoundTable& rt, bool early) {
   const SmallShape s = small_shape(ea.bucket, ct, rt);
   r.img_words = s.img_words; r.off_img = s.off_img; r.off_sym = s.off_sym; r.off_tab = s.off_tab;
   cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr;
-  small_config(s, ea.K, ea.nb - ea.b_first, c->stream, &cfg, &attr);
+  cudaLaunchAttribute attr[2];
+  small_config(s, ea.K, ea.nb - ea.b_first, c->stream, &cfg, attr);
+  std::memset(attr + 1, 0, sizeof(attr[1]));
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // see launch_next
+  attr[1].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  cfg.numAttrs = 2;
   void* args[] = {(void*)&ea, (void*)&r, (void*)&lt, (void*)&lt_kept, (void*)&ct, (void*)&key, (void*)&rt};
   const cudaError_t err = cudaLaunchKernelExC(&cfg, s.fn, args);
   count_launch(c);

@@ -78,6 +78,8 @@ k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ Level
   __shared__ double s_red[2][32];
   fill_bin_table(s_bin, rt, BinKind::kFixed);
   if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
+  start_next();
+  await_previous();
   __syncthreads();
   constexpr bool kTeams = P == 1;
   const int lane = threadIdx.x & 31;
@@ -191,6 +193,8 @@ __global__ void __launch_bounds__(256) k_average(const float* __restrict__ norms
                                                  int bucket, size_t nb, const __grid_constant__ LevelTable lt, float* __restrict__ out, DevStatus* st) {
   __shared__ float s_lev[QGX_MAX_LEVELS * 32];
   for (int i = threadIdx.x; i < QGX_MAX_LEVELS * 32; i += blockDim.x) s_lev[i] = (i >> 5) < lt.nlev ? lt.lev[i >> 5] : 0.0f;
+  start_next();
+  await_previous();
   __syncthreads();
   const size_t groups = (d + V - 1) / V;
   const float Kf = (float)K;
@@ -281,9 +285,9 @@ qgx_status launch_quantize(qgx_ctx* c, DualSource src, int K, size_t d, int buck
   const unsigned per_sm = (unsigned)std::max(2, 1024 / threads);      // registers: 1024 threads
   const unsigned grid = (unsigned)std::min<size_t>((a.total + (size_t)a.teams - 1) / (size_t)a.teams, (size_t)c->num_sms * per_sm);
   switch (pp) {
-    case 1: k_quantize<1><<<grid, threads, 0, c->stream>>>(a, lt, key, *rt); break;
-    case 2: k_quantize<2><<<grid, threads, 0, c->stream>>>(a, lt, key, *rt); break;
-    default: k_quantize<4><<<grid, threads, 0, c->stream>>>(a, lt, key, *rt); break;
+    case 1: launch_next(true, k_quantize<1>, grid, threads, 0, c->stream, a, lt, key, *rt); break;
+    case 2: launch_next(true, k_quantize<2>, grid, threads, 0, c->stream, a, lt, key, *rt); break;
+    default: launch_next(true, k_quantize<4>, grid, threads, 0, c->stream, a, lt, key, *rt); break;
   }
   count_launch(c);
   return cuda_status(cudaGetLastError());
@@ -324,9 +328,9 @@ qgx_status qgx_average(qgx_ctx* c, const float* norms, const uint8_t* sym, int K
   const bool quads = d % 4 == 0 && bucket % 4 == 0 && (reinterpret_cast<uintptr_t>(sym) & 3u) == 0;
   const size_t groups = wide ? d / 16 : (quads ? d / 4 : d);
   const unsigned blocks = (unsigned)std::min<size_t>((groups + 255) / 256, (size_t)c->num_sms * 16u);
-  if (wide) k_average<16><<<blocks, 256, 0, c->stream>>>(norms, sym, K, d, bucket, nb, lt, out, c->dstatus);
-  else if (quads) k_average<4><<<blocks, 256, 0, c->stream>>>(norms, sym, K, d, bucket, nb, lt, out, c->dstatus);
-  else k_average<1><<<blocks, 256, 0, c->stream>>>(norms, sym, K, d, bucket, nb, lt, out, c->dstatus);
+  if (wide) launch_next(true, k_average<16>, blocks, 256, 0, c->stream, norms, sym, K, d, bucket, nb, lt, out, c->dstatus);
+  else if (quads) launch_next(true, k_average<4>, blocks, 256, 0, c->stream, norms, sym, K, d, bucket, nb, lt, out, c->dstatus);
+  else launch_next(true, k_average<1>, blocks, 256, 0, c->stream, norms, sym, K, d, bucket, nb, lt, out, c->dstatus);
   count_launch(c);
   return cuda_status(cudaGetLastError());
 }

@@ -30,6 +30,6 @@ bool small_exchange_size(const qgx_ctx* c, int K, size_t nb, int bucket);   // n
 bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct, const RoundTable& rt, bool octets);
 // After small_exchange_fits.  ea.status [K][nb] and ea.ticket [2] are zero before the launch and again after it.
 qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, const LevelTable& lt, const LevelTable& lt_kept,
-                                 const CodeTable& ct, const PhiloxKey& key, const RoundTable& rt);
+                                 const CodeTable& ct, const PhiloxKey& key, const RoundTable& rt, bool early);
 
 }  // namespace qgx

@@ -72,6 +72,8 @@ __global__ void __launch_bounds__(1024, 1) k_unpack_rows(const __grid_constant__
     return r;
   };
 
+  start_next();
+  await_previous();                      // (the table, too, is the kernel's before this one)
   uint32_t it = blockIdx.x + gridDim.x * (uint32_t)warp;
   Bucket bucket = ask_bucket(it);
   {
@@ -212,7 +214,7 @@ static qgx_status launch_unpack_g(qgx_ctx* c, const UnpackRowsArgs& a, int bucke
   const size_t smem = table + (size_t)warps * each;
   const unsigned grid = std::min((uint32_t)c->num_sms, h.items);
   allow_max_dynamic_smem((const void*)k_unpack_rows<G>, c->device);
-  k_unpack_rows<G><<<grid, 32 * warps, smem, c->stream>>>(a, h);
+  launch_next(true, k_unpack_rows<G>, grid, 32 * warps, smem, c->stream, a, h);
   count_launch(c);
   return cuda_status(cudaGetLastError());
 }
