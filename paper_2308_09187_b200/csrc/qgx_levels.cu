@@ -47,14 +47,16 @@ __device__ __forceinline__ FastBin fast_bin(float x, float c) {
 // counters per bin, one for every second, fourth or eighth lane, made both slower.)  A coordinate counts for the bin that
 // fast_bin gives it; where that may be wrong (a few in a million for bins of small index) the thread's coordinates are read
 // again afterwards and the count moved to the bin of the defining operations, so that the common path has neither a select
-// nor a clamp.  The next bucket is fetched into registers before this one's norm is formed, where a CTA has few enough
-// per thread and more than a few warps.  8 workers of 2^24 coordinates, 1024 bins, L2: bucket 8192 196 -> 178 us, 16384 167 ->
-// 149, 2048 279 -> 234, 256 621 -> 514 (four counters a read in the fold); DRAM alone would take 82.
+// nor a clamp.  A CTA works on its bucket phase by phase (load, norm, count, fold, a barrier between them), so the SM is kept
+// busy by its other CTAs: the fewer threads a bucket has -- the more coordinates each -- the more of them there are.  Fetching
+// the next bucket into registers early bought less than the CTAs it cost.  8 workers of 2^24 coordinates, 1024 bins, L2 and
+// L-infinity: buckets of 16384 with eight quads per thread 145 and 216 us; 8192 with four, fetched early, 177 and 262, with eight
+// 143 and 218; 4096 177 and 265, 142 and 234; 2048 with two 238 and 324, with four 166 and 269; 1024 with two 246 and 361, with
+// four 199 (L2), with two and not early 351; 512 with one 360 and 534, with two 295 and 495.  DRAM alone would take 82.
 template <int V4>
 __global__ void __launch_bounds__(512, 2) k_histogram(DualSource src, size_t d, int bucket, size_t nb, int K, int norm_type,
                                                       int nbins, int weighted, bool vec_ok, double* __restrict__ hist,
                                                       DevStatus* st) {
-  constexpr bool kPrefetch = V4 == 2 || V4 == 4;
   extern __shared__ __align__(16) unsigned char s_raw[];
   double* s_hist = reinterpret_cast<double*>(s_raw);                 // [nbins], then 4 words, then the counters
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_hist + ((nbins + 1) & ~1)) + 4;   // [-1 .. nbins]
@@ -65,22 +67,12 @@ __global__ void __launch_bounds__(512, 2) k_histogram(DualSource src, size_t d, 
   const float nbf = (float)nbins;
   const uint32_t cnt_base = smem_addr(s_cnt) - 4u * kBinZero;         // a bin: base + 4 * pattern, modulo 2^32
   const unsigned long long total = (unsigned long long)nb * (unsigned long long)K;
-  BucketRegs<V4> r, next;
-  const auto load = [&](BucketRegs<V4>& to, unsigned long long t) {
-    const size_t lo = (size_t)(t / (unsigned long long)K) * (size_t)bucket;
-    load_bucket<V4>(to, src, (size_t)(t % (unsigned long long)K), d, lo, (int)min((size_t)bucket, d - lo), vec_ok);
-  };
-  if (kPrefetch) load(next, blockIdx.x);                             // grid <= total
+  BucketRegs<V4> r;
   for (unsigned long long t = blockIdx.x; t < total; t += gridDim.x) {
     const size_t b = (size_t)(t / (unsigned long long)K), k = (size_t)(t % (unsigned long long)K);
     const size_t lo = b * (size_t)bucket;
     const int len = (int)min((size_t)bucket, d - lo);
-    if (kPrefetch) {
-      r = next;
-      if (t + gridDim.x < total) load(next, t + gridDim.x);
-    } else {
-      load(r, t);
-    }
+    load_bucket<V4>(r, src, k, d, lo, len, vec_ok);
     const float norm = V4 == 1 ? bucket_norm<V4>(r, norm_type, s_red) : bucket_norm_all<V4>(r, norm_type, s_red);
     const bool finite = (norm - norm) == 0.0f;
     if (!finite) {
@@ -156,7 +148,7 @@ qgx_status launch_histogram(qgx_ctx* c, DualSource src, int K, size_t d, int buc
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
   const bool vec_ok = (d % kQuad == 0) && ((reinterpret_cast<uintptr_t>(src.v) & 15u) == 0) &&
                       ((reinterpret_cast<uintptr_t>(src.a) & 15u) == 0);
-  const int v4 = bucket_v4(bucket);
+  const int v4 = bucket <= 256 ? 1 : (bucket <= 512 ? 2 : (bucket <= 1024 ? (norm_type == QGX_NORM_L2 ? 4 : 2) : (bucket <= 2048 ? 4 : 8)));
   const int threads = bucket_threads(bucket, v4);
   const size_t smem = sizeof(double) * (size_t)((nbins + 1) & ~1) + sizeof(uint32_t) * (4 + (((size_t)nbins + 1 + 3) & ~(size_t)3));
   const unsigned long long total = (unsigned long long)nb * (unsigned long long)K;
