@@ -4,6 +4,7 @@
 // offsets (k_scan_offsets, which also builds the decoder's table) -> k_unpack_rows or k_unpack.
 #include "qgx_bucket.cuh"
 #include "qgx_codec.cuh"
+#include "qgx_pack.cuh"
 #include "qgx_unpack.cuh"
 
 #include <algorithm>
@@ -231,31 +232,9 @@ __global__ void __launch_bounds__(512) k_bit_scatter(const float* __restrict__ n
 }
 
 // ---- encode in one pass ----------------------------------------------------------------------------
-// The status word of a bucket in the look-back carries two sums at once: words in bits 0..32, unused bits at the ends of
-// the buckets' last words in bits 33..61 -- so the last bucket of a worker knows the stream's bits, too.
-constexpr int kPadShift = 33;
-
-struct PackArgs {
-  const float* norms;
-  const uint8_t* sym;
-  size_t d;
-  int bucket, K;
-  size_t nb;
-  int load;                              // bytes per symbol load: 8, 4 or 1
-  uint32_t* stream;
-  size_t cap_words;
-  uint32_t* bucket_bits;
-  uint64_t* total_bits;
-  unsigned long long* status;            // [K][nb], zeroed before the launch
-  unsigned int* ticket;                  // zeroed before the launch
-  unsigned int first_ticket;             // K times the first bucket of every worker to encode (0 but for the diagnostic)
-  int spin_limit;                        // polls of a wait for another bucket's words before it gives up
-  DevStatus* st;
-};
-
 // Persistent CTAs, a bucket at a time (in the order b-major, k-minor, by a ticket counter: see lookback_prefix), P octets of
 // eight symbols per thread.  One pass over the symbols instead of three kernels and two passes; the symbols' codewords come
-// from a table of pairs.  For streams whose capacity is the worst case, so that no worker can turn out not to fit after
+// from a table of pairs.  Buckets of 1024 2^j symbols go through k_pack_chunks instead.  For streams whose capacity is the worst case, so that no worker can turn out not to fit after
 // its first buckets are written; codes with sub-blocks of 32, 64 or 128 or with none.  Instruction-bound, about 20 per symbol.
 template <int P>
 __global__ void __launch_bounds__(P == 1 ? 256 : 512, P == 1 ? 4 : 2)
@@ -572,16 +551,17 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
   const bool layout = !ct.has_header || ct.G == 32 || ct.G == 64 || ct.G == 128;
   const size_t worst = qgx_stream_capacity_words(d, bucket, cb->subblock, ct.maxlen);
   if (layout && cap_words >= worst && worst < ((size_t)1 << (kPadShift - 1)) && nb < ((size_t)1 << 23) && nb * (size_t)K < ((size_t)1 << 31)) {
-    unsigned long long* status = (unsigned long long*)ws_get(c, 0, sizeof(uint64_t) * ((size_t)K * nb + 2));
+    unsigned long long* status = (unsigned long long*)ws_get(c, 0, sizeof(uint64_t) * ((size_t)K * (nb + 1) + 2));
     if (!status) return QGX_ERR_CUDA;
-    if (cudaMemsetAsync(status, 0, sizeof(uint64_t) * ((size_t)K * nb + 2), c->stream) != cudaSuccess) return QGX_ERR_CUDA;
+    if (cudaMemsetAsync(status, 0, sizeof(uint64_t) * ((size_t)K * (nb + 1) + 2), c->stream) != cudaSuccess) return QGX_ERR_CUDA;
     PackArgs a;
     a.norms = norms; a.sym = sym; a.d = d; a.bucket = bucket; a.K = K; a.nb = nb; a.stream = stream; a.cap_words = cap_words;
     a.bucket_bits = bucket_bits; a.total_bits = total_bits; a.status = status + 2; a.ticket = reinterpret_cast<unsigned int*>(status);
-    const size_t todo = (nb - std::min(c->skip_buckets, nb)) * (size_t)K;
+    const size_t b_first = std::min(c->skip_buckets, nb), todo = (nb - b_first) * (size_t)K;
     a.first_ticket = (unsigned int)(nb * (size_t)K - todo); a.spin_limit = c->wait_limit; a.st = c->dstatus;
     c->skip_buckets = 0;
     if (todo == 0) return QGX_OK;
+    if (pack_chunks_fits(K, nb, bucket)) return launch_pack_chunks(c, a, b_first, ct);
     const uintptr_t at = reinterpret_cast<uintptr_t>(sym);
     a.load = (d % 8 == 0 && bucket % 8 == 0 && (at & 7u) == 0) ? 8 : ((d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
     const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);

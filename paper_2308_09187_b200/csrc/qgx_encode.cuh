@@ -2,6 +2,7 @@
 #pragma once
 
 #include "qgx_bucket.cuh"
+#include "qgx_chunk.cuh"
 #include "qgx_codec.cuh"
 
 namespace qgx {

@@ -27,7 +27,6 @@
 
 namespace qgx {
 
-constexpr int kLaneCoords = 32;                          // coordinates per lane: one 128-byte line of the stage
 constexpr int kQuantizers = 16, kDispatchers = 1, kScanners = 2, kCopiers = 5;
 constexpr int kPipeThreads = 32 * (kQuantizers + kDispatchers + kScanners + kCopiers);
 constexpr unsigned kUnitRing = 64;                       // unit descriptors: more than are ever under way
@@ -55,7 +54,6 @@ struct __align__(16) PipePlace {
   uint32_t nbits;                                        // the bucket's bits; 0: do not write
 };
 
-__host__ __device__ constexpr int pipe_lane_stride(int maxlen) { return (maxlen + 1) | 1; }   // words per lane, odd: no bank conflicts
 struct PipeSmem {                                        // byte offsets into the dynamic shared memory
   uint32_t stage, image, bin, pair, lut, lev, cnt, tot, inorm, last, unit, norm, place, bars, part, posted, bytes;
 };
@@ -138,32 +136,6 @@ __device__ __forceinline__ void copy_async4(uint32_t dst, const float* src, int 
 // so that both a loader's lanes (consecutive pieces) and a quantizer's (the same piece of 8 consecutive lines) spread
 // over the banks
 __device__ __forceinline__ uint32_t piece_at(uint32_t u) { return ((u & ~7u) | ((u ^ (u >> 3)) & 7u)) << 4; }
-
-// Stream bits of a lane as they are produced: a 64-bit window that new bits enter at the top (two funnel shifts, no masks);
-// the oldest 32 go to the lane's words in shared memory once they are there.
-struct LaneBits {
-  uint32_t lo, hi;
-  int pos;                                               // 64 - bits waiting in the window
-  uint32_t wa;                                           // shared address of the next word
-  __device__ __forceinline__ void open(uint32_t addr) { lo = hi = 0u; pos = 64; wa = addr; }
-  // the low n bits of e (n <= 26, the entry's upper 6 bits; fewer than 32 bits are waiting)
-  __device__ __forceinline__ void put(uint32_t e) {
-    const uint32_t n = e >> 26;
-    lo = __funnelshift_r(lo, hi, n);
-    hi = __funnelshift_r(hi, e, n);
-    pos -= (int)n;
-    if (pos <= 32) {
-      sts32(wa, __funnelshift_rc(lo, hi, (uint32_t)pos));
-      wa += 4u;
-      pos += 32;
-    }
-  }
-  // stores what is waiting; the bits put since open(addr)
-  __device__ __forceinline__ uint32_t close(uint32_t addr) {
-    if (pos < 64) sts32(wa, hi >> ((uint32_t)pos - 32u));
-    return 8u * (wa - addr) + (uint32_t)(64 - pos);
-  }
-};
 
 // Two octets (first, first + 1) of one lane's 32 coordinates (of the first `count` of them when MASKED): lx = the shared
 // address of its line, plus 16 times the line's permutation (piece p is at lx ^ 16 p), q0 the generator's counter of its
@@ -623,65 +595,10 @@ k_encode_pipeline(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
         const unsigned cs = ci0 + (unsigned)i, cs2 = cs + par * (unsigned)(NT * kQuantizers);   // the image; of twice the ring
         const PipePlace pp = s_place[cs];
         if (pp.nbits == 0u) continue;                               // no place was found for the unit
-        uint32_t* dst = a.stream + (size_t)pu.k * a.cap_words + pp.word;
         const int ib = i & (m - 1);                                    // the chunk's place in its bucket
-        const uint32_t cnt_sa = sa + L.cnt + cs2 * 64u;                // its 32 lane counts, two bytes each
         const uint32_t nsub = (uint32_t)((min(a.bucket, pu.len - (i - ib) * kChunk) + G - 1) / G);
-        // The header's words of this chunk: two sub-blocks each, G / 32 lane counts per sub-block.
-        constexpr uint32_t kWords = kChunk / G / 2;                    // 16, 8 or 4
-        if ((uint32_t)lane < kWords && (uint32_t)ib * kWords + (uint32_t)lane < nsub / 2u) {
-          uint32_t h;
-          if (G == 32) {
-            h = lds32(cnt_sa + 4u * (uint32_t)lane);
-          } else {
-            uint32_t f0 = 0, f1 = 0;
-#pragma unroll
-            for (int j = 0; j < G / 64; ++j) {
-              const uint32_t c0 = lds32(cnt_sa + (uint32_t)lane * (G / 8) + 4u * j), c1 = lds32(cnt_sa + (uint32_t)lane * (G / 8) + (G / 16) + 4u * j);
-              f0 += (c0 & 0xffffu) + (c0 >> 16);
-              f1 += (c1 & 0xffffu) + (c1 >> 16);
-            }
-            h = f0 | (f1 << 16);
-          }
-          dst[1u + (uint32_t)ib * kWords + (uint32_t)lane] = h;
-        }
-        if (ib == 0 && lane == 0) dst[0] = __float_as_uint(s_inorm[cs]);
-        const uint32_t n_l = s_cnt[cs2 * 32u + (unsigned)lane];
-        const uint32_t p = pp.bit + warp_incl_scan(n_l, lane) - n_l, sh = p & 31u, nw = ((p + n_l) >> 5) - (p >> 5);
-        uint32_t* out = dst + (p >> 5);
-        const uint32_t img = sa + L.image + (cs * 32u + (unsigned)lane) * lane_words * 4u;
-        // Word j of the lane's part of the stream takes the end of its bits' word j - 1 and the beginning of word j; words
-        // 0 .. nw - 1 end inside its bits, word nw is for the lane after it (past the lane's words the reads run into its
-        // neighbour's: those bits are masked off).
-        const uint32_t most = __reduce_max_sync(0xffffffffu, nw);
-        uint32_t prev = lds32(img), tail = 0;
-        const uint32_t first = prev << sh;
-#pragma unroll
-        for (uint32_t j = 1; j <= (uint32_t)QGX_MAX_CODE_LEN + 2u; ++j) {
-          if (j > most) break;
-          const uint32_t cur = lds32(img + 4u * j), x = __funnelshift_l(prev, cur, sh);
-          if (j < nw) out[j] = x;
-          if (j == nw) tail = x;
-          prev = cur;
-        }
-        const uint32_t over = (p + n_l) & 31u, mask = (1u << over) - 1u;
-        tail &= mask;
-        uint32_t before = __shfl_up_sync(0xffffffffu, tail, 1);
-        if (lane == 0) {
-          before = 0;
-          if (sh != 0u) {
-            if (ib != 0) {
-              before = s_last[cs2 - 1u] >> (32u - sh);                 // the last bits of the chunk before
-            } else {                                                   // an odd number of sub-blocks: the last length shares a word
-              const uint16_t* cnt = s_cnt + cs2 * 32u;
-#pragma unroll
-              for (int j = 0; j < G / kLaneCoords; ++j) before += cnt[(nsub - 1u) * (G / kLaneCoords) + j];
-            }
-          }
-        }
-        if (nw > 0u) out[0] = first | before;
-        // the bucket's last word, when it is not whole
-        if (n_l > 0u && p + n_l == pp.nbits && over != 0u) out[nw] = nw > 0u ? tail : ((first & mask) | before);
+        place_chunk<G>(a.stream + (size_t)pu.k * a.cap_words + pp.word, pp.bit, pp.nbits, ib, nsub, s_inorm[cs], s_cnt + cs2 * 32u, s_last + cs2,
+                       sa + L.image + (cs * 32u + (unsigned)lane) * lane_words * 4u, lane);
       }
       __syncwarp();
       if (lane == 0) bar_arrive(written + 8u * ui);

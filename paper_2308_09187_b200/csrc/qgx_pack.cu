@@ -1,0 +1,186 @@
+// qgx_encode in one pass for buckets of 1024, 2048, 4096, 8192 or 16384 symbols, with sub-blocks of 32, 64 or 128 or none, where the
+// capacity fits any outcome.  A CTA takes a unit of chunks of 1024 symbols of one worker, a warp each: a lane turns 32
+// consecutive symbols into bits of its own (pairs of symbols from a table), the CTA finds the unit's place by look-back, and the
+// warps shift their lanes' bits to where they belong -- as the fused encoder does, without its quantizer.
+// What bounds it: instructions (21 per symbol) and the wait for the units before, at 55 % issue.  8 x 2^22 symbols of 17 fitted
+// levels in buckets of 8192: a thread per eight symbols, which ORs them into an image of the bucket (k_pack), 72 us, this 42.  A
+// warp of its own for the look-back, with the next unit written meanwhile, is 1 % faster.
+#include "qgx_chunk.cuh"
+#include "qgx_pack.cuh"
+
+#include <algorithm>
+
+namespace qgx {
+
+constexpr int kPackChunk = 1024;
+struct PackShape {
+  int unit, m_log;                       // chunks per unit, log2 of the chunks per bucket
+  size_t units;                          // per worker
+  size_t first;                          // the first coordinate (0 but for the diagnostic that leaves buckets out)
+  size_t status_ld, status_first;        // status words per worker, the first one used
+  uint32_t lane_words;                   // words per lane of an image
+  uint32_t off_image, off_cnt, off_last; // bytes of dynamic shared memory, after the pair table
+};
+
+template <int G>
+__global__ void __launch_bounds__(512, 3) k_pack_chunks(const __grid_constant__ PackArgs a, const __grid_constant__ PackShape h, const __grid_constant__ CodeTable ct) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  __shared__ EncLut s_lut;
+  __shared__ uint32_t s_tot[2][16];
+  __shared__ unsigned int s_ticket[2];
+  __shared__ unsigned long long s_base[2];
+  __shared__ int s_skip[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, U = h.unit, m = 1 << h.m_log;
+  const int nlev = ct.nlev, n2 = 2 * nlev;
+  uint32_t* s_pair = reinterpret_cast<uint32_t*>(s_raw);               // first + 2 nlev second; a symbol is its level, plus nlev when negative
+  fill_enc_lut(&s_lut, ct);
+  __syncthreads();
+  for (int i = threadIdx.x; i < n2 * n2; i += blockDim.x) {
+    const int f = i % n2, g = i / n2;
+    const uint32_t x = s_lut.e[f < nlev ? f : f - nlev + 32], y = s_lut.e[g < nlev ? g : g - nlev + 32];
+    s_pair[i] = ((x & 0xffffu) | ((y & 0xffffu) << (x >> 16))) | (((x >> 16) + (y >> 16)) << 26);
+  }
+  start_next();
+  await_previous();
+  if (threadIdx.x == 0) s_ticket[0] = atomicAdd(a.ticket, 1u);
+  __syncthreads();
+  const uint32_t pair_sa = smem_addr(s_pair), weights = 4u | ((uint32_t)(8 * nlev) << 16);
+  const uint32_t limit4 = (uint32_t)(128 - nlev) * 0x01010101u;        // carries into bit 7 of a byte >= nlev
+  const uint32_t img = smem_addr(s_raw) + h.off_image + (uint32_t)(warp * 32 + lane) * h.lane_words * 4u;
+  const unsigned total = (unsigned)h.units * (unsigned)a.K;            // below 2^31: the host checks
+  const size_t unit_coords = (size_t)(U * kPackChunk);
+  bool bad = false;
+  for (int par = 0;; par ^= 1) {
+    const unsigned t = s_ticket[par];
+    if (t >= total) break;
+    const unsigned u = t / (unsigned)a.K, k = t - u * (unsigned)a.K;
+    const size_t lo = h.first + (size_t)u * unit_coords;
+    const int len = (int)min(unit_coords, a.d - lo);                  // of the unit
+    const int at = warp * kPackChunk + lane * kLaneCoords, count = max(0, min(kLaneCoords, len - at));
+    const uint8_t* src = a.sym + (size_t)k * a.d + lo + at;
+    uint16_t* cnt = reinterpret_cast<uint16_t*>(s_raw + h.off_cnt) + (par * U + warp) * 32;
+    uint32_t* last = reinterpret_cast<uint32_t*>(s_raw + h.off_last) + par * U + warp;
+    LaneBits out;
+    out.open(img);
+    auto put4 = [&](uint32_t s4) {                                     // four symbols
+      uint32_t lv = s4 & 0x1f1f1f1fu;
+      if ((lv + limit4) & 0x80808080u) {                               // not a level of this code: sent as level 0
+        bad = true;
+        lv = 0u; s4 = 0u;
+      }
+      const uint32_t c4 = lv + ((s4 >> 7) & 0x01010101u) * (uint32_t)nlev;
+      out.put(lds_table32(__dp2a_lo(weights, c4, pair_sa)));
+      out.put(lds_table32(__dp2a_hi(weights, c4, pair_sa)));
+    };
+    if (count == kLaneCoords && a.load == 16) {
+      const uint4 x = __ldcs(reinterpret_cast<const uint4*>(src)), y = __ldcs(reinterpret_cast<const uint4*>(src) + 1);
+      put4(x.x); put4(x.y); put4(x.z); put4(x.w);
+      put4(y.x); put4(y.y); put4(y.z); put4(y.w);
+    } else if (count == kLaneCoords && a.load == 4) {
+      uint32_t w[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) w[j] = __ldcs(reinterpret_cast<const uint32_t*>(src) + j);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) put4(w[j]);
+    } else {
+#pragma unroll 1
+      for (int i = 0; i < count; ++i) {
+        uint32_t s = src[i];
+        if ((int)(s & 31u) >= nlev) { bad = true; s = 0u; }
+        const uint32_t e = s_lut.e[(s & 31u) | ((s >> 7) << 5)];
+        out.put((e & 0xffffu) | ((e >> 16) << 26));
+      }
+    }
+    if (lane == 31) *last = out.hi;                                    // the chunk's last 32 bits, for the chunk after it
+    const uint32_t bits = out.close(img);
+    cnt[lane] = (uint16_t)bits;
+    const uint32_t chunk_bits = __reduce_add_sync(0xffffffffu, bits);
+    if (lane == 0) s_tot[par][warp] = chunk_bits;
+    __syncthreads();
+    // Lane i: chunk i.  Its first bit in the bucket's payload, the bucket's words, the words before the bucket.
+    const uint32_t mine = lane < U ? s_tot[par][lane & 15] : 0u;
+    uint32_t upto = mine;
+    for (int o = 1; o < m; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, upto, o);
+      if ((lane & (m - 1)) >= o) upto += y;
+    }
+    const uint32_t payload = __shfl_sync(0xffffffffu, upto, lane | (m - 1));
+    const int blen = min(a.bucket, len - (lane & ~(m - 1)) * kPackChunk);
+    const bool first = lane < U && (lane & (m - 1)) == 0 && blen > 0;  // the bucket's first chunk
+    const uint32_t nsub = blen > 0 && ct.has_header ? (uint32_t)((blen + G - 1) / G) : 0u, hdr_bits = kNormBits + 16u * nsub;
+    const uint32_t nbits = hdr_bits + payload, nwords = (nbits + 31u) >> 5;
+    const uint32_t words_upto = warp_incl_scan(first ? nwords : 0u, lane);
+    const uint32_t before = __shfl_sync(0xffffffffu, words_upto - (first ? nwords : 0u), lane & ~(m - 1));   // words before the bucket
+    const size_t b0 = lo >> (10 + h.m_log);
+    if (warp == 0) {
+      const uint32_t words = __shfl_sync(0xffffffffu, words_upto, 31);
+      const uint32_t pads = __reduce_add_sync(0xffffffffu, first ? 32u * nwords - nbits : 0u);
+      const unsigned long long sums = (unsigned long long)words | ((unsigned long long)pads << kPadShift);
+      unsigned long long* row = a.status + (size_t)k * h.status_ld;
+      const size_t su = (size_t)u + h.status_first;
+      if (lane == 0) st_status(row + su, kStAggregate | sums);
+      if (first) a.bucket_bits[(size_t)k * a.nb + b0 + (size_t)(lane >> h.m_log)] = nbits;
+      bool timed_out = false;
+      const unsigned long long excl = lookback_prefix(row, (long long)su, lane, a.spin_limit, &timed_out);
+      if (lane == 0) {
+        const unsigned long long incl = excl + sums, upto_here = incl & ((1ull << kPadShift) - 1ull);
+        st_status(row + su, kStPrefix | incl);
+        if (timed_out) latch_error(a.st, QGX_ERR_TIMEOUT);
+        if ((size_t)u + 1 == h.units) a.total_bits[k] = 32ull * upto_here - (incl >> kPadShift);
+        s_base[par] = excl & ((1ull << kPadShift) - 1ull);
+        s_skip[par] = timed_out || upto_here > (unsigned long long)a.cap_words ? 1 : 0;
+        s_ticket[par ^ 1] = atomicAdd(a.ticket, 1u);
+      }
+    }
+    __syncthreads();
+    if (!s_skip[par] && len - warp * kPackChunk > 0) {
+      const uint32_t bit = __shfl_sync(0xffffffffu, hdr_bits + upto - mine, warp), bucket_bits = __shfl_sync(0xffffffffu, nbits, warp & ~(m - 1));
+      const uint32_t word = __shfl_sync(0xffffffffu, before, warp), subs = __shfl_sync(0xffffffffu, nsub, warp);
+      place_chunk<G>(a.stream + (size_t)k * a.cap_words + s_base[par] + word, bit, bucket_bits, warp & (m - 1), subs,
+                     a.norms[(size_t)k * a.nb + b0 + (size_t)(warp >> h.m_log)], cnt, last, img, lane);
+    }
+    // No barrier here: the next unit's counts and last bits go to the other half, the images are the warps' own.
+  }
+  if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
+}
+
+bool pack_chunks_fits(int K, size_t nb, int bucket) {
+  return bucket % kPackChunk == 0 && (bucket & (bucket - 1)) == 0 && (unsigned long long)K * nb < (1ull << 31);
+}
+
+qgx_status launch_pack_chunks(qgx_ctx* c, PackArgs a, size_t b_first, const CodeTable& ct) {
+  const int m = a.bucket / kPackChunk;
+  PackShape h;
+  h.m_log = 31 - __builtin_clz((unsigned)m);
+  // units of 16 chunks; fewer where that would leave SMs without any
+  const size_t chunks = (a.nb - b_first) * (size_t)m;
+  h.unit = 16;
+  while (h.unit > std::max(m, 4) && (chunks + (size_t)h.unit - 1) / (size_t)h.unit * (size_t)a.K < 4 * (size_t)c->num_sms) h.unit /= 2;
+  h.units = (chunks + (size_t)h.unit - 1) / (size_t)h.unit;
+  h.first = b_first * (size_t)a.bucket;
+  h.status_first = (b_first * (size_t)m + (size_t)h.unit - 1) / (size_t)h.unit;
+  h.status_ld = h.status_first + h.units;                              // at most nb + 1
+  h.lane_words = (uint32_t)pipe_lane_stride(ct.maxlen);
+  h.off_image = (uint32_t)(4 * 4 * ct.nlev * ct.nlev);
+  h.off_cnt = h.off_image + (uint32_t)h.unit * 32u * h.lane_words * 4u + 64u;    // a lane's reads may run past its words
+  h.off_last = h.off_cnt + 2u * (uint32_t)h.unit * 64u;
+  const size_t smem = h.off_last + 2u * (uint32_t)h.unit * 4u;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(a.sym);
+  a.load = (a.d % 16 == 0 && (at & 15u) == 0) ? 16 : ((a.d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
+  const unsigned threads = 32u * (unsigned)h.unit, per_sm = std::min(1536u / threads, (unsigned)((220u * 1024u) / (smem + 2048u)));
+  const size_t units = h.units * (size_t)a.K;
+  const unsigned grid = (unsigned)std::min<size_t>(units, (size_t)c->num_sms * per_sm);
+#define QGX_LAUNCH_C(GG)                                                       \
+  do {                                                                         \
+    allow_max_dynamic_smem((const void*)k_pack_chunks<GG>, c->device);         \
+    launch_next(true, k_pack_chunks<GG>, grid, threads, smem, c->stream, a, h, ct);  \
+  } while (0)
+  if (!ct.has_header || ct.G == 32) QGX_LAUNCH_C(32);
+  else if (ct.G == 64) QGX_LAUNCH_C(64);
+  else QGX_LAUNCH_C(128);
+#undef QGX_LAUNCH_C
+  count_launch(c);
+  return cuda_status(cudaGetLastError());
+}
+
+}  // namespace qgx
