@@ -169,8 +169,8 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     if (kCompare) fill_signed_values(reinterpret_cast<float*>(s_raw + h.off_kept), lt_kept);
   }
   __syncthreads();
-  start_next();
   await_previous();
+  start_next();
   // for the next exchange's scan and totals; nobody reads them after the encode pass
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.scan_words; i += (size_t)gridDim.x * blockDim.x) a.scan[i] = 0ull;
   if (blockIdx.x == 0 && a.sums) {

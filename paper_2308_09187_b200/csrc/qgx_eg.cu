@@ -51,8 +51,8 @@ __device__ __forceinline__ double gemv_row(const float* __restrict__ m, size_t n
 __global__ void __launch_bounds__(256) k_gemv_rows(const float* __restrict__ mat, size_t nrows, size_t ncols,
                                                    const float* __restrict__ x, const float* __restrict__ bias,
                                                    float* __restrict__ out, bool vec_ok) {
-  start_next();
   await_previous();
+  start_next();
   const int lane = threadIdx.x & 31;
   const size_t warp = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const size_t nwarps = ((size_t)gridDim.x * blockDim.x) >> 5;
@@ -68,8 +68,8 @@ __global__ void __launch_bounds__(256) k_gemv_rows(const float* __restrict__ mat
 __global__ void __launch_bounds__(1024) k_bilinear(const float* __restrict__ mat, size_t n, const float* __restrict__ z,
                                                    float* __restrict__ out_all, bool vec_ok) {
   __shared__ double s_part[32][33];
-  start_next();
   await_previous();
+  start_next();
   const int cx = threadIdx.x, ry = threadIdx.y;
   const size_t col_blocks = (n + 31) / 32;
   if (blockIdx.x >= col_blocks) {
@@ -109,8 +109,8 @@ __global__ void __launch_bounds__(1024) k_bilinear(const float* __restrict__ mat
 }
 
 __global__ void __launch_bounds__(256) k_diag(const float* __restrict__ D, const float* __restrict__ x, float* __restrict__ out, size_t d) {
-  start_next();
   await_previous();
+  start_next();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (size_t)gridDim.x * blockDim.x)
     out[i] = __fmul_rn(D[i], x[i]);
 }
@@ -128,8 +128,8 @@ __global__ void __launch_bounds__(256) k_eg_init(float* X, float* Y, float* Xbar
 __global__ void __launch_bounds__(256) k_eg_finish(float* __restrict__ X, const float* __restrict__ Y, float* __restrict__ Xbar,
                                                    const float* __restrict__ Xhalf, const float* __restrict__ anchor,
                                                    double* scalars, size_t d, int K, int t) {
-  start_next();
   await_previous();
+  start_next();
   const float gamma = (float)((double)K / sqrt(1.0 + scalars[0]));
   const float tf = (float)t;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (size_t)gridDim.x * blockDim.x) {
@@ -144,8 +144,8 @@ __global__ void __launch_bounds__(256) k_eg_finish(float* __restrict__ X, const 
 // X_{t+1/2} = X_t - gamma_t * m (optimistic dual averaging: m is the mean of the previous iteration's quantized vectors)
 __global__ void __launch_bounds__(256) k_half_from_mean(const float* __restrict__ X, const float* __restrict__ m,
                                                         const double* __restrict__ scalars, float* __restrict__ Xhalf, size_t d) {
-  start_next();
   await_previous();
+  start_next();
   const float gamma = (float)scalars[1];
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (size_t)gridDim.x * blockDim.x)
     Xhalf[i] = __fsub_rn(X[i], __fmul_rn(gamma, m[i]));

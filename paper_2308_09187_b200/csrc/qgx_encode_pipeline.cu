@@ -265,8 +265,8 @@ k_encode_pipeline(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
   if (threadIdx.x == 0) { s_quit[0] = 0; s_quit[1] = kBarLooksBase + a.spin_limit / kBarLooksPolls; }
   if (threadIdx.x < kTurnRing) bar_init(turned + 8u * threadIdx.x, kQuantizers);
   __syncthreads();
-  start_next();
   await_previous();
+  start_next();
   volatile int* quit = s_quit;
   // a wait that ran out: everybody gives up, the launch ends and reports it
   auto give_up = [&]() {

@@ -136,8 +136,8 @@ k_exchange_encode(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
   }
   if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
   for (int i = threadIdx.x; i < 2 * img_words; i += blockDim.x) s_dyn[i] = 0;
-  start_next();
   await_previous();
+  start_next();
   if (threadIdx.x == 0) s_ticket[0] = atomicAdd(a.ticket, 1u);
   __syncthreads();
   const int nlev = lt.nlev;

@@ -71,8 +71,8 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
     s_lev_kept[tid] = tid < lt_kept.nlev ? lt_kept.lev[tid] : 0.0f;
   }
   for (uint32_t i = (uint32_t)tid; i < r.img_words; i += blockDim.x) s_img[i] = 0u;
-  start_next();
   await_previous();
+  start_next();
   // which bucket: a ticket per cluster, so that the buckets a bucket looks back at are already under way
   unsigned ticket = 0;
   if (k == 0 && tid == 0) ticket = atomicAdd(a.ticket, 1u);

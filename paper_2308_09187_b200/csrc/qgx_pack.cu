@@ -40,8 +40,8 @@ __global__ void __launch_bounds__(512, 3) k_pack_chunks(const __grid_constant__ 
     const uint32_t x = s_lut.e[f < nlev ? f : f - nlev + 32], y = s_lut.e[g < nlev ? g : g - nlev + 32];
     s_pair[i] = ((x & 0xffffu) | ((y & 0xffffu) << (x >> 16))) | (((x >> 16) + (y >> 16)) << 26);
   }
-  start_next();
   await_previous();
+  start_next();
   if (threadIdx.x == 0) s_ticket[0] = atomicAdd(a.ticket, 1u);
   __syncthreads();
   const uint32_t pair_sa = smem_addr(s_pair), weights = 4u | ((uint32_t)(8 * nlev) << 16);

@@ -78,8 +78,8 @@ k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ Level
   __shared__ double s_red[2][32];
   fill_bin_table(s_bin, rt, BinKind::kFixed);
   if (threadIdx.x < QGX_MAX_LEVELS) s_lev[threadIdx.x] = threadIdx.x < lt.nlev ? lt.lev[threadIdx.x] : 1.0f;
-  start_next();
   await_previous();
+  start_next();
   __syncthreads();
   constexpr bool kTeams = P == 1;
   const int lane = threadIdx.x & 31;
@@ -193,8 +193,8 @@ __global__ void __launch_bounds__(256) k_average(const float* __restrict__ norms
                                                  int bucket, size_t nb, const __grid_constant__ LevelTable lt, float* __restrict__ out, DevStatus* st) {
   __shared__ float s_lev[QGX_MAX_LEVELS * 32];
   for (int i = threadIdx.x; i < QGX_MAX_LEVELS * 32; i += blockDim.x) s_lev[i] = (i >> 5) < lt.nlev ? lt.lev[i >> 5] : 0.0f;
-  start_next();
   await_previous();
+  start_next();
   __syncthreads();
   const size_t groups = (d + V - 1) / V;
   const float Kf = (float)K;
