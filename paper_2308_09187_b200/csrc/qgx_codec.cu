@@ -1,7 +1,7 @@
 // qgx_encode and qgx_decode as separate steps.  Encoding takes one pass (k_pack: pack a bucket, find its place by look-back,
 // copy it out) where the capacity fits any outcome and the sub-blocks are a warp's, else three kernels: bucket bit lengths ->
 // exclusive scan of the word-aligned lengths (offsets) -> bit scatter; qgx_encode_noalloc takes the three always.  Decoding:
-// offsets (k_scan_offsets, which also builds the decoder's table) -> k_unpack_rows or k_unpack.
+// offsets (k_scan_offsets, which also builds the decoder's table) -> k_unpack_rows, k_unpack_parts or k_unpack.
 #include "qgx_bucket.cuh"
 #include "qgx_codec.cuh"
 #include "qgx_pack.cuh"
@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_offsets(const uint32_t* _
                                                                uint64_t* __restrict__ off, uint64_t* __restrict__ total_bits,
                                                                uint32_t* __restrict__ flags, unsigned int err_code, DevStatus* st,
                                                                int K, const __grid_constant__ CodeTable ct, uint16_t* table, uint32_t* pair) {
-  start_next();
   await_previous();
+  start_next();
   if (blockIdx.x >= (unsigned)K) {
     if (pair) build_unpack_pairs(ct, pair, (blockIdx.x - (unsigned)K) * kScanThreads + threadIdx.x, kPairBuilders * kScanThreads);
     else build_unpack_table(ct, table);
@@ -389,11 +389,11 @@ struct UnpackArgs {
 
 // One thread per sub-block (per bucket without sub-blocks), a warp on consecutive ones of one bucket or of several small
 // buckets; persistent CTAs, so that the table is copied once per CTA and not once per bucket.  For what k_unpack_rows does not
-// take: sub-blocks of other lengths, or none.  Every read is bounded by the bucket's words.  A serial walk per thread: latency-bound with few sub-blocks, instruction-bound (14 per symbol) with many.
+// take: sub-blocks of other lengths; and none, where there are many buckets.  Every read is bounded by the bucket's words.  A serial walk per thread: latency-bound with few sub-blocks, instruction-bound (14 per symbol) with many.
 __global__ void __launch_bounds__(128) k_unpack(const __grid_constant__ UnpackArgs a, const __grid_constant__ CodeTable ct) {
   extern __shared__ __align__(16) uint16_t s_tab[];  // [2 << maxlen], see build_unpack_table
-  start_next();
   await_previous();
+  start_next();
   const int tab_n = 2 << ct.maxlen;
   for (int i = threadIdx.x; i < (tab_n + 7) / 8; i += blockDim.x) reinterpret_cast<uint4*>(s_tab)[i] = __ldg(reinterpret_cast<const uint4*>(a.table) + i);
   __syncthreads();
@@ -618,7 +618,7 @@ qgx_status qgx_decode(qgx_ctx* c, const uint32_t* stream, size_t cap_words, cons
   const size_t nb = (d + (size_t)bucket - 1) / (size_t)bucket;
   uint64_t* off = (uint64_t*)ws_get(c, 0, sizeof(uint64_t) * (size_t)K * nb);
   uint32_t* flags = (uint32_t*)ws_get(c, 1, sizeof(uint32_t) * (size_t)K);
-  const bool rows = unpack_rows_fits(K, d, bucket, ct);
+  const bool parts = unpack_parts_fits(c, K, nb, bucket, ct), rows = parts || unpack_rows_fits(K, d, bucket, ct);
   void* table = ws_get(c, 2, std::max(sizeof(uint16_t) * (size_t)kUnpackTableMax, sizeof(uint32_t) << kPairBitsMax));
   if (!off || !flags || !table) return QGX_ERR_CUDA;
   launch_next(true, k_scan_offsets, K + (rows ? kPairBuilders : 1u), kScanThreads, 0, c->stream, bucket_bits, nb, cap_words, off, nullptr, flags,
@@ -626,7 +626,7 @@ qgx_status qgx_decode(qgx_ctx* c, const uint32_t* stream, size_t cap_words, cons
   if (rows) {
     count_launch(c);
     const UnpackRowsArgs r{stream, cap_words, bucket_bits, off, flags, (const uint32_t*)table, d, K, nb, norms, sym, c->dstatus};
-    return launch_unpack_rows(c, r, bucket, ct);
+    return parts ? launch_unpack_parts(c, r, bucket, ct) : launch_unpack_rows(c, r, bucket, ct);
   }
   UnpackArgs a;
   a.stream = stream; a.cap_words = cap_words; a.bucket_bits = bucket_bits; a.off = off; a.flags = flags; a.table = (const uint16_t*)table; a.d = d;

@@ -1,8 +1,8 @@
-// qgx_decode for codes with sub-blocks of 32, 64 or 128 coordinates: a warp takes a row of 32 consecutive sub-blocks of one
+// qgx_decode.  Codes with sub-blocks of 32, 64 or 128 coordinates: a warp takes a row of 32 consecutive sub-blocks of one
 // worker, copies its stream words to shared memory, walks them a lane per sub-block, two symbols per look-up, and copies the
 // symbols out.  The next row's numbers and header are asked for while this one is walked.
 // What bounds it: instructions, 17 per symbol at 64 % issue.  A thread per sub-block with its own window on global memory, one
-// symbol per look-up (k_unpack, which still serves other sub-block lengths and none) takes 45.7 us for 8 x 2^22 symbols of 17
+// symbol per look-up (k_unpack, which still serves other sub-block lengths) takes 45.7 us for 8 x 2^22 symbols of 17
 // fitted levels, this 27.5.
 #include "qgx_unpack.cuh"
 
@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(1024, 1) k_unpack_rows(const __grid_constant__
     return r;
   };
 
-  start_next();
   await_previous();                      // (the table, too, is the kernel's before this one)
+  start_next();
   uint32_t it = blockIdx.x + gridDim.x * (uint32_t)warp;
   Bucket bucket = ask_bucket(it);
   {
@@ -222,6 +222,156 @@ qgx_status launch_unpack_rows(qgx_ctx* c, const UnpackRowsArgs& a, int bucket, c
   if (ct.G == 32) return launch_unpack_g<32>(c, a, bucket, ct);
   if (ct.G == 64) return launch_unpack_g<64>(c, a, bucket, ct);
   return launch_unpack_g<128>(c, a, bucket, ct);
+}
+
+// ---- codes without sub-blocks -----------------------------------------------------------------
+// A bucket is one chain of codewords.  Where there are many buckets a lane walks one (k_unpack).  Where there are few a CTA takes
+// one apart: its bits are cut into parts, and for every part and every bit that its first codeword can start at (the longest
+// symbol's length of them) a thread walks to the next part.  Where the walks end, taken one after the other from the bucket's
+// first codeword on, is where the parts' codewords really start, and the walks' counts give their places; one thread per part
+// walks once more and writes symbols.
+struct BucketWalk {
+  const uint32_t* words;
+  uint32_t nwords, next;                 // the word after w2
+  uint32_t w0, w1, w2, pos, old;         // see Walk; w2: fetched a word early
+  __device__ __forceinline__ uint32_t word(uint32_t i) const { return i < nwords ? __ldg(words + i) : 0u; }
+  __device__ __forceinline__ void open(uint32_t bit) {                 // bit: the next symbol's first, at least 2
+    const uint32_t i = (bit - 2u) >> 5;
+    w0 = word(i);
+    w1 = word(i + 1u);
+    w2 = word(i + 2u);
+    next = i + 3u;
+    pos = old = (bit - 2u) & 31u;
+  }
+  __device__ __forceinline__ uint32_t window() const { return __funnelshift_r(w0, w1, pos); }
+  __device__ __forceinline__ void settle() {
+    if ((pos ^ old) & 32u) {
+      w0 = w1;
+      w1 = w2;
+      w2 = word(next);
+      ++next;
+    }
+    old = pos;
+  }
+  __device__ __forceinline__ uint32_t bit() const { return 32u * (next - 3u) + (pos & 31u) + 2u; }   // of the next symbol
+};
+struct PartsShape {
+  size_t buckets;                        // of all workers
+  int bucket;
+  int starts_log, parts;                 // log2 of the threads per part, parts per bucket
+  uint32_t pair_mask;
+};
+constexpr int kPartThreads = 1024;
+
+struct BucketOf { size_t k, bi, lo; int count; bool sound, dead; uint32_t nbits; };
+__device__ __forceinline__ BucketOf bucket_of(const UnpackRowsArgs& a, const PartsShape& h, size_t bi, BucketWalk* w) {
+  BucketOf b;
+  const bool there = bi < h.buckets;
+  b.bi = bi;
+  b.k = !there ? 0 : (h.buckets <= 0xffffffffull ? (size_t)((uint32_t)bi / (uint32_t)a.nb) : bi / a.nb);
+  b.lo = there ? (bi - b.k * a.nb) * (size_t)h.bucket : 0;
+  b.count = there ? (int)min((size_t)h.bucket, a.d - b.lo) : 0;
+  b.dead = !there || a.flags[b.k] != 0u;                 // the worker's lengths exceed its words: nothing is read
+  b.nbits = b.dead ? 0u : a.bucket_bits[bi];
+  b.sound = b.nbits >= (uint32_t)kNormBits;              // otherwise nothing trustworthy to read: zeros
+  w->words = a.stream + b.k * a.cap_words + (b.sound ? a.off[bi] : 0ull);
+  w->nwords = b.sound ? (b.nbits + 31u) >> 5 : 0u;
+  return b;
+}
+__device__ __forceinline__ WalkTable bring_table(const UnpackRowsArgs& a, const PartsShape& h, unsigned char* s_raw) {
+  const uint4* src = reinterpret_cast<const uint4*>(a.pair);
+  const int n = (int)((h.pair_mask + 4u) >> 4);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) reinterpret_cast<uint4*>(s_raw)[i] = __ldg(src + i);
+  __syncthreads();
+  return WalkTable{smem_addr(s_raw), h.pair_mask};
+}
+
+// What bounds it: latency, a chain of a part's look-ups, a step per part, a part's look-ups again, instead of a bucket's.  A decode
+// call on 68 buckets of 512 symbols 29 -> 11 us, on 1172 of 1024 53 -> 25.
+__global__ void __launch_bounds__(kPartThreads) k_unpack_parts(const __grid_constant__ UnpackRowsArgs a, const __grid_constant__ PartsShape h) {
+  extern __shared__ __align__(128) unsigned char s_raw[];
+  __shared__ uint32_t s_walk[kPartThreads];              // where the walk ends, bits past the next part's first | symbols << 8
+  __shared__ uint32_t s_start[kPartThreads], s_place[kPartThreads + 1];
+  await_previous();
+  start_next();
+  const WalkTable wt = bring_table(a, h, s_raw);
+  const int part = (int)threadIdx.x >> h.starts_log, late = (int)threadIdx.x & ((1 << h.starts_log) - 1);
+  bool bad = false;
+  for (size_t bi = blockIdx.x; bi < h.buckets; bi += gridDim.x) {
+    BucketWalk w;
+    const BucketOf b = bucket_of(a, h, bi, &w);
+    bad = bad || (!b.dead && !b.sound);
+    if (threadIdx.x == 0) a.norms[bi] = __uint_as_float(w.word(0u));
+    const uint32_t payload = b.sound ? b.nbits - (uint32_t)kNormBits : 0u;
+    auto first_of = [&](int p) { return (uint32_t)kNormBits + (uint32_t)((unsigned long long)payload * (unsigned)p / (unsigned)h.parts); };
+    const uint32_t from = first_of(part), to = first_of(part + 1);
+    {
+      uint32_t n = 0;
+      w.open(from + (uint32_t)late);
+      while (w.bit() < to) {
+        const uint32_t e = wt.entry(w.window()), one = first_bits(e);
+        const bool two = !(e & kPairEscape) && w.bit() + one < to;
+        w.pos += two ? e & 31u : one;
+        n += two ? 2u : 1u;
+        w.settle();
+      }
+      s_walk[threadIdx.x] = (w.bit() - to) | (n << 8);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t at = 0, place = 0;
+      for (int p = 0; p < h.parts; ++p) {
+        s_start[p] = at;
+        s_place[p] = place;
+        const uint32_t x = s_walk[(p << h.starts_log) + (int)at];
+        at = x & 0xffu;
+        place += x >> 8;
+      }
+      s_place[h.parts] = place;
+      bad = bad || (b.sound && (at != 0u || place != (uint32_t)b.count));   // the bucket uses exactly its bits
+    }
+    __syncthreads();
+    uint8_t* out = a.sym + b.k * a.d + b.lo;
+    // symbols, as many as there should be (a stream that holds fewer is filled up with zeros)
+    if ((uint32_t)late == s_start[part]) {
+      uint32_t marks = 0;
+      w.open(from + (uint32_t)late);
+      const uint32_t end = min(s_place[part + 1], (uint32_t)b.count);
+      for (uint32_t i = s_place[part]; i < end; ++i) {
+        const uint32_t x = walk_one(w, wt);
+        marks |= x;
+        out[i] = (uint8_t)(x & 0xbfu);
+      }
+      bad = bad || (marks & kNoSymbol) != 0u;
+    }
+    for (uint32_t i = s_place[h.parts] + threadIdx.x; i < (uint32_t)b.count; i += blockDim.x) out[i] = 0;
+    __syncthreads();                                     // the next bucket's walks replace this one's
+  }
+  if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
+}
+
+// threads for every bit that a codeword can start at after a part's first (a symbol's bits, the longest's, of them)
+static int starts_log2(const CodeTable& ct) {
+  int l = 1;
+  while ((1 << l) < ct.maxlen + 1) ++l;
+  return l;
+}
+// Per bucket `starts` times a walk's work, against the time that a walk takes when there are few: in us, on 148 SMs, 1.6 starts per
+// 10^6 symbols against 0.05 per symbol of a bucket and 2.2 per 10^6 -- 4700 buckets where a symbol has up to 8 bits, 2130 up to 13.
+bool unpack_parts_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct) {
+  return !ct.has_header && bucket >= 64 && nb * (size_t)K * ((8u << starts_log2(ct)) - 11u) <= (size_t)c->num_sms * 1700u;
+}
+qgx_status launch_unpack_parts(qgx_ctx* c, const UnpackRowsArgs& a, int bucket, const CodeTable& ct) {
+  PartsShape h;
+  h.buckets = a.nb * (size_t)a.K;
+  h.bucket = bucket;
+  h.pair_mask = (4u << pair_bits(ct.maxlen)) - 4u;
+  h.starts_log = starts_log2(ct);
+  const int threads = bucket <= 1024 ? 256 : kPartThreads;
+  h.parts = threads >> h.starts_log;
+  launch_next(true, k_unpack_parts, (unsigned)h.buckets, threads, h.pair_mask + 4u, c->stream, a, h);
+  count_launch(c);
+  return cuda_status(cudaGetLastError());
 }
 
 }  // namespace qgx

@@ -1,4 +1,4 @@
-// qgx_decode by rows of sub-blocks (qgx_unpack.cu).
+// qgx_decode by rows of sub-blocks or by parts of buckets (qgx_unpack.cu).
 #pragma once
 
 #include "qgx_walk.cuh"
@@ -30,5 +30,8 @@ struct UnpackRowsArgs {
 
 bool unpack_rows_fits(int K, size_t d, int bucket, const CodeTable& ct);
 qgx_status launch_unpack_rows(qgx_ctx* c, const UnpackRowsArgs& a, int bucket, const CodeTable& ct);
+// codes without sub-blocks, a few buckets
+bool unpack_parts_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct);
+qgx_status launch_unpack_parts(qgx_ctx* c, const UnpackRowsArgs& a, int bucket, const CodeTable& ct);
 
 }  // namespace qgx

@@ -100,37 +100,47 @@ struct WalkTable {
 };
 __device__ __forceinline__ uint32_t first_bits(uint32_t entry) { return (entry >> 8) & 31u; }
 
-// G symbols of one sub-block to row[0 .. G / 4) (shared address), four to a word.  A window holds 30 bits to come, so two
-// entries of at most 13; where an entry stands for one symbol only the second is looked up on its own, its bits taken at once
-// and the entry's own cleared.
+// The next four symbols, a byte each.  A window holds 30 bits to come, so two entries of at most 13; where an entry stands for one
+// symbol only the second is looked up on its own, its bits taken at once and the entry's own cleared.
+template <class W>
+__device__ __forceinline__ uint32_t walk_four(W& w, const WalkTable& t) {
+  uint32_t win = w.window();
+  uint32_t e = t.entry(win);
+  if (e & kPairEscape) {
+    const uint32_t f = t.entry(__funnelshift_r(win, 0u, e));
+    w.pos += (e & 31u) + first_bits(f);
+    w.settle();
+    win = w.window();
+    e = prmt(prmt(e, f, 0x6200u), 0u, 0x3244u);                        // the two symbols, nothing taken
+  }
+  w.pos += e;
+  win = __funnelshift_r(win, 0u, e);
+  uint32_t f = t.entry(win);
+  if (f & kPairEscape) {
+    w.settle();
+    w.pos += f & 31u;
+    w.settle();
+    const uint32_t g = t.entry(w.window());
+    w.pos += first_bits(g);
+    f = prmt(prmt(f, g, 0x6200u), 0u, 0x3244u);
+  }
+  w.pos += f;
+  w.settle();
+  return prmt(e, f, 0x7632u);
+}
+template <class W>
+__device__ __forceinline__ uint32_t walk_one(W& w, const WalkTable& t) {
+  const uint32_t e = t.entry(w.window());
+  w.pos += first_bits(e);
+  w.settle();
+  return (e >> 16) & 0xffu;
+}
+
+// G symbols of one sub-block to row[0 .. G / 4) (shared address), four to a word
 template <int G, bool SH>
 __device__ __forceinline__ void walk_whole(Walk<SH>& w, uint32_t row, const WalkTable& t) {
 #pragma unroll
-  for (int i = 0; i < G; i += 4) {
-    uint32_t win = w.window();
-    uint32_t e = t.entry(win);
-    if (e & kPairEscape) {
-      const uint32_t f = t.entry(__funnelshift_r(win, 0u, e));
-      w.pos += (e & 31u) + first_bits(f);
-      w.settle();
-      win = w.window();
-      e = prmt(prmt(e, f, 0x6200u), 0u, 0x3244u);                      // the two symbols, nothing taken
-    }
-    w.pos += e;
-    win = __funnelshift_r(win, 0u, e);
-    uint32_t f = t.entry(win);
-    if (f & kPairEscape) {
-      w.settle();
-      w.pos += f & 31u;
-      w.settle();
-      const uint32_t g = t.entry(w.window());
-      w.pos += first_bits(g);
-      f = prmt(prmt(f, g, 0x6200u), 0u, 0x3244u);
-    }
-    w.pos += f;
-    w.settle();
-    sts32(row + (uint32_t)i, prmt(e, f, 0x7632u));
-  }
+  for (int i = 0; i < G; i += 4) sts32(row + (uint32_t)i, walk_four(w, t));
 }
 // the same, one symbol at a time, for `count` symbols (the vector's last sub-block)
 template <bool SH>
@@ -139,12 +149,7 @@ __device__ __forceinline__ void walk_some(Walk<SH>& w, int count, uint32_t row, 
   for (int i = 0; i < count; i += 4) {
     uint32_t word = 0;
 #pragma unroll 1
-    for (int q = 0; q < 4 && i + q < count; ++q) {
-      const uint32_t e = t.entry(w.window());
-      w.pos += first_bits(e);
-      w.settle();
-      word |= ((e >> 16) & 0xffu) << (8 * q);
-    }
+    for (int q = 0; q < 4 && i + q < count; ++q) word |= walk_one(w, t) << (8 * q);
     sts32(row + (uint32_t)i, word);
   }
 }

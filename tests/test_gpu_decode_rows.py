@@ -87,3 +87,28 @@ def test_separate_decode_and_average(K, d, bucket, nlev, sub, code, shift):
         assert np.array_equal(mean.cpu().numpy(), o.average(norms.cpu().numpy(), sym.cpu().numpy(), bucket, lev))
     finally:
         qgx.qgx_destroy(ctx)
+
+
+@pytest.mark.parametrize("K,d,bucket,nlev,code", [
+    (1, 1, 4, 2, "fixed"), (4, 8200, 512, 9, "fixed"), (3, 16384 + 5, 16384, 32, "elias"), (2, 40 * 1000 + 17, 1000, 17, "steep"),
+    (8, 3000 * 64, 64, 9, "elias"), (1, 148 * 16 * 32 * 20 + 3, 20, 17, "steep"), (5, 2048 * 300 + 1, 2048, 32, "steep")])
+def test_decode_without_sub_blocks(K, d, bucket, nlev, code):
+    """One walk per bucket: rings that turn over many times and not at all, one to thirty-two lanes per walk, ragged ends."""
+    import paper_2308_09187_b200 as qgx
+    ctx = qgx.qgx_create(0)
+    try:
+        g = torch.Generator("cuda").manual_seed(d)
+        sym = torch.randint(0, nlev, (K, d), generator=g, device="cuda", dtype=torch.uint8)     # every level, long codewords too
+        sym |= ((torch.rand((K, d), generator=g, device="cuda") < 0.5) & (sym != 0)).to(torch.uint8) * 128
+        norms = torch.rand((K, o.nbuckets(d, bucket)), generator=g, device="cuda") + 0.5
+        cb = (qgx.qgx_build_codebook_fixed(nlev, 0) if code == "fixed" else qgx.qgx_build_codebook_elias(nlev, 0) if code == "elias" else
+              qgx.qgx_build_codebook_huffman([2.0 ** -(j + 1) for j in range(nlev)], 0))
+        stream, bits, _ = qgx.qgx_encode(ctx, norms, sym, bucket, cb)
+        got_norms, got = qgx.qgx_decode(ctx, stream, bits, d, bucket, cb)
+        qgx.qgx_sync_status(ctx)
+        assert torch.equal(got_norms, norms) and torch.equal(got, sym)
+        bits[K - 1, 0] -= 1                                  # one bit too few for its symbols
+        qgx.qgx_decode(ctx, stream, bits, d, bucket, cb)
+        assert qgx.qgx_sync_status(ctx, check=False) == qgx.QGX_ERR_CORRUPT
+    finally:
+        qgx.qgx_destroy(ctx)
