@@ -306,8 +306,19 @@ k_encode_pipeline(const __grid_constant__ EncodeArgs a, const __grid_constant__ 
             const int bytes = max(0, min(16, 4 * (left - e)));
             copy_async16(dst + 512u * (uint32_t)q + ((q & 1) ? off1 : off0), bytes > 0 ? from + e : from, bytes);
           }
+        } else if (left >= kChunk) {
+          // rows off the 16-byte grid: 32 coordinates at a time, lane l the word l & 3 of piece 8 q + l / 4 -- byte offset 128 q plus
+          // 16 ((l / 4) ^ (q & 7)) plus 4 (l & 3), see piece_at
+          const float* p = from + lane;
+          uint32_t word = dst + (((uint32_t)lane & 3u) << 2);
+          const uint32_t piece = ((uint32_t)lane >> 2) << 4;
+#pragma unroll 1
+          for (int o = 0; o < 4; ++o, word += 1024u, p += 256) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) copy_async4(word + (piece ^ (16u * (uint32_t)q)) + 128u * (uint32_t)q, p + 32 * q, 4);
+          }
         } else {
-#pragma unroll 8
+#pragma unroll 4
           for (int q = 0; q < 32; ++q) {
             const int e = 32 * q + lane;
             copy_async4(dst + piece_at((uint32_t)(e >> 2)) + 4u * (uint32_t)(e & 3), e < left ? from + e : from, e < left ? 4 : 0);
