@@ -15,6 +15,7 @@ namespace qgx {
 // Scratch of qgx_encode_noalloc: bucket word offsets (u64 per bucket) followed by one overflow flag per
 // worker.  It lives in the library image, so every GPU that loads the library carries these bytes
 // until the process exits.
+constexpr int kWsPackScan = 20;          // workspace slot: the scan words of qgx_encode's one-pass kernels
 constexpr size_t kNoAllocMaxBuckets = 65536;            // K * nb
 constexpr size_t kNoAllocMaxWorkers = 1024;             // K
 constexpr size_t kNoAllocBytes = kNoAllocMaxBuckets * sizeof(uint64_t) + kNoAllocMaxWorkers * sizeof(uint32_t);
@@ -250,7 +251,6 @@ k_pack(const __grid_constant__ PackArgs a, const __grid_constant__ CodeTable ct)
   const int img_words = (int)((((((uint32_t)a.bucket * (uint32_t)(ct.maxlen + 1) + 16u * (uint32_t)(a.bucket / ct.G + 1) + kNormBits + 31u) >> 5) + 4) + 3u) & ~3u);
   uint32_t* s_pair = s_dyn + 2 * img_words;
   fill_enc_lut(&s_lut, ct);
-  if (threadIdx.x == 0) s_ticket[0] = a.first_ticket + atomicAdd(a.ticket, 1u);
   for (int i = threadIdx.x; i < 2 * img_words; i += blockDim.x) s_dyn[i] = 0;
   __syncthreads();
   for (int i = threadIdx.x; i < n2 * n2; i += blockDim.x) {            // (first, second): a level, plus nlev for a negative one
@@ -258,6 +258,9 @@ k_pack(const __grid_constant__ PackArgs a, const __grid_constant__ CodeTable ct)
     const uint32_t x = s_lut.e[f < nlev ? f : f - nlev + 32], y = s_lut.e[g < nlev ? g : g - nlev + 32];
     s_pair[i] = ((x & 0xffffu) | ((y & 0xffffu) << (x >> 16))) | (((x >> 16) + (y >> 16)) << 26);
   }
+  await_previous();
+  start_next();
+  if (threadIdx.x == 0) s_ticket[0] = a.first_ticket + atomicAdd(a.ticket, 1u);
   __syncthreads();
   const uint32_t pair_sa = smem_addr(s_pair), weights = 4u | ((uint32_t)(8 * nlev) << 16);
   const uint32_t limit4 = (uint32_t)(128 - nlev) * 0x01010101u;        // carries into bit 7 of a byte >= nlev
@@ -366,6 +369,7 @@ k_pack(const __grid_constant__ PackArgs a, const __grid_constant__ CodeTable ct)
       for (uint32_t i = threadIdx.x; i < nwords; i += blockDim.x) dst[i] = s_img[i];
     }
   }
+  leave_scan_zero(a);
   if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
 }
 
@@ -551,12 +555,14 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
   const bool layout = !ct.has_header || ct.G == 32 || ct.G == 64 || ct.G == 128;
   const size_t worst = qgx_stream_capacity_words(d, bucket, cb->subblock, ct.maxlen);
   if (layout && cap_words >= worst && worst < ((size_t)1 << (kPadShift - 1)) && nb < ((size_t)1 << 23) && nb * (size_t)K < ((size_t)1 << 31)) {
-    unsigned long long* status = (unsigned long long*)ws_get(c, 0, sizeof(uint64_t) * ((size_t)K * (nb + 1) + 2));
+    // zero between calls: the kernels leave it so
+    const size_t had = c->ws_bytes[kWsPackScan];
+    unsigned long long* status = (unsigned long long*)ws_get(c, kWsPackScan, sizeof(uint64_t) * ((size_t)K * (nb + 1) + 2));
     if (!status) return QGX_ERR_CUDA;
-    if (cudaMemsetAsync(status, 0, sizeof(uint64_t) * ((size_t)K * (nb + 1) + 2), c->stream) != cudaSuccess) return QGX_ERR_CUDA;
+    if (c->ws_bytes[kWsPackScan] != had && cudaMemsetAsync(status, 0, c->ws_bytes[kWsPackScan], c->stream) != cudaSuccess) return QGX_ERR_CUDA;
     PackArgs a;
     a.norms = norms; a.sym = sym; a.d = d; a.bucket = bucket; a.K = K; a.nb = nb; a.stream = stream; a.cap_words = cap_words;
-    a.bucket_bits = bucket_bits; a.total_bits = total_bits; a.status = status + 2; a.ticket = reinterpret_cast<unsigned int*>(status);
+    a.bucket_bits = bucket_bits; a.total_bits = total_bits; a.status = status + 2; a.status_words = (size_t)K * nb; a.ticket = reinterpret_cast<unsigned int*>(status);
     const size_t b_first = std::min(c->skip_buckets, nb), todo = (nb - b_first) * (size_t)K;
     a.first_ticket = (unsigned int)(nb * (size_t)K - todo); a.spin_limit = c->wait_limit; a.st = c->dstatus;
     c->skip_buckets = 0;
@@ -572,7 +578,7 @@ qgx_status qgx_encode(qgx_ctx* c, const float* norms, const uint8_t* sym, int K,
 #define QGX_LAUNCH_K(V)                                              \
   do {                                                               \
     allow_max_dynamic_smem((const void*)k_pack<V>, c->device);       \
-    k_pack<V><<<grid, threads, smem, c->stream>>>(a, ct);            \
+    launch_next(true, k_pack<V>, grid, threads, smem, c->stream, a, ct); \
   } while (0)
     if (pp == 1) QGX_LAUNCH_K(1);
     else if (pp == 2) QGX_LAUNCH_K(2);

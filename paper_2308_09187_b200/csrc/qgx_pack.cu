@@ -141,6 +141,7 @@ __global__ void __launch_bounds__(512, 3) k_pack_chunks(const __grid_constant__ 
     }
     // No barrier here: the next unit's counts and last bits go to the other half, the images are the warps' own.
   }
+  leave_scan_zero(a);
   if (bad) latch_error(a.st, QGX_ERR_CORRUPT);
 }
 
@@ -165,6 +166,7 @@ qgx_status launch_pack_chunks(qgx_ctx* c, PackArgs a, size_t b_first, const Code
   h.off_cnt = h.off_image + (uint32_t)h.unit * 32u * h.lane_words * 4u + 64u;    // a lane's reads may run past its words
   h.off_last = h.off_cnt + 2u * (uint32_t)h.unit * 64u;
   const size_t smem = h.off_last + 2u * (uint32_t)h.unit * 4u;
+  a.status_words = (size_t)a.K * h.status_ld;
   const uintptr_t at = reinterpret_cast<uintptr_t>(a.sym);
   a.load = (a.d % 16 == 0 && (at & 15u) == 0) ? 16 : ((a.d % 4 == 0 && (at & 3u) == 0) ? 4 : 1);
   const unsigned threads = 32u * (unsigned)h.unit, per_sm = std::min(1536u / threads, (unsigned)((220u * 1024u) / (smem + 2048u)));

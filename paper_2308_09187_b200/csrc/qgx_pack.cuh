@@ -20,14 +20,29 @@ struct PackArgs {
   size_t cap_words;
   uint32_t* bucket_bits;
   uint64_t* total_bits;
-  unsigned long long* status;            // [K][nb], zeroed before the launch
-  unsigned int* ticket;                  // zeroed before the launch
+  unsigned long long* status;            // [K][nb] or fewer, zero before the launch and after it (see leave_scan_zero)
+  size_t status_words;
+  unsigned int* ticket;                  // [2], zero before the launch and after it
   unsigned int first_ticket;             // K times the first bucket of every worker to encode (0 but for the diagnostic)
   int spin_limit;                        // polls of a wait for another bucket's words before it gives up
   DevStatus* st;
 };
 
-// Buckets of 1024 2^j coordinates, where there is enough of them.
+// By all threads of a CTA that is done: the last CTA leaves the scan's words and tickets zero for the next launch.
+__device__ __forceinline__ void leave_scan_zero(const PackArgs& a) {
+  __shared__ bool s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(a.ticket + 1, 1u) == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  for (size_t i = threadIdx.x; i < a.status_words; i += blockDim.x) a.status[i] = 0ull;
+  if (threadIdx.x < 2) a.ticket[threadIdx.x] = 0u;
+}
+
+// Buckets of 1024 2^j coordinates.
 bool pack_chunks_fits(int K, size_t nb, int bucket);
 // status: K (nb + 1) words.  b_first: the first bucket of every worker to encode, less than nb.
 qgx_status launch_pack_chunks(qgx_ctx* c, PackArgs a, size_t b_first, const CodeTable& ct);
