@@ -34,6 +34,9 @@ __device__ __forceinline__ float value_of(uint32_t sym, float norm, const float*
   return s < nlev ? val : -val;
 }
 
+// Workers whose symbols are asked for at a time: their CTAs' shared memory is a microsecond away, the kept symbols are in global
+// memory.  8 workers of 8192 coordinates compared (an affine step, two exchanges) 129.3 -> 123.2 us.
+constexpr int kAtOnce = 8;
 constexpr int kPadShift = 33;            // status words carry the words (low) and the unused bits (high) of the buckets so far
 
 // Q quads per thread; G coordinates per sub-block.
@@ -250,10 +253,8 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
     const int e = q * kQuad, nv = min(kQuad, len - e);
     const size_t sat = lo + (size_t)e;                                 // see DecodeArgs::sym_out
     float acc[kQuad] = {0.f, 0.f, 0.f, 0.f};
-    for (int kk = 0; kk < K; ++kk) {
-      const uint32_t word = *cluster.map_shared_rank(s_sym + q, kk);
+    auto add = [&](uint32_t word, uint32_t was, int kk) {
       const float nrm = s_norms[kk];
-      const uint32_t was = r.sym_prev ? *reinterpret_cast<const uint32_t*>(r.sym_prev + (size_t)kk * r.sym_ld + sat) : 0u;
 #pragma unroll
       for (int c = 0; c < kQuad; ++c) {
         const float val = value_of(word >> (8 * c), nrm, s_lev, lt.nlev);
@@ -266,7 +267,20 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
         }
       }
       if (r.sym_out) *reinterpret_cast<uint32_t*>(r.sym_out + (size_t)kk * r.sym_ld + sat) = word;
+    };
+    auto kept = [&](int kk) { return r.sym_prev ? *reinterpret_cast<const uint32_t*>(r.sym_prev + (size_t)kk * r.sym_ld + sat) : 0u; };
+    int kk = 0;
+    for (; kk + kAtOnce <= K; kk += kAtOnce) {                         // the symbols of several workers asked for at a time
+      uint32_t words[kAtOnce], was[kAtOnce];
+#pragma unroll
+      for (int u = 0; u < kAtOnce; ++u) {
+        words[u] = *cluster.map_shared_rank(s_sym + q, kk + u);
+        was[u] = kept(kk + u);
+      }
+#pragma unroll
+      for (int u = 0; u < kAtOnce; ++u) add(words[u], was[u], kk + u);
     }
+    for (; kk < K; ++kk) add(*cluster.map_shared_rank(s_sym + q, kk), kept(kk), kk);
 #pragma unroll
     for (int c = 0; c < kQuad; ++c) {
       if (c < nv) {
