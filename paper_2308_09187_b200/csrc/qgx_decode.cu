@@ -7,13 +7,14 @@
 // from global memory is asked for one turn (header words) or two (bucket lengths and offsets) ahead, its stream words are
 // copied while the turn before is added up.
 //
-// What bounds it: instructions and the shared-memory pipe (22 executed instructions per symbol at 60-75 % issue; 24 M
-// wavefronts per 2^27 symbols, 58 %).  The kernel before this one walked and added in the same thread, one look-up per symbol and
-// 64 sums in registers: 16 warps per SM (12 when comparing) that waited for one another's look-ups, 32 % issue.  A look-up of
-// two symbols halves the chain, and without the sums a thread has 64 registers, 32 warps per SM.  Per 2^27 symbols, 8 workers,
-// 17 fitted levels: kept symbols 281 -> 148 us, compared 359 -> 213.  Vectors with few sub-blocks had a walk that wrote every
-// value (4 bytes per symbol, in pieces of four bytes when the length was odd) and a kernel that added them: 16 workers of
-// 1000003 coordinates 120 -> 34 us.
+// What bounds it: instructions (20 per symbol, 22 with divergence: 9 walk, 7 add, 6 find the row) at 75 % issue, and the
+// shared-memory pipe, 64 % busy.  The kernel before this one walked and added in the same thread, one look-up per symbol and 64
+// sums in registers: 16 warps per SM (12 when comparing) that waited for one another's look-ups, 32 % issue.  A look-up of two
+// symbols halves the chain, and without the sums a thread has 64 registers, 32 warps per SM.  Per 2^31 symbols, 32 workers, 17
+// fitted levels: kept symbols 2533 -> 1865 us, compared 3344 -> 2327 (2848 with the kept symbols loaded where they are needed
+// instead of copied to shared memory during the walk).  Vectors with few sub-blocks had a walk that wrote every value (4 bytes
+// per symbol, in pieces of four bytes when the length was odd) and a kernel that added them: 16 workers of 1000003 coordinates
+// 120 -> 29 us.
 #include "qgx_decode.cuh"
 
 #include <algorithm>
@@ -48,7 +49,7 @@ struct DecodeShape {
   uint32_t units;                        // turns of `rows` rows
   uint32_t pair_mask;                    // of byte offsets into the pair table
   uint32_t row_words;                    // room for a warp's stream words, a multiple of 4
-  uint32_t off_val, off_kept, off_norm, off_norm_kept, off_sym, off_row;   // bytes of dynamic shared memory
+  uint32_t off_val, off_kept, off_norm, off_norm_kept, off_sym, off_kept_row, off_row;   // bytes of dynamic shared memory
 };
 
 struct SubBlockAt {
@@ -153,7 +154,7 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
   constexpr bool kStore = (SYM & 1) != 0, kCompare = (SYM & 2) != 0, kSquare = (SYM & 4) != 0;
   constexpr int kWords = G / 4, kStride = kWords + 1;                  // words of a sub-block, and from one to the next
   constexpr int kQuads = 8 * G;                                        // quads of a row
-  constexpr int kTurn = kCompare && G > 32 ? 4 : 8;                              // workers that a thread adds in one go
+  constexpr int kTurn = 8;                              // workers that a thread adds in one go
   constexpr int QT = G / 32;                                           // of them per thread of a team of eight warps
   extern __shared__ __align__(128) unsigned char s_raw[];
   const uint32_t sa = smem_addr(s_raw);
@@ -189,6 +190,8 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
   const uint32_t my_sym = sa + h.off_sym + (uint32_t)warp * sym_row_bytes<G>() + (uint32_t)lane * (uint32_t)(kStride * 4);
   const uint32_t team_sym = sa + h.off_sym + (uint32_t)(team * W) * sym_row_bytes<G>();
   const uint32_t row_sa = sa + h.off_row + (uint32_t)warp * h.row_words * 4u;
+  // comparing: the kept symbols of the worker and row that this warp walks, in coordinate order
+  const uint32_t kept_row = sa + h.off_kept_row + (uint32_t)warp * (32u * G), team_kept = sa + h.off_kept_row + (uint32_t)(team * W) * (32u * G);
   float* s_norm = reinterpret_cast<float*>(s_raw + h.off_norm) + 32 * (team * W);
   float* s_norm_kept = reinterpret_cast<float*>(s_raw + h.off_norm_kept) + 32 * (team * W);
   const int K = a.K;
@@ -244,6 +247,14 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncwarp();
     if (works(now)) {
+      if (kCompare) {                                                  // there when the walk is done
+        const size_t at0 = (size_t)row_at(now) * (32u * G);
+        const uint8_t* from = a.sym_prev + (size_t)(now.g * W + k_of) * a.sym_ld + at0;
+        const uint32_t pieces = (uint32_t)min((size_t)(32 * G), a.sym_ld - at0) / 16u;   // sym_ld is a multiple of 16
+        for (uint32_t c = (uint32_t)lane; c < pieces; c += 32u)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(kept_row + 16u * c), "l"(from + 16u * c) : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
       uint32_t used = 0;
       auto walk = [&](auto w, auto p) {
         w.open(p, at.sh);
@@ -261,6 +272,7 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
     if (works(next)) at = find_row<G>(a, h, row_at(next), next.g * W + k_of, next_bucket, next_header, lane, row_sa);
     asm volatile("cp.async.commit_group;" ::: "memory");
     next_bucket = later_bucket;
+    if (kCompare) asm volatile("cp.async.wait_group 1;" ::: "memory");   // the kept symbols; the next row's words may still be on their way
     team_sync();
 
     // the ordered sums of this turn's workers
@@ -311,22 +323,16 @@ k_exchange_decode(const __grid_constant__ DecodeArgs a, const __grid_constant__ 
 #pragma unroll 1
         for (int k0 = 0; k0 < nk; k0 += kTurn) {
           const uint32_t at_k0 = sym_at + (uint32_t)k0 * sym_row_bytes<G>();
-          const uint8_t* was_at = kCompare ? a.sym_prev + kept_at + (size_t)k0 * a.sym_ld : nullptr;
+          const uint32_t was_at = team_kept + (uint32_t)(r * K + k0) * (32u * G) + 4u * q;
           uint8_t* out = kStore ? a.sym_out + kept_at + (size_t)k0 * a.sym_ld : nullptr;
           auto turn = [&](auto whole_tag) {                            // of kTurn workers, or of what is left
             constexpr bool kWhole = decltype(whole_tag)::value;
-            uint32_t was[kTurn];
-#pragma unroll
-            for (int u = 0; u < kTurn; ++u) {
-              was[u] = 0u;
-              if (kCompare && (kWhole || k0 + u < nk)) was[u] = *reinterpret_cast<const uint32_t*>(was_at + (size_t)u * a.sym_ld) & valid;
-            }
 #pragma unroll
             for (int u = 0; u < kTurn; ++u) {
               if (!kWhole && k0 + u >= nk) break;
               uint32_t word = lds32(at_k0 + (uint32_t)u * sym_row_bytes<G>());
               if (kCompare || kSquare) word &= valid;
-              add(word, was[u], k0 + u);
+              add(word, kCompare ? lds32(was_at + (uint32_t)u * (32u * G)) & valid : 0u, k0 + u);
               if (kStore) *reinterpret_cast<uint32_t*>(out + (size_t)u * a.sym_ld) = word;
             }
           };
@@ -377,27 +383,39 @@ static qgx_status launch_decode_g(qgx_ctx* c, const DecodeArgs& da, const CodeTa
   DecodeShape h;
   h.minus_zero = kMinusZero2;
   if (!make_row_shape(da.d, da.bucket, G, da.nb, &h.row)) return QGX_ERR_INVALID_ARG;
-  // Shared memory: the pair table, small tables, then per warp the symbols of a row and room for its stream words: as many as
-  // any code can need, or what is left.
+  // A team has eight warps, or more where few rows have many workers.  As many teams as registers allow and shared memory holds:
+  // the pair table, small tables, then per warp the symbols of a row, comparing the kept ones, too, and room for its stream words
+  // -- for what the code's lengths make likely (and 15 % more), or as many as any code can need.  A row that does not fit is
+  // walked where it is, in global memory.
   const int max_warps = kDecodeWarps<G>;
   h.team_warps = 8;
   h.rows = std::max(1, h.team_warps / da.K);
   while (2 * h.team_warps <= max_warps && h.team_warps < da.K && (size_t)h.row.rows * 2 * (size_t)h.team_warps <= (size_t)c->num_sms * (size_t)max_warps) h.team_warps *= 2;
-  h.teams = max_warps / h.team_warps;
   h.groups = (da.K + h.team_warps - 1) / h.team_warps;
   h.units = (h.row.rows + (uint32_t)h.rows - 1u) / (uint32_t)h.rows;
-  const int warps = h.teams * h.team_warps;
   h.pair_mask = (4u << pair_bits(ct.maxlen)) - 4u;
-  uint32_t at = 4u << pair_bits(ct.maxlen);
-  auto take = [&](uint32_t bytes) { const uint32_t was = at; at += (bytes + 15u) & ~15u; return was; };
-  h.off_val = take(4u * kSignedValues);
-  h.off_kept = take(4u * kSignedValues);
-  h.off_norm = take((uint32_t)warps * 128u);
-  h.off_norm_kept = take((uint32_t)warps * 128u);
-  h.off_sym = take((uint32_t)warps * sym_row_bytes<G>());
-  h.off_row = at;
-  const uint32_t room = (224u * 1024u - at) / (uint32_t)(4 * warps) & ~3u;
-  h.row_words = std::min(row_words_worst(G, ct.maxlen), room);
+  double likely = 0.0;                                                 // bits of a symbol whose probability is what its length stands for
+  for (int j = 0; j < ct.nlev; ++j) likely += (double)(ct.len[j] + (j != 0)) / (double)(1u << ct.len[j]);
+  const uint32_t spb = h.row.spb, headers = spb % 32u == 0 ? 0u : (32u / spb + 2u) * (spb / 2u + 2u);
+  const uint32_t worst = row_words_worst(G, ct.maxlen);
+  const uint32_t wanted = std::min(worst, ((uint32_t)(1.15 * G * likely) + headers + WalkReach<G>::kWords + 8u) & ~3u);
+  constexpr uint32_t kRoom = 224u * 1024u;
+  uint32_t at = 0;
+  for (h.teams = max_warps / h.team_warps;; --h.teams) {
+    const uint32_t warps = (uint32_t)(h.teams * h.team_warps);
+    at = 4u << pair_bits(ct.maxlen);
+    auto take = [&](uint32_t bytes) { const uint32_t was = at; at += (bytes + 15u) & ~15u; return was; };
+    h.off_val = take(4u * kSignedValues);
+    h.off_kept = take(4u * kSignedValues);
+    h.off_norm = take(warps * 128u);
+    h.off_norm_kept = take(warps * 128u);
+    h.off_sym = take(warps * sym_row_bytes<G>());
+    h.off_kept_row = take((sym_mode & 2) ? warps * (32u * G) : 0u);
+    h.off_row = at;
+    if (h.teams == 1 || at + warps * wanted * 4u <= kRoom) break;
+  }
+  const int warps = h.teams * h.team_warps;
+  h.row_words = std::min(worst, (kRoom - at) / (uint32_t)(4 * warps) & ~3u);
   const size_t smem = at + (size_t)warps * h.row_words * 4u;
   const unsigned grid = (unsigned)std::min<size_t>((size_t)c->num_sms, h.units);
   ScopedKernelTimer timer(c, QGX_KERNEL_DECODE);
