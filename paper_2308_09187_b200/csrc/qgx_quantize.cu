@@ -120,6 +120,7 @@ k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ Level
     rc.thr = fast ? rt.thrfix : 0x10000u;
     uint8_t* out = a.sym + k * a.d + lo;
     const uint64_t q0 = (uint64_t)(lo >> 2);
+    const PhiloxShared ps = philox_shared((uint32_t)(q0 >> 32), ku, a.xid, key);
 #pragma unroll
     for (int j = 0; j < P; ++j) {
       const int o = (warp * P + j) * 32 + lane, e = 8 * o;
@@ -128,8 +129,8 @@ k_quantize(const __grid_constant__ QuantizeArgs a, const __grid_constant__ Level
       if (live) {
         const uint64_t ctr = q0 + 2ull * (uint64_t)o;
         uint32_t w[8];
-        if ((uint32_t)ctr != 0xffffffffu) {
-          philox_pair((uint32_t)ctr, philox_shared((uint32_t)(ctr >> 32), ku, a.xid, key), key, w);
+        if ((uint32_t)ctr != 0xffffffffu && (uint32_t)(ctr >> 32) == (uint32_t)(q0 >> 32)) {
+          philox_pair((uint32_t)ctr, ps, key, w);
         } else {
           uint4 wa, wb;
           philox4x32_10_x2(ctr, ctr + 1ull, ku, a.xid, key, &wa, &wb);
@@ -278,7 +279,10 @@ qgx_status launch_quantize(qgx_ctx* c, DualSource src, int K, size_t d, int buck
   // to 1024 coordinates side by side as they have warps for, unless that would leave SMs without any: the time of a few
   // buckets is that of one, whatever shares its SM.  (Buckets of 1024, where a table per bucket cost least, 8 x 10^6
   // coordinates: 27.1 us with a table each, 27.0 with two to a CTA.)
-  const int pp = bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4);
+  // Half the threads per bucket, twice the octets, where there are buckets enough to fill the SMs that way: more CTAs side by side
+  // hide one another's barriers.  8 x 2^22 coordinates: buckets of 2048 101 -> 77 us, 8192 81 -> 78, 4096 no gain.
+  const bool many = a.total >= 8 * (size_t)c->num_sms;
+  const int pp = bucket <= 1024 ? 1 : (bucket <= 2048 ? (many ? 2 : 1) : (bucket <= 4096 ? 2 : (bucket <= 8192 && !many ? 2 : 4)));
   a.team = bucket_threads(bucket, 2 * pp);
   a.teams = pp == 1 ? (int)std::max<size_t>(1, std::min<size_t>((size_t)(256 / a.team), a.total / (size_t)c->num_sms)) : 1;
   const int threads = pp == 1 ? 256 : a.team;
