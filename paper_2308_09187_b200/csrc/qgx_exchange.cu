@@ -494,7 +494,7 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
   if (!ct.has_header || bucket % ct.G != 0 || (ct.G != 32 && ct.G != 64 && ct.G != 128)) return QGX_ERR_INVALID_ARG;
   // small vectors: everything in one launch (the other ways are there when a caller asks for one of them)
   if (do_encode && c->skip_buckets < nb && c->encode_path == QGX_ENCODE_AUTO && c->decode_split == QGX_SPLIT_AUTO &&
-      small_exchange_fits(c, K, nb, bucket, ct, qt, ea.vec_ok && ea.quad_base % 2 == 0)) {
+      small_exchange_fits(c, K, nb, bucket, ct, qt, ea.vec_ok && ea.quad_base % 2 == 0, sym_mode != 0)) {
     const size_t had_words = c->ws_bytes[WS_SMALL];
     unsigned long long* words = (unsigned long long*)ws_get(c, WS_SMALL, sizeof(uint64_t) * ((size_t)K * nb + 2));
     if (!words) return QGX_ERR_CUDA;

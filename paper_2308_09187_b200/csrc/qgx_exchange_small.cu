@@ -39,8 +39,9 @@ __device__ __forceinline__ float value_of(uint32_t sym, float norm, const float*
 constexpr int kAtOnce = 8;
 constexpr int kPadShift = 33;            // status words carry the words (low) and the unused bits (high) of the buckets so far
 
-// Q quads per thread; G coordinates per sub-block.
-template <int Q, int G>
+// Q quads per thread; G coordinates per sub-block.  kSteps: an iteration's exchange, which keeps its symbols, compares with kept
+// ones or adds the squared values; without, the kernel has fewer registers and more of its CTAs share an SM.
+template <int Q, int G, bool kSteps>
 __global__ void __launch_bounds__(Q == 4 ? 1024 : 512)
 k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ SmallArgs r, const __grid_constant__ LevelTable lt,
                  const __grid_constant__ LevelTable lt_kept, const __grid_constant__ CodeTable ct, const __grid_constant__ PhiloxKey key,
@@ -71,7 +72,7 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
   if (blockDim.x == kWarp) s_lut.e[QGX_MAX_LEVELS + tid] = __ldg(a.tables->lut.e + QGX_MAX_LEVELS + tid);   // a bucket of 128 has one warp
   if (tid < QGX_MAX_LEVELS) {
     s_lev[tid] = tid < lt.nlev ? lt.lev[tid] : 1.0f;
-    s_lev_kept[tid] = tid < lt_kept.nlev ? lt_kept.lev[tid] : 0.0f;
+    if (kSteps) s_lev_kept[tid] = tid < lt_kept.nlev ? lt_kept.lev[tid] : 0.0f;
   }
   for (uint32_t i = (uint32_t)tid; i < r.img_words; i += blockDim.x) s_img[i] = 0u;
   await_previous();
@@ -243,7 +244,7 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
   // ---- ordered sums of this CTA's share of the quads, kept symbols, squared differences, state update ----
   if (tid < K) {
     s_norms[tid] = *cluster.map_shared_rank(&s_norm, tid);
-    s_norms_kept[tid] = r.norms_prev ? r.norms_prev[(size_t)tid * a.nb + b] : 0.0f;
+    if (kSteps) s_norms_kept[tid] = r.norms_prev ? r.norms_prev[(size_t)tid * a.nb + b] : 0.0f;
   }
   __syncthreads();
   const float Kf = (float)K, gam = r.update == 1 ? (float)r.scalars[1] : 1.0f;
@@ -259,26 +260,28 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
       for (int c = 0; c < kQuad; ++c) {
         const float val = value_of(word >> (8 * c), nrm, s_lev, lt.nlev);
         acc[c] = __fadd_rn(acc[c], val);
-        if (c < nv && r.sym_prev) {
+        if (kSteps && c < nv && r.sym_prev) {
           const float dlt = __fsub_rn(value_of(was >> (8 * c), s_norms_kept[kk], s_lev_kept, lt_kept.nlev), val);
           sq = fma((double)dlt, (double)dlt, sq);
-        } else if (c < nv && r.square) {
+        } else if (kSteps && c < nv && r.square) {
           sq = fma((double)val, (double)val, sq);
         }
       }
-      if (r.sym_out) *reinterpret_cast<uint32_t*>(r.sym_out + (size_t)kk * r.sym_ld + sat) = word;
+      if (kSteps && r.sym_out) *reinterpret_cast<uint32_t*>(r.sym_out + (size_t)kk * r.sym_ld + sat) = word;
     };
-    auto kept = [&](int kk) { return r.sym_prev ? *reinterpret_cast<const uint32_t*>(r.sym_prev + (size_t)kk * r.sym_ld + sat) : 0u; };
+    auto kept = [&](int kk) { return kSteps && r.sym_prev ? *reinterpret_cast<const uint32_t*>(r.sym_prev + (size_t)kk * r.sym_ld + sat) : 0u; };
     int kk = 0;
-    for (; kk + kAtOnce <= K; kk += kAtOnce) {                         // the symbols of several workers asked for at a time
-      uint32_t words[kAtOnce], was[kAtOnce];
+    if constexpr (kSteps) {
+      for (; kk + kAtOnce <= K; kk += kAtOnce) {                       // the symbols of several workers asked for at a time
+        uint32_t words[kAtOnce], was[kAtOnce];
 #pragma unroll
-      for (int u = 0; u < kAtOnce; ++u) {
-        words[u] = *cluster.map_shared_rank(s_sym + q, kk + u);
-        was[u] = kept(kk + u);
+        for (int u = 0; u < kAtOnce; ++u) {
+          words[u] = *cluster.map_shared_rank(s_sym + q, kk + u);
+          was[u] = kept(kk + u);
+        }
+#pragma unroll
+        for (int u = 0; u < kAtOnce; ++u) add(words[u], was[u], kk + u);
       }
-#pragma unroll
-      for (int u = 0; u < kAtOnce; ++u) add(words[u], was[u], kk + u);
     }
     for (; kk < K; ++kk) add(*cluster.map_shared_rank(s_sym + q, kk), kept(kk), kk);
 #pragma unroll
@@ -293,7 +296,7 @@ k_exchange_small(const __grid_constant__ EncodeArgs a, const __grid_constant__ S
       }
     }
   }
-  if (r.sym_prev || r.square) {
+  if (kSteps && (r.sym_prev || r.square)) {
     sq = warp_sum(sq);
     if (lane == 0 && sq != 0.0) atomicAdd(r.sum_sq, sq);
   }
@@ -322,7 +325,7 @@ struct SmallShape {
   uint32_t img_words, off_img, off_sym, off_tab;
   size_t smem;
 };
-static SmallShape small_shape(int bucket, const CodeTable& ct, const RoundTable& rt) {
+static SmallShape small_shape(int bucket, const CodeTable& ct, const RoundTable& rt, bool steps) {
   SmallShape s;
   const int Q = bucket <= 2048 ? 1 : (bucket <= 4096 ? 2 : 4);
   const size_t nbins = ((kKeyTop - kKeyBase) >> rt.key_shift) + 1;
@@ -333,8 +336,10 @@ static SmallShape small_shape(int bucket, const CodeTable& ct, const RoundTable&
   s.off_sym = (uint32_t)((s.off_img + s.img_words * 4u + 15u) & ~15u);
   s.off_tab = (uint32_t)((s.off_sym + (uint32_t)bucket + 15u) & ~15u);
   s.smem = s.off_tab + (sizeof(uint16_t) << (ct.maxlen + 1));
-#define QGX_SMALL_G(QQ) (ct.G == 32 ? (const void*)k_exchange_small<QQ, 32> : (ct.G == 64 ? (const void*)k_exchange_small<QQ, 64> : (const void*)k_exchange_small<QQ, 128>))
+#define QGX_SMALL_S(QQ, GG) (steps ? (const void*)k_exchange_small<QQ, GG, true> : (const void*)k_exchange_small<QQ, GG, false>)
+#define QGX_SMALL_G(QQ) (ct.G == 32 ? QGX_SMALL_S(QQ, 32) : (ct.G == 64 ? QGX_SMALL_S(QQ, 64) : QGX_SMALL_S(QQ, 128)))
   s.fn = Q == 1 ? QGX_SMALL_G(1) : (Q == 2 ? QGX_SMALL_G(2) : QGX_SMALL_G(4));
+#undef QGX_SMALL_S
 #undef QGX_SMALL_G
   return s;
 }
@@ -399,9 +404,9 @@ bool small_exchange_size(const qgx_ctx* c, int K, size_t nb, int bucket) {
 // against 53; 12 workers, 9 buckets of 16384, 9 uniform levels, 47 against 37); now 90 are, 1.40 times at most, and 15 lose
 // 8 to 13 %.  Where it holds, 9 uniform levels: 4 workers, 18 buckets of 1024, 13 : 28; 8 workers, 129 of 512, 21 : 33, 16 of
 // 4096, 21 : 27, and 27 of 8192, 25 : 34; 16 workers, 9 of 4096, 23 : 27.
-bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct, const RoundTable& rt, bool octets) {
+bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct, const RoundTable& rt, bool octets, bool steps) {
   if (!small_exchange_size(c, K, nb, bucket)) return false;
-  const SmallShape s = small_shape(bucket, ct, rt);
+  const SmallShape s = small_shape(bucket, ct, rt, steps);
   const SmallResidency r = small_residency(s, c->device, K);
   if (r.clusters < 1) return false;
   const double kilo = 1e-3 * bucket, buckets = (double)nb * K / c->all_sms;              // of an SM
@@ -415,7 +420,7 @@ bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const C
 
 qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, const LevelTable& lt, const LevelTable& lt_kept,
                                  const CodeTable& ct, const PhiloxKey& key, const RoundTable& rt, bool early) {
-  const SmallShape s = small_shape(ea.bucket, ct, rt);
+  const SmallShape s = small_shape(ea.bucket, ct, rt, r.sym_out || r.sym_prev || r.square);
   r.img_words = s.img_words; r.off_img = s.off_img; r.off_sym = s.off_sym; r.off_tab = s.off_tab;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];

@@ -27,7 +27,7 @@ struct SmallArgs {
 };
 
 bool small_exchange_size(const qgx_ctx* c, int K, size_t nb, int bucket);   // necessary, without the tables
-bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct, const RoundTable& rt, bool octets);
+bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct, const RoundTable& rt, bool octets, bool steps);
 // After small_exchange_fits.  ea.status [K][nb] and ea.ticket [2] are zero before the launch and again after it.
 qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, const LevelTable& lt, const LevelTable& lt_kept,
                                  const CodeTable& ct, const PhiloxKey& key, const RoundTable& rt, bool early);
