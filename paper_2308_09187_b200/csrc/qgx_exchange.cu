@@ -615,12 +615,13 @@ qgx_status exchange_impl(qgx_ctx* c, DualSource src, int K, size_t d, const qgx_
 //   50 of 2 * 10^4, 8 workers, bucket 1024:                     855 / 316 / 315 / 312 / 305
 //   10 of 500 to 2.4 * 10^5, 3 workers, bucket 4096:            194 / 81 / 76 / 75 / 75      (18263 coordinates per SM)
 //   24 of 2500, 4 workers, bucket 1024:                         348 / 157 / 156 / 158 / 158  (1621)
-// Below kSegSplitCoordsPerSm there is nothing to share out and each further stream costs two events.  kSegFixed of 0.3 and
-// 4 * 10^6 instead of 10^6: 669 and 693 for the first, 543 and 532 for the second, the others within 3 %.
+// (with the kernels of then: the decode pass has become faster since, the order has not changed).  Below kSegSplitCoordsPerSm there
+// is nothing to share out and each further stream costs two events.  kSegFixed of 0.5, 0.7 and 1 * 10^6 with the kernels as they
+// are: 631, 624 and 641 for the first, 482, 482 and 481 for the second at twice the size, the others within 1 %.
 constexpr int kSegStreams = 8;
 constexpr int kSegStreamsSmall = 4;
 constexpr double kSegSplitCoordsPerSm = 16384.0;        // workers * coordinates per SM
-constexpr double kSegFixed = 1e6;                       // the chain of a tensor's launches, in coordinates of the whole GPU
+constexpr double kSegFixed = 7e5;                       // the chain of a tensor's launches, in coordinates of the whole GPU
 struct SegChildren {
   qgx_ctx* ctx[kSegStreams];
   cudaEvent_t fork, join[kSegStreams];
