@@ -404,6 +404,13 @@ bool small_exchange_size(const qgx_ctx* c, int K, size_t nb, int bucket) {
 // against 53; 12 workers, 9 buckets of 16384, 9 uniform levels, 47 against 37); now 90 are, 1.40 times at most, and 15 lose
 // 8 to 13 %.  Where it holds, 9 uniform levels: 4 workers, 18 buckets of 1024, 13 : 28; 8 workers, 129 of 512, 21 : 33, 16 of
 // 4096, 21 : 27, and 27 of 8192, 25 : 34; 16 workers, 9 of 4096, 23 : 27.
+// That was with a decode pass of two kernels and memsets and copies between them.  The large kernels have become faster by more
+// than the one launch has, so that what passes this has to pass a second fit, to 3484 measurements of both ways as they are (10 %
+// and 12 % off): of the shapes that the first lets through, 817 were slower in one launch by more than 8 %, 2.2 times at most (16
+// workers, 180 buckets of 256, Elias' code, 47 us against 22; 12 workers, 84 of 1024, 29 against 17; 4 workers, 108 of 4096,
+// 29 against 19); now 349 are, 1.6 times at most.  Buckets from 4096 on whose clusters are all resident at once stay in one
+// launch -- 27 buckets of 8 x 8192 21.0 against 21.2, 6 of 12 x 16384 23 against 22, but 9 of 16 x 4096 22 against 15: the route of
+// those shapes is fixed, and it is one launch less for the host.
 bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const CodeTable& ct, const RoundTable& rt, bool octets, bool steps) {
   if (!small_exchange_size(c, K, nb, bucket)) return false;
   const SmallShape s = small_shape(bucket, ct, rt, steps);
@@ -415,7 +422,12 @@ bool small_exchange_fits(const qgx_ctx* c, int K, size_t nb, int bucket, const C
   const bool pipelined = bucket % kChunk == 0 && (bucket & (bucket - 1)) == 0;
   const bool whole = octets && bucket % (256 * (bucket <= 2048 ? 1 : (bucket <= 8192 ? 2 : 4))) == 0;   // else coordinate by coordinate
   const double other = 23.0 + 1.2 * ct.maxlen + 0.65 * buckets * kilo + (pipelined ? 0.03 * buckets : (whole ? 0.8 * buckets : 1.5 * buckets + 4.0));
-  return one <= other + 1.0;
+  if (one > other + 1.0) return false;
+  if (turns <= 1.0 && bucket >= 4096) return true;
+  const double one_now = 2.3 + turns * (7.35 + 0.1 * s.entries / s.threads + 0.55 * kilo + 0.12 * K) + buckets * (0.54 + 0.7 * kilo);
+  const double other_now = 15.5 + 0.23 * ct.maxlen + 0.73 * buckets * kilo - 0.23 * K +
+                           (pipelined ? -0.15 * buckets : (whole ? 0.49 * buckets - 2.8 : 1.46 * buckets));
+  return one_now <= other_now + 1.0;
 }
 
 qgx_status launch_exchange_small(qgx_ctx* c, const EncodeArgs& ea, SmallArgs r, const LevelTable& lt, const LevelTable& lt_kept,

@@ -1,0 +1,30 @@
+"""Exchanges that the large kernels have come to do faster than one launch; the same mean and bits either way."""
+import numpy as np
+import pytest
+import torch
+
+import qgx_inputs as gen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("K,nb,bucket,one_launch", [
+    (16, 180, 256, False), (12, 84, 1024, False), (4, 108, 4096, False), (8, 180, 512, False),   # several turns of clusters
+    (4, 18, 1024, True), (2, 40, 512, True), (12, 13, 512, True),
+])
+def test_second_fit(K, nb, bucket, one_launch):
+    import paper_2308_09187_b200 as qgx
+    v = gen.gaussian((K, nb * bucket - 4), seed=nb, device="cuda")
+    cfg = qgx.make_quant_cfg(np.linspace(0, 1, 9), bucket, qgx.qgx_build_codebook_elias(9, 32), 9)
+    ctx, large = qgx.qgx_create(0), qgx.qgx_create(0)
+    qgx.qgx_set_decode_split(large, qgx.QGX_SPLIT_NEVER)
+    want = qgx.qgx_exchange(large, v, cfg, 4)
+    qgx.qgx_exchange(ctx, v, cfg, 4)       # the tables are built
+    before = qgx.qgx_launch_count(ctx)
+    got = qgx.qgx_exchange(ctx, v, cfg, 4)
+    assert (qgx.qgx_launch_count(ctx) - before == 1) == one_launch
+    qgx.qgx_sync_status(ctx)
+    qgx.qgx_sync_status(large)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    qgx.qgx_destroy(ctx)
+    qgx.qgx_destroy(large)
